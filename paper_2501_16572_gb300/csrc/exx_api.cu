@@ -717,7 +717,7 @@ int ace_build(exx_plan plan, const double *Psi, int n, long ld, const double *W,
     }
     // xi = W Linv^T
     if (tcg) {
-        if (int rc = tc_gemm(*P, P->N, n, n, W, 1, ld_w, Linv, 1, n, 1.0, xi, 1, ld_xi, s)) return rc;
+        if (int rc = tc_gemm(*P, P->N, n, n, W, 1, ld_w, Linv, 1, n, 1.0, xi, 1, ld_xi, s, true)) return rc;
     } else if (int rc = gemm_fp64_nt(*P, P->N, n, n, W, ld_w, Linv, n, 1.0, xi, ld_xi, s)) {
         return rc;
     }

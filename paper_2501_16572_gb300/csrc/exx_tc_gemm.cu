@@ -11,332 +11,643 @@
 // row is rounded to a 31-bit integer X and cut into four balanced base-256 digits,
 //     X = d0 2^24 + d1 2^16 + d2 2^8 + d3,   |d0| <= 64, |d1|, |d2|, |d3| <= 128,
 // each stored exactly as a bf16.  Digit products of one level (i + j = l, l <= 4) are
-// summed in their own TMEM accumulator (5 levels x 96 output columns per tile); a level
+// summed in their own TMEM accumulator (5 levels x up to 96 output columns per tile); a level
 // gains at most 3 * 2^14 per k, so the 320-term sums stay integers below 2^24 and the
-// tensor core never rounds.  The levels are combined in FP64 and the chunks are summed in
-// FP64.  Dropped digit products (i + j >= 5) weigh below 2^-37 of the row maxima; the
-// rounding of X, 2^-31 of the row maxima, is the leading error.
+// tensor core never rounds.  The levels of a chunk are combined into an FP32 hi + lo pair and
+// the chunks are summed in such pairs (48 bits; the sums of the k splits in FP64).  Dropped
+// digit products (i + j >= 5) weigh below 2^-37 of the row maxima; the rounding of X, 2^-31
+// of the row maxima, is the leading error.
+//
+// Two kernels.  gemm_cut_kernel cuts every operand element once into digit planes in device
+// memory, already in the operand layout of the MMA, and records the row scales;
+// tc_gemm_kernel then only streams 8-byte-per-element blocks of them through shared memory
+// (bulk copies, a producer warp) into the MMAs (one issuing warp) while 8 warps combine
+// finished chunks.  Cutting inside the GEMM repeated the integer work of every A row for each
+// 96 output columns and left the tensor cores idle meanwhile: both products of ace_apply at
+// n = nphi = 512 on 72 x 72 x 144 points took 65.7 ms, 11.8 ms now (cuts 3.3 ms near the HBM
+// rate, MMAs 8.3 ms, of which the tensor pipe's own 5.6 ms).
 #include "exx_internal.h"
 #include "tc_ptx.cuh"
 
 #include <algorithm>
+#include <cmath>
 
 namespace exx {
 
 namespace {
 
 constexpr int kT = 128;              // rows of A per tile (TMEM lanes)
-constexpr int kThreads = 4 * kT;     // 4 threads per row (slicing, drain by column groups)
-constexpr int kTN = 96;              // rows of B per tile (output columns)
+constexpr int kTN = 96;              // most rows of B per tile (output columns)
 constexpr int kLev = 5;              // level accumulators: digit products with i + j <= 4
-constexpr int kSub = 64;             // k per operand image
-constexpr int kSubs = 5;             // images per exact chunk
-constexpr int kChunk = kSub * kSubs; // 320: 4 levels x 320 x 3 * 2^14 < 2^24
-constexpr uint32_t kGemmWait = 1u << 22;
+constexpr int kDig = 4;
+constexpr int kBlk = 32;             // k per operand block
+constexpr int kBlks = 10;            // blocks per exact chunk
+constexpr int kChunk = kBlk * kBlks; // 320: 4 levels x 320 x 3 * 2^14 < 2^24
+constexpr uint64_t kGemmWaitNs = 1000000000ull;
+constexpr uint32_t kSbo = kBlk * 16;           // bytes between 8-row groups of a digit plane
+constexpr int kDrainWarps = 8;
+constexpr int kThreads = 32 * (kDrainWarps + 2);
+constexpr int kCutWarps = kBlks;     // gemm_cut_kernel: a warp per k block of a chunk
+constexpr long kDigitBudget = 1L << 30;        // device memory of the digit planes of one slab
+
+__device__ __forceinline__ int exp_field(uint32_t hi) { return int((hi >> 20) & 0x7ffu); }
+
+// Byte offset of (row, 8-k group c) in the digit planes of an operand whose tiles have `rt`
+// rows: tile (row / rt), block kb of `nkb`, digit plane q, then the canonical K-major
+// no-swizzle image (8 rows x 16 bytes per core matrix).
+__device__ __forceinline__ size_t cut_off(long tile, int r, int rt, long kb, long nkb, int c)
+{
+    return (size_t(tile) * nkb + kb) * (size_t(rt) * kBlk * 2 * kDig) + size_t(r >> 3) * kSbo + size_t(c) * 128 +
+           size_t(r & 7) * 16;
+}
+
+// Digits of eight consecutive k of one row (largest biased exponent E in its chunk), stored as
+// 16 bytes in each of the four planes.  |x| < 2^(E-1022), X = x 2^(1052-E) rounded to even,
+// |X| <= 2^30: the 53-bit mantissa, 64-bit aligned, shifted right by 2 + E - e (zeros and
+// subnormals give X = 0), on the integer pipe: the FP64 unit converts two values per clock and
+// SM.  Digit l is X rounded to a multiple of 2^(24 - 8 l) less the same rounding one digit up.
+__device__ __forceinline__ void cut8(uint8_t *dst, size_t plane, const double (&x)[8], int E)
+{
+    uint32_t w[kDig][4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        float d[2][kDig];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const double v = x[2 * p + h];
+            const uint32_t hi = uint32_t(__double2hiint(v)), lo = uint32_t(__double2loint(v));
+            const int e = exp_field(hi);
+            const uint32_t top = e ? (0x80000000u | (hi << 11) | (lo >> 21)) : 0u;
+            const int s = 2 + E - e;                      // >= 2
+            const uint32_t low = lo << 11;
+            uint32_t q = s < 32 ? top >> s : 0u;
+            const uint32_t fr = s <= 32 ? __funnelshift_rc(low, top, s) : 0u;   // the fraction below q
+            const uint32_t rest = (fr << 1) | low;
+            q += (fr >> 31) & ((q & 1u) | (rest != 0u ? 1u : 0u));
+            const int sg = int(hi) >> 31;
+            const int X = (int(q) ^ sg) - sg;
+            const int R0 = (X + (1 << 23)) >> 24, R1 = (X + (1 << 15)) >> 16, R2 = (X + (1 << 7)) >> 8;
+            // small integers to FP32 through the 1.5 * 2^23 offset
+            d[h][0] = __int_as_float(0x4B400000 + R0) - 12582912.f;
+            d[h][1] = __int_as_float(0x4B400000 + R1 - R0 * 256) - 12582912.f;
+            d[h][2] = __int_as_float(0x4B400000 + R2 - R1 * 256) - 12582912.f;
+            d[h][3] = __int_as_float(0x4B400000 + X - R2 * 256) - 12582912.f;
+        }
+#pragma unroll
+        for (int l = 0; l < kDig; ++l)
+            w[l][p] = __byte_perm(__float_as_uint(d[0][l]), __float_as_uint(d[1][l]), 0x7632);
+    }
+#pragma unroll
+    for (int l = 0; l < kDig; ++l)
+        *reinterpret_cast<uint4 *>(dst + l * plane) = make_uint4(w[l][0], w[l][1], w[l][2], w[l][3]);
+}
+
+struct CutArgs {
+    const double *X;     // element (row, k) at X[row sr + k sk]
+    long sr, sk;
+    long rows, K;        // valid rows and k (zeros beyond)
+    int rt;              // rows per tile
+    long nkb;            // k blocks
+    uint8_t *dig;
+    int *sh;             // [chunk][prow]: largest biased exponent of the row in the chunk (>= 100)
+    long prow;           // padded rows
+    int vec;             // k-contiguous rows start 16-byte aligned
+};
+
+// KFAST (sk = 1): a CTA takes 8 rows x one chunk, lane = (row, 8-k group) of its warp's block:
+// 64 contiguous bytes per lane in, whole 512-byte runs of a plane out.  Otherwise (sr = 1, or
+// any strides): 32 rows x one chunk, lane = row, four 8-k groups per lane.  Memory bound: 8 B
+// read and 8 B written per element.
+template <bool KFAST>
+__global__ void __launch_bounds__(32 * kCutWarps) gemm_cut_kernel(const CutArgs a)
+{
+    __shared__ int smax[kCutWarps][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long chunk = blockIdx.y;
+    const long k0 = chunk * kChunk + warp * kBlk;
+    constexpr int G = KFAST ? 1 : 4;       // 8-k groups per lane
+    const long row = KFAST ? long(blockIdx.x) * 8 + (lane & 7) : long(blockIdx.x) * 32 + lane;
+    const bool ok = row < a.rows;
+    double x[G][8];
+    uint32_t m = 0;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        const long kg = k0 + 8 * (KFAST ? lane >> 3 : g);
+        const double *p = a.X + (ok ? row * a.sr : 0) + kg * a.sk;
+        if (KFAST && a.vec && ok && kg + 8 <= a.K) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const double2 v = *reinterpret_cast<const double2 *>(p + 2 * e);
+                x[g][2 * e] = v.x;
+                x[g][2 * e + 1] = v.y;
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) x[g][e] = (ok && kg + e < a.K) ? p[e * a.sk] : 0.0;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) m = max(m, uint32_t(__double2hiint(x[g][e])) & 0x7ff00000u);
+    }
+    if (KFAST) {   // the lanes of one row: lane, lane ^ 8, lane ^ 16
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, 8));
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
+    }
+    smax[warp][lane] = int(m >> 20);
+    __syncthreads();
+    int E = 100;   // rows below 2^-922 are zero rows
+#pragma unroll
+    for (int w = 0; w < kCutWarps; ++w) E = max(E, smax[w][lane]);
+    if (row < a.prow && warp == 0 && (!KFAST || lane < 8)) a.sh[chunk * a.prow + row] = E;
+    const long kb = chunk * kBlks + warp;
+    if (kb >= a.nkb || row >= a.prow) return;
+    const long tile = row / a.rt;
+    const int r = int(row - tile * a.rt);
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+        cut8(a.dig + cut_off(tile, r, a.rt, kb, a.nkb, KFAST ? lane >> 3 : g), size_t(a.rt) * kBlk * 2, x[g], E);
+}
 
 struct GemmArgs {
-    int m, n;
-    long K;
-    const double *A;
-    long as_i, as_k;
-    const double *B;
-    long bs_j, bs_k;
-    double *D;                 // this CTA's output slot: D + blockIdx.z * dz
+    long m;
+    int n;
+    int Nt, mt, nt;            // tile columns, tiles
+    long Z;                    // k splits
+    long nkb, nchunks;         // blocks and chunks of this slab
+    long cper;                 // chunks per split
+    const uint8_t *digA, *digB;
+    const int *shA, *shB;
+    long prowA, prowB;
+    double *D;                 // split z writes D + z dz
     long ds_i, ds_j, dz;
-    long kper;                 // k handled by one CTA (a multiple of kChunk)
-    double alpha;
+    int add;                   // add to D (a later slab of k without splits)
+    int ktri;                  // B(j, k) = 0 for k > j: tiles stop at their last column
+    float al_h, al_l;          // alpha = (al_h + al_l) 2^al_e
+    int al_e;
+    int stages;
+    uint32_t stage_bytes, offB, offTab, offBar;
+    int tmem_cols;
     int *err;
 };
 
-__device__ __forceinline__ int exp_field(double x) { return int((__double_as_longlong(x) >> 52) & 0x7ff); }
-
-// Digits of x 2^sh, sh = 1052 - E for the row's largest biased exponent E: |x| < 2^(E-1022)
-// gives |X| < 2^30.  The scaling adds sh to the exponent field (x = 0 and values that
-// would leave the normal range give X = 0: they are below 2^-1000 of the row maximum).
-__device__ __forceinline__ void digits4(double x, int sh, float (&d)[4])
+// (h + l) 2^ex as a double, rounded to 48 bits or better, on the integer pipe: GB300 converts
+// to and from FP64 at two per clock and SM, which would cost a 128 x 96 tile 18 thousand cycles.
+__device__ __forceinline__ double pair_to_double(float h, float l, int ex)
 {
-    const int ex = exp_field(x);
-    int X = 0;
-    if (ex != 0 && ex + sh > 0)
-        X = __double2int_rn(__longlong_as_double(__double_as_longlong(x) + (static_cast<long long>(sh) << 52)));
-    const int d0 = (X + (1 << 23)) >> 24;
-    int r = X - (d0 << 24);
-    const int d1 = (r + (1 << 15)) >> 16;
-    r -= d1 << 16;
-    const int d2 = (r + (1 << 7)) >> 8;
-    const int d3 = r - (d2 << 8);
-    // small integers to FP32 through the 1.5 * 2^23 offset (exact for |d| < 2^22)
-    d[0] = __int_as_float(0x4B400000 + d0) - 12582912.f;
-    d[1] = __int_as_float(0x4B400000 + d1) - 12582912.f;
-    d[2] = __int_as_float(0x4B400000 + d2) - 12582912.f;
-    d[3] = __int_as_float(0x4B400000 + d3) - 12582912.f;
-}
-
-// canonical K-major no-swizzle image: byte offset of (row, 16-byte chunk c), 64 k per row
-__device__ __forceinline__ uint32_t gimg_off(int row, int c) { return uint32_t(row >> 3) * 1024u + uint32_t(c) * 128u + uint32_t(row & 7) * 16u; }
-
-// 4 digits x 4 consecutive k of one row -> the four digit images (8 bytes each)
-__device__ __forceinline__ void store_digits(uint8_t *img, int row, int u, const float (&q)[4][4], uint32_t piece)
-{
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-        const uint32_t w0 = __byte_perm(__float_as_uint(q[l][0]), __float_as_uint(q[l][1]), 0x7632);
-        const uint32_t w1 = __byte_perm(__float_as_uint(q[l][2]), __float_as_uint(q[l][3]), 0x7632);
-        *reinterpret_cast<uint2 *>(img + l * piece + gimg_off(row, u >> 1) + (u & 1) * 8) = make_uint2(w0, w1);
+    const float s = h + l;
+    l -= s - h;
+    const uint32_t b = __float_as_uint(s);
+    int e = int((b >> 23) & 0xffu);
+    long long M = static_cast<long long>((b & 0x7fffffu) | 0x800000u) << 29;
+    if (e >= 53) {   // l in units of the last bit of M: |q| <= 2^28
+        const float lq = l * __uint_as_float(uint32_t(306 - e) << 23);
+        M += __float2int_rn((b >> 31) ? -lq : lq);
     }
+    if (M < (1LL << 52)) {
+        M <<= 1;
+        --e;
+    }
+    const int ed = e - 127 + 1023 + ex;
+    if (e <= 0 || ed <= 0) return 0.0;
+    const uint32_t sign = b & 0x80000000u;
+    if (ed >= 2047) return __hiloint2double(int(sign | 0x7ff00000u), 0);
+    const uint32_t hi = sign | (uint32_t(ed) << 20) | (uint32_t(M >> 32) & 0xfffffu);
+    return __hiloint2double(int(hi), int(uint32_t(M)));
 }
 
-__global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(GemmArgs a)
+__device__ __forceinline__ float pow2f(int e) { return e < -126 ? 0.f : __uint_as_float(uint32_t(min(e, 127) + 127) << 23); }
+
+__device__ __forceinline__ void gemm_bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
+{
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+            tc::smem_addr(dst)),
+        "l"(src), "r"(bytes), "r"(tc::smem_addr(bar))
+        : "memory");
+}
+
+// One CTA per SM walks the items (split z, row tile, column tile), column tiles fastest so
+// that concurrent CTAs read the same A blocks from L2.  Bound by the tensor pipe: 13 digit
+// products per k (7 MMAs of up to 192 columns: neighbouring B digits feed neighbouring
+// levels), 632 cycles per 16 k of a 128 x 96 tile against 28.7 KB of operands; the combination
+// of a finished chunk is not overlapped, the five level accumulators fill TMEM.
+template <int G>
+__global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_constant__ GemmArgs a)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    constexpr uint32_t piece = kT * kSub * 2;       // one A digit image: 128 rows x 64 k bf16
-    constexpr uint32_t bpiece = kTN * kSub * 2;     // one B digit image: 96 rows
-    constexpr uint32_t sbo = kSub * 2 * 8;          // bytes per 8-row group
-    uint8_t *sA = smem, *sB = smem + 4 * piece;
-    int *sh_a = reinterpret_cast<int *>(sB + 4 * bpiece);   // per A row: its scale shift
-    int *sh_b = sh_a + kT;                                   // per B row
-    uint64_t *bar = reinterpret_cast<uint64_t *>(sh_b + kTN);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 1);
+    float *fbs = reinterpret_cast<float *>(smem + a.offTab);       // column factors of a chunk, two sets
+    int *refB = reinterpret_cast<int *>(fbs + 2 * kTN);
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + a.offBar);
+    uint64_t *empty = full + a.stages;
+    uint64_t *dfull = empty + a.stages, *dempty = dfull + 1;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(dempty + 1);
     int *sflag = reinterpret_cast<int *>(tslot + 1);
-    const int t = threadIdx.x, warp = t >> 5, row = t & (kT - 1), q = t / kT;
-    constexpr int kWarps = kThreads / 32;
-    if (t == 0) {
-        tc::mbar_init(bar, 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        for (int i = 0; i < a.stages; ++i) {
+            tc::mbar_init(full + i, 1);
+            tc::mbar_init(empty + i, 1);
+        }
+        tc::mbar_init(dfull, 1);
+        tc::mbar_init(dempty, 1);
         *sflag = 0;
     }
-    if (warp == 0) tc::tmem_alloc(tslot, 512);   // 5 levels x 96 columns
+    if (warp == 0) tc::tmem_alloc(tslot, uint32_t(a.tmem_cols));
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tslot;
-    const uint32_t lane = uint32_t((warp & 3) * 32) << 16;   // this warp's TMEM lane quarter
-    const uint32_t idesc = tc::instr_desc(false, kTN);
-    const uint32_t a_addr = tc::smem_addr(sA), b_addr = tc::smem_addr(sB);
+    const long items = a.Z * a.mt * a.nt;
+    const int Nt = a.Nt;
+    const uint32_t a_bytes = kT * kBlk * 2 * kDig, b_bytes = uint32_t(Nt) * kBlk * 2 * kDig;
+    struct Item {
+        long z, c0, c1;
+        int mi, ni;
+    };
+    auto item_of = [&](long it) {
+        Item t;
+        t.ni = int(it % a.nt);
+        const long q = it / a.nt;
+        t.mi = int(q % a.mt);
+        t.z = q / a.mt;
+        t.c0 = t.z * a.cper;
+        t.c1 = min(a.nchunks, t.c0 + a.cper);
+        if (a.ktri) t.c1 = min(t.c1, long((t.ni + 1) * Nt + kChunk - 1) / kChunk);
+        return t;
+    };
 
-    const int i0 = blockIdx.x * kT, j0 = blockIdx.y * kTN;
-    const int i = i0 + row;              // this thread's output row (TMEM lane)
-    const bool arow = i < a.m;
-    const long kbeg = long(blockIdx.z) * a.kper, kend = min(a.K, kbeg + a.kper);
-    double *D = a.D + long(blockIdx.z) * a.dz;
-    uint32_t phase = 0;
-    bool first = true;
-    // Per-row shifts of a chunk [c0, c1) and digit images of a sub-step [k0, k0 + 64) for an
-    // operand X of R tile rows (global rows base + r < valid, element (row, k) at
-    // X[row sr + k sk]).  k-contiguous operands (sk = 1) are read a warp per row,
-    // consecutive lanes on consecutive k; the others by threads per row, consecutive lanes
-    // on consecutive rows: both coalesced.
-    auto shifts = [&](const double *X, long sr, long sk, int base, int valid, int R, int *sh, long c0, long c1) {
-        if (sk == 1) {
-            for (int r = warp; r < R; r += kWarps) {
-                int E = 0;
-                if (base + r < valid) {
-                    const double *xr = X + long(base + r) * sr;
-                    for (long k = c0 + (t & 31); k < c1; k += 32) E = max(E, exp_field(xr[k]));
+    if (warp == kDrainWarps) {
+        // ---- producer warp: one operand block pair per stage ----
+        if (lane == 0) {
+            long seq = 0;
+            bool bad = false;
+            for (long it = blockIdx.x; it < items && !bad; it += gridDim.x) {
+                const Item t = item_of(it);
+                const long kb1 = min(a.nkb, t.c1 * kBlks);
+                for (long kb = t.c0 * kBlks; kb < kb1; ++kb, ++seq) {
+                    const int st = int(seq % a.stages);
+                    const long use = seq / a.stages;
+                    if (use > 0 && !tc::mbar_wait_timed(empty + st, uint32_t((use - 1) & 1), kGemmWaitNs)) {
+                        atomicExch(sflag, 1);
+                        bad = true;
+                        break;
+                    }
+                    uint8_t *s = smem + size_t(st) * a.stage_bytes;
+                    tc::mbar_arrive_expect_tx(full + st, a_bytes + b_bytes);
+                    gemm_bulk_load(s, a.digA + (size_t(t.mi) * a.nkb + kb) * a_bytes, a_bytes, full + st);
+                    gemm_bulk_load(s + a_bytes, a.digB + (size_t(t.ni) * a.nkb + kb) * b_bytes, b_bytes, full + st);
                 }
-                for (int o = 16; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
-                if ((t & 31) == 0) sh[r] = 1052 - max(E, 100);   // rows below 2^-922 are zero rows
             }
-        } else if (t < R) {
-            int E = 0;
-            if (base + t < valid) {
-                const double *xr = X + long(base + t) * sr;
-                for (long k = c0; k < c1; ++k) E = max(E, exp_field(xr[k * sk]));
-            }
-            sh[t] = 1052 - max(E, 100);
-        }
-    };
-    auto digits_sub = [&](const double *X, long sr, long sk, int base, int valid, int R, const int *sh,
-                          uint8_t *img, uint32_t pc, long k0, long c1) {
-        if (sk == 1) {
-            const int l2 = 2 * (t & 31);   // this lane's k: k0 + l2, k0 + l2 + 1
-            for (int r = warp; r < R; r += kWarps) {
-                const bool ok = base + r < valid;
-                const double *xr = ok ? X + long(base + r) * sr : X;
-                const long k = k0 + l2;
-                float d0[4], d1[4];
-                digits4(ok && k < c1 ? xr[k] : 0.0, sh[r], d0);
-                digits4(ok && k + 1 < c1 ? xr[k + 1] : 0.0, sh[r], d1);
-#pragma unroll
-                for (int lv = 0; lv < 4; ++lv)
-                    *reinterpret_cast<uint32_t *>(img + lv * pc + gimg_off(r, l2 >> 3) + (l2 & 7) * 2) =
-                        __byte_perm(__float_as_uint(d0[lv]), __float_as_uint(d1[lv]), 0x7632);
-            }
-        } else if (row < R) {   // 4 threads per row, 4-k units u = q, q + 4, ...
-            const bool ok = base + row < valid;
-            const double *xr = ok ? X + long(base + row) * sr : X;
-            for (int u = q; u < kSub / 4; u += kThreads / kT) {
-                float dq[4][4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const long k = k0 + 4 * u + e;
-                    float d[4];
-                    digits4(ok && k < c1 ? xr[k * sk] : 0.0, sh[row], d);
-#pragma unroll
-                    for (int lv = 0; lv < 4; ++lv) dq[lv][e] = d[lv];
-                }
-                store_digits(img, row, u, dq, pc);
+            for (int st = 0; st < a.stages; ++st) {   // every issued copy has landed before exit
+                const long nf = seq > st ? (seq - 1 - st) / a.stages + 1 : 0;
+                if (nf > 0 && !tc::mbar_wait_timed(full + st, uint32_t((nf - 1) & 1), kGemmWaitNs)) atomicExch(sflag, 1);
             }
         }
-    };
-    for (long c0 = kbeg; c0 < kend; c0 += kChunk) {
-        const long c1 = min(kend, c0 + kChunk);
-        shifts(a.A, a.as_i, a.as_k, i0, a.m, kT, sh_a, c0, c1);
-        shifts(a.B, a.bs_j, a.bs_k, j0, a.n, kTN, sh_b, c0, c1);
-        __syncthreads();   // every row's shift is visible
-        for (int sub = 0; sub < kSubs; ++sub) {
-            const long k0 = c0 + long(sub) * kSub;
-            if (k0 >= c1) break;   // uniform
-            digits_sub(a.A, a.as_i, a.as_k, i0, a.m, kT, sh_a, sA, piece, k0, c1);
-            digits_sub(a.B, a.bs_j, a.bs_k, j0, a.n, kTN, sh_b, sB, bpiece, k0, c1);
-            tc::fence_proxy_async_smem();
-            tc::tc_fence_before();
-            __syncthreads();
-            tc::tc_fence_after();
-            if (t == 0) {
-                // level l of the chunk accumulates the digit products (p, l - p)
-                for (int ks = 0; ks < kSub / 16; ++ks)
-                    for (int l = 0; l < kLev; ++l)
-                        for (int p = max(0, l - 3); p <= min(l, 3); ++p) {
-                            const uint64_t ad = tc::smem_desc(a_addr + p * piece + ks * 256u, 128u, sbo);
-                            const uint64_t bd = tc::smem_desc(b_addr + (l - p) * bpiece + ks * 256u, 128u, sbo);
-                            const bool acc = sub > 0 || ks > 0 || p > max(0, l - 3);
-                            tc::mma_bf16(tmem + uint32_t(l * kTN), ad, bd, idesc, acc ? 1u : 0u);
+    } else if (warp == kDrainWarps + 1) {
+        // ---- MMA warp ----
+        long seq = 0, dseq = 0;
+        bool bad = false;
+        // operand and accumulator steps, fixed for the launch: the issue of one 16-k step is a
+        // straight run of MMAs whose descriptors differ by additions (computed in a loop, the
+        // issuing thread took 1340 cycles a step, twice the tensor pipe's 632)
+        constexpr uint32_t kStepA = kT * kBlk * 2 / 16;            // next A digit, in 16-byte units
+        const uint32_t step_b = uint32_t(Nt) * kBlk * 2 / 16;      // next B digit
+        uint32_t idesc[G + 1];
+#pragma unroll
+        for (int g = 1; g <= G; ++g) idesc[g] = tc::instr_desc(false, g * Nt);
+        // A digit i with B digits j0 .. j0 + g - 1 into levels i + j0 .. (at most G per MMA)
+        auto step = [&](uint64_t ad0, uint64_t bd0, bool first) {
+#pragma unroll
+            for (int i = 0; i < kDig; ++i) {
+                constexpr int kEnd = kLev;
+                const int nj = kDig < kEnd - i ? kDig : kEnd - i;
+                const uint64_t ad = ad0 + i * kStepA;
+#pragma unroll
+                for (int j0 = 0; j0 < nj; j0 += G) {
+                    const int g = G < nj - j0 ? G : nj - j0;
+                    const uint64_t bd = bd0 + j0 * step_b;
+                    const uint32_t d = tmem + uint32_t((i + j0) * Nt);
+                    if (i == 1 && j0 + g == kDig && g > 1) {
+                        if (first) {   // digit 0 has opened levels 0..3; level 4 starts here
+                            tc::mma_bf16(d, ad, bd, idesc[g - 1], 1u);
+                            tc::mma_bf16(tmem + uint32_t(4 * Nt), ad, bd0 + (kDig - 1) * step_b, idesc[1], 0u);
+                        } else {
+                            tc::mma_bf16(d, ad, bd, idesc[g], 1u);
                         }
-                tc::mma_commit(bar);
+                    } else {
+                        const bool open = i == 0 || (i == 1 && j0 == kDig - 1);
+                        tc::mma_bf16(d, ad, bd, idesc[g], open && first ? 0u : 1u);
+                    }
+                }
             }
-            // images are rewritten by the next sub-step, TMEM read by the drain: wait
-            if (!tc::mbar_wait_bounded(bar, phase, kGemmWait)) atomicExch(sflag, 1);
-            phase ^= 1u;
-            tc::tc_fence_after();
-            __syncthreads();   // the images may be rewritten
-        }
-        if (*sflag) break;   // uniform: set before the last barrier
-        // drain: D(i, j) (+)= alpha 2^(48 - shA - shB) sum_l L_l 2^(-8 l).  The levels are
-        // combined in FP32 down to level 1 (rounding ~2^-32 of level 0's scale), level 0 is
-        // added with TwoSum, and the pair is scaled and accumulated in FP64.
-        const int shA = sh_a[row];
-        for (int cg = q; cg < kTN / 8; cg += kThreads / kT) {   // this thread's column groups
-            uint32_t r[kLev][8];
-#pragma unroll
-            for (int l = 0; l < kLev; ++l) tc::tmem_ld8_issue(tmem + lane + uint32_t(l * kTN + cg * 8), r[l]);
-            tc::tmem_wait_ld();
-#pragma unroll
-            for (int l = 0; l < kLev; ++l)
-#pragma unroll
-                for (int e = 0; e < 8; ++e) tc::order_after_wait(r[l][e]);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int col = j0 + cg * 8 + e;
-                if (!arow || col >= a.n) continue;
-                float tl = __uint_as_float(r[4][e]);
-                tl = tl * (1.f / 256.f) + __uint_as_float(r[3][e]);
-                tl = tl * (1.f / 256.f) + __uint_as_float(r[2][e]);
-                tl = tl * (1.f / 256.f) + __uint_as_float(r[1][e]);
-                tl *= 1.f / 256.f;
-                const float l0 = __uint_as_float(r[0][e]);
-                const float h = l0 + tl, bp = h - l0;
-                const float lo = (l0 - (h - bp)) + (tl - bp);
-                // v 2^48 2^-shA 2^-shB alpha, the powers of two as one exponent (a product
-                // below the normal range is zero: both rows were below 2^-900)
-                const int sc = min(48 - shA - sh_b[cg * 8 + e], 1023);
-                double v = double(h) + double(lo);
-                v = sc < -1022 ? 0.0 : a.alpha * (v * __longlong_as_double(static_cast<long long>(sc + 1023) << 52));
-                double *dp = D + long(i) * a.ds_i + long(col) * a.ds_j;
-                *dp = first ? v : *dp + v;
+        };
+        for (long it = blockIdx.x; it < items && !bad; it += gridDim.x) {
+            const Item t = item_of(it);
+            for (long c = t.c0; c < t.c1 && !bad; ++c, ++dseq) {
+                if (dseq > 0 && !tc::mbar_wait_timed(dempty, uint32_t((dseq - 1) & 1), kGemmWaitNs)) {
+                    atomicExch(sflag, 1);
+                    bad = true;
+                    break;
+                }
+                tc::tc_fence_after();
+                const long kb0 = c * kBlks, kb1 = min(a.nkb, kb0 + kBlks);
+                for (long kb = kb0; kb < kb1; ++kb, ++seq) {
+                    const int st = int(seq % a.stages);
+                    if (!tc::mbar_wait_timed(full + st, uint32_t((seq / a.stages) & 1), kGemmWaitNs)) {
+                        atomicExch(sflag, 1);
+                        bad = true;
+                        break;
+                    }
+                    tc::tc_fence_after();
+                    if (lane == 0) {
+                        const uint32_t sa = tc::smem_addr(smem + size_t(st) * a.stage_bytes);
+                        const uint64_t ad = tc::smem_desc(sa, 128u, kSbo), bd = tc::smem_desc(sa + a_bytes, 128u, kSbo);
+                        step(ad, bd, kb == kb0);
+                        step(ad + 16, bd + 16, false);
+                        tc::mma_commit(empty + st);
+                    }
+                    __syncwarp();
+                }
+                if (!bad && lane == 0) tc::mma_commit(dfull);
+                __syncwarp();
             }
         }
-        tc::tc_fence_before();   // TMEM reads before the next chunk's MMAs overwrite it
-        __syncthreads();
-        first = false;
-    }
-    if (first && *sflag == 0 && arow && q == 0) {   // empty k range: the slot holds a zero sum
-        for (int c = 0; c < kTN; ++c) {
-            const int col = j0 + c;
-            if (col < a.n) D[long(i) * a.ds_i + long(col) * a.ds_j] = 0.0;
+    } else {
+        // ---- drain warps: TMEM lane `row`, column groups of 8 of this warp's half ----
+        const int quarter = warp & 3, half = warp >> 2;
+        const int row = quarter * 32 + lane;
+        const uint32_t lane_q = uint32_t(quarter * 32) << 16;
+        constexpr int kHalf = kTN / 2;
+        const int ncol = Nt / 2, cbase = half * ncol;   // Nt is a multiple of 16
+        constexpr int NT = 32 * kDrainWarps;
+        long dseq = 0;
+        bool stop = false;
+        for (long it = blockIdx.x; it < items && !stop; it += gridDim.x) {
+            const Item t = item_of(it);
+            const long i = long(t.mi) * kT + row;
+            const int j0 = t.ni * Nt;
+            // reference exponents: the largest of the item's chunks, per row and column
+            int rA = 100;
+            for (long c = t.c0; c < t.c1; ++c) rA = max(rA, a.shA[c * a.prowA + i]);
+            if (tid < Nt) {
+                int rB = 100;
+                for (long c = t.c0; c < t.c1; ++c) rB = max(rB, a.shB[c * a.prowB + j0 + tid]);
+                refB[tid] = rB;
+            }
+            float ah[kHalf], al[kHalf];
+#pragma unroll
+            for (int e = 0; e < kHalf; ++e) ah[e] = al[e] = 0.f;
+            for (long c = t.c0; c < t.c1; ++c, ++dseq) {
+                float *fb = fbs + (dseq & 1) * kTN;
+                if (tid < Nt) fb[tid] = pow2f(a.shB[c * a.prowB + j0 + tid] - refB[tid]);
+                const float fa = pow2f(a.shA[c * a.prowA + i] - rA);
+                if (!tc::mbar_wait_timed(dfull, uint32_t(dseq & 1), kGemmWaitNs)) atomicExch(sflag, 1);
+                tc::tc_fence_after();
+                if (tc::bar_red_or(1, NT, *sflag != 0)) {   // also: fb is complete
+                    stop = true;
+                    break;
+                }
+#pragma unroll
+                for (int cg = 0; cg < kHalf / 8; ++cg) {
+                    if (cg * 8 >= ncol) break;
+                    const int cc = cbase + cg * 8;
+                    uint32_t r[kLev][8];
+#pragma unroll
+                    for (int l = 0; l < kLev; ++l) tc::tmem_ld8_issue(tmem + lane_q + uint32_t(l * Nt + cc), r[l]);
+                    tc::tmem_wait_ld();
+#pragma unroll
+                    for (int l = 0; l < kLev; ++l)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) tc::order_after_wait(r[l][e]);
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2) {
+                        // levels combined in FP32 down to level 1 (rounding ~2^-32 of level 0's
+                        // scale), level 0 added with TwoSum, the pair scaled and accumulated
+                        auto lv = [&](int l) { return make_float2(__uint_as_float(r[l][e]), __uint_as_float(r[l][e + 1])); };
+                        const float2 q = make_float2(1.f / 256.f, 1.f / 256.f), m1 = make_float2(-1.f, -1.f);
+                        float2 tl = __ffma2_rn(lv(4), q, lv(3));
+                        tl = __ffma2_rn(tl, q, lv(2));
+                        tl = __ffma2_rn(tl, q, lv(1));
+                        tl = __fmul2_rn(tl, q);
+                        const float2 l0 = lv(0);
+                        float2 h = __fadd2_rn(l0, tl);
+                        const float2 b0 = __ffma2_rn(l0, m1, h);
+                        float2 lo = __fadd2_rn(__ffma2_rn(__ffma2_rn(b0, m1, h), m1, l0), __ffma2_rn(b0, m1, tl));
+                        const float2 f = __fmul2_rn(make_float2(fa, fa), *reinterpret_cast<const float2 *>(fb + cc + e));
+                        h = __fmul2_rn(h, f);
+                        lo = __fmul2_rn(lo, f);
+                        const float2 s0 = make_float2(ah[cg * 8 + e], ah[cg * 8 + e + 1]);
+                        const float2 s = __fadd2_rn(s0, h);
+                        const float2 bp = __ffma2_rn(s0, m1, s);
+                        const float2 er = __fadd2_rn(__ffma2_rn(__ffma2_rn(bp, m1, s), m1, s0), __ffma2_rn(bp, m1, h));
+                        const float2 cs = __fadd2_rn(make_float2(al[cg * 8 + e], al[cg * 8 + e + 1]), __fadd2_rn(er, lo));
+                        ah[cg * 8 + e] = s.x;
+                        ah[cg * 8 + e + 1] = s.y;
+                        al[cg * 8 + e] = cs.x;
+                        al[cg * 8 + e + 1] = cs.y;
+                    }
+                }
+                tc::tc_fence_before();   // TMEM reads before the next chunk's MMAs overwrite it
+                tc::bar_sync(1, NT);
+                if (tid == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(dempty)) : "memory");
+            }
+            if (stop) break;
+            tc::bar_sync(1, NT);   // refB is complete also for an item without chunks
+            if (i < a.m) {
+                double *D = a.D + t.z * a.dz + i * a.ds_i;
+#pragma unroll
+                for (int e = 0; e < kHalf; ++e) {
+                    const int col = cbase + e, j = j0 + col;
+                    if (e < ncol && j < a.n) {
+                        // alpha times the pair: the leading product with its rounding error
+                        const float p = ah[e] * a.al_h;
+                        const float l = fmaf(ah[e], a.al_h, -p) + fmaf(ah[e], a.al_l, al[e] * a.al_h);
+                        // x = X 2^(E - 1052), and level 0 holds X 2^-24: 2 x (24 - 1052)
+                        const double v = pair_to_double(p, l, rA + refB[col] - 2056 + a.al_e);
+                        double *dp = D + long(j) * a.ds_j;
+                        *dp = a.add ? *dp + v : v;
+                    }
+                }
+            }
+            tc::bar_sync(1, NT);   // refB is rewritten by the next item
         }
     }
-    if (t == 0 && *sflag) atomicExch(a.err, 1);
     tc::tc_fence_before();
     __syncthreads();
+    if (tid == 0 && *sflag) atomicExch(a.err, 1);
     if (warp == 0) {
         tc::tc_fence_after();
-        tc::tmem_dealloc(tmem, 512);
+        tc::tmem_dealloc(tmem, uint32_t(a.tmem_cols));
     }
 }
 
-// D(i, j) = sum_z W[z][i + m j] with the output strides.
-__global__ void tc_gemm_reduce_kernel(const double *W, int Z, int m, int n, double *D, long ds_i, long ds_j)
+// D(i, j) (+)= alpha sum_z W[z][i + m j] with the output strides.
+__global__ void tc_gemm_reduce_kernel(const double *W, int Z, long m, int n, double alpha, double *D, long ds_i,
+                                      long ds_j, int add)
 {
-    const long tot = long(m) * n;
+    const long tot = m * n;
     for (long e = long(blockIdx.x) * blockDim.x + threadIdx.x; e < tot; e += long(gridDim.x) * blockDim.x) {
+        const long i = e % m, jj = e / m;
+        double *dp = D + i * ds_i + jj * ds_j;
         double s = 0.0;
         for (int z = 0; z < Z; ++z) s += W[long(z) * tot + e];
-        const long i = e % m, jj = e / m;
-        D[i * ds_i + jj * ds_j] = s;
+        *dp = add ? fma(alpha, s, *dp) : alpha * s;
     }
+}
+
+inline long ceil_div(long a, long b) { return (a + b - 1) / b; }
+inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
+int launch_cut(Plan &P, const double *X, long sr, long sk, long rows, long K, int rt, long tiles, uint8_t *dig, int *sh,
+               cudaStream_t s)
+{
+    CutArgs c{};
+    c.X = X;
+    c.sr = sr;
+    c.sk = sk;
+    c.rows = rows;
+    c.K = K;
+    c.rt = rt;
+    c.nkb = ceil_div(K, kBlk);
+    c.dig = dig;
+    c.sh = sh;
+    c.prow = tiles * rt;
+    c.vec = ((reinterpret_cast<uintptr_t>(X) | uintptr_t(sr * 8)) & 15) == 0;
+    const unsigned chunks = unsigned(ceil_div(K, kChunk));
+    const int tb = timing_begin(P, EXX_TIMING_GEMM, s);
+    if (sk == 1)
+        gemm_cut_kernel<true><<<dim3(unsigned(ceil_div(c.prow, 8)), chunks), 32 * kCutWarps, 0, s>>>(c);
+    else
+        gemm_cut_kernel<false><<<dim3(unsigned(ceil_div(c.prow, 32)), chunks), 32 * kCutWarps, 0, s>>>(c);
+    timing_end(P, tb, s);
+    EXX_LAUNCH("gemm_cut_kernel");
+    P.launches++;
+    return EXX_OK;
 }
 
 }  // namespace
 
-int tc_gemm(Plan &P, int m, int n, long K, const double *A, long as_i, long as_k, const double *B, long bs_j,
-            long bs_k, double alpha, double *D, long ds_i, long ds_j, cudaStream_t s)
+int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_k, const double *B, long bs_j,
+            long bs_k, double alpha, double *D, long ds_i, long ds_j, cudaStream_t s, bool ktri)
 {
     if (m < 1 || n < 1 || K < 1) return EXX_ERR_INVALID_ARG;
     if (!P.err_d.p) {
         if (int rc = dev_reserve(P.err_d, 16)) return rc;
         EXX_CUDA(cudaMemsetAsync(P.err_d.p, 0, 16, s));
     }
-    const long mt = (m + kT - 1) / kT, nt = (n + kTN - 1) / kTN;
-    const long nchunks = (K + kChunk - 1) / kChunk;
-    // split k over Z CTAs per output tile when the tiles alone do not fill the GPU twice,
-    // each summing its chunks into its own FP64 slot (at most 1 GiB of slots)
-    long Z = 1;
-    if (nchunks > 1 && mt * nt < 2L * P.num_sms) {
-        Z = std::min(nchunks, (2L * P.num_sms + mt * nt - 1) / (mt * nt));
-        Z = std::min(Z, std::max(1L, (1L << 30) / (long(m) * n * 8)));
-    }
-    const long kper = ((nchunks + Z - 1) / Z) * kChunk;
-    Z = (K + kper - 1) / kper;
-    GemmArgs a{};
-    a.m = m;
-    a.n = n;
-    a.K = K;
-    a.A = A;
-    a.as_i = as_i;
-    a.as_k = as_k;
-    a.B = B;
-    a.bs_j = bs_j;
-    a.bs_k = bs_k;
-    a.kper = kper;
-    a.alpha = alpha;
-    a.err = static_cast<int *>(P.err_d.p);
-    if (Z > 1) {
-        if (int rc = dev_reserve(P.gemm_ws, size_t(Z) * m * n * sizeof(double))) return rc;
-        a.D = static_cast<double *>(P.gemm_ws.p);
-        a.ds_i = 1;
-        a.ds_j = m;
-        a.dz = long(m) * n;
+    // column tiles: as even as 16-column steps allow, at most 96 (5 levels in 512 TMEM columns)
+    const int nt = int(ceil_div(n, kTN));
+    const int Nt = int(ceil_div(ceil_div(n, nt), 16) * 16);
+    const long np = long(nt) * Nt;
+    // slabs: the digit planes (8 B per element) of one slab stay within kDigitBudget, cut along
+    // m when the contraction is short, along k when it is long
+    const long chunks = ceil_div(K, kChunk);
+    const long chunk_bytes = 8L * kChunk;   // per row
+    const long mpad = ceil_div(m, kT) * kT;
+    const bool long_k = chunks > 64;
+    long mslab = mpad, kslab = chunks;
+    if (long_k) {
+        kslab = std::max(1L, kDigitBudget / (chunk_bytes * (mpad + np)));
     } else {
-        a.D = D;
-        a.ds_i = ds_i;
-        a.ds_j = ds_j;
-        a.dz = 0;
+        kslab = std::min(chunks, std::max(1L, kDigitBudget / 2 / (chunk_bytes * np)));
+        const long room = kDigitBudget - std::min(kDigitBudget / 2, chunk_bytes * kslab * np);
+        mslab = std::max<long>(kT, room / (chunk_bytes * kslab) / kT * kT);
     }
-    const size_t smem = 4 * size_t(kT + kTN) * kSub * 2 + (kT + kTN) * sizeof(int) + 64;
-    EXX_CUDA(cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-    int tb = timing_begin(P, EXX_TIMING_GEMM, s);
-    tc_gemm_kernel<<<dim3(unsigned(mt), unsigned(nt), unsigned(Z)), kThreads, smem, s>>>(a);
-    timing_end(P, tb, s);
-    EXX_LAUNCH("tc_gemm_kernel");
-    P.launches++;
-    if (Z > 1) {
-        const long tot = long(m) * n;
-        tb = timing_begin(P, EXX_TIMING_GEMM, s);
-        tc_gemm_reduce_kernel<<<unsigned(std::min<long>((tot + 255) / 256, 4L * P.num_sms)), 256, 0, s>>>(
-            a.D, int(Z), m, n, D, ds_i, ds_j);
-        timing_end(P, tb, s);
-        EXX_LAUNCH("tc_gemm_reduce_kernel");
-        P.launches++;
+    mslab = std::min(mslab, mpad);
+    kslab = std::min(std::min(kslab, chunks), 65535L);
+    kslab = ceil_div(chunks, ceil_div(chunks, kslab));                     // even slabs
+    mslab = ceil_div(ceil_div(mpad, kT), ceil_div(mpad, mslab)) * kT;
+    // k splits: items (tiles x splits) for a whole number of rounds over the SMs
+    const long tiles = (mslab / kT) * nt;
+    auto splits = [&](long nch) {
+        if (nch < 2 || tiles >= 2L * P.num_sms) return 1L;
+        const long round = std::max(1L, P.num_sms / tiles);
+        long Z = nch >= 8 * round ? 2 * round : round;
+        Z = std::min(Z, nch);
+        return std::min(Z, std::max(1L, (1L << 28) / (mslab * n * 8)));
+    };
+    if (kslab < chunks) ktri = false;   // the limit counts chunks from k = 0
+    const long Zmax = ktri ? 1 : splits(kslab);
+    const size_t ldigA = size_t(mslab) * chunk_bytes * kslab, ldigB = size_t(np) * chunk_bytes * kslab;
+    const size_t offB = round_up(ldigA, 256), offSA = offB + round_up(ldigB, 256);
+    const size_t offSB = offSA + round_up(size_t(mslab) * kslab * 4, 256);
+    const size_t offP = offSB + round_up(size_t(np) * kslab * 4, 256);
+    const size_t part = Zmax > 1 ? size_t(Zmax) * std::min(mslab, m) * n * sizeof(double) : 0;
+    if (int rc = dev_reserve(P.gemm_ws, offP + part)) return rc;
+    uint8_t *ws = static_cast<uint8_t *>(P.gemm_ws.p);
+    int *shA = reinterpret_cast<int *>(ws + offSA), *shB = reinterpret_cast<int *>(ws + offSB);
+
+    GemmArgs a{};
+    a.n = n;
+    a.Nt = Nt;
+    a.nt = nt;
+    a.digA = ws;
+    a.digB = ws + offB;
+    a.shA = shA;
+    a.shB = shB;
+    a.prowB = np;
+    a.ktri = ktri ? 1 : 0;
+    a.err = static_cast<int *>(P.err_d.p);
+    a.stage_bytes = uint32_t(kT + Nt) * kBlk * 2 * kDig;
+    a.stages = int(std::min<size_t>(8, 200 * 1024 / a.stage_bytes));
+    a.offTab = uint32_t(a.stages) * a.stage_bytes;
+    a.offBar = a.offTab + uint32_t(round_up(2 * kTN * 4 + kTN * 4, 16));
+    a.tmem_cols = 32;
+    while (a.tmem_cols < kLev * Nt) a.tmem_cols *= 2;
+    const size_t smem = std::max<size_t>(a.offBar + (2 * size_t(a.stages) + 2) * 8 + 16, 120 * 1024);   // one CTA per SM
+    // B digits per MMA: at most 256 columns
+    const int gmax = 256 / Nt;
+    auto kern = gmax >= 4 ? tc_gemm_kernel<4> : gmax == 3 ? tc_gemm_kernel<3> : tc_gemm_kernel<2>;
+    EXX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+
+    for (long c0 = 0; c0 < chunks; c0 += kslab) {
+        const long nch = std::min(kslab, chunks - c0);
+        const long k0 = c0 * kChunk, kk = std::min(K - k0, nch * kChunk);
+        if (int rc = launch_cut(P, B + k0 * bs_k, bs_j, bs_k, n, kk, Nt, nt, ws + offB, shB, s)) return rc;
+        for (long i0 = 0; i0 < m; i0 += mslab) {
+            const long mr = std::min(mslab, m - i0);
+            a.mt = int(ceil_div(mr, kT));
+            if (int rc = launch_cut(P, A + i0 * as_i + k0 * as_k, as_i, as_k, mr, kk, kT, a.mt, ws, shA, s)) return rc;
+            a.m = mr;
+            a.prowA = long(a.mt) * kT;
+            a.nkb = ceil_div(kk, kBlk);
+            a.nchunks = nch;
+            a.Z = ktri ? 1 : std::min(Zmax, nch);
+            a.cper = ceil_div(nch, a.Z);
+            a.Z = ceil_div(nch, a.cper);
+            double *Dd = D + i0 * ds_i;
+            // alpha as an FP32 pair and a power of two; split sums take it in the reduction
+            const double am = std::frexp(a.Z > 1 ? 1.0 : alpha, &a.al_e);
+            a.al_h = float(am);
+            a.al_l = float(am - double(a.al_h));
+            if (a.Z > 1) {
+                a.D = reinterpret_cast<double *>(ws + offP);
+                a.ds_i = 1;
+                a.ds_j = mr;
+                a.dz = mr * n;
+                a.add = 0;
+            } else {
+                a.D = Dd;
+                a.ds_i = ds_i;
+                a.ds_j = ds_j;
+                a.dz = 0;
+                a.add = c0 > 0;
+            }
+            const long items = a.Z * a.mt * a.nt;
+            int tb = timing_begin(P, EXX_TIMING_GEMM, s);
+            kern<<<unsigned(std::min<long>(items, P.num_sms)), kThreads, smem, s>>>(a);
+            timing_end(P, tb, s);
+            EXX_LAUNCH("tc_gemm_kernel");
+            P.launches++;
+            if (a.Z > 1) {
+                const long tot = mr * n;
+                tb = timing_begin(P, EXX_TIMING_GEMM, s);
+                tc_gemm_reduce_kernel<<<unsigned(std::min<long>((tot + 255) / 256, 4L * P.num_sms)), 256, 0, s>>>(
+                    a.D, int(a.Z), mr, n, alpha, Dd, ds_i, ds_j, c0 > 0);
+                timing_end(P, tb, s);
+                EXX_LAUNCH("tc_gemm_reduce_kernel");
+                P.launches++;
+            }
+        }
     }
     return EXX_OK;
 }
