@@ -658,6 +658,383 @@ __global__ void __launch_bounds__(kRows * TPR + 64, 2) slice_pass_kernel(const _
 }
 
 // ---------------------------------------------------------------------------------------
+// Slice pass, direct form: the same tiles, digits, products and roundings as above with the
+// work laid out for instruction issue, which bounds these passes.
+//   * A group of NT threads owns a tile; two groups share an SM (two CTAs, or two groups of one
+//     CTA sharing the matrix images), so one group's CUDA-core phases run under the other's MMAs.
+//     No helper warps: the group's first warp issues the MMAs, and the next tile's input is
+//     loaded straight into registers while this tile's GEMMs run.
+//   * The operand is cut in units of 8 elements of a row (one 16-byte store per digit plane),
+//     8 rows x 4 units per warp: every load is whole 32-byte sectors, every store
+//     conflict-free, and tiles of fewer than 128 rows spread over all threads.  A row's maximum
+//     is gathered by shared-memory atomics on the bit patterns of the unit maxima.
+//   * The transposed tile takes the place of the consumed operand image.
+// Per pair solve against the staged / pipelined forms: 72 x 72 x 144 points pass A 5.82 -> 3.83 us,
+// C 5.62 -> 3.24; 48^3 A 0.617 -> 0.530, C 0.584 -> 0.420; 117 x 117 x 119 (matrices resident instead
+// of streamed) A 12.6 -> 8.7, C 11.7 -> 5.5.  The bits of every result are the same.
+struct SliceDArgs {
+    int n1, n2, n3, G, tpf;
+    long ntiles;
+    long N;
+    const float *psi;       // pass A: FP32 orbital planes (column c at c N)
+    int occ_off;
+    const int2 *pairs;
+    const float *in;        // pass C: input fields
+    float *out;
+    const uint8_t *img1, *img2;
+    uint32_t img1_bytes, img2_bytes;
+    int Kp1, Kp2;
+    uint32_t offB2, offA, a_bytes, offRm, offBar;   // a_bytes: one group's operand / transposed tile
+    uint32_t a_piece1, a_piece2;
+    int Pj, tmem_cols, tcols;                       // tcols: TMEM columns of one group
+    int vec;                // rows of n1 floats start 16-byte aligned
+    int groups;             // groups per CTA
+    int *err;
+};
+
+// Three digits of eight consecutive elements (hi + lo) * s: 16 bytes in each digit plane.
+template <bool LO>
+__device__ __forceinline__ void store_digits8(uint8_t *dst, uint32_t piece, const float (&h)[8], const float (&l)[8], float s)
+{
+    uint32_t w[3][4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        float2 d0, d1, d2;
+        digits3x2<LO>(make_float2(h[2 * e], h[2 * e + 1]), make_float2(l[2 * e], l[2 * e + 1]), f2(s), d0, d1, d2);
+        w[0][e] = pack2(d0.x, d0.y);
+        w[1][e] = pack2(d1.x, d1.y);
+        w[2][e] = pack2(d2.x, d2.y);
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) *reinterpret_cast<uint4 *>(dst + q * piece) = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
+}
+
+__device__ __forceinline__ float max8(const float (&h)[8])
+{
+    const float a = fmaxf(fmaxf(fabsf(h[0]), fabsf(h[1])), fabsf(h[2]));
+    const float b = fmaxf(fmaxf(fabsf(h[3]), fabsf(h[4])), fabsf(h[5]));
+    return fmaxf(fmaxf(a, b), fmaxf(fabsf(h[6]), fabsf(h[7])));
+}
+
+// The 7 digit products of one GEMM as 6 MMAs per 16-k step: d0 meets p0 and p1 in one MMA of
+// 2 Np columns (lead and rest columns are neighbours, as are the two matrix digits).  Per column
+// the products of the rest accumulator keep issue_x7g's order.  Descriptors advance by additions.
+__device__ __forceinline__ void issue_x7_pair(uint32_t d_lead, uint32_t Np, uint32_t a_base, uint32_t a_piece, uint32_t b_base,
+                                              uint32_t b_piece, uint32_t sbo, int ksteps)
+{
+    uint64_t ad = tc::smem_desc(a_base, 128u, sbo), bd = tc::smem_desc(b_base, 128u, sbo);
+    const uint64_t a1 = a_piece >> 4, b1 = b_piece >> 4;
+    const uint32_t i1 = tc::instr_desc(false, int(Np)), i2 = tc::instr_desc(false, int(2 * Np));
+    const uint32_t d_rest = d_lead + Np;
+#pragma unroll 1
+    for (int ks = 0; ks < ksteps; ++ks, ad += 16, bd += 16) {
+        tc::mma_bf16(d_lead, ad, bd, i2, ks > 0 ? 1u : 0u);           // d0 p0 | d0 p1
+        tc::mma_bf16(d_rest, ad + a1, bd, i1, 1u);                    // d1 p0
+        tc::mma_bf16(d_rest, ad, bd + 2 * b1, i1, 1u);                // d0 p2
+        tc::mma_bf16(d_rest, ad + a1, bd + b1, i1, 1u);               // d1 p1
+        tc::mma_bf16(d_rest, ad + 2 * a1, bd, i1, 1u);                // d2 p0
+        tc::mma_bf16(d_rest, ad, bd + 3 * b1, i1, 1u);                // d0 p3
+    }
+}
+
+// Eight drained columns: (lead + rest) * (rs * cs[e]).
+__device__ __forceinline__ void combine8(uint32_t (&r0)[8], uint32_t (&r1)[8], float rs, const float *cs, float (&v)[8])
+{
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float2 c2 = *reinterpret_cast<const float2 *>(cs + 2 * e);
+        const float2 w = __fmul2_rn(__fadd2_rn(make_float2(__uint_as_float(r0[2 * e]), __uint_as_float(r0[2 * e + 1])),
+                                               make_float2(__uint_as_float(r1[2 * e]), __uint_as_float(r1[2 * e + 1]))),
+                                    __fmul2_rn(f2(rs), c2));
+        v[2 * e] = w.x;
+        v[2 * e + 1] = w.y;
+    }
+}
+
+template <bool PAIR, int NT, int UPT>
+__global__ void __launch_bounds__(512, 1) slice_direct_kernel(const __grid_constant__ SliceDArgs a)
+{
+    extern __shared__ __align__(1024) uint8_t smem[];
+    constexpr int kParts = NT / kRows;    // column parts of the drains
+    const int grp = threadIdx.x / NT, tid = threadIdx.x - grp * NT;
+    const int warp = tid >> 5, lane = tid & 31;
+    uint8_t *sB1 = smem;
+    uint8_t *sB2 = a.offB2 ? smem + a.offB2 : smem;
+    uint8_t *sA = smem + a.offA + size_t(grp) * a.a_bytes;
+    float *Ysm = reinterpret_cast<float *>(sA);
+    uint32_t *rm1 = reinterpret_cast<uint32_t *>(smem + a.offRm) + grp * 2 * kRows, *rm2 = rm1 + kRows;
+    uint64_t *bar_d = reinterpret_cast<uint64_t *>(smem + a.offBar) + grp;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + a.offBar + 16);
+    int *sflag = reinterpret_cast<int *>(tslot + 1);
+
+    for (uint32_t i = threadIdx.x * 16; i < a.img1_bytes; i += blockDim.x * 16)
+        *reinterpret_cast<uint4 *>(sB1 + i) = *reinterpret_cast<const uint4 *>(a.img1 + i);
+    if (a.offB2)
+        for (uint32_t i = threadIdx.x * 16; i < a.img2_bytes; i += blockDim.x * 16)
+            *reinterpret_cast<uint4 *>(sB2 + i) = *reinterpret_cast<const uint4 *>(a.img2 + i);
+    for (uint32_t i = threadIdx.x * 16; i < uint32_t(a.groups) * a.a_bytes; i += blockDim.x * 16)
+        *reinterpret_cast<uint4 *>(smem + a.offA + i) = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < 2 * kRows; i += NT) rm1[i] = 0u;
+    if (tid == 0) tc::mbar_init(bar_d, 1);
+    if (threadIdx.x == 0) *sflag = 0;
+    if (threadIdx.x < 32) tc::tmem_alloc(tslot, uint32_t(a.tmem_cols));
+    tc::fence_proxy_async_smem();
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tmem0 = *tslot, tmem = tmem0 + uint32_t(grp * a.tcols);
+    const int n1 = a.n1, n2 = a.n2;
+    const long R = long(n1) * n2;
+    const int Kp1 = a.Kp1, Kp2 = a.Kp2;
+    const uint32_t sbo1 = uint32_t(Kp1) * 16u, sbo2 = uint32_t(Kp2) * 16u;
+    const float *cs1 = reinterpret_cast<const float *>(sB1 + size_t(kMatDig) * Kp1 * Kp1 * 2);
+    const float *cs2 = reinterpret_cast<const float *>(sB2 + size_t(kMatDig) * Kp2 * Kp2 * 2);
+    const int bar_id = 1 + grp;
+
+    // cut units: quarter-warp number q of the group takes (8-row block q / nu, unit q % nu),
+    // its lane & 7 the row.  Units past the operand are marked by row 128.
+    int ru1[UPT], ru2[UPT];   // row | unit << 8
+#pragma unroll
+    for (int g = 0; g < UPT; ++g) {
+        const int q = ((warp + 2 * grp) % (NT / 32)) * 4 + (lane >> 3) + g * (NT / 8);
+        const int nu1 = Kp1 / 8, nu2 = Kp2 / 8;
+        const int row1 = (q / nu1) * 8 + (lane & 7), row2 = (q / nu2) * 8 + (lane & 7);
+        ru1[g] = min(row1, kRows) | ((q % nu1) << 8);
+        ru2[g] = min(row2, kRows) | ((q % nu2) << 8);
+    }
+    // drains: TMEM lane drow, column units dpart, dpart + kParts, ...
+    const int quarter = warp & 3, dpart = warp >> 2;
+    const int drow = quarter * 32 + lane;
+    const uint32_t lane_q = uint32_t(quarter * 32) << 16;
+    const int s1 = drow / n2, j1 = drow - s1 * n2, s2 = drow / n1, i2 = drow - s2 * n1;
+
+    const long stride = long(gridDim.x) * a.groups;
+    long p = (long(blockIdx.x) * a.groups + grp) / a.tpf;
+    int zt = int((long(blockIdx.x) * a.groups + grp) - p * a.tpf);
+    const long dp = stride / a.tpf;
+    const int dz = int(stride - dp * a.tpf);
+    uint32_t ph = 0;
+    auto wait_d = [&]() {
+        if (!tc::mbar_wait_timed(bar_d, ph, kWaitNs)) atomicExch(sflag, 1);
+        ph ^= 1u;
+        tc::tc_fence_after();
+    };
+    // operand image complete: hand it to the MMAs of this group (true = stop on an error)
+    auto handoff = [&](bool first) {
+        tc::fence_proxy_async_smem();
+        tc::tc_fence_before();
+        if (tc::bar_red_or(bar_id, NT, *sflag != 0)) return true;
+        if (warp == 0) {
+            tc::tc_fence_after();
+            if (lane == 0) {
+                if (first)
+                    issue_x7_pair(tmem, uint32_t(Kp1), tc::smem_addr(sA), a.a_piece1, tc::smem_addr(sB1),
+                                  uint32_t(Kp1) * Kp1 * 2u, sbo1, Kp1 / 16);
+                else
+                    issue_x7_pair(tmem, uint32_t(Kp2), tc::smem_addr(sA), a.a_piece2, tc::smem_addr(sB2),
+                                  uint32_t(Kp2) * Kp2 * 2u, sbo2, Kp2 / 16);
+                tc::mma_commit(bar_d);
+            }
+            __syncwarp();
+        }
+        return false;
+    };
+    // input of tile (pp, zz) for this thread's units: raw values of one or two rows
+    float x0[UPT][8], x1[UPT][8];
+    auto load8 = [&](const float *src, int k, bool ok, float (&v)[8]) {
+        if (a.vec) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float4 w = ok && k + 4 * h < n1 ? *reinterpret_cast<const float4 *>(src + 4 * h) : make_float4(0.f, 0.f, 0.f, 0.f);
+                v[4 * h] = w.x; v[4 * h + 1] = w.y; v[4 * h + 2] = w.z; v[4 * h + 3] = w.w;
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = ok && k + e < n1 ? src[e] : 0.f;
+        }
+    };
+    auto prefetch = [&](long pp, int zz) {
+        const int z0 = zz * a.G, R1 = min(a.G, a.n3 - z0) * n2;
+        const float *b0, *b1 = nullptr;
+        if (PAIR) {
+            const int2 mn = a.pairs[pp];
+            b0 = a.psi + size_t(a.occ_off + mn.x) * a.N + size_t(z0) * R;
+            b1 = a.psi + size_t(mn.y) * a.N + size_t(z0) * R;
+        } else {
+            b0 = a.in + size_t(pp) * a.N + size_t(z0) * R;
+        }
+#pragma unroll
+        for (int g = 0; g < UPT; ++g) {
+            const int row = ru1[g] & 255, k = (ru1[g] >> 8) * 8;
+            const bool ok = row < R1;
+            const int o = row * n1 + k;
+            load8(b0 + o, k, ok, x0[g]);
+            if (PAIR) load8(b1 + o, k, ok, x1[g]);
+        }
+    };
+
+    const long nfields = a.ntiles / a.tpf;
+    if (p < nfields) prefetch(p, zt);
+    while (p < nfields) {
+        const int z0 = zt * a.G, ns = min(a.G, a.n3 - z0);
+        const int R1 = ns * n2, R2 = ns * n1;
+        // ---- GEMM 1 operand: row (s, j), K = i: products (hi, rounding error lo), row maxima ----
+#pragma unroll
+        for (int g = 0; g < UPT; ++g) {
+            if (PAIR) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 x = make_float2(x0[g][2 * e], x0[g][2 * e + 1]);
+                    const float2 y = make_float2(x1[g][2 * e], x1[g][2 * e + 1]);
+                    const float2 hh = __fmul2_rn(x, y);
+                    const float2 ll = __ffma2_rn(x, y, __fmul2_rn(hh, f2(-1.f)));
+                    x0[g][2 * e] = hh.x; x0[g][2 * e + 1] = hh.y;
+                    x1[g][2 * e] = ll.x; x1[g][2 * e + 1] = ll.y;
+                }
+            }
+            const int row = ru1[g] & 255;
+            if (row < R1) atomicMax(rm1 + row, __float_as_uint(max8(x0[g])));
+        }
+        tc::bar_sync(bar_id, NT);
+#pragma unroll
+        for (int g = 0; g < UPT; ++g) {
+            const int row = ru1[g] & 255;
+            if (row < R1) {
+                float sc, inv;
+                row_scales(__uint_as_float(rm1[row]), sc, inv);
+                store_digits8<PAIR>(sA + img_at(row, ru1[g] >> 8, sbo1), a.a_piece1, x0[g], x1[g], sc);
+            }
+        }
+        if (handoff(true)) break;
+        // while GEMM 1 runs: the next tile's input, the second maxima cleared
+        long np = p + dp;
+        int nz = zt + dz;
+        if (nz >= a.tpf) {
+            nz -= a.tpf;
+            ++np;
+        }
+        if (np < nfields) prefetch(np, nz);
+        if (tid < kRows) rm2[tid] = 0u;
+        const float rs1 = [&] {
+            float sc, inv;
+            row_scales(__uint_as_float(rm1[drow]), sc, inv);
+            return inv;
+        }();
+        wait_d();
+        // ---- GEMM 1 result -> transposed tile Y[(s, i')][j], over the consumed operand ----
+        if (quarter * 32 < R1) {
+            float *yb = Ysm + size_t(s1) * n1 * a.Pj + j1;
+            const bool act = drow < R1;
+            const int nu = (n1 + 7) / 8;
+            for (int u = dpart; u < nu; u += kParts) {
+                uint32_t r0[8], r1[8];
+                tc::tmem_ld8_issue(tmem + lane_q + uint32_t(8 * u), r0);
+                tc::tmem_ld8_issue(tmem + lane_q + uint32_t(Kp1 + 8 * u), r1);
+                tc::tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    tc::order_after_wait(r0[e]);
+                    tc::order_after_wait(r1[e]);
+                }
+                float v[8];
+                combine8(r0, r1, rs1, cs1 + 8 * u, v);
+                if (act) {
+                    float *y = yb + 8 * u * a.Pj;
+                    if (8 * u + 8 <= n1) {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) y[e * a.Pj] = v[e];
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            if (8 * u + e < n1) y[e * a.Pj] = v[e];
+                    }
+                }
+            }
+        }
+        tc::tc_fence_before();
+        tc::bar_sync(bar_id, NT);
+        // ---- GEMM 2 operand: row (s, i'), K = j, from the transposed tile ----
+        if (tid < kRows) rm1[tid] = 0u;
+        float y[UPT][8];
+#pragma unroll
+        for (int g = 0; g < UPT; ++g) {
+            const int row = ru2[g] & 255, k = (ru2[g] >> 8) * 8;
+            const bool ok = row < R2;
+            const float *yr = Ysm + (ok ? row * a.Pj + k : 0);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const bool in = ok && k + 4 * h < n2;
+                const float4 w = in ? *reinterpret_cast<const float4 *>(yr + 4 * h) : make_float4(0.f, 0.f, 0.f, 0.f);
+                y[g][4 * h] = w.x; y[g][4 * h + 1] = w.y; y[g][4 * h + 2] = w.z; y[g][4 * h + 3] = w.w;
+            }
+            if (k + 8 > n2) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    if (k + e >= n2) y[g][e] = 0.f;   // pitch padding
+            }
+            if (ok) atomicMax(rm2 + row, __float_as_uint(max8(y[g])));
+        }
+        tc::bar_sync(bar_id, NT);
+#pragma unroll
+        for (int g = 0; g < UPT; ++g) {
+            const int row = ru2[g] & 255;
+            if (row < R2) {
+                float sc, inv;
+                row_scales(__uint_as_float(rm2[row]), sc, inv);
+                store_digits8<false>(sA + img_at(row, ru2[g] >> 8, sbo2), a.a_piece2, y[g], y[g], sc);
+            }
+        }
+        if (handoff(false)) break;
+        const float rs2 = [&] {
+            float sc, inv;
+            row_scales(__uint_as_float(rm2[drow]), sc, inv);
+            return inv;
+        }();
+        wait_d();
+        // ---- GEMM 2 result -> the field at (z0 + s, j', i') ----
+        if (quarter * 32 < R2) {
+            float *ob = a.out + size_t(p) * a.N + size_t(z0 + s2) * R + i2;
+            const bool act = drow < R2;
+            const int nu = (n2 + 7) / 8;
+            for (int u = dpart; u < nu; u += kParts) {
+                uint32_t r0[8], r1[8];
+                tc::tmem_ld8_issue(tmem + lane_q + uint32_t(8 * u), r0);
+                tc::tmem_ld8_issue(tmem + lane_q + uint32_t(Kp2 + 8 * u), r1);
+                tc::tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    tc::order_after_wait(r0[e]);
+                    tc::order_after_wait(r1[e]);
+                }
+                float v[8];
+                combine8(r0, r1, rs2, cs2 + 8 * u, v);
+                if (act) {
+                    float *o = ob + 8 * u * n1;
+                    if (8 * u + 8 <= n2) {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) o[e * n1] = v[e];
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            if (8 * u + e < n2) o[e * n1] = v[e];
+                    }
+                }
+            }
+        }
+        tc::tc_fence_before();
+        p = np;
+        zt = nz;
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x == 0 && *sflag) atomicExch(a.err, 1);
+    if (threadIdx.x < 32) {
+        tc::tc_fence_after();
+        tc::tmem_dealloc(tmem0, uint32_t(a.tmem_cols));
+    }
+}
+
+// ---------------------------------------------------------------------------------------
 // Pass B.  A tile is 128 consecutive rows r = a + n1 b of one field (pencils along z).
 //   forward GEMM: rows r, K = z, outputs c in NB blocks of WN columns
 //   middle: (D * f(Lambda)) as FP32 hi + lo, re-sliced in place of its own digits
@@ -1152,6 +1529,55 @@ SliceLayout slice_layout(const Plan &P, bool pair = true)
     return ser_two ? ser : pip;
 }
 
+// Layout of the direct form of the slice passes, false when it does not fit: the matrix images
+// stay resident, so slices wider than about 100 points with different x and y matrices keep
+// the streamed form.
+struct SliceDLayout {
+    size_t smem;
+    uint32_t offB2, offA, a_bytes, offRm, offBar, a_piece1, a_piece2;
+    int G, Pj, tcols, tmem_cols, groups, nt, upt;
+};
+
+bool slice_direct_layout(const Plan &P, SliceDLayout &L)
+{
+    const int n1 = P.n[0], n2 = P.n[1];
+    const int Kp1 = pad16i(n1), Kp2 = pad16i(n2);
+    L = SliceDLayout{};
+    L.G = kRows / std::max(n1, n2);
+    L.Pj = (n2 + 3) & ~3;
+    if (((L.Pj / 4) & 1) == 0) L.Pj += 4;   // odd number of 16-byte units: conflict-free rows
+    const int R1 = L.G * n2, R2 = L.G * n1;
+    size_t off = mat_image_bytes(Kp1, Kp1);
+    if (!P.t3_share01) {
+        off = align_up(off, 1024);
+        L.offB2 = uint32_t(off);
+        off += mat_image_bytes(Kp2, Kp2);
+    }
+    L.offA = uint32_t(align_up(off, 1024));
+    L.a_piece1 = uint32_t(pad8i(R1)) * Kp1 * 2u;
+    L.a_piece2 = uint32_t(pad8i(R2)) * Kp2 * 2u;
+    // the MMA reads 128 rows of every digit plane (rows past the tile are never read back)
+    const size_t reach = std::max(2 * size_t(L.a_piece1) + size_t(kRows) * Kp1 * 2, 2 * size_t(L.a_piece2) + size_t(kRows) * Kp2 * 2);
+    L.a_bytes = uint32_t(align_up(std::max(reach, size_t(R2) * L.Pj * 4), 1024));
+    const int np = 2 * std::max(Kp1, Kp2);   // lead and rest columns of one GEMM
+    L.tcols = np;
+    auto finish = [&](int nt, int groups) {
+        L.nt = nt;
+        L.groups = groups;
+        const int q = std::max(pad8i(R1) / 8 * (Kp1 / 8), pad8i(R2) / 8 * (Kp2 / 8));   // quarter-warp units
+        L.upt = (q + nt / 8 - 1) / (nt / 8);
+        L.offRm = uint32_t(L.offA + size_t(groups) * L.a_bytes);
+        L.offBar = L.offRm + uint32_t(groups) * 2 * kRows * 4;
+        L.smem = L.offBar + 32;
+        L.tmem_cols = tmem_pow2(groups * np);
+        return L.upt <= 4 && L.smem <= kSmemLimit && groups * np <= 512;
+    };
+    const size_t two_per_sm = 233472 / 2 - 1024;
+    if (finish(256, 1) && L.smem <= two_per_sm && L.tmem_cols <= 256) return true;
+    if (finish(256, 2)) return true;
+    return finish(512, 1);
+}
+
 struct ZLayout {
     size_t smem;
     uint32_t offB, offCs, offMax, offBar, blk_bytes;
@@ -1376,7 +1802,65 @@ int tc3_solve_batch(Plan &P, const int2 *pairs_d, int nfields, float *bufA, floa
 {
     const int n1 = P.n[0], n2 = P.n[1], n3 = P.n[2];
     // passes A and C
+    SliceDLayout DL;
+    const bool direct = slice_direct_layout(P, DL);
+    auto slice_direct = [&](bool pair, const float *in, float *out, int kind) -> int {
+        SliceDArgs a{};
+        a.n1 = n1;
+        a.n2 = n2;
+        a.n3 = n3;
+        a.G = DL.G;
+        a.tpf = (n3 + DL.G - 1) / DL.G;
+        a.ntiles = long(nfields) * a.tpf;
+        a.N = P.N;
+        a.psi = static_cast<const float *>(P.psi32.p);
+        a.occ_off = P.tc_occ_off;
+        a.pairs = pairs_d;
+        a.in = in;
+        a.out = out;
+        const int inv = pair ? 0 : 1;
+        a.img1 = static_cast<const uint8_t *>(P.t3img[0][inv].p);
+        a.img2 = static_cast<const uint8_t *>(P.t3img[1][inv].p);
+        a.Kp1 = pad16i(n1);
+        a.Kp2 = pad16i(n2);
+        a.img1_bytes = uint32_t(mat_image_bytes(a.Kp1, a.Kp1));
+        a.img2_bytes = uint32_t(mat_image_bytes(a.Kp2, a.Kp2));
+        a.offB2 = DL.offB2;
+        a.offA = DL.offA;
+        a.a_bytes = DL.a_bytes;
+        a.offRm = DL.offRm;
+        a.offBar = DL.offBar;
+        a.a_piece1 = DL.a_piece1;
+        a.a_piece2 = DL.a_piece2;
+        a.Pj = DL.Pj;
+        a.tmem_cols = DL.tmem_cols;
+        a.tcols = DL.tcols;
+        a.vec = ((n1 & 3) == 0 && (P.N & 3) == 0) ? 1 : 0;
+        a.groups = DL.groups;
+        a.err = static_cast<int *>(P.err_d.p);
+        void (*kern)(const SliceDArgs) = nullptr;
+        if (DL.nt == 256) {
+            if (DL.upt <= 2) kern = pair ? slice_direct_kernel<true, 256, 2> : slice_direct_kernel<false, 256, 2>;
+            else if (DL.upt == 3) kern = pair ? slice_direct_kernel<true, 256, 3> : slice_direct_kernel<false, 256, 3>;
+            else kern = pair ? slice_direct_kernel<true, 256, 4> : slice_direct_kernel<false, 256, 4>;
+        } else {
+            if (DL.upt <= 3) kern = pair ? slice_direct_kernel<true, 512, 3> : slice_direct_kernel<false, 512, 3>;
+            else kern = pair ? slice_direct_kernel<true, 512, 4> : slice_direct_kernel<false, 512, 4>;
+        }
+        size_t smem = DL.smem;
+        const int threads = DL.nt * DL.groups;
+        int per_sm = 1;
+        if (int rc = launch_setup(kern, threads, smem, DL.tmem_cols, per_sm)) return rc;
+        const int grid = int(std::min<long>((a.ntiles + DL.groups - 1) / DL.groups, long(P.num_sms) * per_sm));
+        const int tb = timing_begin(P, kind, s);
+        kern<<<grid, threads, smem, s>>>(a);
+        timing_end(P, tb, s);
+        EXX_LAUNCH("slice_direct_kernel");
+        P.launches++;
+        return EXX_OK;
+    };
     auto slice = [&](bool pair, const float *in, float *out, int kind) -> int {
+        if (direct) return slice_direct(pair, in, out, kind);
         const SliceLayout L = slice_layout(P, pair);
         SliceArgs a{};
         a.n1 = n1;
