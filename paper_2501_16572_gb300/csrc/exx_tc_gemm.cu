@@ -24,8 +24,8 @@
 // (bulk copies, a producer warp) into the MMAs (one issuing warp) while 8 warps combine
 // finished chunks.  Cutting inside the GEMM repeated the integer work of every A row for each
 // 96 output columns and left the tensor cores idle meanwhile: both products of ace_apply at
-// n = nphi = 512 on 72 x 72 x 144 points took 65.7 ms, 11.8 ms now (cuts 3.3 ms near the HBM
-// rate, MMAs 8.3 ms, of which the tensor pipe's own 5.6 ms).
+// n = nphi = 512 on 72 x 72 x 144 points took 65.7 ms, 11.3 ms now (cuts 3.3 ms near the HBM
+// rate, MMAs 7.8 ms, of which the tensor pipe's own 5.6 ms).
 #include "exx_internal.h"
 #include "tc_ptx.cuh"
 
@@ -278,15 +278,15 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     if (warp == kDrainWarps) {
         // ---- producer warp: one operand block pair per stage ----
         if (lane == 0) {
-            long seq = 0;
-            bool bad = false;
+            // stage and its parity by increments: a division per stage would cost as much as its MMAs
+            int st = 0, filled = 0;
+            uint32_t par = 1;   // of the stage's last release; the first pass over the stages waits for none
+            bool bad = false, first = true;
             for (long it = blockIdx.x; it < items && !bad; it += gridDim.x) {
                 const Item t = item_of(it);
                 const long kb1 = min(a.nkb, t.c1 * kBlks);
-                for (long kb = t.c0 * kBlks; kb < kb1; ++kb, ++seq) {
-                    const int st = int(seq % a.stages);
-                    const long use = seq / a.stages;
-                    if (use > 0 && !tc::mbar_wait_timed(empty + st, uint32_t((use - 1) & 1), kGemmWaitNs)) {
+                for (long kb = t.c0 * kBlks; kb < kb1; ++kb) {
+                    if (!first && !tc::mbar_wait_timed(empty + st, par, kGemmWaitNs)) {
                         atomicExch(sflag, 1);
                         bad = true;
                         break;
@@ -295,17 +295,24 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                     tc::mbar_arrive_expect_tx(full + st, a_bytes + b_bytes);
                     gemm_bulk_load(s, a.digA + (size_t(t.mi) * a.nkb + kb) * a_bytes, a_bytes, full + st);
                     gemm_bulk_load(s + a_bytes, a.digB + (size_t(t.ni) * a.nkb + kb) * b_bytes, b_bytes, full + st);
+                    filled = max(filled, st + 1);
+                    if (++st == a.stages) {
+                        st = 0;
+                        par ^= 1u;
+                        first = false;
+                    }
                 }
             }
-            for (int st = 0; st < a.stages; ++st) {   // every issued copy has landed before exit
-                const long nf = seq > st ? (seq - 1 - st) / a.stages + 1 : 0;
-                if (nf > 0 && !tc::mbar_wait_timed(full + st, uint32_t((nf - 1) & 1), kGemmWaitNs)) atomicExch(sflag, 1);
-            }
+            // every issued copy has landed before exit: the last fill of a stage before `st` belongs
+            // to this pass over the stages (parity par ^ 1), of the others to the one before
+            for (int i = 0; i < filled; ++i)
+                if (!tc::mbar_wait_timed(full + i, i < st ? par ^ 1u : par, kGemmWaitNs)) atomicExch(sflag, 1);
         }
     } else if (warp == kDrainWarps + 1) {
         // ---- MMA warp ----
-        long seq = 0, dseq = 0;
-        bool bad = false;
+        int st = 0;
+        uint32_t par = 0, dpar = 1;
+        bool bad = false, dfirst = true;
         // operand and accumulator steps, fixed for the launch: the issue of one 16-k step is a
         // straight run of MMAs whose descriptors differ by additions (computed in a loop, the
         // issuing thread took 1340 cycles a step, twice the tensor pipe's 632)
@@ -342,17 +349,18 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         };
         for (long it = blockIdx.x; it < items && !bad; it += gridDim.x) {
             const Item t = item_of(it);
-            for (long c = t.c0; c < t.c1 && !bad; ++c, ++dseq) {
-                if (dseq > 0 && !tc::mbar_wait_timed(dempty, uint32_t((dseq - 1) & 1), kGemmWaitNs)) {
+            for (long c = t.c0; c < t.c1 && !bad; ++c) {
+                if (!dfirst && !tc::mbar_wait_timed(dempty, dpar, kGemmWaitNs)) {
                     atomicExch(sflag, 1);
                     bad = true;
                     break;
                 }
+                dfirst = false;
+                dpar ^= 1u;
                 tc::tc_fence_after();
                 const long kb0 = c * kBlks, kb1 = min(a.nkb, kb0 + kBlks);
-                for (long kb = kb0; kb < kb1; ++kb, ++seq) {
-                    const int st = int(seq % a.stages);
-                    if (!tc::mbar_wait_timed(full + st, uint32_t((seq / a.stages) & 1), kGemmWaitNs)) {
+                for (long kb = kb0; kb < kb1; ++kb) {
+                    if (!tc::mbar_wait_timed(full + st, par, kGemmWaitNs)) {
                         atomicExch(sflag, 1);
                         bad = true;
                         break;
@@ -366,6 +374,10 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                         tc::mma_commit(empty + st);
                     }
                     __syncwarp();
+                    if (++st == a.stages) {
+                        st = 0;
+                        par ^= 1u;
+                    }
                 }
                 if (!bad && lane == 0) tc::mma_commit(dfull);
                 __syncwarp();
