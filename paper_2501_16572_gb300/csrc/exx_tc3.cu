@@ -692,15 +692,25 @@ struct SliceDArgs {
     int *err;
 };
 
-// Three digits of eight consecutive elements (hi + lo) * s: 16 bytes in each digit plane.
+// Three digits of eight consecutive elements (hi + lo) * s: 16 bytes in each digit plane.  As
+// digits3x2 on the negated values (rounding to even is symmetric), so that every digit comes
+// out of M - (M - d) with its sign and the only constants are three magics and -1: 8 packed
+// operations for two elements (9 with lo), and no constant has to be rebuilt between them.
 template <bool LO>
 __device__ __forceinline__ void store_digits8(uint8_t *dst, uint32_t piece, const float (&h)[8], const float (&l)[8], float s)
 {
+    const float2 m0 = f2(12582912.f), m1 = f2(12582912.f / 512.f), m2 = f2(12582912.f / 262144.f), neg = f2(-1.f);
+    const float2 ns = f2(-s);
     uint32_t w[3][4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        float2 d0, d1, d2;
-        digits3x2<LO>(make_float2(h[2 * e], h[2 * e + 1]), make_float2(l[2 * e], l[2 * e + 1]), f2(s), d0, d1, d2);
+        const float2 x = make_float2(h[2 * e], h[2 * e + 1]);
+        const float2 d0 = __ffma2_rn(__ffma2_rn(x, ns, m0), neg, m0);
+        float2 r = __ffma2_rn(x, ns, d0);                            // -(t - d0)
+        if (LO) r = __ffma2_rn(make_float2(l[2 * e], l[2 * e + 1]), ns, r);
+        const float2 d1 = __ffma2_rn(__fadd2_rn(r, m1), neg, m1);
+        r = __fadd2_rn(r, d1);
+        const float2 d2 = __ffma2_rn(__fadd2_rn(r, m2), neg, m2);
         w[0][e] = pack2(d0.x, d0.y);
         w[1][e] = pack2(d1.x, d1.y);
         w[2][e] = pack2(d2.x, d2.y);
@@ -734,6 +744,32 @@ __device__ __forceinline__ void issue_x7_pair(uint32_t d_lead, uint32_t Np, uint
         tc::mma_bf16(d_rest, ad + a1, bd + b1, i1, 1u);               // d1 p1
         tc::mma_bf16(d_rest, ad + 2 * a1, bd, i1, 1u);                // d2 p0
         tc::mma_bf16(d_rest, ad, bd + 3 * b1, i1, 1u);                // d0 p3
+    }
+}
+
+// The same for pass B: operand and matrix strides of their own, a K-chunk may continue the sums
+// (`cont`), and axes longer than 128 points take 7 MMAs (2 Np columns would pass 256).
+__device__ __forceinline__ void issue_x7_z(uint32_t d_lead, uint32_t Np, uint32_t a_base, uint32_t a_piece, uint32_t a_sbo,
+                                           uint32_t b_base, uint32_t b_piece, uint32_t b_sbo, int ksteps, bool cont)
+{
+    uint64_t ad = tc::smem_desc(a_base, 128u, a_sbo), bd = tc::smem_desc(b_base, 128u, b_sbo);
+    const uint64_t a1 = a_piece >> 4, b1 = b_piece >> 4;
+    const uint32_t i1 = tc::instr_desc(false, int(Np)), i2 = tc::instr_desc(false, int(min(2 * Np, 256u)));
+    const uint32_t d_rest = d_lead + Np;
+#pragma unroll 1
+    for (int ks = 0; ks < ksteps; ++ks, ad += 16, bd += 16) {
+        const uint32_t acc = cont || ks > 0 ? 1u : 0u;
+        if (Np <= 128) {
+            tc::mma_bf16(d_lead, ad, bd, i2, acc);                    // d0 p0 | d0 p1
+        } else {
+            tc::mma_bf16(d_lead, ad, bd, i1, acc);
+            tc::mma_bf16(d_rest, ad, bd + b1, i1, acc);
+        }
+        tc::mma_bf16(d_rest, ad + a1, bd, i1, 1u);
+        tc::mma_bf16(d_rest, ad, bd + 2 * b1, i1, 1u);
+        tc::mma_bf16(d_rest, ad + a1, bd + b1, i1, 1u);
+        tc::mma_bf16(d_rest, ad + 2 * a1, bd, i1, 1u);
+        tc::mma_bf16(d_rest, ad, bd + 3 * b1, i1, 1u);
     }
 }
 
@@ -1383,6 +1419,338 @@ __global__ void __launch_bounds__(kRows * TPR + 64, (UPT <= 4 ? 2 : 1)) zpass_ke
     }
 }
 
+// Pass B, direct form: the tiles, products and roundings of zpass_kernel, laid out as the direct
+// slice form.  A group of NT threads owns a tile of 128 pencils, lane = pencil, each thread
+// 8-long units of z (u = part + g parts); the first warp issues the MMAs.  The values between
+// the two GEMMs stay in registers (FP32 hi, lo as bf16) instead of going through the operand
+// image, f(Lambda) arrives as (hi, lo) pairs during the forward GEMM.
+//   STREAM = false: both matrix images resident, one or two groups per SM.
+//   STREAM = true (long axes): one group of 512, the images pass through `nbuf` buffers as
+//     K-chunks of KC; the thread that issues the MMAs also issues the copies: those of the first
+//     nbuf chunks when the previous GEMM has finished, the others as the chunks are consumed.
+struct ZDArgs {
+    long ntiles;
+    int tpfz, R, n3, Kp;
+    long N;
+    const float *in;
+    float *out;
+    const float2 *F;             // f(Lambda) (hi, lo), natural layout (c R + r)
+    const uint8_t *imgF, *imgI;  // whole images, or nkc chunks each
+    uint32_t img_bytes;          // of one image or chunk
+    int KC, nkc, nbuf;
+    uint32_t offA, a_bytes, offCs, offRm, offBar;
+    int tcols, tmem_cols, groups;
+    int *err;
+};
+
+template <int NT, int UPT, bool STREAM>
+__global__ void __launch_bounds__(512, 1) zpass_direct_kernel(const __grid_constant__ ZDArgs a)
+{
+    extern __shared__ __align__(1024) uint8_t smem[];
+    constexpr int kParts = NT / kRows;
+    constexpr int FD = UPT < 3 ? UPT : UPT <= 4 ? 3 : 2;   // units of f(Lambda) in flight
+    const int grp = STREAM ? 0 : threadIdx.x / NT, tid = threadIdx.x - grp * NT;
+    const int warp = tid >> 5, lane = tid & 31;
+    uint8_t *sA = smem + a.offA + size_t(grp) * a.a_bytes;
+    float *csF = reinterpret_cast<float *>(smem + a.offCs), *csI = csF + a.Kp;
+    uint32_t *rm1 = reinterpret_cast<uint32_t *>(smem + a.offRm) + grp * 2 * kRows, *rm2 = rm1 + kRows;
+    uint64_t *bar_d = reinterpret_cast<uint64_t *>(smem + a.offBar) + grp;
+    uint64_t *bfull = reinterpret_cast<uint64_t *>(smem + a.offBar) + 2, *bempty = bfull + 16;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(bempty + 16);
+    int *sflag = reinterpret_cast<int *>(tslot + 1);
+    const int Kp = a.Kp, KC = STREAM ? a.KC : a.Kp;
+    const uint32_t sbo = uint32_t(Kp) * 16u, a_piece = uint32_t(kRows) * Kp * 2u;
+    const uint32_t b_piece = uint32_t(Kp) * KC * 2u, b_sbo = uint32_t(KC) * 16u;
+
+    if (!STREAM)
+        for (uint32_t i = threadIdx.x * 16; i < a.img_bytes; i += blockDim.x * 16) {
+            *reinterpret_cast<uint4 *>(smem + i) = *reinterpret_cast<const uint4 *>(a.imgF + i);
+            *reinterpret_cast<uint4 *>(smem + a.img_bytes + i) = *reinterpret_cast<const uint4 *>(a.imgI + i);
+        }
+    for (uint32_t i = threadIdx.x * 16; i < uint32_t(a.groups) * a.a_bytes; i += blockDim.x * 16)
+        *reinterpret_cast<uint4 *>(smem + a.offA + i) = make_uint4(0, 0, 0, 0);
+    for (int i = threadIdx.x; i < Kp; i += blockDim.x) {   // column scales (the same in every chunk)
+        csF[i] = reinterpret_cast<const float *>(a.imgF + size_t(kMatDig) * b_piece)[i];
+        csI[i] = reinterpret_cast<const float *>(a.imgI + size_t(kMatDig) * b_piece)[i];
+    }
+    for (int i = tid; i < 2 * kRows; i += NT) rm1[i] = 0u;
+    if (tid == 0) tc::mbar_init(bar_d, 1);
+    if (threadIdx.x == 0) {
+        *sflag = 0;
+        if (STREAM)
+            for (int b = 0; b < a.nbuf; ++b) {
+                tc::mbar_init(bfull + b, 1);
+                tc::mbar_init(bempty + b, 1);
+            }
+    }
+    if (threadIdx.x < 32) tc::tmem_alloc(tslot, uint32_t(a.tmem_cols));
+    tc::fence_proxy_async_smem();
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tmem0 = *tslot, tmem = tmem0 + uint32_t(grp * a.tcols);
+    const int quarter = warp & 3, dq = warp >> 2;
+    const int row = quarter * 32 + lane;
+    const uint32_t lane_q = uint32_t(quarter * 32) << 16;
+    const int n3 = a.n3, R = a.R, bar_id = 1 + grp;
+    uint8_t *arow = sA + img_at(row, 0, sbo);
+
+    const long stride = long(gridDim.x) * a.groups;
+    const long first = long(blockIdx.x) * a.groups + grp;
+    long p = first / a.tpfz;
+    int rt = int(first - p * a.tpfz);
+    const long dp = stride / a.tpfz;
+    const int dr = int(stride - dp * a.tpfz);
+    const long nfields = a.ntiles / a.tpfz;
+    uint32_t ph = 0;
+
+    // ---- streamed chunks (thread 0): buffer and phase parity of the next load and the next use,
+    //      kept by increments (a division per chunk would cost more than its MMAs) ----
+    int ld_slot = 0, us_slot = 0, ld_count = 0;   // ld_count: chunks of the current GEMM loaded so far
+    uint32_t us_par = 0, fills = 0;               // fills: buffers that have been filled at least once
+    auto load_chunk = [&](int g) {                // chunk ld_count into the next buffer, which is free
+        tc::mbar_arrive_expect_tx(bfull + ld_slot, a.img_bytes);
+        bulk_load(smem + uint32_t(ld_slot) * a.img_bytes, (g ? a.imgI : a.imgF) + size_t(ld_count) * a.img_bytes, a.img_bytes,
+                  bfull + ld_slot);
+        fills = max(fills, uint32_t(ld_slot) + 1u);
+        ld_slot = ld_slot + 1 == a.nbuf ? 0 : ld_slot + 1;
+        ++ld_count;
+    };
+    auto load_first = [&](int g) {           // when the previous GEMM has finished
+        if (STREAM && tid == 0) {
+            ld_count = 0;
+            for (int kc = 0; kc < min(a.nbuf, a.nkc); ++kc) load_chunk(g);
+        }
+    };
+    auto wait_d = [&]() {
+        if (!tc::mbar_wait_timed(bar_d, ph, kWaitNs)) atomicExch(sflag, 1);
+        ph ^= 1u;
+        tc::tc_fence_after();
+    };
+    // one GEMM over the whole operand image (lane 0 of warp 0)
+    auto gemm = [&](int g) {
+        const uint32_t ab = tc::smem_addr(sA);
+        if (!STREAM) {
+            issue_x7_z(tmem, uint32_t(Kp), ab, a_piece, sbo, tc::smem_addr(smem + (g ? a.img_bytes : 0u)), b_piece, sbo, Kp / 16, false);
+        } else {
+            int pv_slot = 0;
+            uint32_t pv_par = 0;
+            for (int kc = 0; kc < a.nkc; ++kc) {
+                if (!tc::mbar_wait_timed(bfull + us_slot, us_par, kWaitNs)) {
+                    atomicExch(sflag, 1);
+                    return;
+                }
+                issue_x7_z(tmem, uint32_t(Kp), ab + uint32_t(kc * KC) * 16u, a_piece, sbo,
+                           tc::smem_addr(smem) + uint32_t(us_slot) * a.img_bytes, b_piece, b_sbo, KC / 16, kc > 0);
+                tc::mma_commit(bempty + us_slot);
+                // the buffer of the chunk before this one takes the next chunk of this GEMM
+                if (kc > 0 && ld_count < a.nkc) {
+                    if (!tc::mbar_wait_timed(bempty + pv_slot, pv_par, kWaitNs)) {
+                        atomicExch(sflag, 1);
+                        return;
+                    }
+                    load_chunk(g);
+                }
+                pv_slot = us_slot;
+                pv_par = us_par;
+                if (++us_slot == a.nbuf) {
+                    us_slot = 0;
+                    us_par ^= 1u;
+                }
+            }
+        }
+        tc::mma_commit(bar_d);
+    };
+    auto handoff = [&](int g) {
+        tc::fence_proxy_async_smem();
+        tc::tc_fence_before();
+        if (tc::bar_red_or(bar_id, NT, *sflag != 0)) return true;
+        if (warp == 0) {
+            tc::tc_fence_after();
+            if (lane == 0) gemm(g);
+            __syncwarp();
+        }
+        return false;
+    };
+
+    float x[UPT][8];
+    auto prefetch = [&](long pp, int t) {
+        const int r = t * kRows + row;
+        const float *src = a.in + size_t(pp) * a.N + min(r, R - 1);
+#pragma unroll
+        for (int g = 0; g < UPT; ++g) {
+            const int z0 = 8 * (dq + g * kParts);
+            const float *q = src + size_t(z0) * R;
+            if (z0 + 8 <= n3) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) x[g][e] = q[e * R];
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) x[g][e] = z0 + e < n3 ? q[e * R] : 0.f;
+            }
+        }
+    };
+    if (p < nfields) {
+        prefetch(p, rt);
+        load_first(0);
+    }
+    while (p < nfields) {
+        const int r0 = rt * kRows + row;
+        const bool act = r0 < R;
+        const int r = min(r0, R - 1);      // rows past the field repeat the last one and are not stored
+        // ---- forward operand ----
+        {
+            float mx = 0.f;
+#pragma unroll
+            for (int g = 0; g < UPT; ++g) mx = fmaxf(mx, max8(x[g]));
+            atomicMax(rm1 + row, __float_as_uint(mx));
+        }
+        tc::bar_sync(bar_id, NT);
+        float sc, rs_f, rs_i;
+        row_scales(__uint_as_float(rm1[row]), sc, rs_f);
+#pragma unroll
+        for (int g = 0; g < UPT; ++g) {
+            const int u = dq + g * kParts;
+            if (8 * u < n3) store_digits8<false>(arow + u * 128, a_piece, x[g], x[g], sc);
+        }
+        if (handoff(0)) break;
+        rm2[row] = 0u;
+        // ---- while the forward GEMM runs: f(Lambda) of the first units ----
+        float2 f[FD][8];
+        auto load_f = [&](int g) {
+            const int c0 = 8 * (dq + g * kParts);
+            const float2 *q = a.F + size_t(c0) * R + r;
+            if (c0 + 8 <= n3) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) f[g % FD][e] = q[e * R];
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) f[g % FD][e] = c0 + e < n3 ? q[e * R] : make_float2(0.f, 0.f);
+            }
+        };
+#pragma unroll
+        for (int g = 0; g < FD; ++g) load_f(g);
+        wait_d();
+        load_first(1);
+        // ---- middle: D f(Lambda) as FP32 hi and bf16 lo, in registers ----
+        uint32_t lo[UPT][4];
+        float mx2 = 0.f;
+#pragma unroll
+        for (int g = 0; g < UPT; ++g) {
+            const int u = dq + g * kParts;
+            if (8 * u < n3) {   // uniform across the warp
+                uint32_t q0[8], q1[8];
+                tc::tmem_ld8_issue(tmem + lane_q + uint32_t(8 * u), q0);
+                tc::tmem_ld8_issue(tmem + lane_q + uint32_t(Kp + 8 * u), q1);
+                tc::tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    tc::order_after_wait(q0[e]);
+                    tc::order_after_wait(q1[e]);
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    // TwoSum of the accumulators, times the scales, times f (hi and lo)
+                    const float2 a0 = make_float2(__uint_as_float(q0[2 * e]), __uint_as_float(q0[2 * e + 1]));
+                    const float2 a1 = make_float2(__uint_as_float(q1[2 * e]), __uint_as_float(q1[2 * e + 1]));
+                    const float2 fhh = make_float2(f[g % FD][2 * e].x, f[g % FD][2 * e + 1].x);
+                    const float2 fll = make_float2(f[g % FD][2 * e].y, f[g % FD][2 * e + 1].y);
+                    const float2 scl = __fmul2_rn(f2(rs_f), *reinterpret_cast<const float2 *>(csF + 8 * u + 2 * e));
+                    const float2 h0 = __fadd2_rn(a0, a1);
+                    const float2 bp = sub2(h0, a0);
+                    const float2 l0 = __fmul2_rn(__fadd2_rn(sub2(a0, sub2(h0, bp)), sub2(a1, bp)), scl);
+                    const float2 h = __fmul2_rn(h0, scl);
+                    const float2 prh = __fmul2_rn(h, fhh);   // zero past n3 (f = 0 there)
+                    const float2 prl = __fadd2_rn(__ffma2_rn(h, fhh, __fmul2_rn(prh, f2(-1.f))),
+                                                  __ffma2_rn(h, fll, __fmul2_rn(l0, fhh)));
+                    x[g][2 * e] = prh.x;
+                    x[g][2 * e + 1] = prh.y;
+                    const __nv_bfloat162 lb = __float22bfloat162_rn(prl);
+                    lo[g][e] = *reinterpret_cast<const uint32_t *>(&lb);
+                }
+                mx2 = fmaxf(mx2, max8(x[g]));
+            }
+            if (g + FD < UPT) load_f(g + FD);
+        }
+        tc::tc_fence_before();
+        atomicMax(rm2 + row, __float_as_uint(mx2));
+        tc::bar_sync(bar_id, NT);
+        rm1[row] = 0u;
+        row_scales(__uint_as_float(rm2[row]), sc, rs_i);
+#pragma unroll
+        for (int g = 0; g < UPT; ++g) {
+            const int u = dq + g * kParts;
+            if (8 * u < n3) {
+                float l[8];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    l[2 * e] = __uint_as_float(lo[g][e] << 16);
+                    l[2 * e + 1] = __uint_as_float(lo[g][e] & 0xffff0000u);
+                }
+                store_digits8<true>(arow + u * 128, a_piece, x[g], l, sc);
+            }
+        }
+        if (handoff(1)) break;
+        long np = p + dp;
+        int nr = rt + dr;
+        if (nr >= a.tpfz) {
+            nr -= a.tpfz;
+            ++np;
+        }
+        if (np < nfields) prefetch(np, nr);   // the next tile, while the inverse GEMM runs
+        wait_d();
+        if (np < nfields) load_first(0);
+        // ---- inverse result -> (r, z) of the output field ----
+        float *dst = a.out + size_t(p) * a.N + r;
+#pragma unroll
+        for (int g = 0; g < UPT; ++g) {
+            const int u = dq + g * kParts;
+            if (8 * u >= n3) break;
+            uint32_t q0[8], q1[8];
+            tc::tmem_ld8_issue(tmem + lane_q + uint32_t(8 * u), q0);
+            tc::tmem_ld8_issue(tmem + lane_q + uint32_t(Kp + 8 * u), q1);
+            tc::tmem_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                tc::order_after_wait(q0[e]);
+                tc::order_after_wait(q1[e]);
+            }
+            float v[8];
+            combine8(q0, q1, rs_i, csI + 8 * u, v);
+            if (act) {
+                float *q = dst + size_t(8 * u) * R;
+                if (8 * u + 8 <= n3) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) q[e * R] = v[e];
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        if (8 * u + e < n3) q[e * R] = v[e];
+                }
+            }
+        }
+        tc::tc_fence_before();
+        p = np;
+        rt = nr;
+    }
+    if (STREAM && tid == 0 && *sflag) {
+        // a run that gave up leaves copies that nothing has waited for: none may target shared
+        // memory at exit.  The last fill of a buffer before ld_slot has the parity of the next
+        // load's pass, of the others the one before; both are waited for (one is over already).
+        for (uint32_t b = 0; b < fills; ++b) {
+            tc::mbar_wait_timed(bfull + b, 0u, kWaitNs / 4);
+            tc::mbar_wait_timed(bfull + b, 1u, kWaitNs / 4);
+        }
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x == 0 && *sflag) atomicExch(a.err, 1);
+    if (threadIdx.x < 32) {
+        tc::tc_fence_after();
+        tc::tmem_dealloc(tmem0, uint32_t(a.tmem_cols));
+    }
+}
+
 // ---- host: matrix images -----------------------------------------------------------------
 // Image of C(n, k), n < nout rows (outputs), k < nk (contraction), in a WN x Kp block of
 // rows n0.. and contraction indices k0..: 4 base-512 digit planes (every row scaled by the
@@ -1543,6 +1911,7 @@ bool slice_direct_layout(const Plan &P, SliceDLayout &L)
     const int n1 = P.n[0], n2 = P.n[1];
     const int Kp1 = pad16i(n1), Kp2 = pad16i(n2);
     L = SliceDLayout{};
+    if (P.t3_stage >= 0 || P.t3_pipe >= 0) return false;   // a form asked for by hand
     L.G = kRows / std::max(n1, n2);
     L.Pj = (n2 + 3) & ~3;
     if (((L.Pj / 4) & 1) == 0) L.Pj += 4;   // odd number of 16-byte units: conflict-free rows
@@ -1635,6 +2004,45 @@ bool z_layout(int n3, ZLayout &L, int want_wn = 0, int want_nbuf = 0)
         }
     }
     return false;
+}
+
+// Layout of the direct form of pass B.
+struct ZDLayout {
+    size_t smem;
+    uint32_t img_bytes, offA, a_bytes, offCs, offRm, offBar;
+    int stream, KC, nkc, nbuf, groups, nt, upt, tcols, tmem_cols;
+};
+
+bool z_direct_layout(int n3, ZDLayout &L)
+{
+    const int Kp = pad16i(n3), nu = (n3 + 7) / 8;
+    auto finish = [&](int nt, int groups, bool stream) {
+        L = ZDLayout{};
+        L.nt = nt;
+        L.groups = groups;
+        L.stream = stream ? 1 : 0;
+        L.upt = (nu + nt / kRows - 1) / (nt / kRows);
+        L.KC = stream ? 16 : Kp;
+        L.nkc = Kp / L.KC;
+        L.img_bytes = uint32_t(mat_image_bytes(Kp, L.KC));
+        L.a_bytes = 3u * kRows * Kp * 2u;
+        const size_t tail = 2 * size_t(Kp) * 4 + size_t(groups) * 2 * kRows * 4 + (2 + 32) * 8 + 64;
+        L.nbuf = 2;
+        if (stream) L.nbuf = int(std::min<size_t>(16, (kSmemLimit - L.a_bytes - 1024 - tail) / L.img_bytes));
+        L.offA = uint32_t(align_up(size_t(L.nbuf) * L.img_bytes, 1024));
+        L.offCs = L.offA + uint32_t(groups) * L.a_bytes;
+        L.offRm = L.offCs + 2 * uint32_t(Kp) * 4;
+        L.offBar = uint32_t(align_up(L.offRm + size_t(groups) * 2 * kRows * 4, 16));
+        L.smem = L.offBar + (2 + 32) * 8 + 16;
+        L.tcols = 2 * Kp;
+        L.tmem_cols = groups * 2 * Kp <= 512 ? tmem_pow2(groups * 2 * Kp) : 1024;
+        return L.smem <= kSmemLimit && L.tmem_cols <= 512 && L.upt <= (stream ? 7 : 4) && L.nbuf >= 2;
+    };
+    const size_t two_per_sm = 233472 / 2 - 1024;
+    if (finish(256, 1, false) && L.smem <= two_per_sm && L.tmem_cols <= 256) return true;
+    if (finish(256, 2, false)) return true;
+    if (finish(512, 1, false)) return true;
+    return finish(512, 1, true);
 }
 
 }  // namespace
@@ -1758,20 +2166,26 @@ int tc3_upload(Plan &P)
                 }
             }
     }
-    // z: NB blocks of WN outputs each
+    // z: the direct form's whole image or K-chunks, or (a choice made by hand) NB blocks
+    ZDLayout ZD;
+    const bool zdirect = P.t3_zwn == 0 && z_direct_layout(P.n[2], ZD);
     ZLayout Z;
     if (!z_layout(P.n[2], Z, P.t3_zwn, P.t3_znbuf)) z_layout(P.n[2], Z);
     {
         const int nd = P.n[2], Kp = pad16i(nd);
         const std::vector<double> &V = P.V[2];
+        const int nblk = zdirect ? ZD.nkc : Z.NB;
+        const size_t blk = zdirect ? ZD.img_bytes : Z.blk_bytes;
         for (int inv = 0; inv < 2; ++inv) {
-            std::vector<uint8_t> img(size_t(Z.NB) * Z.blk_bytes, 0);
+            std::vector<uint8_t> img(size_t(nblk) * blk, 0);
             auto coef = [&](int n, int k) {
                 return inv ? V[size_t(n) + size_t(nd) * k] : V[size_t(k) + size_t(nd) * n];
             };
-            for (int nb = 0; nb < Z.NB; ++nb) {
-                uint8_t *dst = img.data() + size_t(nb) * Z.blk_bytes;
-                if (Z.kchunk)   // all outputs, contraction indices nb KC ..
+            for (int nb = 0; nb < nblk; ++nb) {
+                uint8_t *dst = img.data() + size_t(nb) * blk;
+                if (zdirect)
+                    build_block(dst, Kp, ZD.KC, 0, nd, nd, coef, nb * ZD.KC);
+                else if (Z.kchunk)   // all outputs, contraction indices nb KC ..
                     build_block(dst, Z.NC, Z.KC, 0, nd, nd, coef, nb * Z.KC);
                 else
                     build_block(dst, Z.WN, Kp, nb * Z.WN, nd, nd, coef);
@@ -1781,13 +2195,13 @@ int tc3_upload(Plan &P)
             EXX_CUDA(cudaMemcpy(b.p, img.data(), img.size(), cudaMemcpyHostToDevice));
         }
     }
-    // f(Lambda) in the natural layout as FP32 hi and lo planes
+    // f(Lambda) in the natural layout, FP32 hi and lo: as pairs (direct form) or as two planes
     {
         std::vector<float> fl(2 * size_t(P.N));
         for (size_t i = 0; i < size_t(P.N); ++i) {
-            const float h = float(P.F[i]);
-            fl[i] = h;
-            fl[size_t(P.N) + i] = float(P.F[i] - double(h));
+            const float h = float(P.F[i]), l = float(P.F[i] - double(h));
+            fl[zdirect ? 2 * i : i] = h;
+            fl[zdirect ? 2 * i + 1 : size_t(P.N) + i] = l;
         }
         if (int rc = dev_reserve(P.F32n, fl.size() * sizeof(float))) return rc;
         EXX_CUDA(cudaMemcpy(P.F32n.p, fl.data(), fl.size() * sizeof(float), cudaMemcpyHostToDevice));
@@ -1924,7 +2338,57 @@ int tc3_solve_batch(Plan &P, const int2 *pairs_d, int nfields, float *bufA, floa
     };
     if (int rc = slice(true, nullptr, bufA, EXX_TIMING_PASS1)) return rc;
     // pass B
-    {
+    ZDLayout ZD;
+    if (P.t3_zwn == 0 && z_direct_layout(n3, ZD)) {
+        ZDArgs a{};
+        a.R = n1 * n2;
+        a.tpfz = (a.R + kRows - 1) / kRows;
+        a.ntiles = long(nfields) * a.tpfz;
+        a.n3 = n3;
+        a.Kp = pad16i(n3);
+        a.N = P.N;
+        a.in = bufA;
+        a.out = bufB;
+        a.F = static_cast<const float2 *>(P.F32n.p);
+        a.imgF = static_cast<const uint8_t *>(P.t3img[2][0].p);
+        a.imgI = static_cast<const uint8_t *>(P.t3img[2][1].p);
+        a.img_bytes = ZD.img_bytes;
+        a.KC = ZD.KC;
+        a.nkc = ZD.nkc;
+        a.nbuf = ZD.nbuf;
+        a.offA = ZD.offA;
+        a.a_bytes = ZD.a_bytes;
+        a.offCs = ZD.offCs;
+        a.offRm = ZD.offRm;
+        a.offBar = ZD.offBar;
+        a.tcols = ZD.tcols;
+        a.tmem_cols = ZD.tmem_cols;
+        a.groups = ZD.groups;
+        a.err = static_cast<int *>(P.err_d.p);
+        void (*kern)(const ZDArgs) = nullptr;
+        if (ZD.stream) {
+            kern = ZD.upt <= 4   ? zpass_direct_kernel<512, 4, true>
+                   : ZD.upt == 5 ? zpass_direct_kernel<512, 5, true>
+                   : ZD.upt == 6 ? zpass_direct_kernel<512, 6, true>
+                                 : zpass_direct_kernel<512, 7, true>;
+        } else if (ZD.nt == 512) {
+            kern = ZD.upt <= 3 ? zpass_direct_kernel<512, 3, false> : zpass_direct_kernel<512, 4, false>;
+        } else {
+            kern = ZD.upt <= 2   ? zpass_direct_kernel<256, 2, false>
+                   : ZD.upt == 3 ? zpass_direct_kernel<256, 3, false>
+                                 : zpass_direct_kernel<256, 4, false>;
+        }
+        const int threads = ZD.nt * ZD.groups;
+        size_t smem = ZD.smem;
+        int per_sm = 1;
+        if (int rc = launch_setup(kern, threads, smem, ZD.tmem_cols, per_sm)) return rc;
+        const int grid = int(std::min<long>((a.ntiles + ZD.groups - 1) / ZD.groups, long(P.num_sms) * per_sm));
+        const int tb = timing_begin(P, EXX_TIMING_PASS3, s);
+        kern<<<grid, threads, smem, s>>>(a);
+        timing_end(P, tb, s);
+        EXX_LAUNCH("zpass_direct_kernel");
+        P.launches++;
+    } else {
         ZLayout Z;
         if (!z_layout(n3, Z, P.t3_zwn, P.t3_znbuf)) z_layout(n3, Z);
         ZArgs a{};
