@@ -248,13 +248,15 @@ Schedule build_schedule(int n_occ, int n_in, bool aliased, int B, int max_pairs)
     }
     const int nt = n_in - t_begin;
     if (nt > 0) {
+        // one-sided blocks write only their J outputs, so a block may hold many occupied orbitals:
+        // as many (in steps of B) as let all column groups share one batch
         const int Gt = (nt + B - 1) / B;
-        for (int r = 0; r < Go; ++r) {
+        const int C = std::min(Go * B, std::max(B, max_pairs / nt / B * B));
+        for (int I0 = 0; I0 < n_occ; I0 += C) {
             std::vector<Block> blks;
             for (int t = 0; t < Gt; ++t) {
-                int g = (t + r) % Go;
-                int I0 = g * B, J0 = t_begin + t * B;
-                blks.push_back({I0, gsize(I0, n_occ), J0, std::min(B, n_in - J0), BLK_ONE_SIDE, 0});
+                const int J0 = t_begin + t * B;
+                blks.push_back({I0, std::min(C, n_occ - I0), J0, std::min(B, n_in - J0), BLK_ONE_SIDE, 0});
             }
             rounds.push_back(blks);
         }

@@ -186,6 +186,7 @@ struct Plan {
     Timing timing;
     // cached schedule
     int sched_key[4] = {-1, -1, -1, -1};
+    int sched_block = 8;  // orbitals per pair block of the cached schedule
     uint64_t epoch = 0;   // changes whenever device data or settings that launches read change
     Schedule sched;
 };

@@ -1113,97 +1113,181 @@ __device__ __forceinline__ void sub_product(float &s, float &c, float gh, float 
     c -= e + fmaf(gh, vl, gl * vh);
 }
 
+// The same for two sums at once in the packed FP32x2 instructions (nv = -v).
+template <bool HL>
+__device__ __forceinline__ void sub_product2(float2 &s, float2 &c, float2 gh, float2 gl, float2 v, float2 nv, float2 vl)
+{
+    const float2 neg = make_float2(-1.f, -1.f);
+    const float2 q = __fmul2_rn(gh, nv);
+    const float2 e = __ffma2_rn(gh, v, q);
+    const float2 t = __fadd2_rn(s, q);
+    const float2 bp = __ffma2_rn(s, neg, t);
+    const float2 w = __fadd2_rn(__ffma2_rn(__ffma2_rn(bp, neg, t), neg, s), __ffma2_rn(bp, neg, q));
+    float2 x = __ffma2_rn(gl, v, e);
+    if (HL) x = __ffma2_rn(gh, vl, x);
+    c = __fadd2_rn(c, __ffma2_rn(x, neg, w));
+    s = t;
+}
+
 __device__ __forceinline__ int diag_idx(int i, int j, int nI) { return i * nI - (i * (i - 1)) / 2 + (j - i); }
 
-constexpr int kAccBlock = 8;    // widest block edge whose one-sweep J sums live in registers
-constexpr int kAccWide = 16;   // widest edge of the one-sweep form with the J sums in shared memory
+// One launch per batch: CUDA block (x, y) = 128 grid points of the outputs of Block y, one
+// thread per point.  Blocks of one batch have disjoint outputs, so no atomics are needed.
+// Blocks of up to 2 NP columns: every pair field is read once, its value added to both sides.
+// The J-side sums and sources stay in registers, two columns per packed instruction; the next
+// row's fields are loaded while this row's are added.  Bound by the loads of V and of the
+// accumulators (2.25 B of those per 4 B of V at 16 x 16).  Against one column per instruction with
+// the sources re-read for every field, and 8-wide default blocks: 48^3 x 128 3.52 -> 1.69 ms,
+// 72 x 72 x 144 (75 of 96) 9.38 -> 5.84 ms.
+constexpr int kAccThreads = 128;
+struct AccArgs {
+    long N;
+    const Block *blocks;
+    const float *V;
+    long lo_off;
+    const float *g, *g_lo;
+    float *acc_hi, *acc_lo;
+};
 
-// One launch per batch: CUDA block (x, y) = 256 grid points of the outputs of Block y.
-// Blocks of one batch have disjoint outputs, so no atomics are needed.  WIDE: plans with
-// 16-orbital blocks keep the J-side sums of a block in shared memory ([j][thread], 32 KB
-// per CTA), so each pair field is still read once without spending registers on them.
-template <bool HL, bool WIDE>
-__global__ void __launch_bounds__(256, 6) tc_accum_kernel(long N, const Block *blocks, const float *__restrict__ V,
-                                                       long lo_off, const float *__restrict__ g,
-                                                       const float *__restrict__ g_lo, float *__restrict__ acc_hi,
-                                                       float *__restrict__ acc_lo)
+// A load the compiler keeps in its place (volatile), zero when !ok.
+__device__ __forceinline__ float ld_here(const float *p, bool ok)
+{
+    float x;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\tmov.f32 %0, 0f00000000;\n\t@p ld.global.nc.f32 %0, [%1];\n\t}"
+                 : "=f"(x)
+                 : "l"(p), "r"(int(ok)));
+    return x;
+}
+
+template <bool HL, int NP, int KIND>
+__device__ __forceinline__ void accum_block(const AccArgs &a, const Block &b, long r)
+{
+    constexpr bool kDiag = KIND == BLK_SYM_DIAG, kBoth = KIND != BLK_ONE_SIDE;
+    const long N = a.N;
+    const int nI = b.nI, J0 = kDiag ? b.I0 : b.J0, nJ = kDiag ? b.nI : b.nJ;
+    float2 sj[NP], cj[NP], gh[NP], gl[NP];
+#pragma unroll
+    for (int jp = 0; jp < NP; ++jp) {
+        const bool ok0 = 2 * jp < nJ, ok1 = 2 * jp + 1 < nJ;
+        const size_t o = size_t(J0 + 2 * jp) * N + r;
+        sj[jp] = make_float2(ok0 ? a.acc_hi[o] : 0.f, ok1 ? a.acc_hi[o + N] : 0.f);
+        cj[jp] = make_float2(ok0 ? a.acc_lo[o] : 0.f, ok1 ? a.acc_lo[o + N] : 0.f);
+        if (kBoth) {
+            gh[jp] = make_float2(ok0 ? a.g[o] : 0.f, ok1 ? a.g[o + N] : 0.f);
+            gl[jp] = make_float2(ok0 ? a.g_lo[o] : 0.f, ok1 ? a.g_lo[o + N] : 0.f);
+        }
+    }
+    auto finish = [&](int t, float s, float c) {
+        const float hs = s + c;
+        a.acc_lo[size_t(t) * N + r] = c - (hs - s);
+        a.acc_hi[size_t(t) * N + r] = hs;
+    };
+    const float *row = a.V + size_t(b.field0) * N + r;   // field (i, 0), also where a diagonal block has none
+    float2 v[NP];
+#pragma unroll
+    for (int jp = 0; jp < NP; ++jp)
+        v[jp] = make_float2(ld_here(row + 2 * jp * N, 2 * jp < nJ), ld_here(row + (2 * jp + 1) * N, 2 * jp + 1 < nJ));
+#pragma unroll 1
+    for (int i = 0; i < nI; ++i) {
+        const size_t oi = size_t(b.I0 + i) * N + r;
+        const float gih = a.g[oi], gil = a.g_lo[oi];
+        const float2 gi = make_float2(gih, gih), gi_l = make_float2(gil, gil), neg = make_float2(-1.f, -1.f);
+        // the I side starts from its accumulator; on the diagonal it joins the J side below
+        float2 si = make_float2(kBoth && !kDiag ? a.acc_hi[oi] : 0.f, 0.f);
+        float2 ci = make_float2(kBoth && !kDiag ? a.acc_lo[oi] : 0.f, 0.f);
+        const float *next = row + size_t(kDiag ? nI - 1 - i : nJ) * N;
+        const bool more = i + 1 < nI;
+        // this row's fields have arrived before the next row's are asked for: loads share a few
+        // scoreboards, and a value waited for after newer loads on the same one waits for those
+        float2 w[NP];
+#pragma unroll
+        for (int jp = 0; jp < NP; ++jp) {
+            asm volatile("" : "+f"(v[jp].x), "+f"(v[jp].y));
+            w[jp] = v[jp];
+        }
+#pragma unroll
+        for (int jp = 0; jp < NP; ++jp) {   // a diagonal block holds j >= i only, the others count as zero
+            v[jp].x = ld_here(next + 2 * jp * N, more && 2 * jp < nJ && (!kDiag || 2 * jp > i));
+            v[jp].y = ld_here(next + (2 * jp + 1) * N, more && 2 * jp + 1 < nJ && (!kDiag || 2 * jp + 1 > i));
+        }
+#pragma unroll
+        for (int jp = 0; jp < NP; ++jp) {
+            float2 wl = make_float2(0.f, 0.f);
+            const bool ok0 = 2 * jp < nJ, ok1 = 2 * jp + 1 < nJ;
+            if (HL) {
+                wl.x = ok0 && (!kDiag || 2 * jp >= i) ? row[a.lo_off + 2 * jp * N] : 0.f;
+                wl.y = ok1 && (!kDiag || 2 * jp + 1 >= i) ? row[a.lo_off + (2 * jp + 1) * N] : 0.f;
+            }
+            if (!ok0 || (kDiag && 2 * jp + 1 < i)) continue;   // uniform
+            const float2 nw = __fmul2_rn(w[jp], neg);
+            sub_product2<HL>(sj[jp], cj[jp], gi, gi_l, w[jp], nw, wl);
+            if (kBoth) {
+                float2 x = w[jp], nx = nw, xl = wl;
+                if (kDiag) {   // field (i, i) belongs to one side only
+                    if (2 * jp == i) x.x = nx.x = xl.x = 0.f;
+                    if (2 * jp + 1 == i) x.y = nx.y = xl.y = 0.f;
+                }
+                sub_product2<HL>(si, ci, gh[jp], gl[jp], x, nx, xl);
+            }
+        }
+        row = next;
+        if (kBoth && !kDiag) {
+            two_sum_add(si.x, ci.x, si.y);
+            finish(b.I0 + i, si.x, ci.x + ci.y);
+        }
+        if (kDiag) {
+            two_sum_add(si.x, ci.x, si.y);
+            const float cs = ci.x + ci.y;
+#pragma unroll
+            for (int jp = 0; jp < NP; ++jp) {
+                if (2 * jp == i) {
+                    two_sum_add(sj[jp].x, cj[jp].x, si.x);
+                    cj[jp].x += cs;
+                }
+                if (2 * jp + 1 == i) {
+                    two_sum_add(sj[jp].y, cj[jp].y, si.x);
+                    cj[jp].y += cs;
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int jp = 0; jp < NP; ++jp) {
+        if (2 * jp < nJ) finish(J0 + 2 * jp, sj[jp].x, cj[jp].x);
+        if (2 * jp + 1 < nJ) finish(J0 + 2 * jp + 1, sj[jp].y, cj[jp].y);
+    }
+}
+
+template <bool HL, int NP>
+__global__ void __launch_bounds__(kAccThreads, NP > 4 ? 4 : 6) tc_accum_kernel(const __grid_constant__ AccArgs a)
+{
+    const Block b = a.blocks[blockIdx.y];
+    const long r = long(blockIdx.x) * kAccThreads + threadIdx.x;
+    if (r >= a.N) return;
+    if (b.kind == BLK_SYM_OFF) accum_block<HL, NP, BLK_SYM_OFF>(a, b, r);
+    else if (b.kind == BLK_SYM_DIAG) accum_block<HL, NP, BLK_SYM_DIAG>(a, b, r);
+    else accum_block<HL, NP, BLK_ONE_SIDE>(a, b, r);
+}
+
+// Blocks wider than 16 orbitals (exx_plan_set_batch takes up to 32): one output at a time.
+template <bool HL>
+__global__ void __launch_bounds__(256, 6) tc_accum_any_kernel(long N, const Block *blocks, const float *__restrict__ V,
+                                                              long lo_off, const float *__restrict__ g,
+                                                              const float *__restrict__ g_lo, float *__restrict__ acc_hi,
+                                                              float *__restrict__ acc_lo)
 {
     const Block b = blocks[blockIdx.y];
     const long r = long(blockIdx.x) * blockDim.x + threadIdx.x;
     if (r >= N) return;
     const float *Vb = V + size_t(b.field0) * N + r;
-    auto vh_at = [&](size_t fo) { return Vb[fo]; };
-    auto vl_at = [&](size_t fo) { return HL ? Vb[lo_off + fo] : 0.f; };
     auto add = [&](float &s, float &c, int src, size_t fo) {
-        sub_product(s, c, g[size_t(src) * N + r], g_lo[size_t(src) * N + r], vh_at(fo), vl_at(fo));
+        sub_product(s, c, g[size_t(src) * N + r], g_lo[size_t(src) * N + r], Vb[fo], HL ? Vb[lo_off + fo] : 0.f);
     };
     auto finish = [&](int t, float s, float c) {
         float hs = s + c;
         acc_lo[size_t(t) * N + r] = c - (hs - s);
         acc_hi[size_t(t) * N + r] = hs;
     };
-    if constexpr (WIDE) {
-        if (b.kind == BLK_SYM_OFF && b.nJ > kAccBlock && b.nJ <= kAccWide) {
-            __shared__ float shs[kAccWide][256], shc[kAccWide][256];
-            const int t = threadIdx.x;
-            for (int j = 0; j < b.nJ; ++j) {
-                shs[j][t] = acc_hi[size_t(b.J0 + j) * N + r];
-                shc[j][t] = acc_lo[size_t(b.J0 + j) * N + r];
-            }
-#pragma unroll 1
-            for (int i = 0; i < b.nI; ++i) {
-                const int oi = b.I0 + i;
-                const float gih = g[size_t(oi) * N + r], gil = g_lo[size_t(oi) * N + r];
-                float si = acc_hi[size_t(oi) * N + r], ci = acc_lo[size_t(oi) * N + r];
-#pragma unroll 4
-                for (int j = 0; j < b.nJ; ++j) {
-                    const size_t fo = size_t(i * b.nJ + j) * N;
-                    const float vh = vh_at(fo), vl = vl_at(fo);
-                    float sj = shs[j][t], cj = shc[j][t];
-                    sub_product(sj, cj, gih, gil, vh, vl);
-                    shs[j][t] = sj;
-                    shc[j][t] = cj;
-                    const size_t src = size_t(b.J0 + j) * N + r;
-                    sub_product(si, ci, g[src], g_lo[src], vh, vl);
-                }
-                finish(oi, si, ci);
-            }
-            for (int j = 0; j < b.nJ; ++j) finish(b.J0 + j, shs[j][t], shc[j][t]);
-            return;
-        }
-    }
-    if (b.kind == BLK_SYM_OFF && b.nJ <= kAccBlock) {
-        // Both sides in one sweep over the block's fields: field (i, j) adds to output J0+j
-        // (source I0+i) and to output I0+i (source J0+j), so each field is read from memory
-        // once. Per output the terms still come in the order of the other index, as below.
-        float sj[kAccBlock], cj[kAccBlock];
-#pragma unroll
-        for (int j = 0; j < kAccBlock; ++j)
-            if (j < b.nJ) {
-                sj[j] = acc_hi[size_t(b.J0 + j) * N + r];
-                cj[j] = acc_lo[size_t(b.J0 + j) * N + r];
-            }
-#pragma unroll 1
-        for (int i = 0; i < b.nI; ++i) {
-            const int oi = b.I0 + i;
-            const float gih = g[size_t(oi) * N + r], gil = g_lo[size_t(oi) * N + r];
-            float si = acc_hi[size_t(oi) * N + r], ci = acc_lo[size_t(oi) * N + r];
-#pragma unroll
-            for (int j = 0; j < kAccBlock; ++j)
-                if (j < b.nJ) {
-                    const size_t fo = size_t(i * b.nJ + j) * N;
-                    const float vh = vh_at(fo), vl = vl_at(fo);
-                    sub_product(sj[j], cj[j], gih, gil, vh, vl);
-                    const size_t src = size_t(b.J0 + j) * N + r;
-                    sub_product(si, ci, g[src], g_lo[src], vh, vl);
-                }
-            finish(oi, si, ci);
-        }
-#pragma unroll
-        for (int j = 0; j < kAccBlock; ++j)
-            if (j < b.nJ) finish(b.J0 + j, sj[j], cj[j]);
-        return;
-    }
     if (b.kind == BLK_SYM_DIAG) {
         for (int t = 0; t < b.nI; ++t) {
             const int o = b.I0 + t;
@@ -1614,21 +1698,20 @@ int tc_solve_batch(Plan &P, int prec, const int2 *pairs_d, int nfields, float *b
 
 int tc_accumulate(Plan &P, const Block *blocks_d, int nblocks, const float *V, cudaStream_t s)
 {
-    dim3 grid(unsigned((P.N + 255) / 256), unsigned(nblocks));
-    int tb = timing_begin(P, EXX_TIMING_ACCUM, s);
+    const int tb = timing_begin(P, EXX_TIMING_ACCUM, s);
     const float *g = static_cast<const float *>(P.g32.p), *g_lo = g + size_t(P.tc_n_occ) * P.N;
     float *ah = static_cast<float *>(P.acc_hi.p), *al = static_cast<float *>(P.acc_lo.p);
-    const bool wide = P.block_orbitals > kAccBlock;
-    if (prec_info(P.prec).hl) {
-        if (wide)
-            tc_accum_kernel<true, true><<<grid, 256, 0, s>>>(P.N, blocks_d, V, P.tc_lo_off, g, g_lo, ah, al);
-        else
-            tc_accum_kernel<true, false><<<grid, 256, 0, s>>>(P.N, blocks_d, V, P.tc_lo_off, g, g_lo, ah, al);
+    const bool hl = prec_info(P.prec).hl != 0;
+    const long lo = hl ? P.tc_lo_off : 0;
+    if (P.sched_block <= 16) {
+        const dim3 grid(unsigned((P.N + kAccThreads - 1) / kAccThreads), unsigned(nblocks));
+        auto kern = P.sched_block <= 8 ? (hl ? tc_accum_kernel<true, 4> : tc_accum_kernel<false, 4>)
+                                       : (hl ? tc_accum_kernel<true, 8> : tc_accum_kernel<false, 8>);
+        kern<<<grid, kAccThreads, 0, s>>>(AccArgs{P.N, blocks_d, V, lo, g, g_lo, ah, al});
     } else {
-        if (wide)
-            tc_accum_kernel<false, true><<<grid, 256, 0, s>>>(P.N, blocks_d, V, 0, g, g_lo, ah, al);
-        else
-            tc_accum_kernel<false, false><<<grid, 256, 0, s>>>(P.N, blocks_d, V, 0, g, g_lo, ah, al);
+        const dim3 grid(unsigned((P.N + 255) / 256), unsigned(nblocks));
+        auto kern = hl ? tc_accum_any_kernel<true> : tc_accum_any_kernel<false>;
+        kern<<<grid, 256, 0, s>>>(P.N, blocks_d, V, lo, g, g_lo, ah, al);
     }
     timing_end(P, tb, s);
     EXX_LAUNCH("tc_accum_kernel");
