@@ -660,18 +660,18 @@ __global__ void __launch_bounds__(kRows * TPR + 64, 2) slice_pass_kernel(const _
 // ---------------------------------------------------------------------------------------
 // Slice pass, direct form: the same tiles, digits, products and roundings as above with the
 // work laid out for instruction issue, which bounds these passes.
-//   * A group of NT threads owns a tile; two groups share an SM (two CTAs, or two groups of one
-//     CTA sharing the matrix images), so one group's CUDA-core phases run under the other's MMAs.
-//     No helper warps: the group's first warp issues the MMAs, and the next tile's input is
-//     loaded straight into registers while this tile's GEMMs run.
+//   * A group of NT threads owns a tile; two or three groups share an SM (CTAs of one group, or
+//     groups of one CTA sharing the matrix images), so one group's CUDA-core phases run under
+//     the others' MMAs.  No helper warps: the group's first warp issues the MMAs, and the next
+//     tile's input is copied to shared memory by the group's threads while this tile's GEMMs run.
 //   * The operand is cut in units of 8 elements of a row (one 16-byte store per digit plane),
 //     8 rows x 4 units per warp: every load is whole 32-byte sectors, every store
 //     conflict-free, and tiles of fewer than 128 rows spread over all threads.  A row's maximum
 //     is gathered by shared-memory atomics on the bit patterns of the unit maxima.
 //   * The transposed tile takes the place of the consumed operand image.
-// Per pair solve against the staged / pipelined forms: 72 x 72 x 144 points pass A 5.82 -> 3.83 us,
-// C 5.62 -> 3.24; 48^3 A 0.617 -> 0.530, C 0.584 -> 0.420; 117 x 117 x 119 (matrices resident instead
-// of streamed) A 12.6 -> 8.7, C 11.7 -> 5.5.  The bits of every result are the same.
+// Per pair solve, staged / pipelined form -> this: 72 x 72 x 144 points pass A 5.82 -> 3.40 us, C 5.62
+// -> 2.73; 48^3 A 0.617 -> 0.426, C 0.584 -> 0.360; 117 x 117 x 119 (matrices resident instead of
+// streamed) A 12.6 -> 8.7, C 11.7 -> 5.6.  The bits of every result are the same.
 struct SliceDArgs {
     int n1, n2, n3, G, tpf;
     long ntiles;
@@ -687,8 +687,9 @@ struct SliceDArgs {
     uint32_t offB2, offA, a_bytes, offRm, offBar;   // a_bytes: one group's operand / transposed tile
     uint32_t a_piece1, a_piece2;
     int Pj, tmem_cols, tcols;                       // tcols: TMEM columns of one group
-    int vec;                // rows of n1 floats start 16-byte aligned
-    int groups;             // groups per CTA
+    uint32_t offS, stg_plane;   // staged input: plane stride
+    int P1;                 // row pitch (floats) of the staged input
+    int cpw;                // bytes per asynchronous copy (rows start so aligned): 16, 8 or 4
     int *err;
 };
 
@@ -697,11 +698,10 @@ struct SliceDArgs {
 // out of M - (M - d) with its sign and the only constants are three magics and -1: 8 packed
 // operations for two elements (9 with lo), and no constant has to be rebuilt between them.
 template <bool LO>
-__device__ __forceinline__ void store_digits8(uint8_t *dst, uint32_t piece, const float (&h)[8], const float (&l)[8], float s)
+__device__ __forceinline__ void cut_digits8(uint32_t (&w)[3][4], const float (&h)[8], const float (&l)[8], float s)
 {
     const float2 m0 = f2(12582912.f), m1 = f2(12582912.f / 512.f), m2 = f2(12582912.f / 262144.f), neg = f2(-1.f);
     const float2 ns = f2(-s);
-    uint32_t w[3][4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         const float2 x = make_float2(h[2 * e], h[2 * e + 1]);
@@ -715,8 +715,23 @@ __device__ __forceinline__ void store_digits8(uint8_t *dst, uint32_t piece, cons
         w[1][e] = pack2(d1.x, d1.y);
         w[2][e] = pack2(d2.x, d2.y);
     }
+}
+template <bool LO>
+__device__ __forceinline__ void store_digits8(uint8_t *dst, uint32_t piece, const float (&h)[8], const float (&l)[8], float s)
+{
+    uint32_t w[3][4];
+    cut_digits8<LO>(w, h, l, s);
 #pragma unroll
     for (int q = 0; q < 3; ++q) *reinterpret_cast<uint4 *>(dst + q * piece) = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
+}
+// The same into TMEM: this warp's 32 rows, four columns of each digit plane (`plane` columns apart).
+template <bool LO>
+__device__ __forceinline__ void tmem_digits8(uint32_t dst, uint32_t plane, const float (&h)[8], const float (&l)[8], float s)
+{
+    uint32_t w[3][4];
+    cut_digits8<LO>(w, h, l, s);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) tc::tmem_st4(dst + uint32_t(q) * plane, w[q][0], w[q][1], w[q][2], w[q][3]);
 }
 
 __device__ __forceinline__ float max8(const float (&h)[8])
@@ -726,11 +741,11 @@ __device__ __forceinline__ float max8(const float (&h)[8])
     return fmaxf(fmaxf(a, b), fmaxf(fabsf(h[6]), fabsf(h[7])));
 }
 
-// The 7 digit products of one GEMM as 6 MMAs per 16-k step: d0 meets p0 and p1 in one MMA of
+// The 7 digit products of one GEMM (by a whole warp, el: tc::elect_one) as 6 MMAs per 16-k step: d0 meets p0 and p1 in one MMA of
 // 2 Np columns (lead and rest columns are neighbours, as are the two matrix digits).  Per column
 // the products of the rest accumulator keep issue_x7g's order.  Descriptors advance by additions.
 __device__ __forceinline__ void issue_x7_pair(uint32_t d_lead, uint32_t Np, uint32_t a_base, uint32_t a_piece, uint32_t b_base,
-                                              uint32_t b_piece, uint32_t sbo, int ksteps)
+                                              uint32_t b_piece, uint32_t sbo, int ksteps, uint32_t el)
 {
     uint64_t ad = tc::smem_desc(a_base, 128u, sbo), bd = tc::smem_desc(b_base, 128u, sbo);
     const uint64_t a1 = a_piece >> 4, b1 = b_piece >> 4;
@@ -738,19 +753,19 @@ __device__ __forceinline__ void issue_x7_pair(uint32_t d_lead, uint32_t Np, uint
     const uint32_t d_rest = d_lead + Np;
 #pragma unroll 1
     for (int ks = 0; ks < ksteps; ++ks, ad += 16, bd += 16) {
-        tc::mma_bf16(d_lead, ad, bd, i2, ks > 0 ? 1u : 0u);           // d0 p0 | d0 p1
-        tc::mma_bf16(d_rest, ad + a1, bd, i1, 1u);                    // d1 p0
-        tc::mma_bf16(d_rest, ad, bd + 2 * b1, i1, 1u);                // d0 p2
-        tc::mma_bf16(d_rest, ad + a1, bd + b1, i1, 1u);               // d1 p1
-        tc::mma_bf16(d_rest, ad + 2 * a1, bd, i1, 1u);                // d2 p0
-        tc::mma_bf16(d_rest, ad, bd + 3 * b1, i1, 1u);                // d0 p3
+        tc::mma_bf16_warp(d_lead, ad, bd, i2, ks > 0 ? 1u : 0u, el);           // d0 p0 | d0 p1
+        tc::mma_bf16_warp(d_rest, ad + a1, bd, i1, 1u, el);                    // d1 p0
+        tc::mma_bf16_warp(d_rest, ad, bd + 2 * b1, i1, 1u, el);                // d0 p2
+        tc::mma_bf16_warp(d_rest, ad + a1, bd + b1, i1, 1u, el);               // d1 p1
+        tc::mma_bf16_warp(d_rest, ad + 2 * a1, bd, i1, 1u, el);                // d2 p0
+        tc::mma_bf16_warp(d_rest, ad, bd + 3 * b1, i1, 1u, el);                // d0 p3
     }
 }
 
 // The same for pass B: operand and matrix strides of their own, a K-chunk may continue the sums
 // (`cont`), and axes longer than 128 points take 7 MMAs (2 Np columns would pass 256).
 __device__ __forceinline__ void issue_x7_z(uint32_t d_lead, uint32_t Np, uint32_t a_base, uint32_t a_piece, uint32_t a_sbo,
-                                           uint32_t b_base, uint32_t b_piece, uint32_t b_sbo, int ksteps, bool cont)
+                                           uint32_t b_base, uint32_t b_piece, uint32_t b_sbo, int ksteps, bool cont, uint32_t el)
 {
     uint64_t ad = tc::smem_desc(a_base, 128u, a_sbo), bd = tc::smem_desc(b_base, 128u, b_sbo);
     const uint64_t a1 = a_piece >> 4, b1 = b_piece >> 4;
@@ -760,16 +775,41 @@ __device__ __forceinline__ void issue_x7_z(uint32_t d_lead, uint32_t Np, uint32_
     for (int ks = 0; ks < ksteps; ++ks, ad += 16, bd += 16) {
         const uint32_t acc = cont || ks > 0 ? 1u : 0u;
         if (Np <= 128) {
-            tc::mma_bf16(d_lead, ad, bd, i2, acc);                    // d0 p0 | d0 p1
+            tc::mma_bf16_warp(d_lead, ad, bd, i2, acc, el);                    // d0 p0 | d0 p1
         } else {
-            tc::mma_bf16(d_lead, ad, bd, i1, acc);
-            tc::mma_bf16(d_rest, ad, bd + b1, i1, acc);
+            tc::mma_bf16_warp(d_lead, ad, bd, i1, acc, el);
+            tc::mma_bf16_warp(d_rest, ad, bd + b1, i1, acc, el);
         }
-        tc::mma_bf16(d_rest, ad + a1, bd, i1, 1u);
-        tc::mma_bf16(d_rest, ad, bd + 2 * b1, i1, 1u);
-        tc::mma_bf16(d_rest, ad + a1, bd + b1, i1, 1u);
-        tc::mma_bf16(d_rest, ad + 2 * a1, bd, i1, 1u);
-        tc::mma_bf16(d_rest, ad, bd + 3 * b1, i1, 1u);
+        tc::mma_bf16_warp(d_rest, ad + a1, bd, i1, 1u, el);
+        tc::mma_bf16_warp(d_rest, ad, bd + 2 * b1, i1, 1u, el);
+        tc::mma_bf16_warp(d_rest, ad + a1, bd + b1, i1, 1u, el);
+        tc::mma_bf16_warp(d_rest, ad + 2 * a1, bd, i1, 1u, el);
+        tc::mma_bf16_warp(d_rest, ad, bd + 3 * b1, i1, 1u, el);
+    }
+}
+
+// issue_x7_z with the data digits in TMEM (planes a_plane columns apart, 8 columns per 16-k step).
+__device__ __forceinline__ void issue_x7_ts(uint32_t d_lead, uint32_t Np, uint32_t a_tmem, uint32_t a_plane, uint32_t b_base,
+                                            uint32_t b_piece, uint32_t b_sbo, int ksteps, bool cont, uint32_t el)
+{
+    uint64_t bd = tc::smem_desc(b_base, 128u, b_sbo);
+    const uint64_t b1 = b_piece >> 4;
+    const uint32_t i1 = tc::instr_desc(false, int(Np)), i2 = tc::instr_desc(false, int(min(2 * Np, 256u)));
+    const uint32_t d_rest = d_lead + Np;
+#pragma unroll 1
+    for (int ks = 0; ks < ksteps; ++ks, a_tmem += 8, bd += 16) {
+        const uint32_t acc = cont || ks > 0 ? 1u : 0u;
+        if (Np <= 128) {
+            tc::mma_bf16_ts_warp(d_lead, a_tmem, bd, i2, acc, el);                    // d0 p0 | d0 p1
+        } else {
+            tc::mma_bf16_ts_warp(d_lead, a_tmem, bd, i1, acc, el);
+            tc::mma_bf16_ts_warp(d_rest, a_tmem, bd + b1, i1, acc, el);
+        }
+        tc::mma_bf16_ts_warp(d_rest, a_tmem + a_plane, bd, i1, 1u, el);
+        tc::mma_bf16_ts_warp(d_rest, a_tmem, bd + 2 * b1, i1, 1u, el);
+        tc::mma_bf16_ts_warp(d_rest, a_tmem + a_plane, bd + b1, i1, 1u, el);
+        tc::mma_bf16_ts_warp(d_rest, a_tmem + 2 * a_plane, bd, i1, 1u, el);
+        tc::mma_bf16_ts_warp(d_rest, a_tmem, bd + 3 * b1, i1, 1u, el);
     }
 }
 
@@ -787,20 +827,22 @@ __device__ __forceinline__ void combine8(uint32_t (&r0)[8], uint32_t (&r1)[8], f
     }
 }
 
-template <bool PAIR, int NT, int UPT>
-__global__ void __launch_bounds__(512, 1) slice_direct_kernel(const __grid_constant__ SliceDArgs a)
+template <bool PAIR, int NT, int UPT, int GROUPS, bool STG>
+__global__ void __launch_bounds__(NT * GROUPS, 512 / (NT * GROUPS) > 0 ? 512 / (NT * GROUPS) : 1) slice_direct_kernel(const __grid_constant__ SliceDArgs a)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     constexpr int kParts = NT / kRows;    // column parts of the drains
-    const int grp = threadIdx.x / NT, tid = threadIdx.x - grp * NT;
-    const int warp = tid >> 5, lane = tid & 31;
+    const int wid = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0);   // warp-uniform
+    const int grp = wid / (NT / 32), warp = wid - grp * (NT / 32), lane = threadIdx.x & 31, tid = warp * 32 + lane;
     uint8_t *sB1 = smem;
     uint8_t *sB2 = a.offB2 ? smem + a.offB2 : smem;
     uint8_t *sA = smem + a.offA + size_t(grp) * a.a_bytes;
     float *Ysm = reinterpret_cast<float *>(sA);
     uint32_t *rm1 = reinterpret_cast<uint32_t *>(smem + a.offRm) + grp * 2 * kRows, *rm2 = rm1 + kRows;
+    float *stg = reinterpret_cast<float *>(smem + a.offS + size_t(grp) * (PAIR ? 2 : 1) * a.stg_plane);
+    const float *stg1 = reinterpret_cast<const float *>(reinterpret_cast<const uint8_t *>(stg) + a.stg_plane);
     uint64_t *bar_d = reinterpret_cast<uint64_t *>(smem + a.offBar) + grp;
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + a.offBar + 16);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + a.offBar + 32);
     int *sflag = reinterpret_cast<int *>(tslot + 1);
 
     for (uint32_t i = threadIdx.x * 16; i < a.img1_bytes; i += blockDim.x * 16)
@@ -808,7 +850,7 @@ __global__ void __launch_bounds__(512, 1) slice_direct_kernel(const __grid_const
     if (a.offB2)
         for (uint32_t i = threadIdx.x * 16; i < a.img2_bytes; i += blockDim.x * 16)
             *reinterpret_cast<uint4 *>(sB2 + i) = *reinterpret_cast<const uint4 *>(a.img2 + i);
-    for (uint32_t i = threadIdx.x * 16; i < uint32_t(a.groups) * a.a_bytes; i += blockDim.x * 16)
+    for (uint32_t i = threadIdx.x * 16; i < uint32_t(GROUPS) * a.a_bytes; i += blockDim.x * 16)
         *reinterpret_cast<uint4 *>(smem + a.offA + i) = make_uint4(0, 0, 0, 0);
     for (int i = tid; i < 2 * kRows; i += NT) rm1[i] = 0u;
     if (tid == 0) tc::mbar_init(bar_d, 1);
@@ -818,7 +860,7 @@ __global__ void __launch_bounds__(512, 1) slice_direct_kernel(const __grid_const
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
-    const uint32_t tmem0 = *tslot, tmem = tmem0 + uint32_t(grp * a.tcols);
+    const uint32_t tmem0 = __shfl_sync(0xffffffffu, *tslot, 0), tmem = tmem0 + uint32_t(grp * a.tcols);
     const int n1 = a.n1, n2 = a.n2;
     const long R = long(n1) * n2;
     const int Kp1 = a.Kp1, Kp2 = a.Kp2;
@@ -844,15 +886,18 @@ __global__ void __launch_bounds__(512, 1) slice_direct_kernel(const __grid_const
     const uint32_t lane_q = uint32_t(quarter * 32) << 16;
     const int s1 = drow / n2, j1 = drow - s1 * n2, s2 = drow / n1, i2 = drow - s2 * n1;
 
-    const long stride = long(gridDim.x) * a.groups;
-    long p = (long(blockIdx.x) * a.groups + grp) / a.tpf;
-    int zt = int((long(blockIdx.x) * a.groups + grp) - p * a.tpf);
+    const long stride = long(gridDim.x) * GROUPS;
+    long p = (long(blockIdx.x) * GROUPS + grp) / a.tpf;
+    int zt = int((long(blockIdx.x) * GROUPS + grp) - p * a.tpf);
     const long dp = stride / a.tpf;
     const int dz = int(stride - dp * a.tpf);
     uint32_t ph = 0;
+    // GEMM complete: the first warp polls, the others sleep in the barrier (eight polling warps
+    // took a quarter of the issue slots from the other groups and from the warp issuing MMAs)
     auto wait_d = [&]() {
-        if (!tc::mbar_wait_timed(bar_d, ph, kWaitNs)) atomicExch(sflag, 1);
+        if (warp == 0 && !tc::mbar_wait_timed(bar_d, ph, kWaitNs)) atomicExch(sflag, 1);
         ph ^= 1u;
+        tc::bar_sync(bar_id, NT);
         tc::tc_fence_after();
     };
     // operand image complete: hand it to the MMAs of this group (true = stop on an error)
@@ -862,33 +907,75 @@ __global__ void __launch_bounds__(512, 1) slice_direct_kernel(const __grid_const
         if (tc::bar_red_or(bar_id, NT, *sflag != 0)) return true;
         if (warp == 0) {
             tc::tc_fence_after();
-            if (lane == 0) {
-                if (first)
-                    issue_x7_pair(tmem, uint32_t(Kp1), tc::smem_addr(sA), a.a_piece1, tc::smem_addr(sB1),
-                                  uint32_t(Kp1) * Kp1 * 2u, sbo1, Kp1 / 16);
-                else
-                    issue_x7_pair(tmem, uint32_t(Kp2), tc::smem_addr(sA), a.a_piece2, tc::smem_addr(sB2),
-                                  uint32_t(Kp2) * Kp2 * 2u, sbo2, Kp2 / 16);
-                tc::mma_commit(bar_d);
-            }
+            const uint32_t el = tc::elect_one();
+            if (first)
+                issue_x7_pair(tmem, uint32_t(Kp1), tc::smem_addr(sA), a.a_piece1, tc::smem_addr(sB1), uint32_t(Kp1) * Kp1 * 2u,
+                              sbo1, Kp1 / 16, el);
+            else
+                issue_x7_pair(tmem, uint32_t(Kp2), tc::smem_addr(sA), a.a_piece2, tc::smem_addr(sB2), uint32_t(Kp2) * Kp2 * 2u,
+                              sbo2, Kp2 / 16, el);
+            if (el) tc::mma_commit(bar_d);
             __syncwarp();
         }
         return false;
     };
-    // input of tile (pp, zz) for this thread's units: raw values of one or two rows
-    float x0[UPT][8], x1[UPT][8];
-    auto load8 = [&](const float *src, int k, bool ok, float (&v)[8]) {
-        if (a.vec) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float4 w = ok && k + 4 * h < n1 ? *reinterpret_cast<const float4 *>(src + 4 * h) : make_float4(0.f, 0.f, 0.f, 0.f);
-                v[4 * h] = w.x; v[4 * h + 1] = w.y; v[4 * h + 2] = w.z; v[4 * h + 3] = w.w;
-            }
+    // input of tile (pp, zz) into the staging rows (one plane or two, pitch P1), by asynchronous
+    // copies of `cpw` bytes: the tile's rows are consecutive in memory
+    const int cpe = a.cpw >> 2, cpr = n1 / cpe;          // floats per copy, copies per row
+    const int srow0 = tid / cpr, sc0 = tid - srow0 * cpr, sdr = NT / cpr, sdc = NT - sdr * cpr;
+    auto stage = [&](long pp, int zz) {
+        const int z0 = zz * a.G, R1 = min(a.G, a.n3 - z0) * n2;
+        const float *b0, *b1 = nullptr;
+        if (PAIR) {
+            const int2 mn = a.pairs[pp];
+            b0 = a.psi + size_t(a.occ_off + mn.x) * a.N + size_t(z0) * R;
+            b1 = a.psi + size_t(mn.y) * a.N + size_t(z0) * R;
         } else {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = ok && k + e < n1 ? src[e] : 0.f;
+            b0 = a.in + size_t(pp) * a.N + size_t(z0) * R;
+        }
+        int row = srow0, c = sc0, i = tid * cpe;
+        while (row < R1) {
+            float *d = stg + row * a.P1 + c * cpe;
+            float *d1 = const_cast<float *>(stg1) + row * a.P1 + c * cpe;
+            if (a.cpw == 16) {
+                tc::cp_async16(d, b0 + i);
+                if (PAIR) tc::cp_async16(d1, b1 + i);
+            } else if (a.cpw == 8) {
+                tc::cp_async8(d, b0 + i);
+                if (PAIR) tc::cp_async8(d1, b1 + i);
+            } else {
+                tc::cp_async4(d, b0 + i);
+                if (PAIR) tc::cp_async4(d1, b1 + i);
+            }
+            i += NT * cpe;
+            c += sdc;
+            row += sdr;
+            if (c >= cpr) {
+                c -= cpr;
+                ++row;
+            }
         }
     };
+    auto load8 = [&](const float *src, int k, bool ok, float (&v)[8]) {
+        if (!STG && a.cpw != 16) {   // unaligned rows in global memory
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = ok && k + e < n1 ? src[e] : 0.f;
+            return;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 w = ok && k + 4 * h < n1 ? *reinterpret_cast<const float4 *>(src + 4 * h) : make_float4(0.f, 0.f, 0.f, 0.f);
+            v[4 * h] = w.x; v[4 * h + 1] = w.y; v[4 * h + 2] = w.z; v[4 * h + 3] = w.w;
+        }
+        if (k + 8 > n1) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (k + e >= n1) v[e] = 0.f;   // pitch padding
+        }
+    };
+
+    // without staging (slices too wide for it): the same units straight into registers
+    float x0[UPT][8], x1[UPT][8];
     auto prefetch = [&](long pp, int zz) {
         const int z0 = zz * a.G, R1 = min(a.G, a.n3 - z0) * n2;
         const float *b0, *b1 = nullptr;
@@ -901,22 +988,33 @@ __global__ void __launch_bounds__(512, 1) slice_direct_kernel(const __grid_const
         }
 #pragma unroll
         for (int g = 0; g < UPT; ++g) {
-            const int row = ru1[g] & 255, k = (ru1[g] >> 8) * 8;
-            const bool ok = row < R1;
-            const int o = row * n1 + k;
-            load8(b0 + o, k, ok, x0[g]);
-            if (PAIR) load8(b1 + o, k, ok, x1[g]);
+            const int row = ru1[g] & 255, k = (ru1[g] >> 8) * 8, o = row * n1 + k;
+            load8(b0 + o, k, row < R1, x0[g]);
+            if (PAIR) load8(b1 + o, k, row < R1, x1[g]);
         }
     };
 
     const long nfields = a.ntiles / a.tpf;
-    if (p < nfields) prefetch(p, zt);
+    if (p < nfields) {
+        if (STG) {
+            stage(p, zt);
+            tc::cp_async_wait_all();
+            tc::bar_sync(bar_id, NT);
+        } else {
+            prefetch(p, zt);
+        }
+    }
     while (p < nfields) {
         const int z0 = zt * a.G, ns = min(a.G, a.n3 - z0);
         const int R1 = ns * n2, R2 = ns * n1;
         // ---- GEMM 1 operand: row (s, j), K = i: products (hi, rounding error lo), row maxima ----
 #pragma unroll
         for (int g = 0; g < UPT; ++g) {
+            if (STG) {
+                const int urow = ru1[g] & 255, uk = (ru1[g] >> 8) * 8, so = urow < R1 ? urow * a.P1 + uk : 0;
+                load8(stg + so, uk, urow < R1, x0[g]);
+                if (PAIR) load8(stg1 + so, uk, urow < R1, x1[g]);
+            }
             if (PAIR) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -942,14 +1040,16 @@ __global__ void __launch_bounds__(512, 1) slice_direct_kernel(const __grid_const
             }
         }
         if (handoff(true)) break;
-        // while GEMM 1 runs: the next tile's input, the second maxima cleared
+        // while GEMM 1 runs: the next tile's input (everyone has read this tile's), rm2 cleared.
+        // Copies, not loads: loads in flight hold the scoreboards that the shared-memory reads of
+        // the phases below wait for
         long np = p + dp;
         int nz = zt + dz;
         if (nz >= a.tpf) {
             nz -= a.tpf;
             ++np;
         }
-        if (np < nfields) prefetch(np, nz);
+        if (STG && np < nfields) stage(np, nz);
         if (tid < kRows) rm2[tid] = 0u;
         const float rs1 = [&] {
             float sc, inv;
@@ -972,8 +1072,17 @@ __global__ void __launch_bounds__(512, 1) slice_direct_kernel(const __grid_const
                     tc::order_after_wait(r0[e]);
                     tc::order_after_wait(r1[e]);
                 }
+                // the column scale of i' is the same for all of row (s, i') of GEMM 2: it goes into
+                // that row's scale (rs2), exactly, as all scales are powers of two
                 float v[8];
-                combine8(r0, r1, rs1, cs1 + 8 * u, v);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 w = __fmul2_rn(__fadd2_rn(make_float2(__uint_as_float(r0[2 * e]), __uint_as_float(r0[2 * e + 1])),
+                                                           make_float2(__uint_as_float(r1[2 * e]), __uint_as_float(r1[2 * e + 1]))),
+                                                f2(rs1));
+                    v[2 * e] = w.x;
+                    v[2 * e + 1] = w.y;
+                }
                 if (act) {
                     float *y = yb + 8 * u * a.Pj;
                     if (8 * u + 8 <= n1) {
@@ -1020,12 +1129,14 @@ __global__ void __launch_bounds__(512, 1) slice_direct_kernel(const __grid_const
                 store_digits8<false>(sA + img_at(row, ru2[g] >> 8, sbo2), a.a_piece2, y[g], y[g], sc);
             }
         }
+        if (STG) tc::cp_async_wait_all();   // this thread's part of the next tile; the barrier shows it to the others
         if (handoff(false)) break;
         const float rs2 = [&] {
             float sc, inv;
             row_scales(__uint_as_float(rm2[drow]), sc, inv);
-            return inv;
+            return inv * cs1[min(i2, n1 - 1)];
         }();
+        if (!STG && np < nfields) prefetch(np, nz);
         wait_d();
         // ---- GEMM 2 result -> the field at (z0 + s, j', i') ----
         if (quarter * 32 < R2) {
@@ -1424,10 +1535,14 @@ __global__ void __launch_bounds__(kRows * TPR + 64, (UPT <= 4 ? 2 : 1)) zpass_ke
 // 8-long units of z (u = part + g parts); the first warp issues the MMAs.  The values between
 // the two GEMMs stay in registers (FP32 hi, lo as bf16) instead of going through the operand
 // image, f(Lambda) arrives as (hi, lo) pairs during the forward GEMM.
-//   STREAM = false: both matrix images resident, one or two groups per SM.
+//   TS: the data digits live in TMEM (rows are lanes already), which takes the MMAs' 4 KB per
+//     instruction off shared memory: N / 2 cycles per MMA instead of (128 + N) / 4.
+//   STREAM = false: both matrix images resident, up to three groups per SM.
 //   STREAM = true (long axes): one group of 512, the images pass through `nbuf` buffers as
 //     K-chunks of KC; the thread that issues the MMAs also issues the copies: those of the first
 //     nbuf chunks when the previous GEMM has finished, the others as the chunks are consumed.
+// Per pair solve against zpass_kernel: 48^3 0.621 -> 0.292 us, 72 x 72 x 144 5.15 -> 3.14, 117 x 117 x
+// 119 8.9 -> 5.1.  Of that the MMA issue by a converged warp gave 0.373 -> 0.292 and 4.34 -> 3.14.
 struct ZDArgs {
     long ntiles;
     int tpfz, R, n3, Kp;
@@ -1439,23 +1554,23 @@ struct ZDArgs {
     uint32_t img_bytes;          // of one image or chunk
     int KC, nkc, nbuf;
     uint32_t offA, a_bytes, offCs, offRm, offBar;
-    int tcols, tmem_cols, groups;
+    int tcols, tmem_cols;
     int *err;
 };
 
-template <int NT, int UPT, bool STREAM>
-__global__ void __launch_bounds__(512, 1) zpass_direct_kernel(const __grid_constant__ ZDArgs a)
+template <int NT, int UPT, bool STREAM, bool TS, int GROUPS>
+__global__ void __launch_bounds__(NT * GROUPS, NT * GROUPS <= 256 ? 2 : 1) zpass_direct_kernel(const __grid_constant__ ZDArgs a)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     constexpr int kParts = NT / kRows;
-    constexpr int FD = UPT < 3 ? UPT : UPT <= 4 ? 3 : 2;   // units of f(Lambda) in flight
-    const int grp = STREAM ? 0 : threadIdx.x / NT, tid = threadIdx.x - grp * NT;
-    const int warp = tid >> 5, lane = tid & 31;
+    constexpr int FD = GROUPS == 3 ? 1 : UPT < 3 ? UPT : UPT <= 4 ? 3 : 2;   // units of f(Lambda) in flight
+    const int wid = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0);   // warp-uniform
+    const int grp = STREAM ? 0 : wid / (NT / 32), warp = wid - grp * (NT / 32), lane = threadIdx.x & 31, tid = warp * 32 + lane;
     uint8_t *sA = smem + a.offA + size_t(grp) * a.a_bytes;
     float *csF = reinterpret_cast<float *>(smem + a.offCs), *csI = csF + a.Kp;
     uint32_t *rm1 = reinterpret_cast<uint32_t *>(smem + a.offRm) + grp * 2 * kRows, *rm2 = rm1 + kRows;
     uint64_t *bar_d = reinterpret_cast<uint64_t *>(smem + a.offBar) + grp;
-    uint64_t *bfull = reinterpret_cast<uint64_t *>(smem + a.offBar) + 2, *bempty = bfull + 16;
+    uint64_t *bfull = reinterpret_cast<uint64_t *>(smem + a.offBar) + 3, *bempty = bfull + 16;
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bempty + 16);
     int *sflag = reinterpret_cast<int *>(tslot + 1);
     const int Kp = a.Kp, KC = STREAM ? a.KC : a.Kp;
@@ -1467,8 +1582,9 @@ __global__ void __launch_bounds__(512, 1) zpass_direct_kernel(const __grid_const
             *reinterpret_cast<uint4 *>(smem + i) = *reinterpret_cast<const uint4 *>(a.imgF + i);
             *reinterpret_cast<uint4 *>(smem + a.img_bytes + i) = *reinterpret_cast<const uint4 *>(a.imgI + i);
         }
-    for (uint32_t i = threadIdx.x * 16; i < uint32_t(a.groups) * a.a_bytes; i += blockDim.x * 16)
-        *reinterpret_cast<uint4 *>(smem + a.offA + i) = make_uint4(0, 0, 0, 0);
+    if (!TS)
+        for (uint32_t i = threadIdx.x * 16; i < uint32_t(GROUPS) * a.a_bytes; i += blockDim.x * 16)
+            *reinterpret_cast<uint4 *>(smem + a.offA + i) = make_uint4(0, 0, 0, 0);
     for (int i = threadIdx.x; i < Kp; i += blockDim.x) {   // column scales (the same in every chunk)
         csF[i] = reinterpret_cast<const float *>(a.imgF + size_t(kMatDig) * b_piece)[i];
         csI[i] = reinterpret_cast<const float *>(a.imgI + size_t(kMatDig) * b_piece)[i];
@@ -1488,15 +1604,21 @@ __global__ void __launch_bounds__(512, 1) zpass_direct_kernel(const __grid_const
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
-    const uint32_t tmem0 = *tslot, tmem = tmem0 + uint32_t(grp * a.tcols);
+    const uint32_t tmem0 = __shfl_sync(0xffffffffu, *tslot, 0), tmem = tmem0 + uint32_t(grp * a.tcols);
     const int quarter = warp & 3, dq = warp >> 2;
     const int row = quarter * 32 + lane;
     const uint32_t lane_q = uint32_t(quarter * 32) << 16;
     const int n3 = a.n3, R = a.R, bar_id = 1 + grp;
     uint8_t *arow = sA + img_at(row, 0, sbo);
+    const uint32_t ta = tmem + 2u * uint32_t(Kp), a_plane = uint32_t(Kp) / 2u;   // digit planes in TMEM (TS)
+    if (TS) {   // units past n3 stay zero
+        for (int u = dq; u < Kp / 8; u += kParts)
+            for (int q = 0; q < 3; ++q) tc::tmem_st4(ta + lane_q + q * a_plane + 4u * u, 0u, 0u, 0u, 0u);
+        tc::tmem_wait_st();
+    }
 
-    const long stride = long(gridDim.x) * a.groups;
-    const long first = long(blockIdx.x) * a.groups + grp;
+    const long stride = long(gridDim.x) * GROUPS;
+    const long first = long(blockIdx.x) * GROUPS + grp;
     long p = first / a.tpfz;
     int rt = int(first - p * a.tpfz);
     const long dp = stride / a.tpfz;
@@ -1504,34 +1626,43 @@ __global__ void __launch_bounds__(512, 1) zpass_direct_kernel(const __grid_const
     const long nfields = a.ntiles / a.tpfz;
     uint32_t ph = 0;
 
-    // ---- streamed chunks (thread 0): buffer and phase parity of the next load and the next use,
+    // ---- streamed chunks (warp 0, copies issued by one lane): buffer and phase parity of the next load and the next use,
     //      kept by increments (a division per chunk would cost more than its MMAs) ----
     int ld_slot = 0, us_slot = 0, ld_count = 0;   // ld_count: chunks of the current GEMM loaded so far
     uint32_t us_par = 0, fills = 0;               // fills: buffers that have been filled at least once
-    auto load_chunk = [&](int g) {                // chunk ld_count into the next buffer, which is free
-        tc::mbar_arrive_expect_tx(bfull + ld_slot, a.img_bytes);
-        bulk_load(smem + uint32_t(ld_slot) * a.img_bytes, (g ? a.imgI : a.imgF) + size_t(ld_count) * a.img_bytes, a.img_bytes,
-                  bfull + ld_slot);
+    auto load_chunk = [&](int g, uint32_t el) {   // chunk ld_count into the next buffer, which is free
+        if (el) {
+            tc::mbar_arrive_expect_tx(bfull + ld_slot, a.img_bytes);
+            bulk_load(smem + uint32_t(ld_slot) * a.img_bytes, (g ? a.imgI : a.imgF) + size_t(ld_count) * a.img_bytes, a.img_bytes,
+                      bfull + ld_slot);
+        }
         fills = max(fills, uint32_t(ld_slot) + 1u);
         ld_slot = ld_slot + 1 == a.nbuf ? 0 : ld_slot + 1;
         ++ld_count;
     };
     auto load_first = [&](int g) {           // when the previous GEMM has finished
-        if (STREAM && tid == 0) {
+        if (STREAM && warp == 0) {
+            const uint32_t el = tc::elect_one();
             ld_count = 0;
-            for (int kc = 0; kc < min(a.nbuf, a.nkc); ++kc) load_chunk(g);
+            for (int kc = 0; kc < min(a.nbuf, a.nkc); ++kc) load_chunk(g, el);
         }
     };
+    // GEMM complete: the first warp polls, the others sleep in the barrier (eight polling warps
+    // took a quarter of the issue slots from the other groups and from the warp issuing MMAs)
     auto wait_d = [&]() {
-        if (!tc::mbar_wait_timed(bar_d, ph, kWaitNs)) atomicExch(sflag, 1);
+        if (warp == 0 && !tc::mbar_wait_timed(bar_d, ph, kWaitNs)) atomicExch(sflag, 1);
         ph ^= 1u;
+        tc::bar_sync(bar_id, NT);
         tc::tc_fence_after();
     };
-    // one GEMM over the whole operand image (lane 0 of warp 0)
+    // one GEMM over the whole operand image (warp 0)
     auto gemm = [&](int g) {
+        const uint32_t el = tc::elect_one();
         const uint32_t ab = tc::smem_addr(sA);
         if (!STREAM) {
-            issue_x7_z(tmem, uint32_t(Kp), ab, a_piece, sbo, tc::smem_addr(smem + (g ? a.img_bytes : 0u)), b_piece, sbo, Kp / 16, false);
+            const uint32_t bb = tc::smem_addr(smem) + (g ? a.img_bytes : 0u);
+            if (TS) issue_x7_ts(tmem, uint32_t(Kp), ta, a_plane, bb, b_piece, sbo, Kp / 16, false, el);
+            else issue_x7_z(tmem, uint32_t(Kp), ab, a_piece, sbo, bb, b_piece, sbo, Kp / 16, false, el);
         } else {
             int pv_slot = 0;
             uint32_t pv_par = 0;
@@ -1540,16 +1671,19 @@ __global__ void __launch_bounds__(512, 1) zpass_direct_kernel(const __grid_const
                     atomicExch(sflag, 1);
                     return;
                 }
-                issue_x7_z(tmem, uint32_t(Kp), ab + uint32_t(kc * KC) * 16u, a_piece, sbo,
-                           tc::smem_addr(smem) + uint32_t(us_slot) * a.img_bytes, b_piece, b_sbo, KC / 16, kc > 0);
-                tc::mma_commit(bempty + us_slot);
+                const uint32_t bb = tc::smem_addr(smem) + uint32_t(us_slot) * a.img_bytes;
+                if (TS)
+                    issue_x7_ts(tmem, uint32_t(Kp), ta + uint32_t(kc * KC) / 2u, a_plane, bb, b_piece, b_sbo, KC / 16, kc > 0, el);
+                else
+                    issue_x7_z(tmem, uint32_t(Kp), ab + uint32_t(kc * KC) * 16u, a_piece, sbo, bb, b_piece, b_sbo, KC / 16, kc > 0, el);
+                if (el) tc::mma_commit(bempty + us_slot);
                 // the buffer of the chunk before this one takes the next chunk of this GEMM
                 if (kc > 0 && ld_count < a.nkc) {
                     if (!tc::mbar_wait_timed(bempty + pv_slot, pv_par, kWaitNs)) {
                         atomicExch(sflag, 1);
                         return;
                     }
-                    load_chunk(g);
+                    load_chunk(g, el);
                 }
                 pv_slot = us_slot;
                 pv_par = us_par;
@@ -1559,15 +1693,16 @@ __global__ void __launch_bounds__(512, 1) zpass_direct_kernel(const __grid_const
                 }
             }
         }
-        tc::mma_commit(bar_d);
+        if (el) tc::mma_commit(bar_d);
     };
     auto handoff = [&](int g) {
-        tc::fence_proxy_async_smem();
+        if (TS) tc::tmem_wait_st();
+        else tc::fence_proxy_async_smem();
         tc::tc_fence_before();
         if (tc::bar_red_or(bar_id, NT, *sflag != 0)) return true;
         if (warp == 0) {
             tc::tc_fence_after();
-            if (lane == 0) gemm(g);
+            gemm(g);
             __syncwarp();
         }
         return false;
@@ -1611,7 +1746,10 @@ __global__ void __launch_bounds__(512, 1) zpass_direct_kernel(const __grid_const
 #pragma unroll
         for (int g = 0; g < UPT; ++g) {
             const int u = dq + g * kParts;
-            if (8 * u < n3) store_digits8<false>(arow + u * 128, a_piece, x[g], x[g], sc);
+            if (8 * u < n3) {
+                if (TS) tmem_digits8<false>(ta + lane_q + 4u * u, a_plane, x[g], x[g], sc);
+                else store_digits8<false>(arow + u * 128, a_piece, x[g], x[g], sc);
+            }
         }
         if (handoff(0)) break;
         rm2[row] = 0u;
@@ -1687,7 +1825,8 @@ __global__ void __launch_bounds__(512, 1) zpass_direct_kernel(const __grid_const
                     l[2 * e] = __uint_as_float(lo[g][e] << 16);
                     l[2 * e + 1] = __uint_as_float(lo[g][e] & 0xffff0000u);
                 }
-                store_digits8<true>(arow + u * 128, a_piece, x[g], l, sc);
+                if (TS) tmem_digits8<true>(ta + lane_q + 4u * u, a_plane, x[g], l, sc);
+                else store_digits8<true>(arow + u * 128, a_piece, x[g], l, sc);
             }
         }
         if (handoff(1)) break;
@@ -1733,7 +1872,7 @@ __global__ void __launch_bounds__(512, 1) zpass_direct_kernel(const __grid_const
         p = np;
         rt = nr;
     }
-    if (STREAM && tid == 0 && *sflag) {
+    if (STREAM && warp == 0 && *sflag) {
         // a run that gave up leaves copies that nothing has waited for: none may target shared
         // memory at exit.  The last fill of a buffer before ld_slot has the parity of the next
         // load's pass, of the others the one before; both are waited for (one is over already).
@@ -1902,19 +2041,25 @@ SliceLayout slice_layout(const Plan &P, bool pair = true)
 // the streamed form.
 struct SliceDLayout {
     size_t smem;
-    uint32_t offB2, offA, a_bytes, offRm, offBar, a_piece1, a_piece2;
-    int G, Pj, tcols, tmem_cols, groups, nt, upt;
+    uint32_t offB2, offA, a_bytes, offRm, offBar, a_piece1, a_piece2, offS, stg_plane;
+    int G, Pj, P1, cpw, tcols, tmem_cols, groups, nt, upt, staged;
 };
 
-bool slice_direct_layout(const Plan &P, SliceDLayout &L)
+// pair: pass A (two staged planes) or pass C (one).
+bool slice_direct_layout(const Plan &P, bool pair, SliceDLayout &L)
 {
     const int n1 = P.n[0], n2 = P.n[1];
     const int Kp1 = pad16i(n1), Kp2 = pad16i(n2);
     L = SliceDLayout{};
     if (P.t3_stage >= 0 || P.t3_pipe >= 0) return false;   // a form asked for by hand
     L.G = kRows / std::max(n1, n2);
-    L.Pj = (n2 + 3) & ~3;
-    if (((L.Pj / 4) & 1) == 0) L.Pj += 4;   // odd number of 16-byte units: conflict-free rows
+    auto odd_pitch = [](int n) {   // an odd number of 16-byte units: conflict-free rows
+        const int p = (n + 3) & ~3;
+        return ((p / 4) & 1) ? p : p + 4;
+    };
+    L.Pj = odd_pitch(n2);
+    L.P1 = odd_pitch(n1);
+    L.cpw = (n1 % 4 == 0) ? 16 : (n1 % 2 == 0) ? 8 : 4;   // n1 divides N, so fields start as aligned as rows
     const int R1 = L.G * n2, R2 = L.G * n1;
     size_t off = mat_image_bytes(Kp1, Kp1);
     if (!P.t3_share01) {
@@ -1925,26 +2070,35 @@ bool slice_direct_layout(const Plan &P, SliceDLayout &L)
     L.offA = uint32_t(align_up(off, 1024));
     L.a_piece1 = uint32_t(pad8i(R1)) * Kp1 * 2u;
     L.a_piece2 = uint32_t(pad8i(R2)) * Kp2 * 2u;
-    // the MMA reads 128 rows of every digit plane (rows past the tile are never read back)
+    // the MMA reads 128 rows of every digit plane: the reach past a group's image falls into the
+    // next group's or the staging (rows past the tile are never read back)
     const size_t reach = std::max(2 * size_t(L.a_piece1) + size_t(kRows) * Kp1 * 2, 2 * size_t(L.a_piece2) + size_t(kRows) * Kp2 * 2);
-    L.a_bytes = uint32_t(align_up(std::max(reach, size_t(R2) * L.Pj * 4), 1024));
+    L.a_bytes = uint32_t(align_up(std::max({3 * size_t(L.a_piece1), 3 * size_t(L.a_piece2), size_t(R2) * L.Pj * 4}), 1024));
+    L.stg_plane = uint32_t(align_up(size_t(R1) * L.P1 * 4, 128));
     const int np = 2 * std::max(Kp1, Kp2);   // lead and rest columns of one GEMM
     L.tcols = np;
-    auto finish = [&](int nt, int groups) {
+    auto finish = [&](int nt, int groups, bool staged = true) {
         L.nt = nt;
         L.groups = groups;
+        L.staged = staged ? 1 : 0;
         const int q = std::max(pad8i(R1) / 8 * (Kp1 / 8), pad8i(R2) / 8 * (Kp2 / 8));   // quarter-warp units
         L.upt = (q + nt / 8 - 1) / (nt / 8);
-        L.offRm = uint32_t(L.offA + size_t(groups) * L.a_bytes);
+        L.offS = uint32_t(L.offA + size_t(groups) * L.a_bytes);
+        size_t end = L.offS + (staged ? size_t(groups) * (pair ? 2 : 1) * L.stg_plane : 0);
+        end = std::max(end, L.offA + size_t(groups - 1) * L.a_bytes + reach);
+        L.offRm = uint32_t(align_up(end, 16));
         L.offBar = L.offRm + uint32_t(groups) * 2 * kRows * 4;
-        L.smem = L.offBar + 32;
-        L.tmem_cols = tmem_pow2(groups * np);
-        return L.upt <= 4 && L.smem <= kSmemLimit && groups * np <= 512;
+        L.smem = L.offBar + 48;
+        L.tmem_cols = groups * np <= 512 ? tmem_pow2(groups * np) : 1024;
+        return L.upt <= (groups == 3 ? 3 : 4) && L.smem <= kSmemLimit && L.tmem_cols <= 512;
     };
+    // three groups of one CTA (80 registers a thread), else two groups as two CTAs or in one, else
+    // one group of 512
+    if (finish(256, 3)) return true;
     const size_t two_per_sm = 233472 / 2 - 1024;
     if (finish(256, 1) && L.smem <= two_per_sm && L.tmem_cols <= 256) return true;
     if (finish(256, 2)) return true;
-    return finish(512, 1);
+    return finish(512, 1) || finish(512, 1, false);
 }
 
 struct ZLayout {
@@ -2010,39 +2164,41 @@ bool z_layout(int n3, ZLayout &L, int want_wn = 0, int want_nbuf = 0)
 struct ZDLayout {
     size_t smem;
     uint32_t img_bytes, offA, a_bytes, offCs, offRm, offBar;
-    int stream, KC, nkc, nbuf, groups, nt, upt, tcols, tmem_cols;
+    int stream, ts, KC, nkc, nbuf, groups, nt, upt, tcols, tmem_cols;
 };
 
 bool z_direct_layout(int n3, ZDLayout &L)
 {
     const int Kp = pad16i(n3), nu = (n3 + 7) / 8;
-    auto finish = [&](int nt, int groups, bool stream) {
+    auto finish = [&](int nt, int groups, bool stream, bool ts) {
         L = ZDLayout{};
         L.nt = nt;
         L.groups = groups;
         L.stream = stream ? 1 : 0;
+        L.ts = ts ? 1 : 0;
         L.upt = (nu + nt / kRows - 1) / (nt / kRows);
         L.KC = stream ? 16 : Kp;
         L.nkc = Kp / L.KC;
         L.img_bytes = uint32_t(mat_image_bytes(Kp, L.KC));
-        L.a_bytes = 3u * kRows * Kp * 2u;
-        const size_t tail = 2 * size_t(Kp) * 4 + size_t(groups) * 2 * kRows * 4 + (2 + 32) * 8 + 64;
+        L.a_bytes = ts ? 0u : 3u * kRows * Kp * 2u;
+        const size_t tail = 2 * size_t(Kp) * 4 + size_t(groups) * 2 * kRows * 4 + (3 + 32) * 8 + 64;
         L.nbuf = 2;
         if (stream) L.nbuf = int(std::min<size_t>(16, (kSmemLimit - L.a_bytes - 1024 - tail) / L.img_bytes));
         L.offA = uint32_t(align_up(size_t(L.nbuf) * L.img_bytes, 1024));
         L.offCs = L.offA + uint32_t(groups) * L.a_bytes;
         L.offRm = L.offCs + 2 * uint32_t(Kp) * 4;
         L.offBar = uint32_t(align_up(L.offRm + size_t(groups) * 2 * kRows * 4, 16));
-        L.smem = L.offBar + (2 + 32) * 8 + 16;
-        L.tcols = 2 * Kp;
-        L.tmem_cols = groups * 2 * Kp <= 512 ? tmem_pow2(groups * 2 * Kp) : 1024;
-        return L.smem <= kSmemLimit && L.tmem_cols <= 512 && L.upt <= (stream ? 7 : 4) && L.nbuf >= 2;
+        L.smem = L.offBar + (3 + 32) * 8 + 16;
+        L.tcols = 2 * Kp + (ts ? 3 * Kp / 2 : 0);
+        L.tmem_cols = groups * L.tcols <= 512 ? tmem_pow2(groups * L.tcols) : 1024;
+        const int upt_max = stream ? 7 : groups == 3 ? 3 : 4;
+        return L.smem <= kSmemLimit && L.tmem_cols <= 512 && L.upt <= upt_max && L.nbuf >= 2;
     };
-    const size_t two_per_sm = 233472 / 2 - 1024;
-    if (finish(256, 1, false) && L.smem <= two_per_sm && L.tmem_cols <= 256) return true;
-    if (finish(256, 2, false)) return true;
-    if (finish(512, 1, false)) return true;
-    return finish(512, 1, true);
+    if (finish(256, 3, false, true)) return true;    // up to 48 points
+    if (finish(256, 2, false, true)) return true;    // up to 64
+    if (finish(512, 1, false, true)) return true;    // up to 96
+    if (finish(512, 1, true, true)) return true;     // up to 144
+    return finish(512, 1, true, false);
 }
 
 }  // namespace
@@ -2216,9 +2372,7 @@ int tc3_solve_batch(Plan &P, const int2 *pairs_d, int nfields, float *bufA, floa
 {
     const int n1 = P.n[0], n2 = P.n[1], n3 = P.n[2];
     // passes A and C
-    SliceDLayout DL;
-    const bool direct = slice_direct_layout(P, DL);
-    auto slice_direct = [&](bool pair, const float *in, float *out, int kind) -> int {
+    auto slice_direct = [&](const SliceDLayout &DL, bool pair, const float *in, float *out, int kind) -> int {
         SliceDArgs a{};
         a.n1 = n1;
         a.n2 = n2;
@@ -2249,17 +2403,25 @@ int tc3_solve_batch(Plan &P, const int2 *pairs_d, int nfields, float *bufA, floa
         a.Pj = DL.Pj;
         a.tmem_cols = DL.tmem_cols;
         a.tcols = DL.tcols;
-        a.vec = ((n1 & 3) == 0 && (P.N & 3) == 0) ? 1 : 0;
-        a.groups = DL.groups;
+        a.offS = DL.offS;
+        a.stg_plane = DL.stg_plane;
+        a.P1 = DL.P1;
+        a.cpw = DL.cpw;
         a.err = static_cast<int *>(P.err_d.p);
         void (*kern)(const SliceDArgs) = nullptr;
-        if (DL.nt == 256) {
-            if (DL.upt <= 2) kern = pair ? slice_direct_kernel<true, 256, 2> : slice_direct_kernel<false, 256, 2>;
-            else if (DL.upt == 3) kern = pair ? slice_direct_kernel<true, 256, 3> : slice_direct_kernel<false, 256, 3>;
-            else kern = pair ? slice_direct_kernel<true, 256, 4> : slice_direct_kernel<false, 256, 4>;
+        if (DL.groups == 3) {
+            if (DL.upt <= 2) kern = pair ? slice_direct_kernel<true, 256, 2, 3, true> : slice_direct_kernel<false, 256, 2, 3, true>;
+            else kern = pair ? slice_direct_kernel<true, 256, 3, 3, true> : slice_direct_kernel<false, 256, 3, 3, true>;
+        } else if (DL.groups == 2) {
+            if (DL.upt <= 3) kern = pair ? slice_direct_kernel<true, 256, 3, 2, true> : slice_direct_kernel<false, 256, 3, 2, true>;
+            else kern = pair ? slice_direct_kernel<true, 256, 4, 2, true> : slice_direct_kernel<false, 256, 4, 2, true>;
+        } else if (DL.nt == 256) {
+            if (DL.upt <= 3) kern = pair ? slice_direct_kernel<true, 256, 3, 1, true> : slice_direct_kernel<false, 256, 3, 1, true>;
+            else kern = pair ? slice_direct_kernel<true, 256, 4, 1, true> : slice_direct_kernel<false, 256, 4, 1, true>;
         } else {
-            if (DL.upt <= 3) kern = pair ? slice_direct_kernel<true, 512, 3> : slice_direct_kernel<false, 512, 3>;
-            else kern = pair ? slice_direct_kernel<true, 512, 4> : slice_direct_kernel<false, 512, 4>;
+            if (!DL.staged) kern = pair ? slice_direct_kernel<true, 512, 4, 1, false> : slice_direct_kernel<false, 512, 4, 1, false>;
+            else if (DL.upt <= 3) kern = pair ? slice_direct_kernel<true, 512, 3, 1, true> : slice_direct_kernel<false, 512, 3, 1, true>;
+            else kern = pair ? slice_direct_kernel<true, 512, 4, 1, true> : slice_direct_kernel<false, 512, 4, 1, true>;
         }
         size_t smem = DL.smem;
         const int threads = DL.nt * DL.groups;
@@ -2274,7 +2436,8 @@ int tc3_solve_batch(Plan &P, const int2 *pairs_d, int nfields, float *bufA, floa
         return EXX_OK;
     };
     auto slice = [&](bool pair, const float *in, float *out, int kind) -> int {
-        if (direct) return slice_direct(pair, in, out, kind);
+        SliceDLayout DL;
+        if (slice_direct_layout(P, pair, DL)) return slice_direct(DL, pair, in, out, kind);
         const SliceLayout L = slice_layout(P, pair);
         SliceArgs a{};
         a.n1 = n1;
@@ -2363,20 +2526,20 @@ int tc3_solve_batch(Plan &P, const int2 *pairs_d, int nfields, float *bufA, floa
         a.offBar = ZD.offBar;
         a.tcols = ZD.tcols;
         a.tmem_cols = ZD.tmem_cols;
-        a.groups = ZD.groups;
         a.err = static_cast<int *>(P.err_d.p);
         void (*kern)(const ZDArgs) = nullptr;
-        if (ZD.stream) {
-            kern = ZD.upt <= 4   ? zpass_direct_kernel<512, 4, true>
-                   : ZD.upt == 5 ? zpass_direct_kernel<512, 5, true>
-                   : ZD.upt == 6 ? zpass_direct_kernel<512, 6, true>
-                                 : zpass_direct_kernel<512, 7, true>;
+        if (ZD.stream && !ZD.ts) {
+            kern = ZD.upt <= 5   ? zpass_direct_kernel<512, 5, true, false, 1>
+                   : ZD.upt == 6 ? zpass_direct_kernel<512, 6, true, false, 1>
+                                 : zpass_direct_kernel<512, 7, true, false, 1>;
+        } else if (ZD.stream) {
+            kern = ZD.upt <= 4 ? zpass_direct_kernel<512, 4, true, true, 1> : zpass_direct_kernel<512, 5, true, true, 1>;
         } else if (ZD.nt == 512) {
-            kern = ZD.upt <= 3 ? zpass_direct_kernel<512, 3, false> : zpass_direct_kernel<512, 4, false>;
+            kern = zpass_direct_kernel<512, 3, false, true, 1>;
+        } else if (ZD.groups == 2) {
+            kern = zpass_direct_kernel<256, 4, false, true, 2>;
         } else {
-            kern = ZD.upt <= 2   ? zpass_direct_kernel<256, 2, false>
-                   : ZD.upt == 3 ? zpass_direct_kernel<256, 3, false>
-                                 : zpass_direct_kernel<256, 4, false>;
+            kern = ZD.upt <= 2 ? zpass_direct_kernel<256, 2, false, true, 3> : zpass_direct_kernel<256, 3, false, true, 3>;
         }
         const int threads = ZD.nt * ZD.groups;
         size_t smem = ZD.smem;

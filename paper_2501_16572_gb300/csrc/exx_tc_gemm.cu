@@ -24,8 +24,8 @@
 // (bulk copies, a producer warp) into the MMAs (one issuing warp) while 8 warps combine
 // finished chunks.  Cutting inside the GEMM repeated the integer work of every A row for each
 // 96 output columns and left the tensor cores idle meanwhile: both products of ace_apply at
-// n = nphi = 512 on 72 x 72 x 144 points took 65.7 ms, 11.3 ms now (cuts 3.3 ms near the HBM
-// rate, MMAs 7.8 ms, of which the tensor pipe's own 5.6 ms).
+// n = nphi = 512 on 72 x 72 x 144 points took 65.7 ms, 10.9 ms now (cuts 3.3 ms near the HBM
+// rate, MMAs 7.5 ms, of which the tensor pipe's own 5.6 ms).
 #include "exx_internal.h"
 #include "tc_ptx.cuh"
 
@@ -241,7 +241,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     uint64_t *dfull = empty + a.stages, *dempty = dfull + 1;
     uint32_t *tslot = reinterpret_cast<uint32_t *>(dempty + 1);
     int *sflag = reinterpret_cast<int *>(tslot + 1);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform
     if (tid == 0) {
         for (int i = 0; i < a.stages; ++i) {
             tc::mbar_init(full + i, 1);
@@ -255,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
-    const uint32_t tmem = *tslot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
     const long items = a.Z * a.mt * a.nt;
     const int Nt = a.Nt;
     const uint32_t a_bytes = kT * kBlk * 2 * kDig, b_bytes = uint32_t(Nt) * kBlk * 2 * kDig;
@@ -314,14 +315,15 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         uint32_t par = 0, dpar = 1;
         bool bad = false, dfirst = true;
         // operand and accumulator steps, fixed for the launch: the issue of one 16-k step is a
-        // straight run of MMAs whose descriptors differ by additions (computed in a loop, the
-        // issuing thread took 1340 cycles a step, twice the tensor pipe's 632)
+        // straight run of MMAs by the whole warp whose descriptors differ by additions (computed in
+        // a loop by one lane, a step took 1340 cycles, twice the tensor pipe's 632)
         constexpr uint32_t kStepA = kT * kBlk * 2 / 16;            // next A digit, in 16-byte units
         const uint32_t step_b = uint32_t(Nt) * kBlk * 2 / 16;      // next B digit
         uint32_t idesc[G + 1];
 #pragma unroll
         for (int g = 1; g <= G; ++g) idesc[g] = tc::instr_desc(false, g * Nt);
         // A digit i with B digits j0 .. j0 + g - 1 into levels i + j0 .. (at most G per MMA)
+        const uint32_t el = tc::elect_one();
         auto step = [&](uint64_t ad0, uint64_t bd0, bool first) {
 #pragma unroll
             for (int i = 0; i < kDig; ++i) {
@@ -335,14 +337,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                     const uint32_t d = tmem + uint32_t((i + j0) * Nt);
                     if (i == 1 && j0 + g == kDig && g > 1) {
                         if (first) {   // digit 0 has opened levels 0..3; level 4 starts here
-                            tc::mma_bf16(d, ad, bd, idesc[g - 1], 1u);
-                            tc::mma_bf16(tmem + uint32_t(4 * Nt), ad, bd0 + (kDig - 1) * step_b, idesc[1], 0u);
+                            tc::mma_bf16_warp(d, ad, bd, idesc[g - 1], 1u, el);
+                            tc::mma_bf16_warp(tmem + uint32_t(4 * Nt), ad, bd0 + (kDig - 1) * step_b, idesc[1], 0u, el);
                         } else {
-                            tc::mma_bf16(d, ad, bd, idesc[g], 1u);
+                            tc::mma_bf16_warp(d, ad, bd, idesc[g], 1u, el);
                         }
                     } else {
                         const bool open = i == 0 || (i == 1 && j0 == kDig - 1);
-                        tc::mma_bf16(d, ad, bd, idesc[g], open && first ? 0u : 1u);
+                        tc::mma_bf16_warp(d, ad, bd, idesc[g], open && first ? 0u : 1u, el);
                     }
                 }
             }
@@ -366,20 +368,18 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                         break;
                     }
                     tc::tc_fence_after();
-                    if (lane == 0) {
-                        const uint32_t sa = tc::smem_addr(smem + size_t(st) * a.stage_bytes);
-                        const uint64_t ad = tc::smem_desc(sa, 128u, kSbo), bd = tc::smem_desc(sa + a_bytes, 128u, kSbo);
-                        step(ad, bd, kb == kb0);
-                        step(ad + 16, bd + 16, false);
-                        tc::mma_commit(empty + st);
-                    }
+                    const uint32_t sa = tc::smem_addr(smem) + uint32_t(st) * a.stage_bytes;
+                    const uint64_t ad = tc::smem_desc(sa, 128u, kSbo), bd = tc::smem_desc(sa + a_bytes, 128u, kSbo);
+                    step(ad, bd, kb == kb0);
+                    step(ad + 16, bd + 16, false);
+                    if (el) tc::mma_commit(empty + st);
                     __syncwarp();
                     if (++st == a.stages) {
                         st = 0;
                         par ^= 1u;
                     }
                 }
-                if (!bad && lane == 0) tc::mma_commit(dfull);
+                if (!bad && el) tc::mma_commit(dfull);
                 __syncwarp();
             }
         }
@@ -412,12 +412,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
                 float *fb = fbs + (dseq & 1) * kTN;
                 if (tid < Nt) fb[tid] = pow2f(a.shB[c * a.prowB + j0 + tid] - refB[tid]);
                 const float fa = pow2f(a.shA[c * a.prowA + i] - rA);
-                if (!tc::mbar_wait_timed(dfull, uint32_t(dseq & 1), kGemmWaitNs)) atomicExch(sflag, 1);
-                tc::tc_fence_after();
+                // one warp polls, the others sleep in the barrier: polls take issue slots from the MMAs'
+                if (warp == 0 && !tc::mbar_wait_timed(dfull, uint32_t(dseq & 1), kGemmWaitNs)) atomicExch(sflag, 1);
                 if (tc::bar_red_or(1, NT, *sflag != 0)) {   // also: fb is complete
                     stop = true;
                     break;
                 }
+                tc::tc_fence_after();
 #pragma unroll
                 for (int cg = 0; cg < kHalf / 8; ++cg) {
                     if (cg * 8 >= ncol) break;
