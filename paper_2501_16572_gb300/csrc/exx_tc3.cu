@@ -2196,7 +2196,7 @@ bool z_direct_layout(int n3, ZDLayout &L)
     };
     if (finish(256, 3, false, true)) return true;    // up to 48 points
     if (finish(256, 2, false, true)) return true;    // up to 64
-    if (finish(512, 1, false, true)) return true;    // up to 96
+    if (finish(512, 1, false, true)) return true;    // up to 112
     if (finish(512, 1, true, true)) return true;     // up to 144
     return finish(512, 1, true, false);
 }
@@ -2535,7 +2535,7 @@ int tc3_solve_batch(Plan &P, const int2 *pairs_d, int nfields, float *bufA, floa
         } else if (ZD.stream) {
             kern = ZD.upt <= 4 ? zpass_direct_kernel<512, 4, true, true, 1> : zpass_direct_kernel<512, 5, true, true, 1>;
         } else if (ZD.nt == 512) {
-            kern = zpass_direct_kernel<512, 3, false, true, 1>;
+            kern = ZD.upt <= 3 ? zpass_direct_kernel<512, 3, false, true, 1> : zpass_direct_kernel<512, 4, false, true, 1>;
         } else if (ZD.groups == 2) {
             kern = zpass_direct_kernel<256, 4, false, true, 2>;
         } else {
