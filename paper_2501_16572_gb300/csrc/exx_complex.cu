@@ -46,31 +46,120 @@ __global__ void c_pair_kernel(long N, int nfields, const cd *psi_occ, long ld_oc
     }
 }
 
-// Contraction of axis d (length nd, stride sd in the natural layout) of every field:
-// out(..., o, ...) = sum_k C[k nd + o] in(..., k, ...), times S(r) when S is set (real).
-__global__ void c_mode_kernel(long N, int nfields, int nd, long sd, const cd *C, const cd *in, cd *out,
-                              const double *S)
+// Contraction of one axis (length nd, stride sd in the natural layout) of every field with its
+// eigenbasis, times S(r) when S is set.  Bound by the FP64 pipe (2 FMA per clock and SM), so every
+// basis is used as real coefficients, 2 FMA per complex input and output instead of 4:
+//   * Dirichlet axes have real eigenvectors;
+//   * a periodic axis pairs the points j and n - j, where U_p(n - j) = e^{i theta} conj(U_p(j)):
+//     forward   out_p = sum_j (x_j + y_j) cos(phi_p j) - i (x_j - y_j) sin(phi_p j),
+//               y_j = e^{-i theta} x_{n-j}, j = 0 .. n/2 (x_0 and, for even n, x_{n/2} alone);
+//     inverse   C + i S = out_j and e^{i theta} (C - i S) = out_{n-j} from C = sum_p t_p cos(phi_p j),
+//               S = sum_p t_p sin(phi_p j).
+// A CTA stages 32 pencils (folded, forward periodic) in shared memory; a thread has one pencil
+// and kCOut outputs at a time.  Coefficients T[k nc + o], cosines then sines for periodic axes.
+constexpr int kCPen = 32, kCThreads = 256, kCOut = 4;
+enum { C_REAL = 0, C_FWD = 1, C_INV = 2 };
+struct CAxis {
+    long npen;           // pencils: fields x N / nd
+    int nd, nk, no;      // points, staged values (nd, or n/2 + 1 pairs), outputs or output pairs
+    long sd, N;
+    const double *T;     // nk x no (twice for periodic axes)
+    double cth, sth;     // e^{i theta}
+    const cd *in;
+    cd *out;
+    const double *S;
+};
+
+template <int MODE>
+__global__ void __launch_bounds__(kCThreads) c_axis_kernel(const CAxis a)
 {
-    const long total = long(nfields) * N;
-    for (long e = long(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += long(gridDim.x) * blockDim.x) {
-        const long p = e / N, r = e - p * N;
-        const int o = int((r / sd) % nd);
-        const cd *src = in + p * N + (r - long(o) * sd);
-        cd acc = {0.0, 0.0};
-        for (int k = 0; k < nd; ++k) acc = cfma(C[size_t(k) * nd + o], src[size_t(k) * sd], acc);
-        if (S) {
-            acc.re *= S[r];
-            acc.im *= S[r];
+    extern __shared__ cd sx[];                       // [k][32]; forward periodic: x + y, then x - y
+    cd *sy = sx + size_t(a.nk) * kCPen;
+    const int pl = threadIdx.x & 31, og = threadIdx.x >> 5;
+    const long q0 = long(blockIdx.x) * kCPen;
+    auto base = [&](long q) { return (q / a.sd) * (a.sd * a.nd) + q % a.sd; };   // first point of pencil q
+    const int nfull = int(min(long(kCPen), a.npen - q0));
+    const cd zero = {0.0, 0.0};
+    // e^{i theta} or its conjugate times v
+    auto turn = [&](cd v, double s) { return cd{v.re * a.cth - s * v.im * a.sth, v.im * a.cth + s * v.re * a.sth}; };
+    if (MODE != C_FWD) {
+        if (a.sd == 1) {   // consecutive pencils are one run of memory
+            for (int i = threadIdx.x; i < kCPen * a.nd; i += kCThreads) {
+                const int r = i / a.nd, k = i - r * a.nd;
+                sx[k * kCPen + r] = r < nfull ? a.in[q0 * a.nd + i] : zero;
+            }
+        } else {
+            const long b = pl < nfull ? base(q0 + pl) : 0;
+            for (int k = og; k < a.nd; k += kCThreads / 32) sx[k * kCPen + pl] = pl < nfull ? a.in[b + k * a.sd] : zero;
         }
-        out[e] = acc;
+    } else {
+        const long b = pl < nfull ? base(q0 + pl) : 0;
+        for (int j = og; j < a.nk; j += kCThreads / 32) {
+            cd x = zero, y = zero;
+            if (pl < nfull) {
+                x = a.in[b + j * a.sd];
+                if (j > 0 && 2 * j != a.nd) y = turn(a.in[b + (a.nd - j) * a.sd], -1.0);
+            }
+            sx[j * kCPen + pl] = {x.re + y.re, x.im + y.im};
+            sy[j * kCPen + pl] = {x.re - y.re, x.im - y.im};
+        }
+    }
+    __syncthreads();
+    if (pl >= nfull) return;
+    const long b = base(q0 + pl);
+    const double *Ts = a.T + size_t(a.nk) * a.no;
+    for (int o0 = og * kCOut; o0 < a.no; o0 += (kCThreads / 32) * kCOut) {
+        double cr[kCOut] = {}, ci[kCOut] = {}, sr[kCOut] = {}, si[kCOut] = {};
+        int oc[kCOut];
+#pragma unroll
+        for (int t = 0; t < kCOut; ++t) oc[t] = min(o0 + t, a.no - 1);
+        for (int k = 0; k < a.nk; ++k) {
+            const cd x = sx[k * kCPen + pl];
+            const cd y = MODE == C_FWD ? sy[k * kCPen + pl] : x;
+            const double *tk = a.T + size_t(k) * a.no, *ts = Ts + size_t(k) * a.no;
+#pragma unroll
+            for (int t = 0; t < kCOut; ++t) {
+                const double c = tk[oc[t]];
+                cr[t] = fma(x.re, c, cr[t]);
+                ci[t] = fma(x.im, c, ci[t]);
+                if (MODE != C_REAL) {
+                    const double s = ts[oc[t]];
+                    sr[t] = fma(y.re, s, sr[t]);
+                    si[t] = fma(y.im, s, si[t]);
+                }
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < kCOut; ++t) {
+            const int o = o0 + t;
+            if (o >= a.no) break;
+            auto put = [&](int at, cd v) {
+                const long r = b + at * a.sd;
+                if (a.S) {
+                    const double f = a.S[r % a.N];
+                    v.re *= f;
+                    v.im *= f;
+                }
+                a.out[r] = v;
+            };
+            if (MODE == C_REAL) put(o, {cr[t], ci[t]});
+            else if (MODE == C_FWD) put(o, {cr[t] + si[t], ci[t] - sr[t]});      // C - i S
+            else {
+                put(o, {cr[t] - si[t], ci[t] + sr[t]});                          // C + i S
+                if (o > 0 && 2 * o != a.nd) put(a.nd - o, turn({cr[t] + si[t], ci[t] - sr[t]}, 1.0));
+            }
+        }
     }
 }
 
-// out_n(r) (-)= sum_{j < cnt} f_{m_j} psi_occ[m_j](r) V_j(r) for one output column: the fields
-// V_j of the batch all belong to output n, in the order of m.
+// out_n(r) (-)= sum_{j < cnt} f_{m_j} psi_occ[m_j](r) V_j(r): column n = blockIdx.y of the group has the
+// cnt fields V_{n cnt} .., in the order of m.
 __global__ void c_accum_kernel(long N, int cnt, const int2 *pairs, const cd *psi_occ, long ld_occ, const double *f,
-                               const cd *V, cd *out_n, int add)
+                               const cd *V, cd *out, long ld_out, int add)
 {
+    cd *out_n = out + size_t(blockIdx.y) * ld_out;
+    pairs += size_t(blockIdx.y) * cnt;
+    V += size_t(blockIdx.y) * cnt * N;
     for (long r = long(blockIdx.x) * blockDim.x + threadIdx.x; r < N; r += long(gridDim.x) * blockDim.x) {
         cd acc = add ? out_n[r] : cd{0.0, 0.0};
         for (int j = 0; j < cnt; ++j) {
@@ -227,32 +316,27 @@ int invalid_c(const char *msg)
 
 }  // namespace
 
-// Host setup of a Bloch plan: complex eigenbases, the eigenvalue sums and f on them, uploaded
-// as the forward (conj(U)^T) and inverse (U) contraction matrices C[k nd + o] per axis.
+// Host setup of a Bloch plan: the eigenvalue sums and f on them, and the coefficient tables of the
+// forward (conj(U)^T) and inverse (U) contractions per axis.
 int bloch_setup(Plan &P, const double theta[3])
 {
     P.cplx = 1;
     std::vector<double> lam[3];
-    std::vector<std::complex<double>> U[3];
     const int p = P.fd_order / 2;
     std::vector<double> w(size_t(p) + 1);
     fd_weights(p, w.data());
     for (int d = 0; d < 3; ++d) {
         const int nd = P.n[d];
         P.theta[d] = theta[d];
-        U[d].assign(size_t(nd) * nd, 0.0);
         lam[d].assign(nd, 0.0);
         if (P.bc[d] == EXX_BC_PERIODIC) {
-            const double inv = 1.0 / std::sqrt(double(nd));
             for (int q = 0; q < nd; ++q) {
                 const double phi = (2.0 * kPi * q + theta[d]) / nd;
                 double l = w[0];
                 for (int k = 1; k <= p; ++k) l += 2.0 * w[k] * std::cos(k * phi);
                 lam[d][q] = l / (P.h * P.h);
-                for (int j = 0; j < nd; ++j) U[d][size_t(j) + size_t(nd) * q] = std::polar(inv, phi * j);
             }
         } else {
-            for (size_t e = 0; e < size_t(nd) * nd; ++e) U[d][e] = P.V[d][e];
             lam[d] = P.lam[d];
         }
     }
@@ -273,21 +357,32 @@ int bloch_setup(Plan &P, const double theta[3])
                     kernel_f(lam[0][a] + lam[1][b] + lam[2][c], P.kernel, P.omega);
     for (int d = 0; d < 3; ++d) P.clam[d] = lam[d];
     P.cF = F;
-    size_t total = 0;
-    for (int d = 0; d < 3; ++d) total += 2 * size_t(P.n[d]) * P.n[d];
-    std::vector<std::complex<double>> mats(total);
-    size_t off = 0;
+    // coefficient tables of c_axis_kernel, per axis forward then inverse
+    std::vector<double> tab;
     for (int d = 0; d < 3; ++d) {
-        const int nd = P.n[d];
-        for (int k = 0; k < nd; ++k)
-            for (int o = 0; o < nd; ++o) {
-                mats[off + size_t(k) * nd + o] = std::conj(U[d][size_t(k) + size_t(nd) * o]);   // forward
-                mats[off + size_t(nd) * nd + size_t(k) * nd + o] = U[d][size_t(o) + size_t(nd) * k];   // inverse
+        const int nd = P.n[d], np = nd / 2 + 1;
+        if (P.bc[d] != EXX_BC_PERIODIC) {
+            for (int inv = 0; inv < 2; ++inv) {
+                P.ctab_off[d][inv] = tab.size();
+                for (int k = 0; k < nd; ++k)
+                    for (int o = 0; o < nd; ++o)
+                        tab.push_back(inv ? P.V[d][size_t(o) + size_t(nd) * k] : P.V[d][size_t(k) + size_t(nd) * o]);
             }
-        off += 2 * size_t(nd) * nd;
+            continue;
+        }
+        const double s = 1.0 / std::sqrt(double(nd));
+        auto ang = [&](int p, int j) { return (2.0 * kPi * p + theta[d]) / nd * j; };
+        P.ctab_off[d][0] = tab.size();   // forward: [pair j][output p], cosines then sines
+        for (int q = 0; q < 2; ++q)
+            for (int j = 0; j < np; ++j)
+                for (int p = 0; p < nd; ++p) tab.push_back(s * (q ? std::sin(ang(p, j)) : std::cos(ang(p, j))));
+        P.ctab_off[d][1] = tab.size();   // inverse: [p][output pair j]
+        for (int q = 0; q < 2; ++q)
+            for (int p = 0; p < nd; ++p)
+                for (int j = 0; j < np; ++j) tab.push_back(s * (q ? std::sin(ang(p, j)) : std::cos(ang(p, j))));
     }
-    if (int rc = dev_reserve(P.cmats, mats.size() * sizeof(std::complex<double>))) return rc;
-    EXX_CUDA(cudaMemcpy(P.cmats.p, mats.data(), mats.size() * sizeof(std::complex<double>), cudaMemcpyHostToDevice));
+    if (int rc = dev_reserve(P.cmats, tab.size() * sizeof(double))) return rc;
+    EXX_CUDA(cudaMemcpy(P.cmats.p, tab.data(), tab.size() * sizeof(double), cudaMemcpyHostToDevice));
     if (int rc = dev_reserve(P.cFd, F.size() * sizeof(double))) return rc;
     EXX_CUDA(cudaMemcpy(P.cFd.p, F.data(), F.size() * sizeof(double), cudaMemcpyHostToDevice));
     if (int rc = dev_reserve(P.err_d, 16)) return rc;
@@ -295,8 +390,8 @@ int bloch_setup(Plan &P, const double theta[3])
     return EXX_OK;
 }
 
-// The complex exchange: fields batched per output column (all occupied partners of one n,
-// in chunks that fit the workspace).
+// The complex exchange: fields batched over whole groups of output columns (all occupied
+// partners of each), or, when one column's partners do not fit the workspace, over chunks of a column.
 int complex_apply(Plan &P, const double *psi_occ_d, int n_occ, long ld_occ, const double *f, const double *psi_in_d,
                   int n_in, long ld_in, double *out_d, long ld_out, int accumulate, cudaStream_t s)
 {
@@ -304,8 +399,10 @@ int complex_apply(Plan &P, const double *psi_occ_d, int n_occ, long ld_occ, cons
     cd *out = reinterpret_cast<cd *>(out_d);
     const long N = P.N;
     const size_t field = size_t(N) * sizeof(cd);
-    const int chunk = int(std::max<size_t>(1, std::min<size_t>(size_t(n_occ), (size_t(1) << 30) / field)));
-    if (int rc = dev_reserve(P.cwork, 2 * size_t(chunk) * field)) return rc;
+    const long room = std::max(1L, (1L << 30) / long(field));           // fields per buffer
+    const int chunk = int(std::min<long>(n_occ, room));
+    const int group = int(std::max(1L, std::min<long>({long(n_in), room / n_occ, 65535L})));
+    if (int rc = dev_reserve(P.cwork, 2 * size_t(chunk) * group * field)) return rc;
     if (int rc = dev_reserve(P.cpairs, size_t(n_occ) * size_t(n_in) * sizeof(int2))) return rc;
     std::vector<int2> pairs(size_t(n_occ) * n_in);
     for (int n = 0; n < n_in; ++n)
@@ -313,39 +410,53 @@ int complex_apply(Plan &P, const double *psi_occ_d, int n_occ, long ld_occ, cons
     EXX_CUDA(cudaMemcpyAsync(P.cpairs.p, pairs.data(), pairs.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
     EXX_CUDA(cudaStreamSynchronize(s));   // the host vector goes out of scope
     const int2 *pairs_d = static_cast<const int2 *>(P.cpairs.p);
-    cd *A = static_cast<cd *>(P.cwork.p), *B = A + size_t(chunk) * N;
-    const cd *mats = static_cast<const cd *>(P.cmats.p);
-    const cd *Cf[3], *Ci[3];
-    size_t off = 0;
-    for (int d = 0; d < 3; ++d) {
-        Cf[d] = mats + off;
-        Ci[d] = mats + off + size_t(P.n[d]) * P.n[d];
-        off += 2 * size_t(P.n[d]) * P.n[d];
-    }
+    cd *A = static_cast<cd *>(P.cwork.p), *B = A + size_t(chunk) * group * N;
+    const double *tab = static_cast<const double *>(P.cmats.p);
     const long sd[3] = {1, long(P.n[0]), long(P.n[0]) * P.n[1]};
     const double *F = static_cast<const double *>(P.cFd.p);
-    for (int n = 0; n < n_in; ++n) {
+    auto axis = [&](int d, int inv, int fields, const cd *in, cd *o, const double *S) -> int {
+        const bool per = P.bc[d] == EXX_BC_PERIODIC;
+        const int nd = P.n[d], np = nd / 2 + 1;
+        CAxis a{};
+        a.nd = nd;
+        a.npen = long(fields) * (N / nd);
+        a.nk = per && !inv ? np : nd;
+        a.no = per && inv ? np : nd;
+        a.sd = sd[d];
+        a.N = N;
+        a.T = tab + P.ctab_off[d][inv];
+        a.cth = std::cos(P.theta[d]);
+        a.sth = std::sin(P.theta[d]);
+        a.in = in;
+        a.out = o;
+        a.S = S;
+        auto kern = !per ? c_axis_kernel<C_REAL> : inv ? c_axis_kernel<C_INV> : c_axis_kernel<C_FWD>;
+        const size_t smem = size_t(a.nk) * kCPen * sizeof(cd) * (per && !inv ? 2 : 1);   // at most 132 KB
+        if (smem > 48 * 1024) EXX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+        kern<<<unsigned((a.npen + kCPen - 1) / kCPen), kCThreads, smem, s>>>(a);
+        EXX_LAUNCH("c_axis_kernel");
+        P.launches++;
+        return EXX_OK;
+    };
+    for (int n = 0; n < n_in; n += group) {
+        const int gn = std::min(group, n_in - n);
         for (int m0 = 0; m0 < n_occ; m0 += chunk) {
-            const int cnt = std::min(chunk, n_occ - m0);
+            const int cnt = std::min(chunk, n_occ - m0);   // n_occ whenever gn > 1
+            const int fields = cnt * gn;
             const int2 *pp = pairs_d + size_t(n) * n_occ + m0;
-            const long tot = long(cnt) * N;
-            const int g = grid_for(P, tot);
-            c_pair_kernel<<<g, 256, 0, s>>>(N, cnt, po, ld_occ, pi, ld_in, pp, A);
+            c_pair_kernel<<<grid_for(P, long(fields) * N), 256, 0, s>>>(N, fields, po, ld_occ, pi, ld_in, pp, A);
             EXX_LAUNCH("c_pair_kernel");
             // forward x, y, z (z scaled by f(Lambda)), inverse z, y, x: A -> B -> A -> ...
             cd *src = A, *dst = B;
             const int order[6] = {0, 1, 2, 2, 1, 0};
             for (int st = 0; st < 6; ++st) {
-                const int d = order[st];
-                c_mode_kernel<<<g, 256, 0, s>>>(N, cnt, P.n[d], sd[d], st < 3 ? Cf[d] : Ci[d], src, dst,
-                                                st == 2 ? F : nullptr);
-                EXX_LAUNCH("c_mode_kernel");
+                if (int rc = axis(order[st], st < 3 ? 0 : 1, fields, src, dst, st == 2 ? F : nullptr)) return rc;
                 std::swap(src, dst);
             }
-            c_accum_kernel<<<grid_for(P, N), 256, 0, s>>>(N, cnt, pp, po, ld_occ, f, src, out + size_t(n) * ld_out,
-                                                          (accumulate || m0 > 0) ? 1 : 0);
+            c_accum_kernel<<<dim3(unsigned(grid_for(P, N)), unsigned(gn)), 256, 0, s>>>(
+                N, cnt, pp, po, ld_occ, f, src, out + size_t(n) * ld_out, ld_out, (accumulate || m0 > 0) ? 1 : 0);
             EXX_LAUNCH("c_accum_kernel");
-            P.launches += 8;
+            P.launches += 2;
         }
     }
     return EXX_OK;

@@ -170,6 +170,7 @@ struct Plan {
     int cplx = 0;
     double theta[3] = {0.0, 0.0, 0.0};
     std::vector<double> clam[3], cF;
+    size_t ctab_off[3][2] = {};     // coefficient tables in cmats, forward and inverse per axis
     DevBuf cmats, cFd, cwork, cpairs, cred, cace;
     // workspace
     DevBuf work[3];                 // batch buffers (fields x N)
