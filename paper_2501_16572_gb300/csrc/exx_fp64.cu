@@ -1,37 +1,46 @@
 // FP64 path of the batched Kronecker Poisson solve (Sec. II.B) and of the
 // exchange accumulation (Eq. 1), on the CUDA cores.
 //
-// GB300 runs FP64 at a small fraction of its FP32 rate, so these kernels are bound by
-// the double-precision FMA pipe, not by memory: a mode product of length n does 2n
-// flops per 8-byte element.  Each thread owns one row (a pencil along the contracted
-// axis) and produces 16 outputs at a time from the K x 16 slice of the contraction
-// matrix staged in shared memory (every thread of a warp reads the same entry, a
-// broadcast).
+// GB300 runs FP64 at a small fraction of its FP32 rate (2 FMA per clock and SM), so these
+// kernels are bound by the double-precision FMA pipe, not by memory.  Every 1D operator commutes
+// with the reflection of its axis (Toeplitz or circulant, and symmetric), so its eigenvectors are
+// taken even or odd: a forward contraction works on x_k + x_{n-1-k} for the even outputs and on
+// x_k - x_{n-1-k} for the odd ones, an inverse one gives y_k and y_{n-1-k} as the sum and the
+// difference of an even and an odd part: n flops a point instead of 2n.  Each thread owns one row (a
+// pencil along the contracted axis) and produces up to 20 outputs at a time from the slice of
+// the matrix staged in shared memory (every thread of a warp reads the same entry, a
+// broadcast); the slice width is the one that pads the axis least.
+// 28 x 30 x 33 points, 24 of 32 orbitals: 6.05 ms without the reflection and with slices of 16.
 #include "exx_internal.h"
+
+#include <algorithm>
+#include <cmath>
+#include <numeric>
 
 namespace exx {
 
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kChunk = 16;
 
 struct Fp64PassArgs {
     int nfields, R, K;
     const double *in;            // field stride N
     double *out;                 // field stride N
     long N;
-    const double *B;             // K x K, B[k*K + j]
+    const double *B;             // ne x K: B[k*K + j], modes j even (ne of them) then odd
     const double *F;             // [j][r] scaling (R*K values) or null
     const double *psi_a, *psi_b; // pair prologue: psi_a[m*lda + ...], psi_b[n*ldb + ...]
     long lda, ldb;
     const int2 *pairs;
 };
 
-template <int LOAD, int STORE, bool SCALE>
+// Forward: C modes of one parity per sweep over the row.  Inverse: C / 2 point pairs per sweep.
+template <int LOAD, int STORE, bool SCALE, bool INV, int C>
 __global__ void __launch_bounds__(kThreads) fp64_pass_kernel(Fp64PassArgs a)
 {
-    extern __shared__ double Bs[];   // [K][kChunk]
+    extern __shared__ double Bs[];   // [k][C]
+    const int K = a.K, no = K / 2, ne = K - no;
     const long rows = long(a.nfields) * a.R;
     const long g = long(blockIdx.x) * blockDim.x + threadIdx.x;
     const bool active = g < rows;
@@ -45,50 +54,106 @@ __global__ void __launch_bounds__(kThreads) fp64_pass_kernel(Fp64PassArgs a)
         pb = a.psi_b + size_t(mn.y) * a.ldb;
     }
     double *out = a.out + size_t(p) * a.N;
-    for (int j0 = 0; j0 < a.K; j0 += kChunk) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < a.K * kChunk; i += blockDim.x) {
-            int k = i / kChunk, j = i - k * kChunk;
-            Bs[i] = (j0 + j < a.K) ? a.B[size_t(k) * a.K + j0 + j] : 0.0;
-        }
-        __syncthreads();
-        if (!active) continue;
-        double acc[kChunk];
+    auto load = [&](int k) {
+        if (LOAD == LOAD_PAIR) return pa[size_t(k) * a.R + r] * pb[size_t(k) * a.R + r];
+        if (LOAD == LOAD_KSLOW) return in[size_t(k) * a.R + r];
+        return in[size_t(r) * a.K + k];
+    };
+    auto store = [&](int j, double v) {
+        if (SCALE) v *= a.F[size_t(j) * a.R + r];
+        if (STORE == STORE_NSLOW) out[size_t(j) * a.R + r] = v;
+        else out[size_t(r) * a.K + j] = v;
+    };
+    if (!INV) {
+        for (int par = 0; par < 2; ++par) {
+            const int first = par ? ne : 0, cnt = par ? no : ne;   // modes of this parity
+            for (int j0 = 0; j0 < cnt; j0 += C) {
+                __syncthreads();
+                for (int i = threadIdx.x; i < ne * C; i += blockDim.x) {
+                    const int k = i / C, j = i - k * C;
+                    Bs[i] = j0 + j < cnt ? a.B[size_t(k) * K + first + j0 + j] : 0.0;
+                }
+                __syncthreads();
+                if (!active) continue;
+                double acc[C];
 #pragma unroll
-        for (int j = 0; j < kChunk; ++j) acc[j] = 0.0;
-        for (int k = 0; k < a.K; ++k) {
-            double x;
-            if (LOAD == LOAD_PAIR) x = pa[size_t(k) * a.R + r] * pb[size_t(k) * a.R + r];
-            else if (LOAD == LOAD_KSLOW) x = in[size_t(k) * a.R + r];
-            else x = in[size_t(r) * a.K + k];
-            const double2 *bk = reinterpret_cast<const double2 *>(Bs + k * kChunk);
+                for (int j = 0; j < C; ++j) acc[j] = 0.0;
+                for (int k = 0; k < ne; ++k) {   // k = no < ne: the middle point of an odd axis (even modes only)
+                    double x = load(k);
+                    if (k < no) x += par ? -load(K - 1 - k) : load(K - 1 - k);
+                    const double2 *bk = reinterpret_cast<const double2 *>(Bs + k * C);
 #pragma unroll
-            for (int j = 0; j < kChunk / 2; ++j) {
-                double2 b = bk[j];
-                acc[2 * j] = fma(x, b.x, acc[2 * j]);
-                acc[2 * j + 1] = fma(x, b.y, acc[2 * j + 1]);
+                    for (int j = 0; j < C / 2; ++j) {
+                        const double2 b = bk[j];
+                        acc[2 * j] = fma(x, b.x, acc[2 * j]);
+                        acc[2 * j + 1] = fma(x, b.y, acc[2 * j + 1]);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < C; ++j)
+                    if (j0 + j < cnt) store(first + j0 + j, acc[j]);
             }
         }
-        const int jn = min(kChunk, a.K - j0);
+    } else {
+        constexpr int H = C / 2;
+        for (int k0 = 0; k0 < ne; k0 += H) {
+            __syncthreads();
+            for (int i = threadIdx.x; i < K * H; i += blockDim.x) {
+                const int j = i / H, k = k0 + i - j * H;
+                Bs[i] = k < ne ? a.B[size_t(k) * K + j] : 0.0;
+            }
+            __syncthreads();
+            if (!active) continue;
+            double ev[H], od[H];
 #pragma unroll
-        for (int j = 0; j < kChunk; ++j) {
-            if (j >= jn) break;
-            double v = acc[j];
-            if (SCALE) v *= a.F[size_t(j0 + j) * a.R + r];
-            if (STORE == STORE_NSLOW) out[size_t(j0 + j) * a.R + r] = v;
-            else out[size_t(r) * a.K + j0 + j] = v;
+            for (int k = 0; k < H; ++k) ev[k] = od[k] = 0.0;
+            for (int j = 0; j < ne; ++j) {
+                const double t = load(j);
+#pragma unroll
+                for (int k = 0; k < H; ++k) ev[k] = fma(t, Bs[j * H + k], ev[k]);
+            }
+            for (int j = ne; j < K; ++j) {
+                const double t = load(j);
+#pragma unroll
+                for (int k = 0; k < H; ++k) od[k] = fma(t, Bs[j * H + k], od[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < H; ++k) {
+                if (k0 + k >= ne) break;
+                store(k0 + k, ev[k] + od[k]);                            // od = 0 at the middle point
+                if (k0 + k < no) store(K - 1 - k0 - k, ev[k] - od[k]);
+            }
         }
     }
 }
 
-template <int LOAD, int STORE, bool SCALE>
+// The slice width that pads `count` modes (or point pairs, half a width each) least, the widest of equals.
+inline int slice_width(int count, bool inv)
+{
+    int best = 0, cost = 1 << 30;
+    for (int c : {20, 18, 16, 14, 12}) {
+        const int w = inv ? c / 2 : c;
+        const int padded = (count + w - 1) / w * w;
+        if (padded < cost) {
+            cost = padded;
+            best = c;
+        }
+    }
+    return best;
+}
+
+template <int LOAD, int STORE, bool SCALE, bool INV>
 int launch_pass(Plan &P, int kind, const Fp64PassArgs &a, cudaStream_t s)
 {
     const long rows = long(a.nfields) * a.R;
     const int grid = int((rows + kThreads - 1) / kThreads);
-    const size_t smem = size_t(a.K) * kChunk * sizeof(double);
-    auto kern = fp64_pass_kernel<LOAD, STORE, SCALE>;
-    if (smem > 48 * 1024) EXX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    const int ne = a.K - a.K / 2, C = slice_width(ne, INV);
+    const size_t smem = size_t(INV ? a.K * (C / 2) : ne * C) * sizeof(double);   // at most 20.5 KB
+    auto kern = C == 20   ? fp64_pass_kernel<LOAD, STORE, SCALE, INV, 20>
+                : C == 18 ? fp64_pass_kernel<LOAD, STORE, SCALE, INV, 18>
+                : C == 16 ? fp64_pass_kernel<LOAD, STORE, SCALE, INV, 16>
+                : C == 14 ? fp64_pass_kernel<LOAD, STORE, SCALE, INV, 14>
+                          : fp64_pass_kernel<LOAD, STORE, SCALE, INV, 12>;
     int tb = timing_begin(P, kind, s);
     kern<<<grid, kThreads, smem, s>>>(a);
     timing_end(P, tb, s);
@@ -181,25 +246,25 @@ int fp64_solve_batch(Plan &P, const double *psi_occ, long ld_occ, const double *
             // forward y with the Hadamard scaling by f(Lambda), then inverse y
             a.in = src;
             a.out = dst;
-            a.B = static_cast<const double *>(P.B64[2].p);
+            a.B = static_cast<const double *>(P.B64[1].p);
             a.F = static_cast<const double *>(P.F64.p);
-            rc = launch_pass<LOAD_KFAST, STORE_NFAST, true>(P, EXX_TIMING_PASS3, a, s);
+            rc = launch_pass<LOAD_KFAST, STORE_NFAST, true, false>(P, EXX_TIMING_PASS3, a, s);
             if (rc) return rc;
             P.launches++;
             std::swap(src, dst);
             a.in = src;
             a.out = dst;
-            a.B = static_cast<const double *>(P.B64[3].p);
+            a.B = static_cast<const double *>(P.B64[1].p);
             a.F = nullptr;
-            rc = launch_pass<LOAD_KFAST, STORE_NFAST, false>(P, EXX_TIMING_PASS3, a, s);
+            rc = launch_pass<LOAD_KFAST, STORE_NFAST, false, true>(P, EXX_TIMING_PASS3, a, s);
         } else {
             a.in = src;
             a.out = dst;
-            a.B = static_cast<const double *>(P.B64[pass < 2 ? pass : pass + 1].p);
-            if (pass == 0) rc = launch_pass<LOAD_PAIR, STORE_NSLOW, false>(P, EXX_TIMING_PASS1, a, s);
-            else if (pass == 1) rc = launch_pass<LOAD_KFAST, STORE_NSLOW, false>(P, EXX_TIMING_PASS2, a, s);
-            else if (pass == 3) rc = launch_pass<LOAD_KSLOW, STORE_NFAST, false>(P, EXX_TIMING_PASS4, a, s);
-            else rc = launch_pass<LOAD_KSLOW, STORE_NSLOW, false>(P, EXX_TIMING_PASS5, a, s);
+            a.B = static_cast<const double *>(P.B64[g.axis].p);
+            if (pass == 0) rc = launch_pass<LOAD_PAIR, STORE_NSLOW, false, false>(P, EXX_TIMING_PASS1, a, s);
+            else if (pass == 1) rc = launch_pass<LOAD_KFAST, STORE_NSLOW, false, false>(P, EXX_TIMING_PASS2, a, s);
+            else if (pass == 3) rc = launch_pass<LOAD_KSLOW, STORE_NFAST, false, true>(P, EXX_TIMING_PASS4, a, s);
+            else rc = launch_pass<LOAD_KSLOW, STORE_NSLOW, false, true>(P, EXX_TIMING_PASS5, a, s);
         }
         if (rc) return rc;
         P.launches++;
@@ -234,30 +299,62 @@ int fp64_accumulate(Plan &P, const double *psi_occ, long ld_occ, const double *p
     return EXX_OK;
 }
 
+// Even and odd eigenvectors of one axis, ne x n: B[k n + j] is mode j (the ne even ones, then the
+// odd ones) at point k, over sqrt(2) except at the middle point of an odd axis; order[j] = the mode's
+// place among the ascending eigenvalues.
+static int fold_axis(const Plan &P, int d, std::vector<double> &B, std::vector<int> &order)
+{
+    const int n = P.n[d], no = n / 2, ne = n - no;
+    std::vector<double> D(size_t(n) * n), lam(n);
+    second_derivative(n, P.h, P.bc[d], P.fd_order / 2, D.data());
+    B.assign(size_t(ne) * n, 0.0);
+    const double r2 = std::sqrt(0.5);
+    for (int par = 0; par < 2; ++par) {
+        const int m = par ? no : ne, first = par ? ne : 0;
+        if (m == 0) continue;
+        std::vector<double> A(size_t(m) * m), U(size_t(m) * m);
+        for (int l = 0; l < m; ++l)
+            for (int k = 0; k < m; ++k) {
+                const bool mk = k == no, ml = l == no;   // the middle point is its own mirror image
+                const double direct = D[size_t(k) + size_t(n) * l];
+                const double mirror = D[size_t(k) + size_t(n) * (n - 1 - l)];
+                A[size_t(k) + size_t(m) * l] = mk && ml ? direct : (mk || ml) ? direct / r2 : par ? direct - mirror : direct + mirror;
+            }
+        if (sym_eig(m, A.data(), U.data(), lam.data() + first)) {
+            set_error("exx_plan_create: eigen-decomposition did not converge");
+            return EXX_ERR_UNSUPPORTED;
+        }
+        for (int j = 0; j < m; ++j)
+            for (int k = 0; k < m; ++k) B[size_t(k) * n + first + j] = U[size_t(k) + size_t(m) * j] * (k == no ? 1.0 : r2);
+    }
+    std::vector<int> rank(n);
+    std::iota(rank.begin(), rank.end(), 0);
+    std::stable_sort(rank.begin(), rank.end(), [&](int x, int y) { return lam[x] < lam[y]; });
+    order.resize(n);
+    for (int i = 0; i < n; ++i) order[rank[i]] = i;
+    return EXX_OK;
+}
+
 int fp64_upload(Plan &P)
 {
-    // contraction matrices: forward B[k][j] = V(k, j); inverse B[k][j] = V(j, k)
-    const int axis_of[6] = {2, 0, 1, 1, 0, 2};
-    const int inv_of[6] = {0, 0, 0, 1, 1, 1};
-    for (int slot = 0; slot < 6; ++slot) {
-        int d = axis_of[slot], nd = P.n[d];
-        std::vector<double> B(size_t(nd) * nd);
-        for (int k = 0; k < nd; ++k)
-            for (int j = 0; j < nd; ++j)
-                B[size_t(k) * nd + j] = inv_of[slot] ? P.V[d][j + size_t(nd) * k] : P.V[d][k + size_t(nd) * j];
-        if (int rc = dev_reserve(P.B64[slot], B.size() * sizeof(double))) return rc;
-        EXX_CUDA(cudaMemcpy(P.B64[slot].p, B.data(), B.size() * sizeof(double), cudaMemcpyHostToDevice));
+    std::vector<int> order[3];
+    for (int d = 0; d < 3; ++d) {
+        std::vector<double> B;
+        if (int rc = fold_axis(P, d, B, order[d])) return rc;
+        if (int rc = dev_reserve(P.B64[d], B.size() * sizeof(double))) return rc;
+        EXX_CUDA(cudaMemcpy(P.B64[d].p, B.data(), B.size() * sizeof(double), cudaMemcpyHostToDevice));
     }
-    // F in the P3 layout: [b][a][c] -> F(a, b, c)
+    // F in the P3 layout: [b][a][c] -> F(a, b, c); FP64 in the folded order of the modes, the
+    // FP32 planes (hi, then lo) of the five-pass split modes in ascending order
     const int n1 = P.n[0], n2 = P.n[1], n3 = P.n[2];
     std::vector<double> F3(size_t(P.N));
-    std::vector<float> F3f(2 * size_t(P.N));   // hi plane, then lo plane
+    std::vector<float> F3f(2 * size_t(P.N));
     for (int b = 0; b < n2; ++b)
         for (int a = 0; a < n1; ++a)
             for (int c = 0; c < n3; ++c) {
-                double v = P.F[a + size_t(n1) * (b + size_t(n2) * c)];
                 size_t idx = size_t(b) * n1 * n3 + size_t(a) * n3 + c;
-                F3[idx] = v;
+                F3[idx] = P.F[order[0][a] + size_t(n1) * (order[1][b] + size_t(n2) * order[2][c])];
+                const double v = P.F[a + size_t(n1) * (b + size_t(n2) * c)];
                 F3f[idx] = float(v);
                 F3f[idx + size_t(P.N)] = float(v - double(float(v)));
             }

@@ -144,10 +144,10 @@ struct Plan {
     int device = 0;
     int num_sms = 0;
     std::vector<double> V[3], lam[3], F;   // host copies
-    // FP64 path: per pass the K x K contraction matrix B[k*K + j] (output j, input k)
-    DevBuf B64[6];                  // P1, P2, P3-forward, P3-inverse, P4, P5
-    DevBuf F64;                     // F in the P3 layout [b][a][c]
-    DevBuf F32;                     // same as two float planes, hi then lo
+    // FP64 path: per axis the even, then the odd eigenvectors at the first half of the points
+    DevBuf B64[3];
+    DevBuf F64;                     // F in the P3 layout [b][a][c], modes in that order
+    DevBuf F32;                     // F in the P3 layout as two float planes, hi then lo (ascending modes)
     // tensor path: per pass and precision the B operand pieces, canonical SMEM image
     DevBuf Btc[5][6];               // [prec][pass slot]: nblk^2 block images, (c, h) at (c nblk + h)
     int tc_nblk[5][3] = {};         // [prec][axis]: blocks the axis is cut into (1 = whole axis)
