@@ -176,89 +176,20 @@ gemm_rows_kernel(long M, int Nc, int K, const double *A, long lda, const double 
         }
 }
 
-constexpr int kCholThreads = 1024;
-
-// n <= kCholSmemMax: one CTA with everything in shared memory (column-major n x n):
-// right-looking Cholesky (column j: pivot, scale, rank-1 update of the trailing lower
-// triangle), then the inverse in place, columns from the right (unblocked triangular
-// inverse): X_jj = 1 / L_jj and X(j+1:, j) = -X_jj X(j+1:, j+1:) L(j+1:, j), the
-// triangular product into a scratch column.
-constexpr int kCholSmemMax = 128;
-__global__ void __launch_bounds__(kCholThreads)
-cholesky_inverse_smem_kernel(int n, const double *M, double *Linv, int *info_d)
-{
-    extern __shared__ double S[];   // n x n, S[i + n j], then n scratch values
-    double *y = S + n * n;
-    __shared__ int failed;
-    const int tid = threadIdx.x;
-    for (int e = tid; e < n * n; e += blockDim.x) {
-        const int i = e % n, j = e / n;
-        S[e] = (i >= j) ? -0.5 * (M[i + size_t(n) * j] + M[j + size_t(n) * i]) : 0.0;
-    }
-    if (tid == 0) {
-        failed = 0;
-        info_d[0] = 0;
-    }
-    __syncthreads();
-    for (int j = 0; j < n; ++j) {
-        if (tid == 0) {
-            const double d = S[j + n * j];
-            if (!(d > 0.0)) {
-                failed = 1;
-                info_d[0] = j + 1;
-            } else {
-                S[j + n * j] = sqrt(d);
-            }
-        }
-        __syncthreads();
-        if (failed) return;   // uniform: read after the barrier
-        const double djj = S[j + n * j];
-        for (int i = j + 1 + tid; i < n; i += blockDim.x) S[i + n * j] /= djj;
-        __syncthreads();
-        // trailing lower triangle: warps over its columns k, lanes over consecutive rows i
-        for (int k = j + 1 + (tid >> 5); k < n; k += blockDim.x >> 5) {
-            const double lk = S[k + n * j];
-            for (int i = k + (tid & 31); i < n; i += 32) S[i + n * k] -= S[i + n * j] * lk;
-        }
-        __syncthreads();
-    }
-    for (int j = n - 1; j >= 0; --j) {
-        const double xjj = 1.0 / S[j + n * j];
-        // y_i = sum_{k = j+1..i} X(i, k) L(k, j), rows i > j (X(j+1:, j+1:) is final): a
-        // thread per row (consecutive lanes read consecutive rows of a column), four
-        // partial sums against the FMA latency
-        for (int i = j + 1 + tid; i < n; i += blockDim.x) {
-            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-            int k = j + 1;
-            for (; k + 3 <= i; k += 4) {
-                s0 = fma(S[i + n * k], S[k + n * j], s0);
-                s1 = fma(S[i + n * (k + 1)], S[k + 1 + n * j], s1);
-                s2 = fma(S[i + n * (k + 2)], S[k + 2 + n * j], s2);
-                s3 = fma(S[i + n * (k + 3)], S[k + 3 + n * j], s3);
-            }
-            for (; k <= i; ++k) s0 = fma(S[i + n * k], S[k + n * j], s0);
-            y[i] = (s0 + s1) + (s2 + s3);
-        }
-        __syncthreads();
-        for (int i = j + 1 + tid; i < n; i += blockDim.x) S[i + n * j] = -xjj * y[i];
-        if (tid == 0) S[j + n * j] = xjj;
-        __syncthreads();
-    }
-    for (int e = tid; e < n * n; e += blockDim.x) {
-        const int i = e % n, j = e / n;
-        Linv[e] = (i >= j) ? S[e] : 0.0;
-    }
-}
-
-// ---- blocked Cholesky and triangular inverse for n > kCholSmemMax (many CTAs) -----------
-// A = -(M + M^T)/2 is factored in place, right-looking, in column blocks of kCb:
-//   diagonal block: A_kk = L_kk L_kk^T and D_k = L_kk^{-1} (one CTA, shared memory);
-//   panel:          L_ik = A_ik D_k^T for the row blocks i > k (a CTA per row block);
-//   trailing:       A_ij -= L_ik L_jk^T for i >= j > k (a CTA per lower 64 x 64 tile).
-// Then X = L^{-1} block row by block row: X_ii = D_i (written with the factorisation),
-// X_ij = -D_i sum_{k=j}^{i-1} L_ik X_kj (a CTA per block j < i).
+// ---- blocked Cholesky and triangular inverse --------------------------------------------
+// A = -(M + M^T)/2 is factored in place, right-looking, in column blocks of kCb = 32:
+//   diagonal block: A_kk = L_kk L_kk^T and D_k = L_kk^{-1} (one warp, rows and columns in registers);
+//   panel:          L_ik = A_ik D_k^T for the rows below (a CTA per kPanel rows);
+//   trailing:       A_ij -= L_ik L_jk^T for i >= j > k (a CTA per lower 32 x 32 tile).
+// Then X = L^{-1} by doubling: with the inverses X11, X22 of neighbouring diagonal blocks of s
+// points known, X21 = -X22 (L21 X11), all pairs of a level at once.
+// Everything here is a chain of small steps on the FP64 pipe (2 FMA per clock and SM: a 64 x 64 x 64 tile
+// takes one SM 65 us, a 32 x 32 x 32 tile 8 us), so the tiles are small, spread over the SMs, and the
+// diagonal block runs on shuffles instead of 1024 threads and three barriers a column.
+// ace_build of n = 512 (72 x 72 x 144): 16.40 -> 12.09 ms against 64-wide blocks on one CTA of 1024
+// threads and block rows of X in sequence.
 // A failed pivot sets info_d[0] = 1 + its index; every later kernel then returns at once.
-constexpr int kCb = 64;
+constexpr int kCb = 32, kPanel = 8, kCholThreads = 256;
 
 __global__ void chol_prep_kernel(int n, const double *M, double *A, double *X, int *info_d)
 {
@@ -270,227 +201,150 @@ __global__ void chol_prep_kernel(int n, const double *M, double *A, double *X, i
     if (blockIdx.x == 0 && threadIdx.x == 0) info_d[0] = 0;
 }
 
-// One CTA: the diagonal block at (k0, k0) of size b <= kCb: factor, write L_kk into A and
-// D = L_kk^{-1} (lower, b x b, leading dimension kCb) into Dk and into X's diagonal block.
-__global__ void __launch_bounds__(kCholThreads) chol_diag_kernel(int n, double *A, int k0, int b, double *Dk,
-                                                                 double *X, int *info_d)
+// One warp: the diagonal block at (k0, k0) of size b <= 32 (padded with the identity): lane i holds
+// row i.  Writes L_kk into A, D = L_kk^{-1} (leading dimension kCb, zeros above) into Dk and X.
+__global__ void __launch_bounds__(32) chol_diag_kernel(int n, double *A, int k0, int b, double *Dk, double *X, int *info_d)
 {
-    __shared__ double S[kCb * kCb];
-    __shared__ double y[kCb];
-    __shared__ int failed;
-    const int tid = threadIdx.x;
-    if (tid == 0) failed = info_d[0] != 0;
-    __syncthreads();
-    if (failed) return;
-    for (int e = tid; e < b * b; e += blockDim.x) {
-        const int i = e % b, j = e / b;
-        S[i + kCb * j] = (i >= j) ? A[(k0 + i) + size_t(n) * (k0 + j)] : 0.0;
-    }
-    __syncthreads();
-    for (int j = 0; j < b; ++j) {
-        if (tid == 0) {
-            const double d = S[j + kCb * j];
-            if (!(d > 0.0)) {
-                failed = 1;
-                info_d[0] = k0 + j + 1;
-            } else {
-                S[j + kCb * j] = sqrt(d);
-            }
+    const int lane = threadIdx.x;
+    if (info_d[0]) return;
+    double a[kCb], rd[kCb];
+#pragma unroll
+    for (int j = 0; j < kCb; ++j)
+        a[j] = lane < b && j <= lane ? A[(k0 + lane) + size_t(n) * (k0 + j)] : (j == lane ? 1.0 : 0.0);
+#pragma unroll
+    for (int j = 0; j < kCb; ++j) {
+        const double d = __shfl_sync(0xffffffffu, a[j], j);
+        if (!(d > 0.0)) {   // uniform
+            if (lane == 0) info_d[0] = k0 + j + 1;
+            return;
         }
-        __syncthreads();
-        if (failed) return;
-        const double djj = S[j + kCb * j];
-        for (int i = j + 1 + tid; i < b; i += blockDim.x) S[i + kCb * j] /= djj;
-        __syncthreads();
-        for (int k = j + 1 + (tid >> 5); k < b; k += blockDim.x >> 5) {
-            const double lk = S[k + kCb * j];
-            for (int i = k + (tid & 31); i < b; i += 32) S[i + kCb * k] -= S[i + kCb * j] * lk;
+        const double djj = sqrt(d);
+        rd[j] = 1.0 / djj;
+        const double l = lane == j ? djj : a[j] * rd[j];
+        a[j] = l;
+#pragma unroll
+        for (int k = j + 1; k < kCb; ++k) a[k] = fma(-l, __shfl_sync(0xffffffffu, l, k), a[k]);
+    }
+#pragma unroll
+    for (int j = 0; j < kCb; ++j)
+        if (lane < b && j <= lane) A[(k0 + lane) + size_t(n) * (k0 + j)] = a[j];
+    // column `lane` of the inverse by forward substitution
+    double x[kCb];
+#pragma unroll
+    for (int i = 0; i < kCb; ++i) {
+        double s0 = i == lane ? 1.0 : 0.0, s1 = 0.0;
+#pragma unroll
+        for (int k = 0; k < i; ++k) {
+            const double t = __shfl_sync(0xffffffffu, a[k], i);
+            if (k & 1) s1 = fma(-t, x[k], s1);
+            else s0 = fma(-t, x[k], s0);
         }
-        __syncthreads();
+        x[i] = (s0 + s1) * rd[i];
     }
-    for (int e = tid; e < b * b; e += blockDim.x) {
-        const int i = e % b, j = e / b;
-        if (i >= j) A[(k0 + i) + size_t(n) * (k0 + j)] = S[i + kCb * j];
-    }
-    __syncthreads();
-    // in-place inverse of the b x b lower triangle, columns from the right
-    for (int j = b - 1; j >= 0; --j) {
-        const double xjj = 1.0 / S[j + kCb * j];
-        for (int i = j + 1 + tid; i < b; i += blockDim.x) {
-            double acc = 0.0;
-            for (int k = j + 1; k <= i; ++k) acc = fma(S[i + kCb * k], S[k + kCb * j], acc);
-            y[i] = acc;
-        }
-        __syncthreads();
-        for (int i = j + 1 + tid; i < b; i += blockDim.x) S[i + kCb * j] = -xjj * y[i];
-        if (tid == 0) S[j + kCb * j] = xjj;
-        __syncthreads();
-    }
-    for (int e = tid; e < kCb * kCb; e += blockDim.x) {
-        const int i = e % kCb, j = e / kCb;
-        const double v = (i < b && j < b && i >= j) ? S[i + kCb * j] : 0.0;
-        Dk[e] = v;
-        if (i < b && j < b) X[(k0 + i) + size_t(n) * (k0 + j)] = v;
+#pragma unroll
+    for (int i = 0; i < kCb; ++i) {
+        const double v = i < b && lane < b && i >= lane ? x[i] : 0.0;
+        Dk[i + kCb * lane] = v;
+        if (i < b && lane < b) X[(k0 + i) + size_t(n) * (k0 + lane)] = v;
     }
 }
 
-// C (rows r0.., columns c0.., 64 x 64 tile, leading dimension n) op= sum_t P(r, t) Q(c, t),
-// P(r, t) = Pm[r + ldp t], Q(c, t) = Qm[c + ldq t], t < K; mode 0: C = alpha acc; 1: C += alpha acc.
-__device__ __forceinline__ void tile_gemm_nt(int rows, int cols, int K, const double *Pm, long ldp, const double *Qm,
-                                             long ldq, double alpha, double *C, long ldc, int mode)
+// panel: rows r0 .. r0 + 7 below the diagonal block, L(r, c) = sum_t A(r, k0 + t) D(c, t)
+__global__ void __launch_bounds__(kCholThreads) chol_panel_kernel(int n, double *A, int k0, int b, const double *Dk, const int *info_d)
 {
-    __shared__ double Ps[kKt][kTile + 1];
-    __shared__ double Qs[kKt][kTile + 1];
+    __shared__ double D[kCb][kCb + 1], R[kPanel][kCb + 1];
+    if (info_d[0]) return;
+    const int r0 = k0 + b + blockIdx.x * kPanel;
+    for (int e = threadIdx.x; e < kCb * kCb; e += kCholThreads) D[e / kCb][e % kCb] = Dk[e];   // D[t][c]
+    const int r = threadIdx.x % kPanel, c = threadIdx.x / kPanel;
+    const bool ok = r0 + r < n && c < b;
+    double *at = A + (r0 + r) + size_t(n) * (k0 + c);
+    R[r][c] = ok ? *at : 0.0;
+    __syncthreads();
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+    for (int t = 0; t < kCb; t += 2) {
+        s0 = fma(R[r][t], D[t][c], s0);
+        s1 = fma(R[r][t + 1], D[t + 1][c], s1);
+    }
+    if (ok) *at = s0 + s1;
+}
+
+// A 32 x 32 tile sum_{t < K} P(r, t) Q(t, c), 2 x 2 outputs per thread: P(r, t) = Pm[r + ldp t];
+// Q(t, c) = Qm[c ldc + t ldt].  Rows and columns past rows / cols count as zero.
+__device__ __forceinline__ void tile32(int rows, int cols, int K, const double *Pm, long ldp, const double *Qm, long ldc,
+                                       long ldt, double (&acc)[2][2])
+{
+    __shared__ double Ps[kCb][kCb + 1], Qs[kCb][kCb + 1];
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    double acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += kKt) {
-        for (int t = threadIdx.x; t < kKt * kTile; t += kGemmThreads) {
-            const int rr = t % kTile, kk = t / kTile;
-            Ps[kk][rr] = (rr < rows && k0 + kk < K) ? Pm[rr + ldp * (k0 + kk)] : 0.0;
-            Qs[kk][rr] = (rr < cols && k0 + kk < K) ? Qm[rr + ldq * (k0 + kk)] : 0.0;
+    for (int k0 = 0; k0 < K; k0 += kCb) {
+        for (int e = threadIdx.x; e < kCb * kCb; e += kCholThreads) {
+            const int i = e % kCb, j = e / kCb;
+            Ps[j][i] = i < rows && k0 + j < K ? Pm[i + ldp * (k0 + j)] : 0.0;   // [t][r], r consecutive
+            if (ldt == 1) Qs[i][j] = j < cols && k0 + i < K ? Qm[j * ldc + k0 + i] : 0.0;
+            else Qs[j][i] = i < cols && k0 + j < K ? Qm[i * ldc + (k0 + j) * ldt] : 0.0;
         }
         __syncthreads();
-#pragma unroll 4
-        for (int kk = 0; kk < kKt; ++kk) {
-            double a[4], b[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                a[u] = Ps[kk][tx + 16 * u];
-                b[u] = Qs[kk][ty + 16 * u];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int w = 0; w < 4; ++w) acc[u][w] = fma(a[u], b[w], acc[u][w]);
+#pragma unroll 8
+        for (int t = 0; t < kCb; ++t) {
+            const double p0 = Ps[t][tx], p1 = Ps[t][tx + 16], q0 = Qs[t][ty], q1 = Qs[t][ty + 16];
+            acc[0][0] = fma(p0, q0, acc[0][0]);
+            acc[0][1] = fma(p0, q1, acc[0][1]);
+            acc[1][0] = fma(p1, q0, acc[1][0]);
+            acc[1][1] = fma(p1, q1, acc[1][1]);
         }
         __syncthreads();
     }
-    for (int u = 0; u < 4; ++u)
-        for (int w = 0; w < 4; ++w) {
-            const int r = tx + 16 * u, c = ty + 16 * w;
-            if (r < rows && c < cols) {
-                double *o = C + r + ldc * c;
-                *o = mode ? *o + alpha * acc[u][w] : alpha * acc[u][w];
-            }
-        }
 }
 
-// panel: row block i = k0/kCb + 1 + blockIdx.x, L_ik = A_ik D_k^T (into a scratch copy first:
-// the tile reads A_ik while writing it)
-__global__ void __launch_bounds__(kGemmThreads) chol_panel_kernel(int n, double *A, int k0, int b, const double *Dk,
-                                                                  double *scratch, const int *info_d)
+// trailing update of the lower triangle: tile (bi, bj), bi >= bj, of the part past k0 + b (the strict
+// upper part of a diagonal tile is updated too; it is never read)
+__global__ void __launch_bounds__(kCholThreads) chol_update_kernel(int n, double *A, int k0, int b, const int *info_d)
 {
-    if (info_d[0]) return;
-    const int r0 = k0 + b + blockIdx.x * kCb;
-    const int rows = min(kCb, n - r0);
-    double *tmp = scratch + size_t(blockIdx.x) * kCb * kCb;
-    // tmp(r, c) = sum_t A(r0 + r, k0 + t) D(c, t)
-    tile_gemm_nt(rows, b, b, A + r0 + size_t(n) * k0, n, Dk, kCb, 1.0, tmp, kCb, 0);
-    __syncthreads();
-    for (int e = threadIdx.x; e < kCb * kCb; e += blockDim.x) {
-        const int r = e % kCb, c = e / kCb;
-        if (r < rows && c < b) A[(r0 + r) + size_t(n) * (k0 + c)] = tmp[r + kCb * c];
-    }
-}
-
-// trailing update of the lower triangle: tile (bi, bj), bi >= bj, of the part past k0 + b
-__global__ void __launch_bounds__(kGemmThreads) chol_update_kernel(int n, double *A, int k0, int b, const int *info_d)
-{
-    if (info_d[0]) return;
     const int bi = blockIdx.x, bj = blockIdx.y;
-    if (bi < bj) return;
-    const int base = k0 + b;
-    const int r0 = base + bi * kCb, c0 = base + bj * kCb;
+    if (info_d[0] || bi < bj) return;
+    const int r0 = k0 + b + bi * kCb, c0 = k0 + b + bj * kCb;
     const int rows = min(kCb, n - r0), cols = min(kCb, n - c0);
-    // A(r, c) -= sum_t L(r, k0 + t) L(c, k0 + t)   (the strict upper part of a diagonal tile
-    // is updated too; it is never read and is cleared at the end)
-    tile_gemm_nt(rows, cols, b, A + r0 + size_t(n) * k0, n, A + c0 + size_t(n) * k0, n, -1.0,
-                 A + r0 + size_t(n) * c0, n, 1);
+    double acc[2][2] = {};
+    tile32(rows, cols, b, A + r0 + size_t(n) * k0, n, A + c0 + size_t(n) * k0, 1, n, acc);
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+            const int r = tx + 16 * u, c = ty + 16 * w;
+            if (r < rows && c < cols) A[(r0 + r) + size_t(n) * (c0 + c)] -= acc[u][w];
+        }
 }
 
-// block row i of X = L^{-1}: for bj < i (blockIdx.x): T = sum_{k=bj}^{i-1} L_ik X_kj, X_ij = -D_i T
-__global__ void __launch_bounds__(kGemmThreads) chol_inv_row_kernel(int n, const double *A, double *X, int bi,
-                                                                    const double *Dall, double *scratch,
-                                                                    const int *info_d)
+// Doubling level s: pair blockIdx.z, tile (blockIdx.x, blockIdx.y) of the block below X11.
+// step 0: T = L21 X11 (X11 lower: t >= c); step 1: X21 = -X22 T (X22 lower: t <= r).
+__global__ void __launch_bounds__(kCholThreads) chol_double_kernel(int n, int s, int step, const double *L, double *X, double *T,
+                                                                   const int *info_d)
 {
     if (info_d[0]) return;
-    const int bj = blockIdx.x;
-    const int r0 = bi * kCb, c0 = bj * kCb;
-    const int rows = min(kCb, n - r0), cols = min(kCb, n - c0);
-    double *T = scratch + size_t(blockIdx.x) * kCb * kCb;
-    // T(r, c) = sum_{t = c0 .. r0-1} L(r0 + r, t) X(t, c0 + c): P = L rows, Q(c, t) = X(t, c0 + c)
-    // (Q given transposed: Q(c, t) = Xm[c + ldq t] needs X^T; use the rows form instead)
-    const int K = r0 - c0;
-    {
-        __shared__ double Ps[kKt][kTile + 1];
-        __shared__ double Qs[kKt][kTile + 1];
-        const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-        double acc[4][4] = {};
-        for (int k = 0; k < K; k += kKt) {
-            for (int t = threadIdx.x; t < kKt * kTile; t += kGemmThreads) {
-                const int rr = t % kTile, kk = t / kTile;
-                const int tt = c0 + k + kk;
-                Ps[kk][rr] = (rr < rows && k + kk < K) ? A[(r0 + rr) + size_t(n) * tt] : 0.0;
-                Qs[kk][rr] = (rr < cols && k + kk < K) ? X[tt + size_t(n) * (c0 + rr)] : 0.0;
-            }
-            __syncthreads();
-#pragma unroll 4
-            for (int kk = 0; kk < kKt; ++kk) {
-                double a[4], b[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    a[u] = Ps[kk][tx + 16 * u];
-                    b[u] = Qs[kk][ty + 16 * u];
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-#pragma unroll
-                    for (int w = 0; w < 4; ++w) acc[u][w] = fma(a[u], b[w], acc[u][w]);
-            }
-            __syncthreads();
-        }
-        for (int u = 0; u < 4; ++u)
-            for (int w = 0; w < 4; ++w) {
-                const int r = tx + 16 * u, c = ty + 16 * w;
-                T[r + kCb * c] = (r < rows && c < cols) ? acc[u][w] : 0.0;
-            }
+    const int base = blockIdx.z * 2 * s, r0 = base + s + blockIdx.x * kCb, c0 = base + blockIdx.y * kCb;
+    if (r0 >= n) return;
+    const int rows = min(kCb, min(n, base + 2 * s) - r0), cols = kCb;   // columns lie in a whole block
+    double acc[2][2] = {};
+    double *out;
+    if (step == 0) {
+        tile32(rows, cols, base + s - c0, L + r0 + size_t(n) * c0, n, X + c0 + size_t(n) * c0, n, 1, acc);
+        out = T;
+    } else {
+        const int t0 = base + s;
+        tile32(rows, cols, r0 + rows - t0, X + r0 + size_t(n) * t0, n, T + t0 + size_t(n) * c0, n, 1, acc);
+        out = X;
     }
-    __syncthreads();
-    // X_ij(r, c) = -sum_t D_i(r, t) T(t, c): P = D_i (rows r), Q(c, t) = T(t, c) -> T^T
-    const double *Di = Dall + size_t(bi) * kCb * kCb;
-    {
-        __shared__ double Ps[kKt][kTile + 1];
-        __shared__ double Qs[kKt][kTile + 1];
-        const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-        double acc[4][4] = {};
-        for (int k = 0; k < rows; k += kKt) {
-            for (int t = threadIdx.x; t < kKt * kTile; t += kGemmThreads) {
-                const int rr = t % kTile, kk = t / kTile;
-                Ps[kk][rr] = (k + kk < rows) ? Di[rr + kCb * (k + kk)] : 0.0;
-                Qs[kk][rr] = (k + kk < rows) ? T[(k + kk) + kCb * rr] : 0.0;
-            }
-            __syncthreads();
-#pragma unroll 4
-            for (int kk = 0; kk < kKt; ++kk) {
-                double a[4], b[4];
+    const double sg = step ? -1.0 : 1.0;
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    a[u] = Ps[kk][tx + 16 * u];
-                    b[u] = Qs[kk][ty + 16 * u];
-                }
+    for (int u = 0; u < 2; ++u)
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
-#pragma unroll
-                    for (int w = 0; w < 4; ++w) acc[u][w] = fma(a[u], b[w], acc[u][w]);
-            }
-            __syncthreads();
+        for (int w = 0; w < 2; ++w) {
+            const int r = tx + 16 * u, c = ty + 16 * w;
+            if (r < rows && c < cols) out[(r0 + r) + size_t(n) * (c0 + c)] = sg * acc[u][w];
         }
-        for (int u = 0; u < 4; ++u)
-            for (int w = 0; w < 4; ++w) {
-                const int r = tx + 16 * u, c = ty + 16 * w;
-                if (r < rows && c < cols) X[(r0 + r) + size_t(n) * (c0 + c)] = -acc[u][w];
-            }
-    }
 }
 
 }  // namespace
@@ -568,44 +422,35 @@ int cholesky_neg_sym_and_inverse(Plan &P, int n, const double *M, double *Linv, 
                                  cudaStream_t s)
 {
     int tb = timing_begin(P, EXX_TIMING_CHOL, s);
-    if (n <= kCholSmemMax) {
-        const size_t smem = (size_t(n) * n + n) * sizeof(double);
-        EXX_CUDA(cudaFuncSetAttribute(cholesky_inverse_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      int(smem)));
-        cholesky_inverse_smem_kernel<<<1, kCholThreads, smem, s>>>(n, M, Linv, info_d);
-        timing_end(P, tb, s);
-        EXX_LAUNCH("cholesky_inverse_smem_kernel");
-        P.launches++;
-        return EXX_OK;
-    }
-    // workspace: A (n x n), the diagonal-block inverses (nbk blocks of kCb^2), tile scratch
-    const int nbk = (n + kCb - 1) / kCb;
-    const size_t nn = size_t(n) * n, blk = size_t(kCb) * kCb;
-    if (int rc = dev_reserve(P.small_ws, (nn + 2 * size_t(nbk) * blk) * sizeof(double))) return rc;
+    // workspace: A (n x n), the products of the doubling (n x n), one diagonal-block inverse
+    const size_t nn = size_t(n) * n;
+    if (int rc = dev_reserve(P.small_ws, (2 * nn + kCb * kCb) * sizeof(double))) return rc;
     double *A = static_cast<double *>(P.small_ws.p);
-    double *Dall = A + nn;
-    double *scratch = Dall + size_t(nbk) * blk;
+    double *T = A + nn, *Dk = T + nn;
     const int eg = std::min(4 * P.num_sms, int((nn + 255) / 256));
     chol_prep_kernel<<<eg, 256, 0, s>>>(n, M, A, Linv, info_d);
     EXX_LAUNCH("chol_prep_kernel");
     P.launches++;
-    for (int kb = 0; kb < nbk; ++kb) {
-        const int k0 = kb * kCb, b = std::min(kCb, n - k0);
-        chol_diag_kernel<<<1, kCholThreads, 0, s>>>(n, A, k0, b, Dall + size_t(kb) * blk, Linv, info_d);
+    for (int k0 = 0; k0 < n; k0 += kCb) {
+        const int b = std::min(kCb, n - k0), rest = n - k0 - b;
+        chol_diag_kernel<<<1, 32, 0, s>>>(n, A, k0, b, Dk, Linv, info_d);
         EXX_LAUNCH("chol_diag_kernel");
         P.launches++;
-        const int rest = nbk - kb - 1;
         if (rest == 0) break;
-        chol_panel_kernel<<<rest, kGemmThreads, 0, s>>>(n, A, k0, b, Dall + size_t(kb) * blk, scratch, info_d);
+        chol_panel_kernel<<<(rest + kPanel - 1) / kPanel, kCholThreads, 0, s>>>(n, A, k0, b, Dk, info_d);
         EXX_LAUNCH("chol_panel_kernel");
-        chol_update_kernel<<<dim3(rest, rest), kGemmThreads, 0, s>>>(n, A, k0, b, info_d);
+        const unsigned nt = unsigned((rest + kCb - 1) / kCb);
+        chol_update_kernel<<<dim3(nt, nt), kCholThreads, 0, s>>>(n, A, k0, b, info_d);
         EXX_LAUNCH("chol_update_kernel");
         P.launches += 2;
     }
-    for (int bi = 1; bi < nbk; ++bi) {
-        chol_inv_row_kernel<<<bi, kGemmThreads, 0, s>>>(n, A, Linv, bi, Dall, scratch, info_d);
-        EXX_LAUNCH("chol_inv_row_kernel");
-        P.launches++;
+    for (int sz = kCb; sz < n; sz *= 2) {
+        const dim3 grid(unsigned(sz / kCb), unsigned(sz / kCb), unsigned((n - sz + 2 * sz - 1) / (2 * sz)));
+        for (int step = 0; step < 2; ++step) {
+            chol_double_kernel<<<grid, kCholThreads, 0, s>>>(n, sz, step, A, Linv, T, info_d);
+            EXX_LAUNCH("chol_double_kernel");
+            P.launches++;
+        }
     }
     timing_end(P, tb, s);
     return EXX_OK;
