@@ -156,7 +156,8 @@ __global__ void __launch_bounds__(32 * kCutWarps) gemm_cut_kernel(const CutArgs 
     __syncthreads();
     int E = 100;   // rows below 2^-922 are zero rows
 #pragma unroll
-    for (int w = 0; w < kCutWarps; ++w) E = max(E, smax[w][lane]);
+    for (int w = 0; w < kCutWarps; ++w)
+        if (w < int(blockDim.x >> 5)) E = max(E, smax[w][lane]);   // a short contraction launches fewer warps
     if (row < a.prow && warp == 0 && (!KFAST || lane < 8)) a.sh[chunk * a.prow + row] = E;
     const long kb = chunk * kBlks + warp;
     if (kb >= a.nkb || row >= a.prow) return;
@@ -230,8 +231,10 @@ __device__ __forceinline__ void gemm_bulk_load(void *dst, const void *src, uint3
 // products per k (7 MMAs of up to 192 columns: neighbouring B digits feed neighbouring
 // levels), 632 cycles per 16 k of a 128 x 96 tile against 28.7 KB of operands; the combination
 // of a finished chunk is not overlapped, the five level accumulators fill TMEM.
-template <int G>
-__global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_constant__ GemmArgs a)
+// NH: most columns of a drain warp's half.  Narrow tiles (up to 32 columns) are bound by the operand
+// blocks' way from L2 and by the chain load - MMA - drain - store of one item, so two CTAs share an SM.
+template <int G, int NH>
+__global__ void __launch_bounds__(kThreads, NH <= 16 ? 2 : 1) tc_gemm_kernel(const __grid_constant__ GemmArgs a)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     float *fbs = reinterpret_cast<float *>(smem + a.offTab);       // column factors of a chunk, two sets
@@ -388,7 +391,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         const int quarter = warp & 3, half = warp >> 2;
         const int row = quarter * 32 + lane;
         const uint32_t lane_q = uint32_t(quarter * 32) << 16;
-        constexpr int kHalf = kTN / 2;
+        constexpr int kHalf = NH;
         const int ncol = Nt / 2, cbase = half * ncol;   // Nt is a multiple of 16
         constexpr int NT = 32 * kDrainWarps;
         long dseq = 0;
@@ -493,17 +496,29 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
     }
 }
 
-// D(i, j) (+)= alpha sum_z W[z][i + m j] with the output strides.
-__global__ void tc_gemm_reduce_kernel(const double *W, int Z, long m, int n, double alpha, double *D, long ds_i,
-                                      long ds_j, int add)
+// D(i, j) (+)= alpha sum_z W[z][i + m j] with the output strides: 32 entries per CTA, eight threads
+// each take every eighth split, then a fixed order (one thread per entry left 116 loads in sequence:
+// 20 us for 128 x 16).
+constexpr int kRedZ = 8;
+__global__ void __launch_bounds__(32 * kRedZ) tc_gemm_reduce_kernel(const double *W, int Z, long m, int n, double alpha, double *D,
+                                                                    long ds_i, long ds_j, int add)
 {
+    __shared__ double sh[kRedZ][32];
     const long tot = m * n;
-    for (long e = long(blockIdx.x) * blockDim.x + threadIdx.x; e < tot; e += long(gridDim.x) * blockDim.x) {
-        const long i = e % m, jj = e / m;
-        double *dp = D + i * ds_i + jj * ds_j;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    for (long e0 = long(blockIdx.x) * 32; e0 < tot; e0 += long(gridDim.x) * 32) {
+        const long e = e0 + tx;
         double s = 0.0;
-        for (int z = 0; z < Z; ++z) s += W[long(z) * tot + e];
-        *dp = add ? fma(alpha, s, *dp) : alpha * s;
+        if (e < tot)
+            for (int z = ty; z < Z; z += kRedZ) s += W[long(z) * tot + e];
+        sh[ty][tx] = s;
+        __syncthreads();
+        if (ty == 0 && e < tot) {
+            for (int z = 1; z < kRedZ; ++z) s += sh[z][tx];
+            double *dp = D + (e % m) * ds_i + (e / m) * ds_j;
+            *dp = add ? fma(alpha, s, *dp) : alpha * s;
+        }
+        __syncthreads();
     }
 }
 
@@ -526,11 +541,12 @@ int launch_cut(Plan &P, const double *X, long sr, long sk, long rows, long K, in
     c.prow = tiles * rt;
     c.vec = ((reinterpret_cast<uintptr_t>(X) | uintptr_t(sr * 8)) & 15) == 0;
     const unsigned chunks = unsigned(ceil_div(K, kChunk));
+    const int threads = 32 * int(std::min<long>(kCutWarps, c.nkb));
     const int tb = timing_begin(P, EXX_TIMING_GEMM, s);
     if (sk == 1)
-        gemm_cut_kernel<true><<<dim3(unsigned(ceil_div(c.prow, 8)), chunks), 32 * kCutWarps, 0, s>>>(c);
+        gemm_cut_kernel<true><<<dim3(unsigned(ceil_div(c.prow, 8)), chunks), threads, 0, s>>>(c);
     else
-        gemm_cut_kernel<false><<<dim3(unsigned(ceil_div(c.prow, 32)), chunks), 32 * kCutWarps, 0, s>>>(c);
+        gemm_cut_kernel<false><<<dim3(unsigned(ceil_div(c.prow, 32)), chunks), threads, 0, s>>>(c);
     timing_end(P, tb, s);
     EXX_LAUNCH("gemm_cut_kernel");
     P.launches++;
@@ -571,9 +587,10 @@ int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_
     mslab = ceil_div(ceil_div(mpad, kT), ceil_div(mpad, mslab)) * kT;
     // k splits: items (tiles x splits) for a whole number of rounds over the SMs
     const long tiles = (mslab / kT) * nt;
+    const long slots = long(P.num_sms) * (Nt <= 32 ? 2 : 1);   // CTAs resident at once
     auto splits = [&](long nch) {
-        if (nch < 2 || tiles >= 2L * P.num_sms) return 1L;
-        const long round = std::max(1L, P.num_sms / tiles);
+        if (nch < 2 || tiles >= 2 * slots) return 1L;
+        const long round = std::max(1L, slots / tiles);
         long Z = nch >= 8 * round ? 2 * round : round;
         Z = std::min(Z, nch);
         return std::min(Z, std::max(1L, (1L << 28) / (mslab * n * 8)));
@@ -601,15 +618,19 @@ int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_
     a.ktri = ktri ? 1 : 0;
     a.err = static_cast<int *>(P.err_d.p);
     a.stage_bytes = uint32_t(kT + Nt) * kBlk * 2 * kDig;
-    a.stages = int(std::min<size_t>(8, 200 * 1024 / a.stage_bytes));
+    a.stages = int(std::min<size_t>(8, (Nt <= 32 ? 111 : 200) * 1024 / a.stage_bytes));
     a.offTab = uint32_t(a.stages) * a.stage_bytes;
     a.offBar = a.offTab + uint32_t(round_up(2 * kTN * 4 + kTN * 4, 16));
     a.tmem_cols = 32;
     while (a.tmem_cols < kLev * Nt) a.tmem_cols *= 2;
-    const size_t smem = std::max<size_t>(a.offBar + (2 * size_t(a.stages) + 2) * 8 + 16, 120 * 1024);   // one CTA per SM
+    size_t smem = a.offBar + (2 * size_t(a.stages) + 2) * 8 + 16;
+    if (Nt > 32) smem = std::max<size_t>(smem, 120 * 1024);   // one CTA per SM
     // B digits per MMA: at most 256 columns
     const int gmax = 256 / Nt;
-    auto kern = gmax >= 4 ? tc_gemm_kernel<4> : gmax == 3 ? tc_gemm_kernel<3> : tc_gemm_kernel<2>;
+    auto kern = Nt <= 32    ? tc_gemm_kernel<4, 16>
+                : gmax >= 4 ? tc_gemm_kernel<4, kTN / 2>
+                : gmax == 3 ? tc_gemm_kernel<3, kTN / 2>
+                            : tc_gemm_kernel<2, kTN / 2>;
     EXX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
 
     for (long c0 = 0; c0 < chunks; c0 += kslab) {
@@ -647,14 +668,14 @@ int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_
             }
             const long items = a.Z * a.mt * a.nt;
             int tb = timing_begin(P, EXX_TIMING_GEMM, s);
-            kern<<<unsigned(std::min<long>(items, P.num_sms)), kThreads, smem, s>>>(a);
+            kern<<<unsigned(std::min<long>(items, slots)), kThreads, smem, s>>>(a);
             timing_end(P, tb, s);
             EXX_LAUNCH("tc_gemm_kernel");
             P.launches++;
             if (a.Z > 1) {
                 const long tot = mr * n;
                 tb = timing_begin(P, EXX_TIMING_GEMM, s);
-                tc_gemm_reduce_kernel<<<unsigned(std::min<long>((tot + 255) / 256, 4L * P.num_sms)), 256, 0, s>>>(
+                tc_gemm_reduce_kernel<<<unsigned(std::min<long>((tot + 31) / 32, 32L * P.num_sms)), 32 * kRedZ, 0, s>>>(
                     a.D, int(a.Z), mr, n, alpha, Dd, ds_i, ds_j, c0 > 0);
                 timing_end(P, tb, s);
                 EXX_LAUNCH("tc_gemm_reduce_kernel");
