@@ -525,6 +525,8 @@ __global__ void __launch_bounds__(32 * kRedZ) tc_gemm_reduce_kernel(const double
 inline long ceil_div(long a, long b) { return (a + b - 1) / b; }
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
+// Rows past the last group of 8 (or 32) that holds a valid one are left as they are: a row of an
+// operand only reaches its own row or column of the output, and those are never stored.
 int launch_cut(Plan &P, const double *X, long sr, long sk, long rows, long K, int rt, long tiles, uint8_t *dig, int *sh,
                cudaStream_t s)
 {
@@ -544,9 +546,9 @@ int launch_cut(Plan &P, const double *X, long sr, long sk, long rows, long K, in
     const int threads = 32 * int(std::min<long>(kCutWarps, c.nkb));
     const int tb = timing_begin(P, EXX_TIMING_GEMM, s);
     if (sk == 1)
-        gemm_cut_kernel<true><<<dim3(unsigned(ceil_div(c.prow, 8)), chunks), threads, 0, s>>>(c);
+        gemm_cut_kernel<true><<<dim3(unsigned(ceil_div(c.rows, 8)), chunks), threads, 0, s>>>(c);
     else
-        gemm_cut_kernel<false><<<dim3(unsigned(ceil_div(c.prow, 32)), chunks), threads, 0, s>>>(c);
+        gemm_cut_kernel<false><<<dim3(unsigned(ceil_div(c.rows, 32)), chunks), threads, 0, s>>>(c);
     timing_end(P, tb, s);
     EXX_LAUNCH("gemm_cut_kernel");
     P.launches++;
@@ -570,7 +572,7 @@ int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_
     // slabs: the digit planes (8 B per element) of one slab stay within kDigitBudget, cut along
     // m when the contraction is short, along k when it is long
     const long chunks = ceil_div(K, kChunk);
-    const long chunk_bytes = 8L * kChunk;   // per row
+    const long chunk_bytes = std::min(8L * kChunk, ceil_div(K, kBlk) * kBlk * 8);   // per row (and of a lone short chunk)
     const long mpad = ceil_div(m, kT) * kT;
     const bool long_k = chunks > 64;
     long mslab = mpad, kslab = chunks;
