@@ -112,8 +112,9 @@ int exx_plan_create(exx_plan *out, int Nx, int Ny, int Nz, double h, const int b
 int exx_plan_set_precision(exx_plan plan, int prec);
 
 /* Tuning: pairs per batch (the paper's n_c, Sec. II.B) and orbitals per pair block.
- * 0 = defaults: blocks of 8 orbitals, and as many pairs per batch as fit two plan-owned
- * work buffers of at most 2 GiB each, at most 1024, a multiple of block^2.  Results do
+ * 0 = defaults: blocks of 16 orbitals (8 when 256 pair fields pass a work buffer, or when the plan is
+ * sharded), and as many pairs per batch as fit two plan-owned work buffers of at most 2 GiB
+ * each, at most 1024, a multiple of block^2.  Results do
  * not depend on either (up to the order of the compensated sums). */
 int exx_plan_set_batch(exx_plan plan, int pairs_per_batch, int block_orbitals);
 
@@ -201,7 +202,8 @@ int exx_energy(exx_plan plan, const double *Psi_occ, int n_occ, long ld, const d
  * (NULL to skip).  FP64 plans compute every step on the CUDA cores in FP64.  Split
  * plans compute the products M and xi on the tensor cores: fixed-point digits of 31
  * bits per 320-long chunk of the contraction (rows scaled by their largest entry),
- * exact integer sums per chunk, FP64 across chunks (relative error ~1e-9..1e-8).  The
+ * exact integer sums per chunk, FP32 pairs (48 bits) across chunks, FP64 across splits of the
+ * contraction (relative error ~1e-9..1e-8).  The
  * Cholesky factor and its inverse are FP64 in every mode.
  * *info_h (host) is 0, or 1 + the failing pivot when EXX_ERR_NOT_POSDEF is
  * returned.  Synchronizes `stream`.  n <= 2048. */

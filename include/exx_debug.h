@@ -37,7 +37,8 @@ int exx_debug_tc_gemm(int tf32, int n, int k, const float *A, const float *B, fl
  * (field, row in field) (Granlund & Montgomery 1994, Fig. 4.1), host-side.  d >= 1. */
 int exx_debug_fastdiv(unsigned d, int count, const unsigned *n, unsigned *q);
 
-/* The automatic BF16X7 (three-pass) layouts of an n1 x n2 x n3 grid, host-side (no device):
+/* The BF16X7 (three-pass) layouts of the older kernel forms for an n1 x n2 x n3 grid (what a grid gets
+ * whose x/y matrices do not stay resident, and hand-made settings), host-side (no device):
  * out (HOST int[16]) = supported; shared memory of pass A and pass C; pass A streams its x/y
  * matrices and their chunk width; the same for pass C; pass A pipelined; pass A staged; pass B
  * shared memory (0 = none fits); pass B K-chunks; its chunk or block width; its buffers; its

@@ -16,6 +16,10 @@
 // than about 108 points) a producer warp streams them through two buffers as K-chunks, every
 // chunk holding all outputs of its contraction indices.
 //
+// Each pass has two forms with the same arithmetic: the direct form (slice_direct_kernel,
+// zpass_direct_kernel), the automatic choice, and the older one described above, for slices whose
+// two matrices do not stay resident and for settings made by hand.
+//
 // Arithmetic of one mode product D[row][n] = sum_k A[row][k] C[n][k]:
 //  * every data row gets a power-of-two scale from its largest entry and is cut into three
 //    balanced base-512 digits d0 + d1 + d2 (d0 an integer of magnitude <= 256, d1 a
@@ -1539,7 +1543,7 @@ __global__ void __launch_bounds__(kRows * TPR + 64, (UPT <= 4 ? 2 : 1)) zpass_ke
 //     instruction off shared memory: N / 2 cycles per MMA instead of (128 + N) / 4.
 //   STREAM = false: both matrix images resident, up to three groups per SM.
 //   STREAM = true (long axes): one group of 512, the images pass through `nbuf` buffers as
-//     K-chunks of KC; the thread that issues the MMAs also issues the copies: those of the first
+//     K-chunks of KC; the warp that issues the MMAs also issues the copies: those of the first
 //     nbuf chunks when the previous GEMM has finished, the others as the chunks are consumed.
 // Per pair solve against zpass_kernel: 48^3 0.621 -> 0.292 us, 72 x 72 x 144 5.15 -> 3.14, 117 x 117 x
 // 119 8.9 -> 5.1.  Of that the MMA issue by a converged warp gave 0.373 -> 0.292 and 4.34 -> 3.14.
@@ -2015,7 +2019,7 @@ SliceLayout slice_layout_for(const Plan &P, bool pair, bool pipe, bool bstream =
     return L;
 }
 
-// The plan's choice: pipelined when tuned so, or (automatic) when it fits and the serial form
+// The older form's choice: pipelined when tuned so, or (automatic) when it fits and the serial form
 // cannot run two CTAs per SM.
 SliceLayout slice_layout(const Plan &P, bool pair = true)
 {
@@ -2606,7 +2610,7 @@ int tc3_solve_batch(Plan &P, const int2 *pairs_d, int nfields, float *bufA, floa
     return EXX_OK;
 }
 
-// Host only: the automatic BF16X7 layouts of an n1 x n2 x n3 grid (no device involved).
+// Host only: the BF16X7 layouts of the older forms for an n1 x n2 x n3 grid (no device involved).
 // out[0] supported; [1] [2] shared memory of pass A / pass C; [3] [4] pass A streams its x/y
 // matrices, chunk width; [5] [6] the same for pass C; [7] pass A pipelined, [8] staged;
 // [9] pass B shared memory (0: none fits); [10] pass B K-chunks; [11] chunk or block width;
