@@ -27,6 +27,12 @@ int exx_debug_sym_eig(int n, const double *A, double *V, double *lam);
 int exx_debug_schedule(int n_occ, int n_in, int aliased, int block, int max_pairs, long *npairs,
                        long *nbatches, long *nblocks, int *pairs, int *batches, int *blocks);
 
+/* The batches that exx_apply runs on a plan of N points with these settings (exx_plan_set_precision,
+ * _set_shard, _set_batch): limits = {orbitals per pair block, most pairs per batch}; batches (2 ints
+ * each: pair fields, 1 when its outputs are those of one side only) may be NULL to get the number. */
+int exx_debug_plan_schedule(long N, int prec, int world, int pairs_per_batch, int block_orbitals, int n_occ, int n_in,
+                            int aliased, int *limits, long *nbatches, int *batches);
+
 /* One 128 x n x k tensor-core tile (tcgen05.mma, one bf16 or tf32 piece per operand,
  * FP32 accumulation): D (128 x n, row-major) = A (128 x k, row-major) B (n x k,
  * row-major)^T.  DEVICE pointers; n, k multiples of 16 in [16, 256].  Synchronizes the

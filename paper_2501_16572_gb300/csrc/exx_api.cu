@@ -81,39 +81,13 @@ static void free_plan_buffers(Plan &P)
         dev_free(*b);
 }
 
-constexpr long kBatchBudget = 2048L << 20;   // per work buffer (two of them)
-static long field_bytes(const Plan &P)
-{
-    return long(P.N) * (P.prec == EXX_PREC_FP64 || P.prec == EXX_PREC_BF16X10 ? 8 : 4);
-}
-
-// Default pair block: 16 orbitals.  The accumulation reads and writes its sums once per block
-// (2.25 B per 4 B of pair field at 16 x 16, 4.5 B at 8 x 8), small systems need fewer batches of
-// launches (16 orbitals: one diagonal block instead of two batches), and rounds of the schedule
-// reach the default batch.  8 where a 16 x 16 block passes the batch buffer, and for sharded
-// plans, which deal whole batches to the ranks.
-static int default_block(const Plan &P)
-{
-    return P.shard_world == 1 && kBatchBudget / field_bytes(P) >= 256 ? 16 : 8;
-}
-
-// Default batch size: enough fields per launch that every SM loops over tens of tiles
-// (launch start-up and the last tile's drain are amortised), capped by a memory budget
-// per batch buffer.
-static int default_pairs(const Plan &P, int block)
-{
-    long pairs = std::max<long>(block * block, kBatchBudget / field_bytes(P));
-    pairs = std::min<long>(pairs, 1024);
-    return int((pairs / (block * block)) * (block * block));
-}
-
 static int ensure_schedule(Plan &P, int n_occ, int n_in, bool aliased, cudaStream_t s)
 {
-    const int block = P.block_orbitals > 0 ? P.block_orbitals : default_block(P);
-    const int maxp = P.pairs_per_batch > 0 ? P.pairs_per_batch : default_pairs(P, block);
-    int key[4] = {n_occ, n_in, (aliased ? 1 : 0) | (block << 1), maxp};
+    int block, maxp;
+    schedule_limits(P.N, P.prec, P.shard_world, P.pairs_per_batch, P.block_orbitals, block, maxp);
+    int key[4] = {n_occ, n_in, (aliased ? 1 : 0) | (P.shard_world > 1 ? 2 : 0) | (block << 2), maxp};
     if (std::equal(key, key + 4, P.sched_key)) return EXX_OK;
-    P.sched = build_schedule(n_occ, n_in, aliased, block, maxp);
+    P.sched = build_schedule(n_occ, n_in, aliased, block, maxp, P.shard_world);
     P.sched_block = std::min(block, std::max(n_occ, n_in));
     if (int rc = dev_reserve(P.pairs_d, std::max<size_t>(1, P.sched.pairs.size()) * sizeof(int2))) return rc;
     if (int rc = dev_reserve(P.blocks_d, std::max<size_t>(1, P.sched.blocks.size()) * sizeof(Block))) return rc;

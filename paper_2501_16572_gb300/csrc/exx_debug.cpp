@@ -71,6 +71,23 @@ int exx_debug_schedule(int n_occ, int n_in, int aliased, int block, int max_pair
     return EXX_OK;
 }
 
+int exx_debug_plan_schedule(long N, int prec, int world, int pairs_per_batch, int block_orbitals, int n_occ, int n_in,
+                            int aliased, int *limits, long *nbatches, int *batches)
+{
+    if (N < 1 || world < 1 || pairs_per_batch < 0 || block_orbitals < 0 || block_orbitals > 32 || n_occ < 1 || n_in < 1 ||
+        !limits || !nbatches)
+        return EXX_ERR_INVALID_ARG;
+    exx::schedule_limits(N, prec, world, pairs_per_batch, block_orbitals, limits[0], limits[1]);
+    const exx::Schedule S = exx::build_schedule(n_occ, n_in, aliased != 0, limits[0], limits[1], world);
+    *nbatches = long(S.batches.size());
+    if (batches)
+        for (size_t i = 0; i < S.batches.size(); ++i) {
+            batches[2 * i] = S.batches[i].nfields;
+            batches[2 * i + 1] = S.blocks[S.batches[i].block0].kind == exx::BLK_ONE_SIDE;
+        }
+    return EXX_OK;
+}
+
 int exx_debug_tc_gemm(int tf32, int n, int k, const float *A, const float *B, float *D, int *err)
 {
     if (!A || !B || !D || !err) return EXX_ERR_INVALID_ARG;

@@ -221,7 +221,23 @@ static int block_pairs(const Block &b)
     return b.kind == BLK_SYM_DIAG ? b.nI * (b.nI + 1) / 2 : b.nI * b.nJ;
 }
 
-Schedule build_schedule(int n_occ, int n_in, bool aliased, int B, int max_pairs)
+// Default pair block: 16 orbitals.  The accumulation reads and writes its sums once per block
+// (2.25 B per 4 B of pair field at 16 x 16, 4.5 B at 8 x 8), small systems need fewer batches of
+// launches (16 orbitals: one diagonal block instead of two batches), and rounds of the schedule
+// reach the default batch.  8 where a 16 x 16 block passes the batch buffer, and for sharded
+// plans, which deal whole batches to the ranks.
+// Default batch size: enough fields per launch that every SM loops over tens of tiles
+// (launch start-up and the last tile's drain are amortised), capped by a memory budget
+// per batch buffer (two of them).
+void schedule_limits(long N, int prec, int world, int set_pairs, int set_block, int &block, int &max_pairs)
+{
+    const long fit = (2048L << 20) / (N * (prec == EXX_PREC_FP64 || prec == EXX_PREC_BF16X10 ? 8 : 4));
+    block = set_block > 0 ? set_block : world == 1 && fit >= 256 ? 16 : 8;
+    const int b2 = block * block;
+    max_pairs = set_pairs > 0 ? set_pairs : int(std::min<long>(std::max<long>(b2, fit), 1024) / b2) * b2;
+}
+
+Schedule build_schedule(int n_occ, int n_in, bool aliased, int B, int max_pairs, int world)
 {
     Schedule S;
     if (max_pairs < B * B) max_pairs = B * B;
@@ -249,13 +265,16 @@ Schedule build_schedule(int n_occ, int n_in, bool aliased, int B, int max_pairs)
     const int nt = n_in - t_begin;
     if (nt > 0) {
         // one-sided blocks write only their J outputs, so a block may hold many occupied orbitals:
-        // as many (in steps of B) as let all column groups share one batch
+        // as many (in steps of B) as let all column groups share one batch.  A sharded plan deals
+        // batches to its ranks: B orbitals a round there, rotated so that no round collects a shorter last group
+        // (128 x 16 on 8 ranks: 16 batches of 128 fields; 2 of 1024 left six ranks idle)
         const int Gt = (nt + B - 1) / B;
-        const int C = std::min(Go * B, std::max(B, max_pairs / nt / B * B));
-        for (int I0 = 0; I0 < n_occ; I0 += C) {
+        const int C = world > 1 ? B : std::min(Go * B, std::max(B, max_pairs / nt / B * B));
+        const int Gc = (n_occ + C - 1) / C;
+        for (int r = 0; r < Gc; ++r) {
             std::vector<Block> blks;
             for (int t = 0; t < Gt; ++t) {
-                const int J0 = t_begin + t * B;
+                const int I0 = (world > 1 ? (t + r) % Gc : r) * C, J0 = t_begin + t * B;
                 blks.push_back({I0, std::min(C, n_occ - I0), J0, std::min(B, n_in - J0), BLK_ONE_SIDE, 0});
             }
             rounds.push_back(blks);

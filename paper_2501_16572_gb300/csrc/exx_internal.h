@@ -101,7 +101,10 @@ struct Schedule {
     int max_fields = 0;
     int max_blocks = 0;
 };
-Schedule build_schedule(int n_occ, int n_in, bool aliased, int block, int max_pairs);
+Schedule build_schedule(int n_occ, int n_in, bool aliased, int block, int max_pairs, int world = 1);
+// Orbitals per pair block and pairs per batch of a plan of N points sharded over `world` ranks
+// (set_pairs, set_block: the caller's settings, 0 = automatic).
+void schedule_limits(long N, int prec, int world, int set_pairs, int set_block, int &block, int &max_pairs);
 
 // ---- host FP64 setup -------------------------------------------------------------------
 void fd_weights(int p, double *w);                       // w[0..p]

@@ -161,6 +161,32 @@ def test_schedule_covers_each_pair_once_with_disjoint_outputs(lib, n_occ, n_in, 
     assert p0 == len(pairs)
 
 
+def plan_schedule(lib, N, prec, world, pairs, block, n_occ, n_in, aliased):
+    Ip, L = ctypes.POINTER(ctypes.c_int), ctypes.c_long
+    lib.exx_debug_plan_schedule.argtypes = [L] + [ctypes.c_int] * 7 + [Ip, ctypes.POINTER(L), Ip]
+    lim, nb = (ctypes.c_int * 2)(), L()
+    args = (N, prec, world, pairs, block, n_occ, n_in, aliased, lim, ctypes.byref(nb))
+    assert lib.exx_debug_plan_schedule(*args, None) == 0
+    b = np.zeros((nb.value, 2), dtype=np.int32)
+    assert lib.exx_debug_plan_schedule(*args, b.ctypes.data_as(Ip)) == 0
+    return list(lim), b
+
+
+@pytest.mark.parametrize("n_occ, n_in, aliased", [(128, 16, 0), (60, 8, 0), (40, 30, 0), (160, 8, 0), (5, 100, 0),
+                                                  (100, 128, 1), (31, 40, 1)])
+@pytest.mark.parametrize("world", [2, 4, 8])
+def test_sharded_one_sided_batches_spread_over_the_ranks(lib, n_occ, n_in, aliased, world):
+    """A sharded plan deals batch b to rank b mod world.  One-sided batches hold 8 occupied
+    orbitals each, so no rank gets more of them than ceil(number / world)."""
+    import paper_2501_16572_gb300 as exx
+    lim, b = plan_schedule(lib, 48 ** 3, exx.EXX_PREC_BF16X7, world, 0, 0, n_occ, n_in, aliased)
+    assert lim[0] == 8
+    nt = n_in - n_occ if aliased else n_in
+    share = [int(b[r::world][b[r::world, 1] == 1, 0].sum()) for r in range(world)]
+    assert sum(share) == n_occ * nt
+    assert max(share) <= -(-(-(-n_occ // 8)) // world) * 8 * nt
+
+
 def test_fast_division_matches_integer_division(lib):
     """Row -> (field, row in field) in the pass kernels divides by multiply and shift;
     every quotient must equal the integer one, at the divisor and quotient edges too."""
