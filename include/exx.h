@@ -112,8 +112,8 @@ int exx_plan_create(exx_plan *out, int Nx, int Ny, int Nz, double h, const int b
 int exx_plan_set_precision(exx_plan plan, int prec);
 
 /* Tuning: pairs per batch (the paper's n_c, Sec. II.B) and orbitals per pair block.
- * 0 = defaults: blocks of 16 orbitals (8 when 256 pair fields pass a work buffer, or when the plan is
- * sharded), and as many pairs per batch as fit two plan-owned work buffers of at most 2 GiB
+ * 0 = defaults: blocks of 16 orbitals (8 when 256 pair fields pass a work buffer or the pairs per
+ * batch set here, or when the plan is sharded), and as many pairs per batch as fit two plan-owned work buffers of at most 2 GiB
  * each, at most 1024, a multiple of block^2.  Results do
  * not depend on either (up to the order of the compensated sums). */
 int exx_plan_set_batch(exx_plan plan, int pairs_per_batch, int block_orbitals);

@@ -224,15 +224,15 @@ static int block_pairs(const Block &b)
 // Default pair block: 16 orbitals.  The accumulation reads and writes its sums once per block
 // (2.25 B per 4 B of pair field at 16 x 16, 4.5 B at 8 x 8), small systems need fewer batches of
 // launches (16 orbitals: one diagonal block instead of two batches), and rounds of the schedule
-// reach the default batch.  8 where a 16 x 16 block passes the batch buffer, and for sharded
-// plans, which deal whole batches to the ranks.
+// reach the default batch.  8 where a 16 x 16 block passes the batch buffer or the batch that the
+// caller asked for, and for sharded plans, which deal whole batches to the ranks.
 // Default batch size: enough fields per launch that every SM loops over tens of tiles
 // (launch start-up and the last tile's drain are amortised), capped by a memory budget
 // per batch buffer (two of them).
 void schedule_limits(long N, int prec, int world, int set_pairs, int set_block, int &block, int &max_pairs)
 {
     const long fit = (2048L << 20) / (N * (prec == EXX_PREC_FP64 || prec == EXX_PREC_BF16X10 ? 8 : 4));
-    block = set_block > 0 ? set_block : world == 1 && fit >= 256 ? 16 : 8;
+    block = set_block > 0 ? set_block : world == 1 && (set_pairs > 0 ? set_pairs : fit) >= 256 ? 16 : 8;
     const int b2 = block * block;
     max_pairs = set_pairs > 0 ? set_pairs : int(std::min<long>(std::max<long>(b2, fit), 1024) / b2) * b2;
 }

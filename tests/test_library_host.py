@@ -187,6 +187,17 @@ def test_sharded_one_sided_batches_spread_over_the_ranks(lib, n_occ, n_in, alias
     assert max(share) <= -(-(-(-n_occ // 8)) // world) * 8 * nt
 
 
+@pytest.mark.parametrize("n_occ, n_in, aliased", [(16, 16, 1), (128, 128, 1), (100, 128, 1), (40, 30, 0), (7, 3, 0)])
+@pytest.mark.parametrize("pairs", [0, 1, 64, 100, 255, 256, 600])
+def test_set_batch_limits_the_fields_of_a_batch(lib, n_occ, n_in, aliased, pairs):
+    """exx_plan_set_batch(plan, pairs, 0) runs no batch of more pairs than asked for, down to one
+    8 x 8 block."""
+    import paper_2501_16572_gb300 as exx
+    lim, b = plan_schedule(lib, 24 ** 3, exx.EXX_PREC_BF16X7, 1, pairs, 0, n_occ, n_in, aliased)
+    assert b[:, 0].max() <= (max(pairs, 64) if pairs else 1024)
+    assert lim[0] == (8 if 0 < pairs < 256 else 16)
+
+
 def test_fast_division_matches_integer_division(lib):
     """Row -> (field, row in field) in the pass kernels divides by multiply and shift;
     every quotient must equal the integer one, at the divisor and quotient edges too."""
