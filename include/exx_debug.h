@@ -70,6 +70,11 @@ int exx_debug_matrix_digits(int nout, int nk, const double *C, int WN, int Kp, i
  * The context stays usable.  Returns EXX_ERR_CUDA without a GPU. */
 int exx_debug_wait_timeout(int *status_h);
 
+/* The wait of the MMA-issuing warps: one kernel in which half of a warp's lanes run out of time
+ * before their barrier completes and the other half do not.  *went_on_h (HOST) has a bit for
+ * every lane that took the wait as completed: all or none. */
+int exx_debug_wait_warp(unsigned *went_on_h);
+
 #ifdef __cplusplus
 }
 #endif

@@ -108,4 +108,10 @@ int exx_debug_wait_timeout(int *status_h)
     return exx::tc_wait_timeout_probe(status_h);
 }
 
+int exx_debug_wait_warp(unsigned *went_on_h)
+{
+    if (!went_on_h) return EXX_ERR_INVALID_ARG;
+    return exx::tc_wait_warp_probe(went_on_h);
+}
+
 }  // extern "C"

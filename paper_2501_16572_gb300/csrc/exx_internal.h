@@ -229,6 +229,7 @@ void tc3_debug_matrix_digits(int nout, int nk, const double *C, int WN, int Kp, 
                              float *scales);
 int tc_unit_gemm(int tf32, int n, int k, const float *A, const float *B, float *D, int *err);
 int tc_wait_timeout_probe(int *status_h);
+int tc_wait_warp_probe(unsigned *went_on_h);
 
 // reductions, GEMM, Cholesky (exx_linalg.cu)
 int energy_fp64(Plan &P, const double *psi, int n, long ld, const double *f, const double *v,

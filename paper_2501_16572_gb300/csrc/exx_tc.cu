@@ -1758,7 +1758,36 @@ __global__ void tc_wait_timeout_kernel(uint32_t limit, uint64_t limit_ns, int *e
     if (!tc::mbar_wait_bounded(&bar, 0, limit) && threadIdx.x == 0) atomicOr(err, 1);
     if (!tc::mbar_wait_timed(&bar, 0, limit_ns) && threadIdx.x == 0) atomicOr(err, 2);
 }
+
+// A whole warp's wait whose limit runs out for its first 16 lanes (2 ms) before the barrier completes
+// (10 ms, by the second warp) and for the others after it (1 s): which lanes went on.
+__global__ void tc_wait_warp_kernel(uint32_t *went_on)
+{
+    __shared__ uint64_t bar;
+    if (threadIdx.x == 0) tc::mbar_init(&bar, 1);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const bool ok = tc::mbar_wait_warp(&bar, 0, threadIdx.x < 16 ? 2000000ull : 1000000000ull);
+        const uint32_t on = __ballot_sync(0xffffffffu, ok);
+        if (threadIdx.x == 0) *went_on = on;
+    } else if (threadIdx.x == 32) {
+        const uint64_t t0 = tc::globaltimer_ns();
+        while (tc::globaltimer_ns() - t0 < 10000000ull) {}
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(&bar)) : "memory");
+    }
+}
 }  // namespace
+
+int tc_wait_warp_probe(unsigned *went_on_h)
+{
+    uint32_t *d = nullptr;
+    EXX_CUDA(cudaMalloc(&d, sizeof(uint32_t)));
+    tc_wait_warp_kernel<<<1, 64>>>(d);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpy(went_on_h, d, sizeof(uint32_t), cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    return e == cudaSuccess ? EXX_OK : cuda_fail(e, "tc_wait_warp_probe");
+}
 
 int tc_wait_timeout_probe(int *status_h)
 {

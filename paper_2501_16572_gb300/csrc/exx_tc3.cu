@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kRows * TPR + 64, 2) slice_pass_kernel(const _
         long seq = 0;   // matrix chunks consumed (bstream)
         for (long tile = blockIdx.x; tile < a.ntiles && !bad; tile += gridDim.x) {
             for (int g = 0; g < 2 && !bad; ++g) {
-                if (!tc::mbar_wait_timed(bar_a, ph, kWaitNs)) {
+                if (!tc::mbar_wait_warp(bar_a, ph, kWaitNs)) {
                     atomicExch(sflag, 1);
                     bad = true;
                 }
@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(kRows * TPR + 64, 2) slice_pass_kernel(const _
                     const uint32_t d0 = g ? t2 : tmem;
                     for (int kc = 0; kc < nkc && !bad; ++kc, ++seq) {
                         const int slot = int(seq & 1);
-                        if (!tc::mbar_wait_timed(bfull + slot, uint32_t((seq >> 1) & 1), kWaitNs)) {
+                        if (!tc::mbar_wait_warp(bfull + slot, uint32_t((seq >> 1) & 1), kWaitNs)) {
                             atomicExch(sflag, 1);
                             bad = true;
                             break;
@@ -1322,7 +1322,7 @@ __global__ void __launch_bounds__(kRows * TPR + 64, (UPT <= 4 ? 2 : 1)) zpass_ke
         bool first = true;
         for (long tile = blockIdx.x; tile < a.ntiles && !bad; tile += gridDim.x) {
             for (int g = 0; g < 2 && !bad; ++g) {
-                if (!tc::mbar_wait_timed(bar_a, ph, kWaitNs)) {
+                if (!tc::mbar_wait_warp(bar_a, ph, kWaitNs)) {
                     atomicExch(sflag, 1);
                     bad = true;
                 }
@@ -1342,7 +1342,7 @@ __global__ void __launch_bounds__(kRows * TPR + 64, (UPT <= 4 ? 2 : 1)) zpass_ke
                         par = uint32_t((seq / a.nbuf) & 1);
                         need = true;
                     }
-                    if (need && !tc::mbar_wait_timed(bfull + slot, par, kWaitNs)) {
+                    if (need && !tc::mbar_wait_warp(bfull + slot, par, kWaitNs)) {
                         atomicExch(sflag, 1);
                         bad = true;
                         break;
@@ -1671,7 +1671,7 @@ __global__ void __launch_bounds__(NT * GROUPS, NT * GROUPS <= 256 ? 2 : 1) zpass
             int pv_slot = 0;
             uint32_t pv_par = 0;
             for (int kc = 0; kc < a.nkc; ++kc) {
-                if (!tc::mbar_wait_timed(bfull + us_slot, us_par, kWaitNs)) {
+                if (!tc::mbar_wait_warp(bfull + us_slot, us_par, kWaitNs)) {
                     atomicExch(sflag, 1);
                     return;
                 }
@@ -1683,7 +1683,7 @@ __global__ void __launch_bounds__(NT * GROUPS, NT * GROUPS <= 256 ? 2 : 1) zpass
                 if (el) tc::mma_commit(bempty + us_slot);
                 // the buffer of the chunk before this one takes the next chunk of this GEMM
                 if (kc > 0 && ld_count < a.nkc) {
-                    if (!tc::mbar_wait_timed(bempty + pv_slot, pv_par, kWaitNs)) {
+                    if (!tc::mbar_wait_warp(bempty + pv_slot, pv_par, kWaitNs)) {
                         atomicExch(sflag, 1);
                         return;
                     }

@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(kThreads, NH <= 16 ? 2 : 1) tc_gemm_kernel(con
         for (long it = blockIdx.x; it < items && !bad; it += gridDim.x) {
             const Item t = item_of(it);
             for (long c = t.c0; c < t.c1 && !bad; ++c) {
-                if (!dfirst && !tc::mbar_wait_timed(dempty, dpar, kGemmWaitNs)) {
+                if (!dfirst && !tc::mbar_wait_warp(dempty, dpar, kGemmWaitNs)) {
                     atomicExch(sflag, 1);
                     bad = true;
                     break;
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kThreads, NH <= 16 ? 2 : 1) tc_gemm_kernel(con
                 tc::tc_fence_after();
                 const long kb0 = c * kBlks, kb1 = min(a.nkb, kb0 + kBlks);
                 for (long kb = kb0; kb < kb1; ++kb) {
-                    if (!tc::mbar_wait_timed(full + st, par, kGemmWaitNs)) {
+                    if (!tc::mbar_wait_warp(full + st, par, kGemmWaitNs)) {
                         atomicExch(sflag, 1);
                         bad = true;
                         break;

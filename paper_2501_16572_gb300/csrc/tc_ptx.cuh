@@ -97,6 +97,13 @@ __device__ __forceinline__ bool mbar_wait_timed(uint64_t *bar, uint32_t parity, 
     }
 }
 
+// The same by a whole warp, which goes on or gives up as one: lanes that disagree when the limit
+// runs out would later wait at different warp barriers for each other.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, uint64_t limit_ns)
+{
+    return __all_sync(0xffffffffu, mbar_wait_timed(bar, parity, limit_ns)) != 0;
+}
+
 __device__ __forceinline__ void fence_proxy_async_smem()
 {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

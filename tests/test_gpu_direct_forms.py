@@ -6,6 +6,8 @@ rows).  The pair blocks are held fixed, so that the sums run in the same order.
 
 The other kernels of the exchange path that take new routes by size: the FP64 passes on even and odd
 axes, the complex axis contractions, and the blocked Cholesky with its doubling inverse."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -98,3 +100,12 @@ def test_cholesky_and_doubling_inverse(exx, n):
     low = torch.linalg.cholesky(-p.dV * (psi @ W.mT))
     ref = torch.linalg.solve_triangular(low, W, upper=False)
     assert float(torch.linalg.norm(xi - ref) / torch.linalg.norm(ref)) < 1e-12
+
+
+def test_a_warp_gives_up_a_wait_as_one(exx):
+    """Half of the lanes run out of time, half see the barrier complete: none may go on alone."""
+    L = exx.load()
+    L.exx_debug_wait_warp.argtypes = [ctypes.POINTER(ctypes.c_uint)]
+    on = ctypes.c_uint(1)
+    assert L.exx_debug_wait_warp(ctypes.byref(on)) == 0
+    assert on.value == 0
