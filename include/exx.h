@@ -202,8 +202,7 @@ int exx_energy(exx_plan plan, const double *Psi_occ, int n_occ, long ld, const d
  * (NULL to skip).  FP64 plans compute every step on the CUDA cores in FP64.  Split
  * plans compute the products M and xi on the tensor cores: fixed-point digits of 31
  * bits per 320-long chunk of the contraction (rows scaled by their largest entry),
- * exact integer sums per chunk, FP32 pairs (48 bits) across chunks, FP64 across splits of the
- * contraction (relative error ~1e-9..1e-8).  The
+ * exact integer sums per chunk, FP64 across chunks (relative error ~1e-9..1e-8).  The
  * Cholesky factor and its inverse are FP64 in every mode.
  * *info_h (host) is 0, or 1 + the failing pivot when EXX_ERR_NOT_POSDEF is
  * returned.  Synchronizes `stream`.  n <= 2048. */

@@ -11,21 +11,20 @@
 // row is rounded to a 31-bit integer X and cut into four balanced base-256 digits,
 //     X = d0 2^24 + d1 2^16 + d2 2^8 + d3,   |d0| <= 64, |d1|, |d2|, |d3| <= 128,
 // each stored exactly as a bf16.  Digit products of one level (i + j = l, l <= 4) are
-// summed in their own TMEM accumulator (5 levels x up to 96 output columns per tile); a level
+// summed in their own TMEM accumulator (5 levels x up to 48 output columns per tile, two sets of them); a level
 // gains at most 3 * 2^14 per k, so the 320-term sums stay integers below 2^24 and the
-// tensor core never rounds.  The levels of a chunk are combined into an FP32 hi + lo pair and
-// the chunks are summed in such pairs (48 bits; the sums of the k splits in FP64).  Dropped
-// digit products (i + j >= 5) weigh below 2^-37 of the row maxima; the rounding of X, 2^-31
-// of the row maxima, is the leading error.
+// tensor core never rounds.  The levels of a chunk are combined into an FP32 hi + lo pair, and
+// the chunks are summed in FP64.  Dropped digit products (i + j >= 5) weigh below 2^-37 of the
+// row maxima; the rounding of X, 2^-31 of the row maxima, is the leading error.
 //
 // Two kernels.  gemm_cut_kernel cuts every operand element once into digit planes in device
 // memory, already in the operand layout of the MMA, and records the row scales;
 // tc_gemm_kernel then only streams 8-byte-per-element blocks of them through shared memory
-// (bulk copies, a producer warp) into the MMAs (one issuing warp) while 8 warps combine
+// (bulk copies, a producer warp) into the MMAs (one issuing warp) while 8 or 16 warps combine
 // finished chunks.  Cutting inside the GEMM repeated the integer work of every A row for each
-// 96 output columns and left the tensor cores idle meanwhile: both products of ace_apply at
-// n = nphi = 512 on 72 x 72 x 144 points took 65.7 ms, 10.9 ms now (cuts 3.3 ms near the HBM
-// rate, MMAs 7.5 ms, of which the tensor pipe's own 5.6 ms).
+// column tile and left the tensor cores idle meanwhile: both products of ace_apply at
+// n = nphi = 512 on 72 x 72 x 144 points took 65.7 ms, 10.1 ms now (cuts 3.3 ms near the HBM
+// rate, the GEMMs 6.8 ms, of which the tensor pipe's own about 4.7).
 #include "exx_internal.h"
 #include "tc_ptx.cuh"
 
@@ -37,7 +36,7 @@ namespace exx {
 namespace {
 
 constexpr int kT = 128;              // rows of A per tile (TMEM lanes)
-constexpr int kTN = 96;              // most rows of B per tile (output columns)
+constexpr int kTN = 48;              // most rows of B per tile (output columns): two sets of levels fill TMEM
 constexpr int kLev = 5;              // level accumulators: digit products with i + j <= 4
 constexpr int kDig = 4;
 constexpr int kBlk = 32;             // k per operand block
@@ -45,8 +44,8 @@ constexpr int kBlks = 10;            // blocks per exact chunk
 constexpr int kChunk = kBlk * kBlks; // 320: 4 levels x 320 x 3 * 2^14 < 2^24
 constexpr uint64_t kGemmWaitNs = 1000000000ull;
 constexpr uint32_t kSbo = kBlk * 16;           // bytes between 8-row groups of a digit plane
-constexpr int kDrainWarps = 8;
-constexpr int kThreads = 32 * (kDrainWarps + 2);
+constexpr int kParts = 4;            // drain warps per 32 TMEM lanes (2 for tiles of up to 32 columns)
+constexpr int kNarrow = 32;          // tiles of up to 32 columns: one set of levels, two CTAs per SM
 constexpr int kCutWarps = kBlks;     // gemm_cut_kernel: a warp per k block of a chunk
 constexpr long kDigitBudget = 1L << 30;        // device memory of the digit planes of one slab
 
@@ -182,40 +181,35 @@ struct GemmArgs {
     long ds_i, ds_j, dz;
     int add;                   // add to D (a later slab of k without splits)
     int ktri;                  // B(j, k) = 0 for k > j: tiles stop at their last column
-    float al_h, al_l;          // alpha = (al_h + al_l) 2^al_e
-    int al_e;
+    double alpha;
     int stages;
     uint32_t stage_bytes, offB, offTab, offBar;
     int tmem_cols;
     int *err;
 };
 
-// (h + l) 2^ex as a double, rounded to 48 bits or better, on the integer pipe: GB300 converts
-// to and from FP64 at two per clock and SM, which would cost a 128 x 96 tile 18 thousand cycles.
-__device__ __forceinline__ double pair_to_double(float h, float l, int ex)
+// (h + l) 2^ex rounded to a double, for a chunk's sum h + l: h is its FP32 rounding, l the rest,
+// zero or 2^-32 <= |h| < 2^26.  On the integer pipe: GB300 converts to and from FP64 at two per
+// clock and SM, two conversions and an addition for each of 128 x 96 sums would take 18 thousand
+// cycles.
+__device__ __forceinline__ double chunk_value(float h, float l, int ex)
 {
-    const float s = h + l;
-    l -= s - h;
-    const uint32_t b = __float_as_uint(s);
-    int e = int((b >> 23) & 0xffu);
-    long long M = static_cast<long long>((b & 0x7fffffu) | 0x800000u) << 29;
-    if (e >= 53) {   // l in units of the last bit of M: |q| <= 2^28
-        const float lq = l * __uint_as_float(uint32_t(306 - e) << 23);
-        M += __float2int_rn((b >> 31) ? -lq : lq);
+    const uint32_t b = __float_as_uint(h), sign = b & 0x80000000u, m = (b & 0x7fffffu) | 0x800000u;
+    const int e = int((b >> 23) & 0xffu);
+    int ed = e - 127 + 1023 + ex;
+    if (e == 0 || uint32_t(ed - 2) > 2044u) {   // zero, or near the ends of the range
+        if (e == 0 || ex < -1022) return 0.0;
+        return (double(h) + double(l)) * __hiloint2double((min(ex, 1023) + 1023) << 20, 0);
     }
-    if (M < (1LL << 52)) {
-        M <<= 1;
-        --e;
+    // the mantissa of h as that of a double, l added in units of its last bit
+    const float lq = l * __uint_as_float((uint32_t(306 - e) << 23) | sign);
+    long long M = static_cast<long long>((uint64_t(m >> 3) << 32) | uint32_t(m << 29)) + __float2int_rn(lq);
+    if (M < (1LL << 52)) {   // below a power of two: half the unit
+        M = (1LL << 53) + __float2int_rn(2.f * lq);
+        --ed;
     }
-    const int ed = e - 127 + 1023 + ex;
-    if (e <= 0 || ed <= 0) return 0.0;
-    const uint32_t sign = b & 0x80000000u;
-    if (ed >= 2047) return __hiloint2double(int(sign | 0x7ff00000u), 0);
-    const uint32_t hi = sign | (uint32_t(ed) << 20) | (uint32_t(M >> 32) & 0xfffffu);
-    return __hiloint2double(int(hi), int(uint32_t(M)));
+    return __hiloint2double(int((uint32_t(M >> 32) + (uint32_t(ed - 1) << 20)) | sign), int(uint32_t(M)));
 }
-
-__device__ __forceinline__ float pow2f(int e) { return e < -126 ? 0.f : __uint_as_float(uint32_t(min(e, 127) + 127) << 23); }
 
 __device__ __forceinline__ void gemm_bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
 {
@@ -226,23 +220,29 @@ __device__ __forceinline__ void gemm_bulk_load(void *dst, const void *src, uint3
         : "memory");
 }
 
-// One CTA per SM walks the items (split z, row tile, column tile), column tiles fastest so
-// that concurrent CTAs read the same A blocks from L2.  Bound by the tensor pipe: 13 digit
-// products per k (7 MMAs of up to 192 columns: neighbouring B digits feed neighbouring
-// levels), 632 cycles per 16 k of a 128 x 96 tile against 28.7 KB of operands; the combination
-// of a finished chunk is not overlapped, the five level accumulators fill TMEM.
-// NH: most columns of a drain warp's half.  Narrow tiles (up to 32 columns) are bound by the operand
-// blocks' way from L2 and by the chain load - MMA - drain - store of one item, so two CTAs share an SM.
-template <int G, int NH>
-__global__ void __launch_bounds__(kThreads, NH <= 16 ? 2 : 1) tc_gemm_kernel(const __grid_constant__ GemmArgs a)
+// The CTAs walk the items (split z, row tile, column tile), column tiles fastest so that concurrent
+// CTAs read the same A blocks from L2.  13 digit products per k in 4 MMAs of up to 192 columns
+// (neighbouring B digits feed neighbouring levels): about 284 cycles of the tensor pipe per 16 k of a
+// 128 x 48 tile, against 22.5 KB of operands.
+//   * SETS = 2 (tiles of 48 columns), one CTA per SM: two sets of level accumulators, so that the
+//     drain warps combine a finished chunk under the next chunk's MMAs.  The combination is
+//     integer work for the most part, about 7 thousand cycles per 128 x 48 chunk where the MMAs
+//     take 5.7 thousand: with one set of 96 columns it was not overlapped, and both products of
+//     ace_apply at n = nphi = 512 on 72 x 72 x 144 points took 15.7 ms, now 10.1.
+//   * SETS = 1 (tiles of up to 32 columns), two CTAs per SM: bound by the operand blocks' way from L2
+//     and by the chain load - MMA - drain - store of one item.
+// PARTS: drain warps per 32 TMEM lanes (four: 10.1 ms for that call, three 10.2, two 11.1).
+template <int PARTS, int SETS>
+__global__ void __launch_bounds__(128 * PARTS + 64, 3 - SETS) tc_gemm_kernel(const __grid_constant__ GemmArgs a)
 {
+    constexpr int kDrainWarps = 4 * PARTS;
+    constexpr int NH = ((SETS == 1 ? kNarrow : kTN) / 4 + PARTS - 1) / PARTS * 4;   // most columns of a drain warp
     extern __shared__ __align__(1024) uint8_t smem[];
-    float *fbs = reinterpret_cast<float *>(smem + a.offTab);       // column factors of a chunk, two sets
-    int *refB = reinterpret_cast<int *>(fbs + 2 * kTN);
+    int *eb = reinterpret_cast<int *>(smem + a.offTab);            // column exponents of a chunk, two sets
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + a.offBar);
     uint64_t *empty = full + a.stages;
-    uint64_t *dfull = empty + a.stages, *dempty = dfull + 1;
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(dempty + 1);
+    uint64_t *dfull = empty + a.stages, *dempty = dfull + 2;   // per accumulator set
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(dempty + 2);
     int *sflag = reinterpret_cast<int *>(tslot + 1);
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform
@@ -251,8 +251,10 @@ __global__ void __launch_bounds__(kThreads, NH <= 16 ? 2 : 1) tc_gemm_kernel(con
             tc::mbar_init(full + i, 1);
             tc::mbar_init(empty + i, 1);
         }
-        tc::mbar_init(dfull, 1);
-        tc::mbar_init(dempty, 1);
+        for (int i = 0; i < 2; ++i) {
+            tc::mbar_init(dfull + i, 1);
+            tc::mbar_init(dempty + i, 1);
+        }
         *sflag = 0;
     }
     if (warp == 0) tc::tmem_alloc(tslot, uint32_t(a.tmem_cols));
@@ -314,55 +316,44 @@ __global__ void __launch_bounds__(kThreads, NH <= 16 ? 2 : 1) tc_gemm_kernel(con
         }
     } else if (warp == kDrainWarps + 1) {
         // ---- MMA warp ----
-        int st = 0;
-        uint32_t par = 0, dpar = 1;
-        bool bad = false, dfirst = true;
+        int st = 0, set = 0;
+        uint32_t par = 0, dpar = 3;   // dpar: per accumulator set, of its last release (the first wait passes)
+        bool bad = false;
         // operand and accumulator steps, fixed for the launch: the issue of one 16-k step is a
         // straight run of MMAs by the whole warp whose descriptors differ by additions (computed in
-        // a loop by one lane, a step took 1340 cycles, twice the tensor pipe's 632)
+        // a loop by one lane, a step took 1340 cycles, twice the tensor pipe's time)
         constexpr uint32_t kStepA = kT * kBlk * 2 / 16;            // next A digit, in 16-byte units
         const uint32_t step_b = uint32_t(Nt) * kBlk * 2 / 16;      // next B digit
-        uint32_t idesc[G + 1];
+        uint32_t idesc[kDig + 1];
 #pragma unroll
-        for (int g = 1; g <= G; ++g) idesc[g] = tc::instr_desc(false, g * Nt);
-        // A digit i with B digits j0 .. j0 + g - 1 into levels i + j0 .. (at most G per MMA)
+        for (int g = 1; g <= kDig; ++g) idesc[g] = tc::instr_desc(false, g * Nt);
         const uint32_t el = tc::elect_one();
-        auto step = [&](uint64_t ad0, uint64_t bd0, bool first) {
+        // A digit i with the B digits 0 .. 4 - i, neighbours of levels i .. 4, in one MMA
+        auto step = [&](uint32_t d0, uint64_t ad0, uint64_t bd, bool first) {
 #pragma unroll
             for (int i = 0; i < kDig; ++i) {
-                constexpr int kEnd = kLev;
-                const int nj = kDig < kEnd - i ? kDig : kEnd - i;
+                const int nj = kDig < kLev - i ? kDig : kLev - i;
                 const uint64_t ad = ad0 + i * kStepA;
-#pragma unroll
-                for (int j0 = 0; j0 < nj; j0 += G) {
-                    const int g = G < nj - j0 ? G : nj - j0;
-                    const uint64_t bd = bd0 + j0 * step_b;
-                    const uint32_t d = tmem + uint32_t((i + j0) * Nt);
-                    if (i == 1 && j0 + g == kDig && g > 1) {
-                        if (first) {   // digit 0 has opened levels 0..3; level 4 starts here
-                            tc::mma_bf16_warp(d, ad, bd, idesc[g - 1], 1u, el);
-                            tc::mma_bf16_warp(tmem + uint32_t(4 * Nt), ad, bd0 + (kDig - 1) * step_b, idesc[1], 0u, el);
-                        } else {
-                            tc::mma_bf16_warp(d, ad, bd, idesc[g], 1u, el);
-                        }
-                    } else {
-                        const bool open = i == 0 || (i == 1 && j0 == kDig - 1);
-                        tc::mma_bf16_warp(d, ad, bd, idesc[g], open && first ? 0u : 1u, el);
-                    }
+                const uint32_t d = d0 + uint32_t(i * Nt);
+                if (i == 1 && first) {   // digit 0 has opened levels 0..3; level 4 starts here
+                    tc::mma_bf16_warp(d, ad, bd, idesc[kDig - 1], 1u, el);
+                    tc::mma_bf16_warp(d0 + uint32_t(4 * Nt), ad, bd + (kDig - 1) * step_b, idesc[1], 0u, el);
+                } else {
+                    tc::mma_bf16_warp(d, ad, bd, idesc[nj], i == 0 && first ? 0u : 1u, el);
                 }
             }
         };
         for (long it = blockIdx.x; it < items && !bad; it += gridDim.x) {
             const Item t = item_of(it);
             for (long c = t.c0; c < t.c1 && !bad; ++c) {
-                if (!dfirst && !tc::mbar_wait_warp(dempty, dpar, kGemmWaitNs)) {
+                if (!tc::mbar_wait_warp(dempty + set, (dpar >> set) & 1u, kGemmWaitNs)) {
                     atomicExch(sflag, 1);
                     bad = true;
                     break;
                 }
-                dfirst = false;
-                dpar ^= 1u;
+                dpar ^= 1u << set;
                 tc::tc_fence_after();
+                const uint32_t d0 = tmem + uint32_t(set * kLev * Nt);
                 const long kb0 = c * kBlks, kb1 = min(a.nkb, kb0 + kBlks);
                 for (long kb = kb0; kb < kb1; ++kb) {
                     if (!tc::mbar_wait_warp(full + st, par, kGemmWaitNs)) {
@@ -373,8 +364,8 @@ __global__ void __launch_bounds__(kThreads, NH <= 16 ? 2 : 1) tc_gemm_kernel(con
                     tc::tc_fence_after();
                     const uint32_t sa = tc::smem_addr(smem) + uint32_t(st) * a.stage_bytes;
                     const uint64_t ad = tc::smem_desc(sa, 128u, kSbo), bd = tc::smem_desc(sa + a_bytes, 128u, kSbo);
-                    step(ad, bd, kb == kb0);
-                    step(ad + 16, bd + 16, false);
+                    step(d0, ad, bd, kb == kb0);
+                    step(d0, ad + 16, bd + 16, false);
                     if (el) tc::mma_commit(empty + st);
                     __syncwarp();
                     if (++st == a.stages) {
@@ -382,62 +373,65 @@ __global__ void __launch_bounds__(kThreads, NH <= 16 ? 2 : 1) tc_gemm_kernel(con
                         par ^= 1u;
                     }
                 }
-                if (!bad && el) tc::mma_commit(dfull);
+                if (!bad && el) tc::mma_commit(dfull + set);
                 __syncwarp();
+                if (SETS == 2) set ^= 1;
             }
         }
     } else {
-        // ---- drain warps: TMEM lane `row`, column groups of 8 of this warp's half ----
-        const int quarter = warp & 3, half = warp >> 2;
+        // ---- drain warps: TMEM lane `row`, column groups of 4 of this warp's part ----
+        const int quarter = warp & 3;
         const int row = quarter * 32 + lane;
         const uint32_t lane_q = uint32_t(quarter * 32) << 16;
-        constexpr int kHalf = NH;
-        const int ncol = Nt / 2, cbase = half * ncol;   // Nt is a multiple of 16
-        constexpr int NT = 32 * kDrainWarps;
-        long dseq = 0;
+        const int part = (Nt / 4 + PARTS - 1) / PARTS * 4, cbase = (warp >> 2) * part, ncol = min(part, Nt - cbase);
+        constexpr int NT = 128 * PARTS;
+        int seq = 0;   // chunks drained so far
         bool stop = false;
         for (long it = blockIdx.x; it < items && !stop; it += gridDim.x) {
             const Item t = item_of(it);
             const long i = long(t.mi) * kT + row;
             const int j0 = t.ni * Nt;
-            // reference exponents: the largest of the item's chunks, per row and column
-            int rA = 100;
-            for (long c = t.c0; c < t.c1; ++c) rA = max(rA, a.shA[c * a.prowA + i]);
-            if (tid < Nt) {
-                int rB = 100;
-                for (long c = t.c0; c < t.c1; ++c) rB = max(rB, a.shB[c * a.prowB + j0 + tid]);
-                refB[tid] = rB;
-            }
-            float ah[kHalf], al[kHalf];
+            double acc[NH];
 #pragma unroll
-            for (int e = 0; e < kHalf; ++e) ah[e] = al[e] = 0.f;
-            for (long c = t.c0; c < t.c1; ++c, ++dseq) {
-                float *fb = fbs + (dseq & 1) * kTN;
-                if (tid < Nt) fb[tid] = pow2f(a.shB[c * a.prowB + j0 + tid] - refB[tid]);
-                const float fa = pow2f(a.shA[c * a.prowA + i] - rA);
+            for (int e = 0; e < NH; ++e) acc[e] = 0.0;
+            // row and column exponents, asked for a chunk ahead
+            auto row_exp = [&](long c) { return i < a.m ? a.shA[c * a.prowA + i] : 0; };
+            auto col_exp = [&](long c) { return tid < Nt && j0 + tid < a.n ? a.shB[c * a.prowB + j0 + tid] : 0; };
+            int ea_next = row_exp(t.c0), eb_next = col_exp(t.c0);
+            for (long c = t.c0; c < t.c1; ++c, ++seq) {
+                const int set = SETS == 2 ? seq & 1 : 0;
+                int *ebc = eb + (seq & 1) * kTN;
+                if (tid < Nt) ebc[tid] = eb_next;
+                // x = X 2^(E - 1052), and level 0 holds X 2^-24: 2 x (24 - 1052)
+                const int ea = ea_next - 2056;
+                if (c + 1 < t.c1) {
+                    ea_next = row_exp(c + 1);
+                    eb_next = col_exp(c + 1);
+                }
                 // one warp polls, the others sleep in the barrier: polls take issue slots from the MMAs'
-                if (warp == 0 && !tc::mbar_wait_timed(dfull, uint32_t(dseq & 1), kGemmWaitNs)) atomicExch(sflag, 1);
-                if (tc::bar_red_or(1, NT, *sflag != 0)) {   // also: fb is complete
+                if (warp == 0 && !tc::mbar_wait_timed(dfull + set, uint32_t(seq / SETS) & 1u, kGemmWaitNs)) atomicExch(sflag, 1);
+                if (tc::bar_red_or(1, NT, *sflag != 0)) {   // also: ebc is complete
                     stop = true;
                     break;
                 }
                 tc::tc_fence_after();
+                const uint32_t d0 = tmem + lane_q + uint32_t(set * kLev * Nt);
 #pragma unroll
-                for (int cg = 0; cg < kHalf / 8; ++cg) {
-                    if (cg * 8 >= ncol) break;
-                    const int cc = cbase + cg * 8;
-                    uint32_t r[kLev][8];
+                for (int cg = 0; cg < NH / 4; ++cg) {
+                    if (cg * 4 >= ncol) break;
+                    const int cc = cbase + cg * 4;
+                    uint32_t r[kLev][4];
 #pragma unroll
-                    for (int l = 0; l < kLev; ++l) tc::tmem_ld8_issue(tmem + lane_q + uint32_t(l * Nt + cc), r[l]);
+                    for (int l = 0; l < kLev; ++l) tc::tmem_ld4_issue(d0 + uint32_t(l * Nt + cc), r[l]);
                     tc::tmem_wait_ld();
 #pragma unroll
                     for (int l = 0; l < kLev; ++l)
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) tc::order_after_wait(r[l][e]);
+                        for (int e = 0; e < 4; ++e) tc::order_after_wait(r[l][e]);
 #pragma unroll
-                    for (int e = 0; e < 8; e += 2) {
+                    for (int e = 0; e < 4; e += 2) {
                         // levels combined in FP32 down to level 1 (rounding ~2^-32 of level 0's
-                        // scale), level 0 added with TwoSum, the pair scaled and accumulated
+                        // scale), level 0 added with TwoSum, the pair summed over the chunks in FP64
                         auto lv = [&](int l) { return make_float2(__uint_as_float(r[l][e]), __uint_as_float(r[l][e + 1])); };
                         const float2 q = make_float2(1.f / 256.f, 1.f / 256.f), m1 = make_float2(-1.f, -1.f);
                         float2 tl = __ffma2_rn(lv(4), q, lv(3));
@@ -445,46 +439,30 @@ __global__ void __launch_bounds__(kThreads, NH <= 16 ? 2 : 1) tc_gemm_kernel(con
                         tl = __ffma2_rn(tl, q, lv(1));
                         tl = __fmul2_rn(tl, q);
                         const float2 l0 = lv(0);
-                        float2 h = __fadd2_rn(l0, tl);
+                        const float2 h = __fadd2_rn(l0, tl);
                         const float2 b0 = __ffma2_rn(l0, m1, h);
-                        float2 lo = __fadd2_rn(__ffma2_rn(__ffma2_rn(b0, m1, h), m1, l0), __ffma2_rn(b0, m1, tl));
-                        const float2 f = __fmul2_rn(make_float2(fa, fa), *reinterpret_cast<const float2 *>(fb + cc + e));
-                        h = __fmul2_rn(h, f);
-                        lo = __fmul2_rn(lo, f);
-                        const float2 s0 = make_float2(ah[cg * 8 + e], ah[cg * 8 + e + 1]);
-                        const float2 s = __fadd2_rn(s0, h);
-                        const float2 bp = __ffma2_rn(s0, m1, s);
-                        const float2 er = __fadd2_rn(__ffma2_rn(__ffma2_rn(bp, m1, s), m1, s0), __ffma2_rn(bp, m1, h));
-                        const float2 cs = __fadd2_rn(make_float2(al[cg * 8 + e], al[cg * 8 + e + 1]), __fadd2_rn(er, lo));
-                        ah[cg * 8 + e] = s.x;
-                        ah[cg * 8 + e + 1] = s.y;
-                        al[cg * 8 + e] = cs.x;
-                        al[cg * 8 + e + 1] = cs.y;
+                        const float2 lo = __fadd2_rn(__ffma2_rn(__ffma2_rn(b0, m1, h), m1, l0), __ffma2_rn(b0, m1, tl));
+                        const int2 ebv = *reinterpret_cast<const int2 *>(ebc + cc + e);
+                        acc[cg * 4 + e] += chunk_value(h.x, lo.x, ea + ebv.x);
+                        acc[cg * 4 + e + 1] += chunk_value(h.y, lo.y, ea + ebv.y);
                     }
                 }
-                tc::tc_fence_before();   // TMEM reads before the next chunk's MMAs overwrite it
+                tc::tc_fence_before();   // TMEM reads before a later chunk's MMAs overwrite them
                 tc::bar_sync(1, NT);
-                if (tid == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(dempty)) : "memory");
+                if (tid == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(dempty + set)) : "memory");
             }
             if (stop) break;
-            tc::bar_sync(1, NT);   // refB is complete also for an item without chunks
             if (i < a.m) {
                 double *D = a.D + t.z * a.dz + i * a.ds_i;
 #pragma unroll
-                for (int e = 0; e < kHalf; ++e) {
-                    const int col = cbase + e, j = j0 + col;
+                for (int e = 0; e < NH; ++e) {
+                    const int j = j0 + cbase + e;
                     if (e < ncol && j < a.n) {
-                        // alpha times the pair: the leading product with its rounding error
-                        const float p = ah[e] * a.al_h;
-                        const float l = fmaf(ah[e], a.al_h, -p) + fmaf(ah[e], a.al_l, al[e] * a.al_h);
-                        // x = X 2^(E - 1052), and level 0 holds X 2^-24: 2 x (24 - 1052)
-                        const double v = pair_to_double(p, l, rA + refB[col] - 2056 + a.al_e);
                         double *dp = D + long(j) * a.ds_j;
-                        *dp = a.add ? *dp + v : v;
+                        *dp = a.add ? fma(a.alpha, acc[e], *dp) : a.alpha * acc[e];
                     }
                 }
             }
-            tc::bar_sync(1, NT);   // refB is rewritten by the next item
         }
     }
     tc::tc_fence_before();
@@ -565,7 +543,7 @@ int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_
         if (int rc = dev_reserve(P.err_d, 16)) return rc;
         EXX_CUDA(cudaMemsetAsync(P.err_d.p, 0, 16, s));
     }
-    // column tiles: as even as 16-column steps allow, at most 96 (5 levels in 512 TMEM columns)
+    // column tiles: as even as 16-column steps allow, at most 48 (two sets of 5 levels in 512 TMEM columns)
     const int nt = int(ceil_div(n, kTN));
     const int Nt = int(ceil_div(ceil_div(n, nt), 16) * 16);
     const long np = long(nt) * Nt;
@@ -589,7 +567,7 @@ int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_
     mslab = ceil_div(ceil_div(mpad, kT), ceil_div(mpad, mslab)) * kT;
     // k splits: items (tiles x splits) for a whole number of rounds over the SMs
     const long tiles = (mslab / kT) * nt;
-    const long slots = long(P.num_sms) * (Nt <= 32 ? 2 : 1);   // CTAs resident at once
+    const long slots = long(P.num_sms) * (Nt <= kNarrow ? 2 : 1);   // CTAs resident at once
     auto splits = [&](long nch) {
         if (nch < 2 || tiles >= 2 * slots) return 1L;
         const long round = std::max(1L, slots / tiles);
@@ -620,19 +598,15 @@ int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_
     a.ktri = ktri ? 1 : 0;
     a.err = static_cast<int *>(P.err_d.p);
     a.stage_bytes = uint32_t(kT + Nt) * kBlk * 2 * kDig;
-    a.stages = int(std::min<size_t>(8, (Nt <= 32 ? 111 : 200) * 1024 / a.stage_bytes));
+    const bool narrow = Nt <= kNarrow;
+    a.stages = int(std::min<size_t>(8, (narrow ? 111 : 222) * 1024 / a.stage_bytes));
     a.offTab = uint32_t(a.stages) * a.stage_bytes;
-    a.offBar = a.offTab + uint32_t(round_up(2 * kTN * 4 + kTN * 4, 16));
+    a.offBar = a.offTab + 2 * kTN * 4;
     a.tmem_cols = 32;
-    while (a.tmem_cols < kLev * Nt) a.tmem_cols *= 2;
-    size_t smem = a.offBar + (2 * size_t(a.stages) + 2) * 8 + 16;
-    if (Nt > 32) smem = std::max<size_t>(smem, 120 * 1024);   // one CTA per SM
-    // B digits per MMA: at most 256 columns
-    const int gmax = 256 / Nt;
-    auto kern = Nt <= 32    ? tc_gemm_kernel<4, 16>
-                : gmax >= 4 ? tc_gemm_kernel<4, kTN / 2>
-                : gmax == 3 ? tc_gemm_kernel<3, kTN / 2>
-                            : tc_gemm_kernel<2, kTN / 2>;
+    while (a.tmem_cols < (narrow ? 1 : 2) * kLev * Nt) a.tmem_cols *= 2;
+    const size_t smem = a.offBar + (2 * size_t(a.stages) + 4) * 8 + 16;
+    auto kern = narrow ? tc_gemm_kernel<2, 1> : tc_gemm_kernel<kParts, 2>;
+    const int threads = 128 * (narrow ? 2 : kParts) + 64;
     EXX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
 
     for (long c0 = 0; c0 < chunks; c0 += kslab) {
@@ -651,10 +625,7 @@ int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_
             a.cper = ceil_div(nch, a.Z);
             a.Z = ceil_div(nch, a.cper);
             double *Dd = D + i0 * ds_i;
-            // alpha as an FP32 pair and a power of two; split sums take it in the reduction
-            const double am = std::frexp(a.Z > 1 ? 1.0 : alpha, &a.al_e);
-            a.al_h = float(am);
-            a.al_l = float(am - double(a.al_h));
+            a.alpha = a.Z > 1 ? 1.0 : alpha;   // split sums take it in the reduction
             if (a.Z > 1) {
                 a.D = reinterpret_cast<double *>(ws + offP);
                 a.ds_i = 1;
@@ -670,7 +641,7 @@ int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_
             }
             const long items = a.Z * a.mt * a.nt;
             int tb = timing_begin(P, EXX_TIMING_GEMM, s);
-            kern<<<unsigned(std::min<long>(items, slots)), kThreads, smem, s>>>(a);
+            kern<<<unsigned(std::min<long>(items, slots)), threads, smem, s>>>(a);
             timing_end(P, tb, s);
             EXX_LAUNCH("tc_gemm_kernel");
             P.launches++;
