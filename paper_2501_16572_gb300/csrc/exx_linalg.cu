@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(32) chol_diag_kernel(int n, double *A, int k0,
         }
         const double djj = sqrt(d);
         rd[j] = 1.0 / djj;
-        const double l = lane == j ? djj : a[j] * rd[j];
+        const double l = lane == j ? djj : a[j] / djj;
         a[j] = l;
 #pragma unroll
         for (int k = j + 1; k < kCb; ++k) a[k] = fma(-l, __shfl_sync(0xffffffffu, l, k), a[k]);
