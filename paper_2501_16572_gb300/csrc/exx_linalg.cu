@@ -201,37 +201,60 @@ __global__ void chol_prep_kernel(int n, const double *M, double *A, double *X, i
     if (blockIdx.x == 0 && threadIdx.x == 0) info_d[0] = 0;
 }
 
-// One warp: the diagonal block at (k0, k0) of size b <= 32 (padded with the identity): lane i holds
+// One warp: the diagonal block at (k0, k0) of size b <= NB (padded with the identity): lane i holds
 // row i.  Writes L_kk into A, D = L_kk^{-1} (leading dimension kCb, zeros above) into Dk and X.
-__global__ void __launch_bounds__(32) chol_diag_kernel(int n, double *A, int k0, int b, double *Dk, double *X, int *info_d)
+// A matrix of one block is taken straight from M: no preparation, no workspace.  NB and the
+// stop at row b keep small blocks short; a FULL one (b = NB) has no stops, which would keep the
+// FP64 chains of neighbouring rows from overlapping.
+template <int NB, bool FULL>
+__global__ void __launch_bounds__(32) chol_diag_kernel(int n, const double *M, double *A, int k0, int b, double *Dk, double *X,
+                                                       int *info_d)
 {
     const int lane = threadIdx.x;
-    if (info_d[0]) return;
-    double a[kCb], rd[kCb];
+    if (M) {
+        if (lane == 0) info_d[0] = 0;
+    } else if (info_d[0]) {
+        return;
+    }
+    double a[NB], dg = 1.0;   // dg: L(lane, lane)
 #pragma unroll
-    for (int j = 0; j < kCb; ++j)
-        a[j] = lane < b && j <= lane ? A[(k0 + lane) + size_t(n) * (k0 + j)] : (j == lane ? 1.0 : 0.0);
+    for (int j = 0; j < NB; ++j) {
+        a[j] = j == lane ? 1.0 : 0.0;
+        if (lane < b && j <= lane)
+            a[j] = M ? -0.5 * (M[lane + size_t(n) * j] + M[j + size_t(n) * lane]) : A[(k0 + lane) + size_t(n) * (k0 + j)];
+    }
 #pragma unroll
-    for (int j = 0; j < kCb; ++j) {
+    for (int j = 0; j < NB; ++j) {
+        if (!FULL && j >= b) break;
         const double d = __shfl_sync(0xffffffffu, a[j], j);
         if (!(d > 0.0)) {   // uniform
             if (lane == 0) info_d[0] = k0 + j + 1;
             return;
         }
         const double djj = sqrt(d);
-        rd[j] = 1.0 / djj;
-        const double l = lane == j ? djj : a[j] / djj;
+        if (lane == j) dg = djj;
+        // the quotient from the rounded reciprocal and its remainder, correctly rounded (Markstein,
+        // "Computation of elementary functions on the IBM RISC System/6000 processor", 1990): the
+        // division took 8 us more per block of 32 columns
+        const double r = 1.0 / djj, q = a[j] * r;
+        const double l = lane == j ? djj : fma(fma(-djj, q, a[j]), r, q);
         a[j] = l;
 #pragma unroll
-        for (int k = j + 1; k < kCb; ++k) a[k] = fma(-l, __shfl_sync(0xffffffffu, l, k), a[k]);
+        for (int k = j + 1; k < NB; ++k) a[k] = fma(-l, __shfl_sync(0xffffffffu, l, k), a[k]);
     }
+    if (!M) {
 #pragma unroll
-    for (int j = 0; j < kCb; ++j)
-        if (lane < b && j <= lane) A[(k0 + lane) + size_t(n) * (k0 + j)] = a[j];
+        for (int j = 0; j < NB; ++j)
+            if (lane < b && j <= lane) A[(k0 + lane) + size_t(n) * (k0 + j)] = a[j];
+    }
     // column `lane` of the inverse by forward substitution
-    double x[kCb];
+    const double rdg = 1.0 / dg;
+    double x[NB];
 #pragma unroll
-    for (int i = 0; i < kCb; ++i) {
+    for (int i = 0; i < NB; ++i) x[i] = 0.0;
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        if (!FULL && i >= b) break;
         double s0 = i == lane ? 1.0 : 0.0, s1 = 0.0;
 #pragma unroll
         for (int k = 0; k < i; ++k) {
@@ -239,12 +262,12 @@ __global__ void __launch_bounds__(32) chol_diag_kernel(int n, double *A, int k0,
             if (k & 1) s1 = fma(-t, x[k], s1);
             else s0 = fma(-t, x[k], s0);
         }
-        x[i] = (s0 + s1) * rd[i];
+        x[i] = (s0 + s1) * __shfl_sync(0xffffffffu, rdg, i);
     }
 #pragma unroll
-    for (int i = 0; i < kCb; ++i) {
+    for (int i = 0; i < NB; ++i) {
         const double v = i < b && lane < b && i >= lane ? x[i] : 0.0;
-        Dk[i + kCb * lane] = v;
+        if (Dk) Dk[i + kCb * lane] = v;
         if (i < b && lane < b) X[(k0 + i) + size_t(n) * (k0 + lane)] = v;
     }
 }
@@ -422,6 +445,23 @@ int cholesky_neg_sym_and_inverse(Plan &P, int n, const double *M, double *Linv, 
                                  cudaStream_t s)
 {
     int tb = timing_begin(P, EXX_TIMING_CHOL, s);
+    auto diag = [&](const double *m, double *A, int k0, int b, double *Dk) -> int {
+        auto kern = b == 8    ? chol_diag_kernel<8, true>
+                    : b < 8   ? chol_diag_kernel<8, false>
+                    : b == 16 ? chol_diag_kernel<16, true>
+                    : b < 16  ? chol_diag_kernel<16, false>
+                    : b < kCb ? chol_diag_kernel<kCb, false>
+                              : chol_diag_kernel<kCb, true>;
+        kern<<<1, 32, 0, s>>>(n, m, A, k0, b, b == kCb ? Dk : nullptr, Linv, info_d);   // a last, shorter block has no panel
+        EXX_LAUNCH("chol_diag_kernel");
+        P.launches++;
+        return EXX_OK;
+    };
+    if (n <= kCb) {
+        const int rc = diag(M, nullptr, 0, n, nullptr);
+        timing_end(P, tb, s);
+        return rc;
+    }
     // workspace: A (n x n), the products of the doubling (n x n), one diagonal-block inverse
     const size_t nn = size_t(n) * n;
     if (int rc = dev_reserve(P.small_ws, (2 * nn + kCb * kCb) * sizeof(double))) return rc;
@@ -433,9 +473,7 @@ int cholesky_neg_sym_and_inverse(Plan &P, int n, const double *M, double *Linv, 
     P.launches++;
     for (int k0 = 0; k0 < n; k0 += kCb) {
         const int b = std::min(kCb, n - k0), rest = n - k0 - b;
-        chol_diag_kernel<<<1, 32, 0, s>>>(n, A, k0, b, Dk, Linv, info_d);
-        EXX_LAUNCH("chol_diag_kernel");
-        P.launches++;
+        if (int rc = diag(nullptr, A, k0, b, Dk)) return rc;
         if (rest == 0) break;
         chol_panel_kernel<<<(rest + kPanel - 1) / kPanel, kCholThreads, 0, s>>>(n, A, k0, b, Dk, info_d);
         EXX_LAUNCH("chol_panel_kernel");

@@ -43,3 +43,30 @@ def test_factor_entries_are_correctly_rounded_quotients(exx, n):
         X[i + 1, i] = -((q[b] / root[b]) * (1.0 / root[b])) * 2.0 ** -30
     got = _inverse_factor(exx, A)
     assert np.array_equal(got, X)
+
+
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 15, 16, 17, 31, 32, 33])
+def test_one_block_sizes(exx, n):
+    """Around the widths of the one-block form; A = C C^T + n I is conditioned below 10, so both factors
+    agree to n rounding errors of 2.2e-16 times that: 1e-12.  A negative last diagonal entry is
+    the pivot reported."""
+    rng = np.random.default_rng(n)
+    C = rng.standard_normal((n, n))
+    A = C @ C.T + n * np.eye(n)
+    got = _inverse_factor(exx, A)
+    ref = np.linalg.inv(np.linalg.cholesky(A))
+    assert np.linalg.norm(got - ref) <= 1e-12 * np.linalg.norm(ref)
+    assert not np.triu(got, 1).any()
+    A[n - 1, n - 1] = -1.0
+    with pytest.raises(exx.ExxError) as e:
+        _inverse_factor(exx, A)
+    assert e.value.status == exx.EXX_ERR_NOT_POSDEF and e.value.pivot == n - 1
+
+
+def test_one_block_is_one_launch(exx):
+    """Two kernels for M, one for the factor and its inverse, one for xi."""
+    p = exx.Plan((8, 8, 8), 0.5, (1, 1, 0), 12, exx.EXX_KERNEL_ERFC, 0.106)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    psi = torch.randn((32, p.N), dtype=torch.float64, device="cuda", generator=g)
+    p.ace_build(psi, -psi)
+    assert p.launch_count() == 4
