@@ -56,8 +56,11 @@ __global__ void c_pair_kernel(long N, int nfields, const cd *psi_occ, long ld_oc
 //     inverse   C + i S = out_j and e^{i theta} (C - i S) = out_{n-j} from C = sum_p t_p cos(phi_p j),
 //               S = sum_p t_p sin(phi_p j).
 // A CTA stages 32 pencils (folded, forward periodic) in shared memory; a thread has one pencil
-// and kCOut outputs at a time.  Coefficients T[k nc + o], cosines then sines for periodic axes.
-constexpr int kCPen = 32, kCThreads = 256, kCOut = 4;
+// and CO outputs at a time, the groups of outputs dealt to the blockIdx.y first and then to the warps.
+// Four outputs a thread; one where few pencils leave most SMs idle (a 24 x 20 x 22 field has 17 CTAs of
+// them: a warp's FMAs are 64 cycles apart, so a chain of 4 x 24 steps in few warps took 27 us).
+// Coefficients T[k nc + o], cosines then sines for periodic axes.
+constexpr int kCPen = 32, kCThreads = 256;
 enum { C_REAL = 0, C_FWD = 1, C_INV = 2 };
 struct CAxis {
     long npen;           // pencils: fields x N / nd
@@ -70,7 +73,7 @@ struct CAxis {
     const double *S;
 };
 
-template <int MODE>
+template <int MODE, int CO>
 __global__ void __launch_bounds__(kCThreads) c_axis_kernel(const CAxis a)
 {
     extern __shared__ cd sx[];                       // [k][32]; forward periodic: x + y, then x - y
@@ -108,17 +111,18 @@ __global__ void __launch_bounds__(kCThreads) c_axis_kernel(const CAxis a)
     if (pl >= nfull) return;
     const long b = base(q0 + pl);
     const double *Ts = a.T + size_t(a.nk) * a.no;
-    for (int o0 = og * kCOut; o0 < a.no; o0 += (kCThreads / 32) * kCOut) {
-        double cr[kCOut] = {}, ci[kCOut] = {}, sr[kCOut] = {}, si[kCOut] = {};
-        int oc[kCOut];
+    const int og0 = og * int(gridDim.y) + int(blockIdx.y);
+    for (int o0 = og0 * CO; o0 < a.no; o0 += (kCThreads / 32) * int(gridDim.y) * CO) {
+        double cr[CO] = {}, ci[CO] = {}, sr[CO] = {}, si[CO] = {};
+        int oc[CO];
 #pragma unroll
-        for (int t = 0; t < kCOut; ++t) oc[t] = min(o0 + t, a.no - 1);
+        for (int t = 0; t < CO; ++t) oc[t] = min(o0 + t, a.no - 1);
         for (int k = 0; k < a.nk; ++k) {
             const cd x = sx[k * kCPen + pl];
             const cd y = MODE == C_FWD ? sy[k * kCPen + pl] : x;
             const double *tk = a.T + size_t(k) * a.no, *ts = Ts + size_t(k) * a.no;
 #pragma unroll
-            for (int t = 0; t < kCOut; ++t) {
+            for (int t = 0; t < CO; ++t) {
                 const double c = tk[oc[t]];
                 cr[t] = fma(x.re, c, cr[t]);
                 ci[t] = fma(x.im, c, ci[t]);
@@ -130,7 +134,7 @@ __global__ void __launch_bounds__(kCThreads) c_axis_kernel(const CAxis a)
             }
         }
 #pragma unroll
-        for (int t = 0; t < kCOut; ++t) {
+        for (int t = 0; t < CO; ++t) {
             const int o = o0 + t;
             if (o >= a.no) break;
             auto put = [&](int at, cd v) {
@@ -430,10 +434,14 @@ int complex_apply(Plan &P, const double *psi_occ_d, int n_occ, long ld_occ, cons
         a.in = in;
         a.out = o;
         a.S = S;
-        auto kern = !per ? c_axis_kernel<C_REAL> : inv ? c_axis_kernel<C_INV> : c_axis_kernel<C_FWD>;
+        const long gx = (a.npen + kCPen - 1) / kCPen;
+        const bool few = gx * a.no <= 8L * P.num_sms;   // at most two warps for each quarter of an SM with one output each
+        auto kern = few ? (!per ? c_axis_kernel<C_REAL, 1> : inv ? c_axis_kernel<C_INV, 1> : c_axis_kernel<C_FWD, 1>)
+                        : (!per ? c_axis_kernel<C_REAL, 4> : inv ? c_axis_kernel<C_INV, 4> : c_axis_kernel<C_FWD, 4>);
         const size_t smem = size_t(a.nk) * kCPen * sizeof(cd) * (per && !inv ? 2 : 1);   // at most 132 KB
         if (smem > 48 * 1024) EXX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-        kern<<<unsigned((a.npen + kCPen - 1) / kCPen), kCThreads, smem, s>>>(a);
+        const long gy = few ? (a.no + 3) / 4 : 1;       // four warps of a CTA at work, one on each quarter
+        kern<<<dim3(unsigned(gx), unsigned(gy)), kCThreads, smem, s>>>(a);
         EXX_LAUNCH("c_axis_kernel");
         P.launches++;
         return EXX_OK;

@@ -109,3 +109,16 @@ def test_a_warp_gives_up_a_wait_as_one(exx):
     on = ctypes.c_uint(1)
     assert L.exx_debug_wait_warp(ctypes.byref(on)) == 0
     assert on.value == 0
+
+
+def test_complex_axes_by_one_output_or_four(exx):
+    """Few pencils take one output a thread, many four: the same sums, so the same bits."""
+    n, no, ni = (24, 20, 22), 6, 20
+    g = torch.Generator(device="cuda").manual_seed(7)
+    N = n[0] * n[1] * n[2]
+    z = torch.randn((no + ni, N), dtype=torch.complex128, device="cuda", generator=g)
+    f = torch.rand(no, dtype=torch.float64, device="cuda", generator=g)
+    p = exx.Plan.bloch(n, 0.3, (1, 1, 0), [0.7, -1.3, 0.0], 12, exx.EXX_KERNEL_ERFC, 0.106)
+    out = p.apply_complex(z[:1].contiguous(), f[:1], z[no:].contiguous())
+    for j in (0, 7, 19):
+        assert torch.equal(p.apply_complex(z[:1].contiguous(), f[:1], z[no + j:no + j + 1].contiguous())[0], out[j])
