@@ -891,8 +891,10 @@ __global__ void __launch_bounds__(NT * GROUPS, 512 / (NT * GROUPS) > 0 ? 512 / (
     const int s1 = drow / n2, j1 = drow - s1 * n2, s2 = drow / n1, i2 = drow - s2 * n1;
 
     const long stride = long(gridDim.x) * GROUPS;
-    long p = (long(blockIdx.x) * GROUPS + grp) / a.tpf;
-    int zt = int((long(blockIdx.x) * GROUPS + grp) - p * a.tpf);
+    // tiles go to the CTAs first, then to their groups: few tiles get an SM each
+    const long first = long(grp) * gridDim.x + blockIdx.x;
+    long p = first / a.tpf;
+    int zt = int(first - p * a.tpf);
     const long dp = stride / a.tpf;
     const int dz = int(stride - dp * a.tpf);
     uint32_t ph = 0;
@@ -1622,7 +1624,7 @@ __global__ void __launch_bounds__(NT * GROUPS, NT * GROUPS <= 256 ? 2 : 1) zpass
     }
 
     const long stride = long(gridDim.x) * GROUPS;
-    const long first = long(blockIdx.x) * GROUPS + grp;
+    const long first = long(grp) * gridDim.x + blockIdx.x;   // few tiles get an SM each
     long p = first / a.tpfz;
     int rt = int(first - p * a.tpfz);
     const long dp = stride / a.tpfz;
@@ -2431,7 +2433,7 @@ int tc3_solve_batch(Plan &P, const int2 *pairs_d, int nfields, float *bufA, floa
         const int threads = DL.nt * DL.groups;
         int per_sm = 1;
         if (int rc = launch_setup(kern, threads, smem, DL.tmem_cols, per_sm)) return rc;
-        const int grid = int(std::min<long>((a.ntiles + DL.groups - 1) / DL.groups, long(P.num_sms) * per_sm));
+        const int grid = int(std::min<long>(a.ntiles, long(P.num_sms) * per_sm));
         const int tb = timing_begin(P, kind, s);
         kern<<<grid, threads, smem, s>>>(a);
         timing_end(P, tb, s);
@@ -2549,7 +2551,7 @@ int tc3_solve_batch(Plan &P, const int2 *pairs_d, int nfields, float *bufA, floa
         size_t smem = ZD.smem;
         int per_sm = 1;
         if (int rc = launch_setup(kern, threads, smem, ZD.tmem_cols, per_sm)) return rc;
-        const int grid = int(std::min<long>((a.ntiles + ZD.groups - 1) / ZD.groups, long(P.num_sms) * per_sm));
+        const int grid = int(std::min<long>(a.ntiles, long(P.num_sms) * per_sm));
         const int tb = timing_begin(P, EXX_TIMING_PASS3, s);
         kern<<<grid, threads, smem, s>>>(a);
         timing_end(P, tb, s);
