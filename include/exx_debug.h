@@ -8,6 +8,7 @@
  */
 #ifndef EXX_GB300_DEBUG_H
 #define EXX_GB300_DEBUG_H
+#include "exx.h"
 #ifdef __cplusplus
 extern "C" {
 #endif
@@ -32,6 +33,16 @@ int exx_debug_schedule(int n_occ, int n_in, int aliased, int block, int max_pair
  * each: pair fields, 1 when its outputs are those of one side only) may be NULL to get the number. */
 int exx_debug_plan_schedule(long N, int prec, int world, int pairs_per_batch, int block_orbitals, int n_occ, int n_in,
                             int aliased, int *limits, long *nbatches, int *batches);
+
+/* How an ACE product D (m x n) = A B^T with a contraction of K is cut when its digit planes may take
+ * `budget` bytes: out (HOST long[12]) = rows of a tile, column tiles, columns of each, rows of a slab, 320-long
+ * chunks of a slab, k splits, triangular limit in use, then the byte offsets of B's planes, the row
+ * scales of A and of B, the split sums, and the total.  ktri: B(j, k) = 0 for k > j. */
+int exx_debug_gemm_shape(long m, int n, long K, int ktri, int num_sms, long budget, long *out);
+
+/* A plan's bytes for those digit planes (0 = the default), and the size above which a workspace that
+ * has a smaller form counts as out of memory (0 = no such size). */
+int exx_debug_limits(exx_plan plan, long gemm_budget, long workspace_cap);
 
 /* One 128 x n x k tensor-core tile (tcgen05.mma, one bf16 or tf32 piece per operand,
  * FP32 accumulation): D (128 x n, row-major) = A (128 x k, row-major) B (n x k,

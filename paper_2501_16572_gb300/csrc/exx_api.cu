@@ -47,10 +47,20 @@ int dev_reserve(DevBuf &b, size_t bytes)
     cudaError_t e = cudaMalloc(&b.p, bytes);
     if (e != cudaSuccess) {
         b.p = nullptr;
+        cudaGetLastError();   // reported here, not by the next launch check
         return cuda_fail(e, "cudaMalloc(workspace)");
     }
     b.bytes = bytes;
     return EXX_OK;
+}
+
+int plan_reserve(Plan &P, DevBuf &b, size_t bytes)
+{
+    if (P.ws_cap && bytes > P.ws_cap) {
+        dev_free(b);
+        return cuda_fail(cudaErrorMemoryAllocation, "workspace above the plan's cap");
+    }
+    return dev_reserve(b, bytes);
 }
 
 void dev_free(DevBuf &b)
@@ -691,6 +701,8 @@ int ace_build(exx_plan plan, const double *Psi, int n, long ld, const double *W,
     // CUDA cores; the Cholesky factor and its inverse are FP64 in both
     const bool tcg = P->prec != EXX_PREC_FP64;
     if (tcg) {
+        const GemmDims both[2] = {{n, n, P->N, false}, {P->N, n, n, true}};
+        if (int rc = tc_gemm_reserve(*P, both, 2)) return rc;
         if (int rc = tc_gemm(*P, n, n, P->N, Psi, ld, 1, W, ld_w, 1, P->dV, M, 1, n, s)) return rc;
     } else if (int rc = gemm_fp64_tn_splitk(*P, n, n, P->N, Psi, ld, W, ld_w, P->dV, M, n, s)) {
         return rc;
@@ -729,6 +741,8 @@ int ace_apply(exx_plan plan, const double *xi, int n, long ld_xi, const double *
     double *chi = static_cast<double *>(P->small_ws.p);
     // chi = xi^T Phi (n x nphi), out = -dV xi chi
     if (P->prec != EXX_PREC_FP64) {   // the two products on the tensor cores
+        const GemmDims both[2] = {{n, nphi, P->N, false}, {P->N, nphi, n, false}};
+        if (int rc = tc_gemm_reserve(*P, both, 2)) return rc;
         if (int rc = tc_gemm(*P, n, nphi, P->N, xi, ld_xi, 1, Phi, ld_phi, 1, 1.0, chi, 1, n, s)) return rc;
         return tc_gemm(*P, P->N, nphi, n, xi, 1, ld_xi, chi, n, 1, -P->dV, out, 1, ld_out, s);
     }

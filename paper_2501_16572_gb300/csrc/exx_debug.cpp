@@ -88,6 +88,25 @@ int exx_debug_plan_schedule(long N, int prec, int world, int pairs_per_batch, in
     return EXX_OK;
 }
 
+int exx_debug_gemm_shape(long m, int n, long K, int ktri, int num_sms, long budget, long *out)
+{
+    if (m < 1 || n < 1 || K < 1 || num_sms < 1 || budget < 1 || !out) return EXX_ERR_INVALID_ARG;
+    const exx::GemmShape g = exx::gemm_shape({m, n, K, ktri != 0}, num_sms, budget);
+    const long v[] = {g.rt, g.nt, g.Nt, g.mslab, g.kslab, g.Zmax, g.ktri, long(g.offB), long(g.offSA),
+                      long(g.offSB), long(g.offP), long(g.bytes)};
+    std::copy(v, v + 12, out);
+    return EXX_OK;
+}
+
+int exx_debug_limits(exx_plan plan, long gemm_budget, long workspace_cap)
+{
+    exx::Plan *P = reinterpret_cast<exx::Plan *>(plan);
+    if (!P || gemm_budget < 0 || workspace_cap < 0) return EXX_ERR_INVALID_ARG;
+    P->gemm_budget = gemm_budget ? gemm_budget : exx::Plan().gemm_budget;
+    P->ws_cap = size_t(workspace_cap);
+    return EXX_OK;
+}
+
 int exx_debug_tc_gemm(int tf32, int n, int k, const float *A, const float *B, float *D, int *err)
 {
     if (!A || !B || !D || !err) return EXX_ERR_INVALID_ARG;

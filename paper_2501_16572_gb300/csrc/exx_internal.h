@@ -190,6 +190,8 @@ struct Plan {
     Timing timing;
     // cached schedule
     int sched_key[4] = {-1, -1, -1, -1};
+    long gemm_budget = 1L << 30;   // bytes of the ACE products' digit planes, halved where they do not fit
+    size_t ws_cap = 0;             // exx_debug_limits: larger workspaces count as out of memory
     int sched_block = 8;  // orbitals per pair block of the cached schedule
     uint64_t epoch = 0;   // changes whenever device data or settings that launches read change
     Schedule sched;
@@ -234,6 +236,23 @@ int tc_wait_warp_probe(unsigned *went_on_h);
 // reductions, GEMM, Cholesky (exx_linalg.cu)
 int energy_fp64(Plan &P, const double *psi, int n, long ld, const double *f, const double *v,
                 long ld_v, double *E_h, cudaStream_t s);
+int plan_reserve(Plan &P, DevBuf &b, size_t bytes);   // a workspace that has a smaller form
+// One product of tc_gemm, and how it is cut to a budget of digit planes.
+struct GemmDims {
+    long m;
+    int n;
+    long K;
+    bool ktri;
+};
+struct GemmShape {
+    int rt, nt, Nt;        // rows of a tile, column tiles, columns of each
+    long mslab, kslab;     // rows and 320-long chunks whose digit planes are in memory at a time
+    long Zmax, slots;      // k splits, resident CTAs
+    bool ktri;
+    size_t offB, offSA, offSB, offP, bytes;
+};
+GemmShape gemm_shape(const GemmDims &d, int num_sms, long budget);
+int tc_gemm_reserve(Plan &P, const GemmDims *d, int count);
 // D(i, j) = alpha sum_k A(i, k) B(j, k) on the tensor cores (fixed-point digits, exact
 // 320-long chunks); A(i, k) = A[i as_i + k as_k], same for B and D.  ktri: B(j, k) = 0 for k > j.
 int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_k, const double *B, long bs_j,

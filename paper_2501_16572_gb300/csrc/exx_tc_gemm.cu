@@ -47,7 +47,6 @@ constexpr uint32_t kSbo = kBlk * 16;           // bytes between 8-row groups of 
 constexpr int kParts = 4;            // drain warps per 32 TMEM lanes (2 for tiles of up to 32 columns)
 constexpr int kNarrow = 32;          // tiles of up to 32 columns: one set of levels, two CTAs per SM
 constexpr int kCutWarps = kBlks;     // gemm_cut_kernel: a warp per k block of a chunk
-constexpr long kDigitBudget = 1L << 30;        // device memory of the digit planes of one slab
 
 __device__ __forceinline__ int exp_field(uint32_t hi) { return int((hi >> 20) & 0x7ffu); }
 
@@ -170,7 +169,7 @@ __global__ void __launch_bounds__(32 * kCutWarps) gemm_cut_kernel(const CutArgs 
 struct GemmArgs {
     long m;
     int n;
-    int Nt, mt, nt;            // tile columns, tiles
+    int rt, Nt, mt, nt;        // tile rows and columns, tiles
     long Z;                    // k splits
     long nkb, nchunks;         // blocks and chunks of this slab
     long cper;                 // chunks per split
@@ -264,7 +263,7 @@ __global__ void __launch_bounds__(128 * PARTS + 64, 3 - SETS) tc_gemm_kernel(con
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
     const long items = a.Z * a.mt * a.nt;
     const int Nt = a.Nt;
-    const uint32_t a_bytes = kT * kBlk * 2 * kDig, b_bytes = uint32_t(Nt) * kBlk * 2 * kDig;
+    const uint32_t a_bytes = uint32_t(a.rt) * kBlk * 2 * kDig, b_bytes = uint32_t(Nt) * kBlk * 2 * kDig;
     struct Item {
         long z, c0, c1;
         int mi, ni;
@@ -322,8 +321,7 @@ __global__ void __launch_bounds__(128 * PARTS + 64, 3 - SETS) tc_gemm_kernel(con
         // operand and accumulator steps, fixed for the launch: the issue of one 16-k step is a
         // straight run of MMAs by the whole warp whose descriptors differ by additions (computed in
         // a loop by one lane, a step took 1340 cycles, twice the tensor pipe's time)
-        constexpr uint32_t kStepA = kT * kBlk * 2 / 16;            // next A digit, in 16-byte units
-        const uint32_t step_b = uint32_t(Nt) * kBlk * 2 / 16;      // next B digit
+        const uint32_t step_a = uint32_t(a.rt) * kBlk * 2 / 16, step_b = uint32_t(Nt) * kBlk * 2 / 16;   // next digit, in 16 bytes
         uint32_t idesc[kDig + 1];
 #pragma unroll
         for (int g = 1; g <= kDig; ++g) idesc[g] = tc::instr_desc(false, g * Nt);
@@ -333,7 +331,7 @@ __global__ void __launch_bounds__(128 * PARTS + 64, 3 - SETS) tc_gemm_kernel(con
 #pragma unroll
             for (int i = 0; i < kDig; ++i) {
                 const int nj = kDig < kLev - i ? kDig : kLev - i;
-                const uint64_t ad = ad0 + i * kStepA;
+                const uint64_t ad = ad0 + i * step_a;
                 const uint32_t d = d0 + uint32_t(i * Nt);
                 if (i == 1 && first) {   // digit 0 has opened levels 0..3; level 4 starts here
                     tc::mma_bf16_warp(d, ad, bd, idesc[kDig - 1], 1u, el);
@@ -418,7 +416,7 @@ __global__ void __launch_bounds__(128 * PARTS + 64, 3 - SETS) tc_gemm_kernel(con
                 const uint32_t d0 = tmem + lane_q + uint32_t(set * kLev * Nt);
 #pragma unroll
                 for (int cg = 0; cg < NH / 4; ++cg) {
-                    if (cg * 4 >= ncol) break;
+                    if (cg * 4 >= ncol || i - lane >= a.m) break;   // uniform
                     const int cc = cbase + cg * 4;
                     uint32_t r[kLev][4];
 #pragma unroll
@@ -535,6 +533,70 @@ int launch_cut(Plan &P, const double *X, long sr, long sk, long rows, long K, in
 
 }  // namespace
 
+// Tiles, slabs and workspace of one product whose digit planes may take `budget` bytes.
+GemmShape gemm_shape(const GemmDims &d, int num_sms, long budget)
+{
+    GemmShape g{};
+    // column tiles: as even as 16-column steps allow, at most 48 (two sets of 5 levels in 512 TMEM columns)
+    g.nt = int(ceil_div(d.n, kTN));
+    g.Nt = int(ceil_div(ceil_div(d.n, g.nt), 16) * 16);
+    const long np = long(g.nt) * g.Nt;
+    // slabs: the digit planes (8 B per element) of one slab stay within the budget, cut along m
+    // when the contraction is short, along k when it is long
+    const long chunks = ceil_div(d.K, kChunk);
+    const long chunk_bytes = std::min(8L * kChunk, ceil_div(d.K, kBlk) * kBlk * 8);   // per row (and of a lone short chunk)
+    g.rt = int(std::min<long>(kT, ceil_div(d.m, 8) * 8));   // a lone short tile holds, and moves, no more rows than it has
+    const long mpad = ceil_div(d.m, g.rt) * g.rt;
+    g.mslab = mpad;
+    g.kslab = chunks;
+    if (chunks > 64) {
+        g.kslab = std::max(1L, budget / (chunk_bytes * (mpad + np)));
+    } else {
+        g.kslab = std::min(chunks, std::max(1L, budget / 2 / (chunk_bytes * std::max<long>(np, g.rt))));
+        const long room = budget - std::min(budget / 2, chunk_bytes * g.kslab * np);
+        g.mslab = std::max<long>(g.rt, room / (chunk_bytes * g.kslab) / g.rt * g.rt);
+    }
+    g.mslab = std::min(g.mslab, mpad);
+    g.kslab = std::min(std::min(g.kslab, chunks), 65535L);
+    g.kslab = ceil_div(chunks, ceil_div(chunks, g.kslab));                     // even slabs
+    g.mslab = ceil_div(mpad / g.rt, ceil_div(mpad, g.mslab)) * g.rt;
+    // k splits: items (tiles x splits) for a whole number of rounds over the SMs
+    g.ktri = d.ktri && g.kslab == chunks;   // the limit counts chunks from k = 0
+    g.slots = long(num_sms) * (g.Nt <= kNarrow ? 2 : 1);   // CTAs resident at once
+    g.Zmax = 1;
+    const long tiles = (g.mslab / g.rt) * g.nt;
+    if (!g.ktri && g.kslab > 1 && tiles < 2 * g.slots) {
+        const long round = std::max(1L, g.slots / tiles);
+        const long slot = ceil_div(g.mslab, kT) * kT * d.n * long(sizeof(double));
+        g.Zmax = std::min(g.kslab >= 8 * round ? 2 * round : round, g.kslab);
+        g.Zmax = std::min(g.Zmax, std::max(1L, budget / 4 / slot));
+    }
+    g.offB = round_up(size_t(g.mslab) * chunk_bytes * g.kslab, 256);
+    g.offSA = g.offB + round_up(size_t(np) * chunk_bytes * g.kslab, 256);
+    g.offSB = g.offSA + round_up(size_t(g.mslab) * g.kslab * 4, 256);
+    g.offP = g.offSB + round_up(size_t(np) * g.kslab * 4, 256);
+    g.bytes = g.offP + (g.Zmax > 1 ? size_t(g.Zmax) * std::min(g.mslab, d.m) * d.n * sizeof(double) : 0);
+    return g;
+}
+
+// One workspace for the products of a call.  A device too full for it gets smaller slabs, down to
+// one tile and one chunk; the plan keeps the smaller budget.
+int tc_gemm_reserve(Plan &P, const GemmDims *d, int count)
+{
+    for (;;) {
+        size_t bytes = 0;
+        bool least = true;
+        for (int i = 0; i < count; ++i) {
+            const GemmShape g = gemm_shape(d[i], P.num_sms, P.gemm_budget);
+            bytes = std::max(bytes, g.bytes);
+            least = least && g.mslab == g.rt && g.kslab == 1;
+        }
+        const int rc = plan_reserve(P, P.gemm_ws, bytes);
+        if (rc != EXX_ERR_OOM || least || P.gemm_budget < 2) return rc;
+        P.gemm_budget /= 2;
+    }
+}
+
 int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_k, const double *B, long bs_j,
             long bs_k, double alpha, double *D, long ds_i, long ds_j, cudaStream_t s, bool ktri)
 {
@@ -543,68 +605,40 @@ int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_
         if (int rc = dev_reserve(P.err_d, 16)) return rc;
         EXX_CUDA(cudaMemsetAsync(P.err_d.p, 0, 16, s));
     }
-    // column tiles: as even as 16-column steps allow, at most 48 (two sets of 5 levels in 512 TMEM columns)
-    const int nt = int(ceil_div(n, kTN));
-    const int Nt = int(ceil_div(ceil_div(n, nt), 16) * 16);
-    const long np = long(nt) * Nt;
-    // slabs: the digit planes (8 B per element) of one slab stay within kDigitBudget, cut along
-    // m when the contraction is short, along k when it is long
-    const long chunks = ceil_div(K, kChunk);
-    const long chunk_bytes = std::min(8L * kChunk, ceil_div(K, kBlk) * kBlk * 8);   // per row (and of a lone short chunk)
-    const long mpad = ceil_div(m, kT) * kT;
-    const bool long_k = chunks > 64;
-    long mslab = mpad, kslab = chunks;
-    if (long_k) {
-        kslab = std::max(1L, kDigitBudget / (chunk_bytes * (mpad + np)));
-    } else {
-        kslab = std::min(chunks, std::max(1L, kDigitBudget / 2 / (chunk_bytes * np)));
-        const long room = kDigitBudget - std::min(kDigitBudget / 2, chunk_bytes * kslab * np);
-        mslab = std::max<long>(kT, room / (chunk_bytes * kslab) / kT * kT);
+    const GemmDims dims{m, n, K, ktri};
+    GemmShape g = gemm_shape(dims, P.num_sms, P.gemm_budget);
+    if (P.gemm_ws.bytes < g.bytes) {
+        if (int rc = tc_gemm_reserve(P, &dims, 1)) return rc;
+        g = gemm_shape(dims, P.num_sms, P.gemm_budget);
     }
-    mslab = std::min(mslab, mpad);
-    kslab = std::min(std::min(kslab, chunks), 65535L);
-    kslab = ceil_div(chunks, ceil_div(chunks, kslab));                     // even slabs
-    mslab = ceil_div(ceil_div(mpad, kT), ceil_div(mpad, mslab)) * kT;
-    // k splits: items (tiles x splits) for a whole number of rounds over the SMs
-    const long tiles = (mslab / kT) * nt;
-    const long slots = long(P.num_sms) * (Nt <= kNarrow ? 2 : 1);   // CTAs resident at once
-    auto splits = [&](long nch) {
-        if (nch < 2 || tiles >= 2 * slots) return 1L;
-        const long round = std::max(1L, slots / tiles);
-        long Z = nch >= 8 * round ? 2 * round : round;
-        Z = std::min(Z, nch);
-        return std::min(Z, std::max(1L, (1L << 28) / (mslab * n * 8)));
-    };
-    if (kslab < chunks) ktri = false;   // the limit counts chunks from k = 0
-    const long Zmax = ktri ? 1 : splits(kslab);
-    const size_t ldigA = size_t(mslab) * chunk_bytes * kslab, ldigB = size_t(np) * chunk_bytes * kslab;
-    const size_t offB = round_up(ldigA, 256), offSA = offB + round_up(ldigB, 256);
-    const size_t offSB = offSA + round_up(size_t(mslab) * kslab * 4, 256);
-    const size_t offP = offSB + round_up(size_t(np) * kslab * 4, 256);
-    const size_t part = Zmax > 1 ? size_t(Zmax) * std::min(mslab, m) * n * sizeof(double) : 0;
-    if (int rc = dev_reserve(P.gemm_ws, offP + part)) return rc;
     uint8_t *ws = static_cast<uint8_t *>(P.gemm_ws.p);
-    int *shA = reinterpret_cast<int *>(ws + offSA), *shB = reinterpret_cast<int *>(ws + offSB);
+    int *shA = reinterpret_cast<int *>(ws + g.offSA), *shB = reinterpret_cast<int *>(ws + g.offSB);
+    const int rt = g.rt, nt = g.nt, Nt = g.Nt;
+    const long np = long(nt) * Nt, mslab = g.mslab, kslab = g.kslab, chunks = ceil_div(K, kChunk);
+    ktri = g.ktri;
 
     GemmArgs a{};
     a.n = n;
+    a.rt = rt;
     a.Nt = Nt;
     a.nt = nt;
     a.digA = ws;
-    a.digB = ws + offB;
+    a.digB = ws + g.offB;
     a.shA = shA;
     a.shB = shB;
     a.prowB = np;
     a.ktri = ktri ? 1 : 0;
     a.err = static_cast<int *>(P.err_d.p);
-    a.stage_bytes = uint32_t(kT + Nt) * kBlk * 2 * kDig;
+    a.stage_bytes = uint32_t(rt + Nt) * kBlk * 2 * kDig;
     const bool narrow = Nt <= kNarrow;
     a.stages = int(std::min<size_t>(8, (narrow ? 111 : 222) * 1024 / a.stage_bytes));
     a.offTab = uint32_t(a.stages) * a.stage_bytes;
     a.offBar = a.offTab + 2 * kTN * 4;
     a.tmem_cols = 32;
     while (a.tmem_cols < (narrow ? 1 : 2) * kLev * Nt) a.tmem_cols *= 2;
-    const size_t smem = a.offBar + (2 * size_t(a.stages) + 4) * 8 + 16;
+    size_t smem = a.offBar + (2 * size_t(a.stages) + 4) * 8 + 16;
+    // the MMA reads 128 rows of every A digit: what lies past a short tile's, to lanes nobody reads
+    smem = std::max(smem, size_t(a.stages - 1) * a.stage_bytes + (size_t(3) * rt + kT) * kBlk * 2);
     auto kern = narrow ? tc_gemm_kernel<2, 1> : tc_gemm_kernel<kParts, 2>;
     const int threads = 128 * (narrow ? 2 : kParts) + 64;
     EXX_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
@@ -612,22 +646,22 @@ int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_
     for (long c0 = 0; c0 < chunks; c0 += kslab) {
         const long nch = std::min(kslab, chunks - c0);
         const long k0 = c0 * kChunk, kk = std::min(K - k0, nch * kChunk);
-        if (int rc = launch_cut(P, B + k0 * bs_k, bs_j, bs_k, n, kk, Nt, nt, ws + offB, shB, s)) return rc;
+        if (int rc = launch_cut(P, B + k0 * bs_k, bs_j, bs_k, n, kk, Nt, nt, ws + g.offB, shB, s)) return rc;
         for (long i0 = 0; i0 < m; i0 += mslab) {
             const long mr = std::min(mslab, m - i0);
-            a.mt = int(ceil_div(mr, kT));
-            if (int rc = launch_cut(P, A + i0 * as_i + k0 * as_k, as_i, as_k, mr, kk, kT, a.mt, ws, shA, s)) return rc;
+            a.mt = int(ceil_div(mr, rt));
+            if (int rc = launch_cut(P, A + i0 * as_i + k0 * as_k, as_i, as_k, mr, kk, rt, a.mt, ws, shA, s)) return rc;
             a.m = mr;
-            a.prowA = long(a.mt) * kT;
+            a.prowA = long(a.mt) * rt;
             a.nkb = ceil_div(kk, kBlk);
             a.nchunks = nch;
-            a.Z = ktri ? 1 : std::min(Zmax, nch);
+            a.Z = std::min(g.Zmax, nch);
             a.cper = ceil_div(nch, a.Z);
             a.Z = ceil_div(nch, a.cper);
             double *Dd = D + i0 * ds_i;
             a.alpha = a.Z > 1 ? 1.0 : alpha;   // split sums take it in the reduction
             if (a.Z > 1) {
-                a.D = reinterpret_cast<double *>(ws + offP);
+                a.D = reinterpret_cast<double *>(ws + g.offP);
                 a.ds_i = 1;
                 a.ds_j = mr;
                 a.dz = mr * n;
@@ -641,7 +675,7 @@ int tc_gemm(Plan &P, long m, int n, long K, const double *A, long as_i, long as_
             }
             const long items = a.Z * a.mt * a.nt;
             int tb = timing_begin(P, EXX_TIMING_GEMM, s);
-            kern<<<unsigned(std::min<long>(items, slots)), threads, smem, s>>>(a);
+            kern<<<unsigned(std::min<long>(items, g.slots)), threads, smem, s>>>(a);
             timing_end(P, tb, s);
             EXX_LAUNCH("tc_gemm_kernel");
             P.launches++;

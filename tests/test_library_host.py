@@ -198,6 +198,35 @@ def test_set_batch_limits_the_fields_of_a_batch(lib, n_occ, n_in, aliased, pairs
     assert lim[0] == (8 if 0 < pairs < 256 else 16)
 
 
+def test_ace_product_slabs_cover_the_product_within_the_budget(lib):
+    """Slabs of rows and of 320-long chunks: whole tiles, digit planes (8 bytes an entry) within the
+    budget, or of one chunk where B alone passes half of it (A's then within half, or one tile) or the
+    contraction is long (all rows); regions in order and large enough."""
+    Lp = ctypes.POINTER(ctypes.c_long)
+    lib.exx_debug_gemm_shape.argtypes = [ctypes.c_long, ctypes.c_int, ctypes.c_long, ctypes.c_int, ctypes.c_int,
+                                         ctypes.c_long, Lp]
+    rng = np.random.default_rng(320)
+    keys = "rt nt Nt mslab kslab Z ktri offB offSA offSB offP bytes".split()
+    for _ in range(4000):
+        short = bool(rng.integers(2))
+        m, n, K = (int(np.exp(rng.uniform(0, np.log(v)))) for v in ((2e6, 2048, 2048) if short else (2048, 2048, 2e6)))
+        ktri, budget = int(short and rng.integers(2)), 1 << int(rng.integers(16, 31))
+        out = (ctypes.c_long * 12)()
+        assert lib.exx_debug_gemm_shape(m, n, K, ktri, 152, budget, out) == 0
+        g = dict(zip(keys, out))
+        chunks, row = -(-K // 320), min(2560, -(-K // 32) * 256)   # bytes of a row in one chunk
+        assert g["rt"] == min(128, -(-m // 8) * 8) and g["Nt"] in (16, 32, 48) and g["nt"] * g["Nt"] >= n > (g["nt"] - 1) * g["Nt"]
+        assert g["mslab"] % g["rt"] == 0 and 0 < g["mslab"] <= -(-m // g["rt"]) * g["rt"] and 0 < g["kslab"] <= chunks
+        a, b = g["mslab"] * row * g["kslab"], g["nt"] * g["Nt"] * row * g["kslab"]
+        assert a + b <= budget or g["kslab"] == 1 and (chunks > 64 or a <= budget // 2 or g["mslab"] == g["rt"]), (m, n, K, budget, g)
+        assert g["offB"] >= a and g["offSA"] >= g["offB"] + b
+        assert g["offSB"] >= g["offSA"] + 4 * g["mslab"] * g["kslab"] and g["offP"] >= g["offSB"] + 4 * g["nt"] * g["Nt"] * g["kslab"]
+        assert not g["offB"] % 256 and not g["offP"] % 256
+        split = 8 * g["Z"] * min(g["mslab"], m) * n if g["Z"] > 1 else 0
+        assert g["bytes"] == g["offP"] + split and split <= budget // 4 and 1 <= g["Z"] <= g["kslab"]
+        assert not g["ktri"] or ktri and g["Z"] == 1 and g["kslab"] == chunks
+
+
 def test_fast_division_matches_integer_division(lib):
     """Row -> (field, row in field) in the pass kernels divides by multiply and shift;
     every quotient must equal the integer one, at the divisor and quotient edges too."""
