@@ -83,8 +83,8 @@ __global__ void __launch_bounds__(kCThreads) c_axis_kernel(const CAxis a)
     auto base = [&](long q) { return (q / a.sd) * (a.sd * a.nd) + q % a.sd; };   // first point of pencil q
     const int nfull = int(min(long(kCPen), a.npen - q0));
     const cd zero = {0.0, 0.0};
-    // e^{i theta} or its conjugate times v
-    auto turn = [&](cd v, double s) { return cd{v.re * a.cth - s * v.im * a.sth, v.im * a.cth + s * v.re * a.sth}; };
+    // e^{i theta} or its conjugate times v; explicit fused products, the same for every CO
+    auto turn = [&](cd v, double s) { return cd{fma(v.re, a.cth, -s * v.im * a.sth), fma(v.im, a.cth, s * v.re * a.sth)}; };
     if (MODE != C_FWD) {
         if (a.sd == 1) {   // consecutive pencils are one run of memory
             for (int i = threadIdx.x; i < kCPen * a.nd; i += kCThreads) {
