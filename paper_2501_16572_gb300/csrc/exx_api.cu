@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -94,7 +95,8 @@ static void free_plan_buffers(Plan &P)
 static int ensure_schedule(Plan &P, int n_occ, int n_in, bool aliased, cudaStream_t s)
 {
     int block, maxp;
-    schedule_limits(P.N, P.prec, P.shard_world, P.pairs_per_batch, P.block_orbitals, block, maxp);
+    schedule_limits(P.N, P.prec, P.shard_world, P.pairs_per_batch > 0 ? P.pairs_per_batch : P.pairs_cap, P.block_orbitals, block,
+                    maxp);
     int key[4] = {n_occ, n_in, (aliased ? 1 : 0) | (P.shard_world > 1 ? 2 : 0) | (block << 2), maxp};
     if (std::equal(key, key + 4, P.sched_key)) return EXX_OK;
     P.sched = build_schedule(n_occ, n_in, aliased, block, maxp, P.shard_world);
@@ -249,6 +251,7 @@ int exx_plan_set_precision(exx_plan plan, int prec)
         if (int rc = tc_upload(*P, prec)) return rc;
     }
     P->prec = prec;
+    P->pairs_cap = 0;
     std::fill(P->sched_key, P->sched_key + 4, -1);
     bump_epoch(*P);
     return EXX_OK;
@@ -262,6 +265,7 @@ int exx_plan_set_batch(exx_plan plan, int pairs_per_batch, int block_orbitals)
         return invalid("exx_plan_set_batch: sizes must be >= 0 (block <= 32)");
     P->pairs_per_batch = pairs_per_batch;
     P->block_orbitals = block_orbitals;
+    P->pairs_cap = 0;
     std::fill(P->sched_key, P->sched_key + 4, -1);
     bump_epoch(*P);
     return EXX_OK;
@@ -375,19 +379,23 @@ static int apply_prepare(Plan *P, ApplyCall &c, cudaStream_t s)
     };
     if (overlaps(c.Psi_occ, c.n_occ, c.ld_occ) || overlaps(c.Psi_in, c.n_in, c.ld_in)) return invalid("exx_apply: out overlaps an input");
     c.aliased = (c.Psi_in == c.Psi_occ) && (c.ld_in == c.ld_occ) && (c.n_in >= c.n_occ);
-    if (int rc = ensure_schedule(*P, c.n_occ, c.n_in, c.aliased, s)) return rc;
-    const Schedule &S = P->sched;
-    if (P->prec == EXX_PREC_FP64) {
-        size_t fb = size_t(S.max_fields) * P->N * sizeof(double);
-        if (int rc = dev_reserve(P->work[0], fb)) return rc;
-        return dev_reserve(P->work[1], fb);
+    if (P->prec != EXX_PREC_FP64)
+        if (int rc = tc_reserve_orbitals(*P, c.n_occ, c.n_in, c.aliased)) return rc;
+    // two batch buffers.  A device too full for the automatic batch gets smaller ones, down to one
+    // block of 8 x 8 orbitals (or of the caller's); the plan keeps the smaller batch
+    for (int last = INT_MAX;;) {
+        if (int rc = ensure_schedule(*P, c.n_occ, c.n_in, c.aliased, s)) return rc;
+        const Schedule &S = P->sched;
+        const bool hl = P->prec != EXX_PREC_FP64 && tc_is_hilo(P->prec);
+        P->tc_lo_off = hl ? long(S.max_fields) * P->N : 0;
+        const size_t fb = size_t(S.max_fields) * P->N * (P->prec == EXX_PREC_FP64 || hl ? 8 : 4);
+        int rc = plan_reserve(*P, P->work[0], fb);
+        if (rc == EXX_OK) rc = plan_reserve(*P, P->work[1], fb);
+        if (rc != EXX_ERR_OOM || P->pairs_per_batch > 0 || S.max_fields <= 64 || S.max_fields >= last) return rc;
+        last = S.max_fields;
+        for (int i = 0; i < 2; ++i) dev_free(P->work[i]);
+        P->pairs_cap = std::max(64, S.max_fields / 2);
     }
-    if (int rc = tc_reserve_orbitals(*P, c.n_occ, c.n_in, c.aliased)) return rc;
-    const bool hl = tc_is_hilo(P->prec);
-    P->tc_lo_off = hl ? long(S.max_fields) * P->N : 0;
-    size_t fb = size_t(S.max_fields) * P->N * sizeof(float) * (hl ? 2 : 1);
-    if (int rc = dev_reserve(P->work[0], fb)) return rc;
-    return dev_reserve(P->work[1], fb);
 }
 
 // The launches of one exx_apply (stream work only: capturable into a CUDA graph).  With
