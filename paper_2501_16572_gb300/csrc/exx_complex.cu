@@ -405,8 +405,13 @@ int complex_apply(Plan &P, const double *psi_occ_d, int n_occ, long ld_occ, cons
     const size_t field = size_t(N) * sizeof(cd);
     const long room = std::max(1L, (1L << 30) / long(field));           // fields per buffer
     const int chunk = int(std::min<long>(n_occ, room));
-    const int group = int(std::max(1L, std::min<long>({long(n_in), room / n_occ, 65535L})));
-    if (int rc = dev_reserve(P.cwork, 2 * size_t(chunk) * group * field)) return rc;
+    int group = int(std::max(1L, std::min<long>({long(n_in), room / n_occ, 65535L})));
+    // a device too full for that gets fewer columns at a time; the plan keeps the smaller group
+    if (P.cgroup_cap > 0) group = std::min(group, P.cgroup_cap);
+    for (int rc; (rc = plan_reserve(P, P.cwork, 2 * size_t(chunk) * group * field)) != EXX_OK;) {
+        if (rc != EXX_ERR_OOM || group == 1) return rc;
+        P.cgroup_cap = group /= 2;
+    }
     if (int rc = dev_reserve(P.cpairs, size_t(n_occ) * size_t(n_in) * sizeof(int2))) return rc;
     std::vector<int2> pairs(size_t(n_occ) * n_in);
     for (int n = 0; n < n_in; ++n)

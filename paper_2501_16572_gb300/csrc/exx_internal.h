@@ -192,6 +192,7 @@ struct Plan {
     int sched_key[4] = {-1, -1, -1, -1};
     long gemm_budget = 1L << 30;   // bytes of the ACE products' digit planes, halved where they do not fit
     int pairs_cap = 0;             // pairs per batch that fitted the device, 0 = not tried
+    int cgroup_cap = 0;            // output columns of a complex apply at a time that fitted, 0 = not tried
     size_t ws_cap = 0;             // exx_debug_limits: larger workspaces count as out of memory
     int sched_block = 8;  // orbitals per pair block of the cached schedule
     uint64_t epoch = 0;   // changes whenever device data or settings that launches read change

@@ -48,3 +48,19 @@ def test_apply_takes_smaller_batches(exx, prec, cap, n_occ, n_in, aliased):
     assert e.value.status == exx.EXX_ERR_OOM
     _cap(exx, p, 0)
     assert torch.isfinite(p.apply(psi[:n_occ], f, phi)).all()
+
+
+def test_complex_apply_takes_fewer_columns(exx):
+    """6 occupied x 20 columns of 24 x 20 x 22 points: 2 MB a column, all of them at once without a cap."""
+    n, no, ni = (24, 20, 22), 6, 20
+    g = torch.Generator(device="cuda").manual_seed(3)
+    z = torch.randn((no + ni, n[0] * n[1] * n[2]), dtype=torch.complex128, device="cuda", generator=g)
+    f = torch.rand(no, dtype=torch.float64, device="cuda", generator=g)
+    p = exx.Plan.bloch(n, 0.3, (1, 1, 0), [0.7, -1.3, 0.0], 12, exx.EXX_KERNEL_ERFC, 0.106)
+    ref = p.apply_complex(z[:no].contiguous(), f, z[no:].contiguous())
+    _cap(exx, p, 5 * MB)
+    assert torch.equal(p.apply_complex(z[:no].contiguous(), f, z[no:].contiguous()), ref)
+    _cap(exx, p, MB)   # less than a column
+    with pytest.raises(exx.ExxError) as e:
+        p.apply_complex(z[:no].contiguous(), f, z[no:].contiguous())
+    assert e.value.status == exx.EXX_ERR_OOM
