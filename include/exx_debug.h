@@ -63,6 +63,11 @@ int exx_debug_fastdiv(unsigned d, int count, const unsigned *n, unsigned *q);
  * the same length and boundary condition (one image serves both).  Sizes in [2, 256]. */
 int exx_debug_tc3_layout(int n1, int n2, int n3, int share01, int *out);
 
+/* The layouts of the direct kernel forms, which a grid gets by itself (slices: where both matrices stay
+ * resident), host-side (no device): out (HOST int[59]) = 20 values each for pass A and pass C and 18 for
+ * pass B, in the order that tc3_debug_direct states, and the shared-memory limit. */
+int exx_debug_tc3_direct(int n1, int n2, int n3, int share01, int *out);
+
 /* The base-512 digit image of the 1D matrices, host-side: C (HOST, row-major nout x nk, row n =
  * output n, column k = contraction index k) cut for a WN x Kp block of rows n0.. and indices
  * k0.. (a K-chunk when k0 > 0 or Kp < nk), decoded from the tensor-core layout back to values:

@@ -13,6 +13,13 @@ int exx_debug_tc3_layout(int n1, int n2, int n3, int share01, int *out)
     return EXX_OK;
 }
 
+int exx_debug_tc3_direct(int n1, int n2, int n3, int share01, int *out)
+{
+    if (n1 < 2 || n2 < 2 || n3 < 2 || n1 > 256 || n2 > 256 || n3 > 256 || !out) return EXX_ERR_INVALID_ARG;
+    exx::tc3_debug_direct(n1, n2, n3, share01 != 0, out);
+    return EXX_OK;
+}
+
 int exx_debug_matrix_digits(int nout, int nk, const double *C, int WN, int Kp, int n0, int k0, float *digits,
                             float *scales)
 {

@@ -2107,6 +2107,26 @@ bool slice_direct_layout(const Plan &P, bool pair, SliceDLayout &L)
     return finish(512, 1) || finish(512, 1, false);
 }
 
+// Compiled forms of the slice kernel: groups, threads of one, staged input, units per thread.
+struct SliceInst {
+    int groups, nt, staged, upt;
+    void (*kern[2])(const SliceDArgs);   // [pair]
+};
+#define EXX_SLICE(G, NT, STG, U) {G, NT, STG, U, {slice_direct_kernel<false, NT, U, G, STG != 0>, slice_direct_kernel<true, NT, U, G, STG != 0>}}
+const SliceInst kSliceInst[] = {
+    EXX_SLICE(3, 256, 1, 2), EXX_SLICE(3, 256, 1, 3), EXX_SLICE(2, 256, 1, 3), EXX_SLICE(2, 256, 1, 4),
+    EXX_SLICE(1, 256, 1, 3), EXX_SLICE(1, 256, 1, 4), EXX_SLICE(1, 512, 1, 3), EXX_SLICE(1, 512, 1, 4),
+    EXX_SLICE(1, 512, 0, 4),
+};
+#undef EXX_SLICE
+// The narrowest one that holds the layout's units.
+const SliceInst *slice_instance(const SliceDLayout &L)
+{
+    for (const SliceInst &i : kSliceInst)
+        if (i.groups == L.groups && i.nt == L.nt && i.staged == L.staged && i.upt >= L.upt) return &i;
+    return nullptr;
+}
+
 struct ZLayout {
     size_t smem;
     uint32_t offB, offCs, offMax, offBar, blk_bytes;
@@ -2205,6 +2225,24 @@ bool z_direct_layout(int n3, ZDLayout &L)
     if (finish(512, 1, false, true)) return true;    // up to 112
     if (finish(512, 1, true, true)) return true;     // up to 144
     return finish(512, 1, true, false);
+}
+
+// Compiled forms of the direct pass B: groups, threads of one, streamed matrices, digits in TMEM, units per thread.
+struct ZInst {
+    int groups, nt, stream, ts, upt;
+    void (*kern)(const ZDArgs);
+};
+#define EXX_Z(G, NT, STREAM, TS, U) {G, NT, STREAM, TS, U, zpass_direct_kernel<NT, U, STREAM != 0, TS != 0, G>}
+const ZInst kZInst[] = {
+    EXX_Z(3, 256, 0, 1, 2), EXX_Z(3, 256, 0, 1, 3), EXX_Z(2, 256, 0, 1, 4), EXX_Z(1, 512, 0, 1, 3), EXX_Z(1, 512, 0, 1, 4),
+    EXX_Z(1, 512, 1, 1, 4), EXX_Z(1, 512, 1, 1, 5), EXX_Z(1, 512, 1, 0, 5), EXX_Z(1, 512, 1, 0, 6), EXX_Z(1, 512, 1, 0, 7),
+};
+#undef EXX_Z
+const ZInst *z_instance(const ZDLayout &L)
+{
+    for (const ZInst &i : kZInst)
+        if (i.groups == L.groups && i.nt == L.nt && i.stream == L.stream && i.ts == L.ts && i.upt >= L.upt) return &i;
+    return nullptr;
 }
 
 }  // namespace
@@ -2414,21 +2452,12 @@ int tc3_solve_batch(Plan &P, const int2 *pairs_d, int nfields, float *bufA, floa
         a.P1 = DL.P1;
         a.cpw = DL.cpw;
         a.err = static_cast<int *>(P.err_d.p);
-        void (*kern)(const SliceDArgs) = nullptr;
-        if (DL.groups == 3) {
-            if (DL.upt <= 2) kern = pair ? slice_direct_kernel<true, 256, 2, 3, true> : slice_direct_kernel<false, 256, 2, 3, true>;
-            else kern = pair ? slice_direct_kernel<true, 256, 3, 3, true> : slice_direct_kernel<false, 256, 3, 3, true>;
-        } else if (DL.groups == 2) {
-            if (DL.upt <= 3) kern = pair ? slice_direct_kernel<true, 256, 3, 2, true> : slice_direct_kernel<false, 256, 3, 2, true>;
-            else kern = pair ? slice_direct_kernel<true, 256, 4, 2, true> : slice_direct_kernel<false, 256, 4, 2, true>;
-        } else if (DL.nt == 256) {
-            if (DL.upt <= 3) kern = pair ? slice_direct_kernel<true, 256, 3, 1, true> : slice_direct_kernel<false, 256, 3, 1, true>;
-            else kern = pair ? slice_direct_kernel<true, 256, 4, 1, true> : slice_direct_kernel<false, 256, 4, 1, true>;
-        } else {
-            if (!DL.staged) kern = pair ? slice_direct_kernel<true, 512, 4, 1, false> : slice_direct_kernel<false, 512, 4, 1, false>;
-            else if (DL.upt <= 3) kern = pair ? slice_direct_kernel<true, 512, 3, 1, true> : slice_direct_kernel<false, 512, 3, 1, true>;
-            else kern = pair ? slice_direct_kernel<true, 512, 4, 1, true> : slice_direct_kernel<false, 512, 4, 1, true>;
+        const SliceInst *inst = slice_instance(DL);
+        if (!inst) {
+            set_error("BF16X7: no slice kernel for this layout");
+            return EXX_ERR_UNSUPPORTED;
         }
+        const auto kern = inst->kern[pair];
         size_t smem = DL.smem;
         const int threads = DL.nt * DL.groups;
         int per_sm = 1;
@@ -2533,20 +2562,12 @@ int tc3_solve_batch(Plan &P, const int2 *pairs_d, int nfields, float *bufA, floa
         a.tcols = ZD.tcols;
         a.tmem_cols = ZD.tmem_cols;
         a.err = static_cast<int *>(P.err_d.p);
-        void (*kern)(const ZDArgs) = nullptr;
-        if (ZD.stream && !ZD.ts) {
-            kern = ZD.upt <= 5   ? zpass_direct_kernel<512, 5, true, false, 1>
-                   : ZD.upt == 6 ? zpass_direct_kernel<512, 6, true, false, 1>
-                                 : zpass_direct_kernel<512, 7, true, false, 1>;
-        } else if (ZD.stream) {
-            kern = ZD.upt <= 4 ? zpass_direct_kernel<512, 4, true, true, 1> : zpass_direct_kernel<512, 5, true, true, 1>;
-        } else if (ZD.nt == 512) {
-            kern = ZD.upt <= 3 ? zpass_direct_kernel<512, 3, false, true, 1> : zpass_direct_kernel<512, 4, false, true, 1>;
-        } else if (ZD.groups == 2) {
-            kern = zpass_direct_kernel<256, 4, false, true, 2>;
-        } else {
-            kern = ZD.upt <= 2 ? zpass_direct_kernel<256, 2, false, true, 3> : zpass_direct_kernel<256, 3, false, true, 3>;
+        const ZInst *inst = z_instance(ZD);
+        if (!inst) {
+            set_error("BF16X7: no z kernel for this layout");
+            return EXX_ERR_UNSUPPORTED;
         }
+        const auto kern = inst->kern;
         const int threads = ZD.nt * ZD.groups;
         size_t smem = ZD.smem;
         int per_sm = 1;
@@ -2644,6 +2665,43 @@ void tc3_debug_layout(int n1, int n2, int n3, int share01, int *out)
     out[13] = Z.resident;
     out[14] = z_upt(n3);
     out[15] = int(kSmemLimit);
+}
+
+// Host only: the direct forms of a grid.  Pass A, then pass C (20 values each): fits; shared memory;
+// bytes of the two matrix images; offsets of the second image, the operands, the staging, the row
+// maxima, the barriers; bytes of one group's operand and of all its staged planes; groups, threads
+// of one, units per thread, those of the kernel; slices of a tile; operand digit planes of the two
+// GEMMs; TMEM columns of a group, allocated.  Then pass B (18): fits; shared
+// memory; bytes of an image; images in shared memory; offsets of the operands, scales, row maxima,
+// barriers; operand bytes of a group; groups, threads, units, those of the kernel; TMEM columns of a
+// group, allocated; streamed; digits in TMEM; contraction indices of an image.  Last the limit.
+void tc3_debug_direct(int n1, int n2, int n3, int share01, int *out)
+{
+    Plan P;
+    P.n[0] = n1;
+    P.n[1] = n2;
+    P.n[2] = n3;
+    P.t3_share01 = share01;
+    for (int pass = 0; pass < 2; ++pass) {
+        SliceDLayout L;
+        const bool ok = std::max(n1, n2) <= kRows && slice_direct_layout(P, pass == 0, L);
+        const SliceInst *inst = ok ? slice_instance(L) : nullptr;
+        const int Kp1 = pad16i(n1), Kp2 = pad16i(n2);
+        const int v[20] = {ok, int(L.smem), int(mat_image_bytes(Kp1, Kp1)), int(mat_image_bytes(Kp2, Kp2)), int(L.offB2), int(L.offA),
+                           int(L.offS), int(L.offRm), int(L.offBar), int(L.a_bytes),
+                           L.staged ? int(L.stg_plane) * (pass == 0 ? 2 : 1) : 0, L.groups, L.nt, L.upt, inst ? inst->upt : 0, L.G,
+                           int(L.a_piece1), int(L.a_piece2), L.tcols, L.tmem_cols};
+        if (ok) std::copy(v, v + 20, out);
+        else std::fill(out, out + 20, 0);
+        out += 20;
+    }
+    ZDLayout Z;
+    const bool ok = z_direct_layout(n3, Z);
+    const ZInst *inst = ok ? z_instance(Z) : nullptr;
+    const int v[18] = {ok, int(Z.smem), int(Z.img_bytes), Z.nbuf, int(Z.offA), int(Z.offCs), int(Z.offRm), int(Z.offBar), int(Z.a_bytes),
+                       Z.groups, Z.nt, Z.upt, inst ? inst->upt : 0, Z.tcols, Z.tmem_cols, Z.stream, Z.ts, Z.KC};
+    std::copy(v, v + 18, out);
+    out[18] = int(kSmemLimit);
 }
 
 // Host only: the digit image of C(n, k) (row-major nout x nk, HOST) in a WN x Kp block of rows

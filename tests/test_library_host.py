@@ -303,6 +303,81 @@ def test_three_pass_layouts_fit_shared_memory(lib):
     assert _tc3_layout(lib, 16, 16, 240, 1)["supported"] == 0
 
 
+SLICE_KEYS = ("fits smem img1 img2 offB2 offA offS offRm offBar a_bytes stg groups nt upt inst G piece1 piece2 "
+              "tcols tmem").split()
+Z_KEYS = "fits smem img nbuf offA offCs offRm offBar a_bytes groups nt upt inst tcols tmem stream ts KC".split()
+
+
+def _tc3_direct(lib, n1, n2, n3, share):
+    out = (ctypes.c_int * 59)()
+    lib.exx_debug_tc3_direct.argtypes = [ctypes.c_int] * 4 + [ctypes.c_void_p]
+    assert lib.exx_debug_tc3_direct(n1, n2, n3, share, out) == 0
+    v = list(out)
+    return dict(zip(SLICE_KEYS, v[:20])), dict(zip(SLICE_KEYS, v[20:40])), dict(zip(Z_KEYS, v[40:58])), v[58]
+
+
+def test_direct_slice_layouts(lib):
+    """Every pair of x and y axes up to 128 points: where the direct form fits, the images, each group's
+    operand (all cut units of both GEMMs, the transposed tile), the staging, row maxima and barriers
+    follow each other within the limit, the MMA's reach of 128 rows stays inside, the kernel that runs
+    has at least the layout's units, and those cover both operands.  The bench slab runs two or three
+    groups; 117-point slices stay resident, 110 x 100 with two matrices do not."""
+    r = lambda v, a: -(-v // a) * a
+    fits = 0
+    for n1 in range(2, 129):
+        for n2 in range(2, 129):
+            for share in ((0, 1) if n1 == n2 else (0,)):
+                A, C, _, limit = _tc3_direct(lib, n1, n2, 9, share)
+                for L, planes in ((A, 2), (C, 1)):
+                    if not L["fits"]:
+                        continue
+                    fits += 1
+                    k1, k2, G, g = r(n1, 16), r(n2, 16), L["G"], L["groups"]
+                    assert G == 128 // max(n1, n2) and G * max(n1, n2) <= 128
+                    first = L["img1"]
+                    if not share:
+                        assert L["offB2"] >= first
+                        first = L["offB2"] + L["img2"]
+                    assert L["offA"] >= first and L["offA"] % 1024 == 0
+                    assert L["piece1"] == r(G * n2, 8) * k1 * 2 and L["piece2"] == r(G * n1, 8) * k2 * 2
+                    assert L["a_bytes"] >= max(3 * L["piece1"], 3 * L["piece2"], G * n1 * r(n2, 4) * 4)
+                    ops = L["offA"] + g * L["a_bytes"]
+                    assert L["offS"] >= ops and L["offRm"] >= L["offS"] + g * L["stg"]
+                    assert not L["stg"] or L["stg"] >= planes * G * n2 * r(n1, 4) * 4
+                    reach = max(2 * L["piece1"] + 256 * k1, 2 * L["piece2"] + 256 * k2)
+                    assert L["offA"] + (g - 1) * L["a_bytes"] + reach <= L["smem"]
+                    assert L["offBar"] >= L["offRm"] + g * 1024 and L["smem"] >= L["offBar"] + 40 and L["smem"] <= limit
+                    assert L["inst"] >= L["upt"] >= 1
+                    for rows, k in ((G * n2, k1), (G * n1, k2)):
+                        assert L["upt"] * L["nt"] // 8 >= r(rows, 8) // 8 * (k // 8)
+                    assert L["tcols"] >= 2 * max(k1, k2) and g * L["tcols"] <= L["tmem"] <= 512
+    assert fits > 20000
+    assert _tc3_direct(lib, 48, 48, 48, 1)[0]["groups"] == 3
+    slab = _tc3_direct(lib, 72, 72, 144, 1)[0]
+    assert slab["groups"] >= 2 or slab["nt"] == 256   # groups of one CTA, or two CTAs
+    assert _tc3_direct(lib, 117, 117, 119, 1)[0]["fits"] == 1 and _tc3_direct(lib, 110, 100, 9, 0)[0]["fits"] == 0
+
+
+def test_direct_z_layouts(lib):
+    """Every z axis from 2 to 208 points has the direct form: images, operands, scales, row maxima and
+    barriers within the limit, kernel units that cover the axis (97 to 112 points once ran one too few),
+    accumulators and digits within TMEM; three groups up to 48 points, two up to 64, resident matrices
+    up to 112, digits in TMEM up to 144."""
+    for n in range(2, 209):
+        _, _, L, limit = _tc3_direct(lib, 8, 8, n, 1)
+        kp, g = -(-n // 16) * 16, L["groups"]
+        assert L["fits"] == 1 and g == (3 if n <= 48 else 2 if n <= 64 else 1)
+        assert L["stream"] == (n > 112) and L["ts"] == (n <= 144)
+        assert L["KC"] == (16 if L["stream"] else kp) and L["nbuf"] >= 2
+        assert L["img"] >= kp * L["KC"] * 2 * 4 + kp * 4
+        assert L["offA"] >= L["nbuf"] * L["img"] and L["offCs"] >= L["offA"] + g * L["a_bytes"]
+        assert L["a_bytes"] == (0 if L["ts"] else 3 * 128 * kp * 2)
+        assert L["offRm"] >= L["offCs"] + 8 * kp and L["offBar"] >= L["offRm"] + g * 1024
+        assert L["offBar"] + 35 * 8 + 8 <= L["smem"] <= limit
+        assert L["inst"] >= L["upt"] and L["upt"] * 8 * (L["nt"] // 128) >= n
+        assert L["tcols"] == 2 * kp + (3 * kp // 2 if L["ts"] else 0) and g * L["tcols"] <= L["tmem"] <= 512
+
+
 def test_matrix_digit_images_reproduce_the_matrix(lib):
     """The four base-512 digits of a matrix row (row scaled by the largest entry of the whole row
     into [128, 256)) reproduce every entry to 2^-35 of the row maximum (the last digit rounds
