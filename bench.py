@@ -344,7 +344,7 @@ def run_ours(args):
         dom = max(ktimes, key=lambda k: ktimes[k][0])
         dom_ms, dom_n = ktimes[dom]
         rec["kernel_times_ms"] = {k: round(v[0] / K, 4) for k, v in ktimes.items()}
-        rec["roofline"] = roofline(s, prec_name, dom, dom_ms, dom_n, K, peaks)
+        rec["roofline"] = roofline(s, prec_name, dom, dom_ms, dom_n, K, peaks, tuning or {})
         rec["roofline_apply"] = roofline_apply(s, prec_name, apply_total_ms / K, peaks)
         rec["tensor_roofline"] = tensor_roofline(s, prec_name, apply_total_ms / K, peaks)
     rec["ordered_pair_solves_per_s"] = value * ordered / unique
@@ -526,7 +526,7 @@ def run_batch48(args):
         achieved = bytes_kind[dom] / (ms / 1e3) / 1e9
         pk = peaks.get("hbm_gbs", 6800.0)
         rec["roofline"] = {"bound": "hbm", "achieved": achieved, "peak": pk, "unit": "GB/s", "frac": achieved / pk,
-                           "traffic": None, "kernel": kernel_name(prec_name, dom), "launches": n,
+                           "traffic": None, "kernel": kernel_name(prec_name, dom, {}), "launches": n,
                            "avg_launch_ms": ms / n, "algorithmic_bytes_per_launch": bytes_kind[dom] / n,
                            "timing": "one extra step with CUDA events around each launch (launches issued "
                                      "one by one, not through the graph)",
@@ -697,16 +697,21 @@ def pass_bytes(kind):
 
 
 # kernel behind each timing class, per mode family
-def kernel_name(prec, kind):
+def kernel_name(prec, kind, tuning=None):
     if prec == "fp64":
         return "fp64_pass_kernel" if kind.startswith("pass") else kind
     if prec == "bf16x7":
-        return {"pass1": "slice_pass_kernel (pass A)", "pass3": "zpass_kernel (pass B)",
-                "pass5": "slice_pass_kernel (pass C)", "accum": "tc_accum_kernel"}.get(kind, kind)
+        # the direct forms under a plan's own settings, the older ones where a setting asks for them
+        # (or, for the slices, both matrices do not stay in shared memory: none of the workloads here)
+        t = {"staging": 0, "z_block": 16} if tuning is None else tuning
+        sl = "slice_direct_kernel" if t.get("staging", -1) < 0 and t.get("pipeline", -1) < 0 else "slice_pass_kernel"
+        z = "zpass_kernel" if t.get("z_block", 0) else "zpass_direct_kernel"
+        return {"pass1": f"{sl} (pass A)", "pass3": f"{z} (pass B)", "pass5": f"{sl} (pass C)",
+                "accum": "tc_accum_kernel"}.get(kind, kind)
     return {"accum": "tc_accum_kernel"}.get(kind, f"tc_pass_kernel ({kind})")
 
 
-def roofline(s, prec, kind, ms, nlaunch, K, peaks):
+def roofline(s, prec, kind, ms, nlaunch, K, peaks, tuning=None):
     """Achieved throughput of the dominant kernel class from its live CUDA-event time:
     algorithmic bytes per launch (pass_bytes x N x pair fields per launch, + f(Lambda)) over
     the average launch time, against the measured HBM copy bandwidth."""
@@ -714,7 +719,7 @@ def roofline(s, prec, kind, ms, nlaunch, K, peaks):
     unique = s.unique_pairs()
     fields_per_launch = unique * K / max(1, nlaunch)
     avg_s = ms / max(1, nlaunch) / 1e3
-    name = kernel_name(prec, kind)
+    name = kernel_name(prec, kind, tuning)
     out = {"kernel": name, "launches": nlaunch, "avg_launch_ms": ms / max(1, nlaunch),
            "fields_per_launch": fields_per_launch}
     if prec == "fp64" and kind.startswith("pass"):
