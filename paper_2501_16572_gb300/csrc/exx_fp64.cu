@@ -10,7 +10,7 @@
 // pencil along the contracted axis) and produces up to 20 outputs at a time from the slice of
 // the matrix staged in shared memory (every thread of a warp reads the same entry, a
 // broadcast); the slice width is the one that pads the axis least.
-// 28 x 30 x 33 points, 24 of 32 orbitals: 6.05 ms without the reflection and with slices of 16.
+// 28 x 30 x 33 points, 24 of 32 orbitals: 6.05 ms without the reflection and with slices of 16, 2.97 with both.
 #include "exx_internal.h"
 
 #include <algorithm>

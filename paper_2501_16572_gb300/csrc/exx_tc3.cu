@@ -32,7 +32,7 @@
 //  * the epilogue adds the two accumulators and applies the row and column scales.
 // The result carries ~27 bits of the data rows and ~36 bits of the matrices; the middle of
 // pass B (the fully modal values, the only place where a rounding is common to all terms
-// of the exchange energy) is kept as an FP32 hi + lo pair.
+// of the exchange energy) is kept as an FP32 hi + bf16 lo pair.
 #include "exx_internal.h"
 #include "tc_ptx.cuh"
 
@@ -171,17 +171,6 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_addr(bar)) : "memory");
 }
 
-// Untiled bulk copy global -> shared (16-byte aligned addresses, size a multiple of 16),
-// completing as transaction bytes on `bar`.
-__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
-{
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            tc::smem_addr(dst)),
-        "l"(src), "r"(bytes), "r"(tc::smem_addr(bar))
-        : "memory");
-}
-
 // Four consecutive TMEM columns of this warp's lanes, both accumulators, one wait.
 __device__ __forceinline__ void tmem_pair4(uint32_t lead, uint32_t rest, float (&a)[4], float (&b)[4])
 {
@@ -312,11 +301,11 @@ __global__ void __launch_bounds__(kRows * TPR + 64, 2) slice_pass_kernel(const _
                 tc::mbar_arrive_expect_tx(stg_full, (PAIR ? 2u : 1u) * bytes);
                 if (PAIR) {
                     const int2 mn = a.pairs[p];
-                    bulk_load(stg, a.psi + size_t(a.occ_off + mn.x) * a.N + size_t(z0) * R, bytes, stg_full);
-                    bulk_load(reinterpret_cast<uint8_t *>(stg) + a.stg_plane,
+                    tc::bulk_load(stg, a.psi + size_t(a.occ_off + mn.x) * a.N + size_t(z0) * R, bytes, stg_full);
+                    tc::bulk_load(reinterpret_cast<uint8_t *>(stg) + a.stg_plane,
                               a.psi + size_t(mn.y) * a.N + size_t(z0) * R, bytes, stg_full);
                 } else {
-                    bulk_load(stg, a.in + size_t(p) * a.N + size_t(z0) * R, bytes, stg_full);
+                    tc::bulk_load(stg, a.in + size_t(p) * a.N + size_t(z0) * R, bytes, stg_full);
                 }
             }
             // no copy may still target shared memory at exit: the last fill has landed
@@ -340,7 +329,7 @@ __global__ void __launch_bounds__(kRows * TPR + 64, 2) slice_pass_kernel(const _
                             break;
                         }
                         tc::mbar_arrive_expect_tx(bfull + slot, cb);
-                        bulk_load(smem + size_t(slot) * a.buf_bytes, img + size_t(kc) * cb, cb, bfull + slot);
+                        tc::bulk_load(smem + size_t(slot) * a.buf_bytes, img + size_t(kc) * cb, cb, bfull + slot);
                     }
                 }
             for (int slot = 0; slot < 2; ++slot) {   // every issued copy has landed before exit
@@ -1190,7 +1179,7 @@ __global__ void __launch_bounds__(NT * GROUPS, 512 / (NT * GROUPS) > 0 ? 512 / (
 // ---------------------------------------------------------------------------------------
 // Pass B.  A tile is 128 consecutive rows r = a + n1 b of one field (pencils along z).
 //   forward GEMM: rows r, K = z, outputs c in NB blocks of WN columns
-//   middle: (D * f(Lambda)) as FP32 hi + lo, re-sliced in place of its own digits
+//   middle: (D * f(Lambda)) as FP32 hi + bf16 lo, re-sliced in place of its own digits
 //   inverse GEMM: rows r, K = c, outputs z in NB blocks
 // The matrix images stream through nbuf shared-memory buffers (bulk copies by the producer
 // warp) unless all 2 NB blocks are resident.
@@ -1286,7 +1275,7 @@ __global__ void __launch_bounds__(kRows * TPR + 64, (UPT <= 4 ? 2 : 1)) zpass_ke
             if (a.resident) {
                 for (int j = 0; j < 2 * NB; ++j) {
                     tc::mbar_arrive_expect_tx(bfull + j, a.blk_bytes);
-                    bulk_load(sB + size_t(j) * a.blk_bytes, block_src(j), a.blk_bytes, bfull + j);
+                    tc::bulk_load(sB + size_t(j) * a.blk_bytes, block_src(j), a.blk_bytes, bfull + j);
                 }
                 for (int j = 0; j < 2 * NB; ++j)   // no copy may still target shared memory at exit
                     if (!tc::mbar_wait_timed(bfull + j, 0, kWaitNs)) atomicExch(sflag, 1);
@@ -1303,7 +1292,7 @@ __global__ void __launch_bounds__(kRows * TPR + 64, (UPT <= 4 ? 2 : 1)) zpass_ke
                             break;
                         }
                         tc::mbar_arrive_expect_tx(bfull + slot, a.blk_bytes);
-                        bulk_load(sB + size_t(slot) * a.blk_bytes, block_src(j), a.blk_bytes, bfull + slot);
+                        tc::bulk_load(sB + size_t(slot) * a.blk_bytes, block_src(j), a.blk_bytes, bfull + slot);
                     }
                 }
                 // every issued copy has landed before exit: the last fill of each slot
@@ -1639,7 +1628,7 @@ __global__ void __launch_bounds__(NT * GROUPS, NT * GROUPS <= 256 ? 2 : 1) zpass
     auto load_chunk = [&](int g, uint32_t el) {   // chunk ld_count into the next buffer, which is free
         if (el) {
             tc::mbar_arrive_expect_tx(bfull + ld_slot, a.img_bytes);
-            bulk_load(smem + uint32_t(ld_slot) * a.img_bytes, (g ? a.imgI : a.imgF) + size_t(ld_count) * a.img_bytes, a.img_bytes,
+            tc::bulk_load(smem + uint32_t(ld_slot) * a.img_bytes, (g ? a.imgI : a.imgF) + size_t(ld_count) * a.img_bytes, a.img_bytes,
                       bfull + ld_slot);
         }
         fills = max(fills, uint32_t(ld_slot) + 1u);

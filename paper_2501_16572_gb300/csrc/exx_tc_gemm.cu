@@ -210,15 +210,6 @@ __device__ __forceinline__ double chunk_value(float h, float l, int ex)
     return __hiloint2double(int((uint32_t(M >> 32) + (uint32_t(ed - 1) << 20)) | sign), int(uint32_t(M)));
 }
 
-__device__ __forceinline__ void gemm_bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
-{
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            tc::smem_addr(dst)),
-        "l"(src), "r"(bytes), "r"(tc::smem_addr(bar))
-        : "memory");
-}
-
 // The CTAs walk the items (split z, row tile, column tile), column tiles fastest so that concurrent
 // CTAs read the same A blocks from L2.  13 digit products per k in 4 MMAs of up to 192 columns
 // (neighbouring B digits feed neighbouring levels): about 284 cycles of the tensor pipe per 16 k of a
@@ -298,8 +289,8 @@ __global__ void __launch_bounds__(128 * PARTS + 64, 3 - SETS) tc_gemm_kernel(con
                     }
                     uint8_t *s = smem + size_t(st) * a.stage_bytes;
                     tc::mbar_arrive_expect_tx(full + st, a_bytes + b_bytes);
-                    gemm_bulk_load(s, a.digA + (size_t(t.mi) * a.nkb + kb) * a_bytes, a_bytes, full + st);
-                    gemm_bulk_load(s + a_bytes, a.digB + (size_t(t.ni) * a.nkb + kb) * b_bytes, b_bytes, full + st);
+                    tc::bulk_load(s, a.digA + (size_t(t.mi) * a.nkb + kb) * a_bytes, a_bytes, full + st);
+                    tc::bulk_load(s + a_bytes, a.digB + (size_t(t.ni) * a.nkb + kb) * b_bytes, b_bytes, full + st);
                     filled = max(filled, st + 1);
                     if (++st == a.stages) {
                         st = 0;
