@@ -68,6 +68,11 @@ int exx_debug_tc3_layout(int n1, int n2, int n3, int share01, int *out);
  * pass B, in the order that tc3_debug_direct states, and the shared-memory limit. */
 int exx_debug_tc3_direct(int n1, int n2, int n3, int share01, int *out);
 
+/* The forms of the five-pass kernels of a split mode (not BF16X7) for blocks of Np points (a multiple of
+ * 16), host-side: out (HOST int[36]) = for pass 1, 2, 3 in one kernel, one half of pass 3, 4 and 5 each:
+ * fits, staging buffers, accumulator sets, TMEM columns they take, columns allocated, shared memory. */
+int exx_debug_tc_passes(int prec, int Np, int *out);
+
 /* The base-512 digit image of the 1D matrices, host-side: C (HOST, row-major nout x nk, row n =
  * output n, column k = contraction index k) cut for a WN x Kp block of rows n0.. and indices
  * k0.. (a K-chunk when k0 > 0 or Kp < nk), decoded from the tensor-core layout back to values:

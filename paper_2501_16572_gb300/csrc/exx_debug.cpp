@@ -20,6 +20,13 @@ int exx_debug_tc3_direct(int n1, int n2, int n3, int share01, int *out)
     return EXX_OK;
 }
 
+int exx_debug_tc_passes(int prec, int Np, int *out)
+{
+    if (prec <= EXX_PREC_FP64 || prec >= EXX_PREC_BF16X7 || Np < 16 || Np > 256 || Np % 16 || !out) return EXX_ERR_INVALID_ARG;
+    exx::tc_debug_passes(prec, Np, out);
+    return EXX_OK;
+}
+
 int exx_debug_matrix_digits(int nout, int nk, const double *C, int WN, int Kp, int n0, int k0, float *digits,
                             float *scales)
 {

@@ -233,6 +233,7 @@ void tc3_debug_direct(int n1, int n2, int n3, int share01, int *out);
 void tc3_debug_matrix_digits(int nout, int nk, const double *C, int WN, int Kp, int n0, int k0, float *digits,
                              float *scales);
 int tc_unit_gemm(int tf32, int n, int k, const float *A, const float *B, float *D, int *err);
+void tc_debug_passes(int prec, int Np, int *out);
 int tc_wait_timeout_probe(int *status_h);
 int tc_wait_warp_probe(unsigned *went_on_h);
 

@@ -65,7 +65,8 @@ __host__ __device__ inline PrecInfo prec_info(int prec)
 }
 
 inline int pad16(int n) { return (n + 15) & ~15; }
-inline int pow2_cols(int c) { return c <= 32 ? 32 : c <= 64 ? 64 : c <= 128 ? 128 : c <= 256 ? 256 : 512; }
+// TMEM columns to allocate for c; 1024, more than there are, past 512
+inline int pow2_cols(int c) { return c <= 32 ? 32 : c <= 64 ? 64 : c <= 128 ? 128 : c <= 256 ? 256 : c <= 512 ? 512 : 1024; }
 
 // bytes of one operand image: SB pieces of Np x Np, then (fixed mode) Np column scales
 inline size_t image_bytes(int prec, int Np)
@@ -1378,15 +1379,25 @@ int launch_tc_pass_nb(Plan &P, int kind, int prec, const TcPassArgs &a, cudaStre
 
 // Largest configuration that fits: pipelined with two staging buffers, pipelined with one,
 // or (long axes) one A buffer and one TMEM set.
+struct PassForm {
+    int nbuf, nsets;
+};
+PassForm pass_form(int prec, int Np, bool dbl, int load, int store)
+{
+    const size_t lim = 232448;
+    const bool tm2 = tmem_cols(prec, Np, 2) <= 512;
+    if (load != LOAD_PAIR && tm2 && pass_smem(prec, Np, dbl, load, 2, 2, store) <= lim) return {2, 2};
+    if (tm2 && pass_smem(prec, Np, dbl, load, 1, 2, store) <= lim) return {1, 2};
+    return {1, 1};
+}
+
 template <int MODE, int S, int SB, bool HL, int LOAD, int STORE, bool DOUBLE>
 int launch_tc_pass(Plan &P, int kind, int prec, const TcPassArgs &a, cudaStream_t s)
 {
-    const size_t lim = 232448;
-    const bool tm2 = tmem_cols(prec, a.Np, 2) <= 512;
-    if (LOAD != LOAD_PAIR && tm2 && pass_smem(prec, a.Np, DOUBLE, LOAD, 2, 2, STORE) <= lim)
-        return launch_tc_pass_nb<MODE, S, SB, HL, LOAD, STORE, DOUBLE, 2, 2>(P, kind, prec, a, s);
-    if (tm2 && pass_smem(prec, a.Np, DOUBLE, LOAD, 1, 2, STORE) <= lim)
-        return launch_tc_pass_nb<MODE, S, SB, HL, LOAD, STORE, DOUBLE, 1, 2>(P, kind, prec, a, s);
+    const PassForm form = pass_form(prec, a.Np, DOUBLE, LOAD, STORE);
+    if constexpr (LOAD != LOAD_PAIR)
+        if (form.nbuf == 2) return launch_tc_pass_nb<MODE, S, SB, HL, LOAD, STORE, DOUBLE, 2, 2>(P, kind, prec, a, s);
+    if (form.nsets == 2) return launch_tc_pass_nb<MODE, S, SB, HL, LOAD, STORE, DOUBLE, 1, 2>(P, kind, prec, a, s);
     return launch_tc_pass_nb<MODE, S, SB, HL, LOAD, STORE, DOUBLE, 1, 1>(P, kind, prec, a, s);
 }
 
@@ -1558,6 +1569,26 @@ static bool axis_fits(int prec, int d, int Np, bool split)
     if (d == 1) need = pass_smem(prec, Np, !split, LOAD_KFAST, 1, 1, STORE_NFAST);
     if (d == 2) need = std::max(pass_smem(prec, Np, false, LOAD_PAIR), pass_smem(prec, Np, false, LOAD_KSLOW));
     return need <= 232448 && tmem_cols(prec, Np) <= 512;
+}
+
+// Host only: the five passes of a split mode with blocks of Np points: which of pass 1 (pair), 2, 3 (both
+// GEMMs, or either alone) and 4, 5 a block fits; staging buffers, TMEM sets, TMEM columns that the sets
+// take and that are allocated, shared memory.
+void tc_debug_passes(int prec, int Np, int *out)
+{
+    const struct {
+        int load, store;
+        bool dbl;
+    } pass[6] = {{LOAD_PAIR, STORE_NSLOW, false}, {LOAD_KFAST, STORE_NSLOW, false}, {LOAD_KFAST, STORE_NFAST, true},
+                 {LOAD_KFAST, STORE_NFAST, false}, {LOAD_KSLOW, STORE_NFAST, false}, {LOAD_KSLOW, STORE_NSLOW, false}};
+    for (const auto &p : pass) {
+        const PassForm f = pass_form(prec, Np, p.dbl, p.load, p.store);
+        const size_t smem = pass_smem(prec, Np, p.dbl, p.load, f.nbuf, f.nsets, p.store);
+        const int cols = f.nsets * prec_info(prec).nacc * Np;
+        const int v[6] = {smem <= 232448 && tmem_cols(prec, Np, f.nsets) <= 512, f.nbuf, f.nsets, cols,
+                          tmem_cols(prec, Np, f.nsets), int(smem)};
+        out = std::copy(v, v + 6, out);
+    }
 }
 
 int tc_upload(Plan &P, int prec)

@@ -378,6 +378,23 @@ def test_direct_z_layouts(lib):
         assert L["tcols"] == 2 * kp + (3 * kp // 2 if L["ts"] else 0) and g * L["tcols"] <= L["tmem"] <= 512
 
 
+@pytest.mark.parametrize("mode", ["BF16X3", "BF16X6", "TF32X3", "BF16X10"])
+def test_five_pass_forms_stay_within_tmem(lib, mode):
+    """A pass that runs never takes more tensor memory than it allocates, or than there is: two
+    accumulator sets of a 72-point axis of BF16X6 are 640 columns."""
+    import paper_2501_16572_gb300 as exx
+    lib.exx_debug_tc_passes.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_void_p]
+    some = 0
+    for Np in range(16, 257, 16):
+        out = (ctypes.c_int * 36)()
+        assert lib.exx_debug_tc_passes(getattr(exx, "EXX_PREC_" + mode), Np, out) == 0
+        for fits, nbuf, nsets, cols, alloc, smem in np.array(out).reshape(6, 6):
+            if fits:
+                some += 1
+                assert cols <= alloc <= 512 and smem <= 232448 and nbuf in (1, 2) and nsets in (1, 2), (Np, cols, alloc)
+    assert some >= 12
+
+
 def test_matrix_digit_images_reproduce_the_matrix(lib):
     """The four base-512 digits of a matrix row (row scaled by the largest entry of the whole row
     into [128, 256)) reproduce every entry to 2^-35 of the row maximum (the last digit rounds
