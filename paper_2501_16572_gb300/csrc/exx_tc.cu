@@ -1139,7 +1139,9 @@ __device__ __forceinline__ int diag_idx(int i, int j, int nI) { return i * nI - 
 // row's fields are loaded while this row's are added.  Bound by the loads of V and of the
 // accumulators (2.25 B of those per 4 B of V at 16 x 16).  Against one column per instruction with
 // the sources re-read for every field, and 8-wide default blocks: 48^3 x 128 3.52 -> 1.69 ms,
-// 72 x 72 x 144 (75 of 96) 9.38 -> 5.84 ms.
+// 72 x 72 x 144 (75 of 96) 9.38 -> 5.84 ms.  Fields as hi + lo (BF16X10) load both planes a row ahead, with
+// registers for it (three CTAs of 16 columns): 48^3 x 128 4.24 -> 2.28 ms against lo read where it is used,
+// 3.48 for one column per instruction.
 constexpr int kAccThreads = 128;
 struct AccArgs {
     long N;
@@ -1184,10 +1186,14 @@ __device__ __forceinline__ void accum_block(const AccArgs &a, const Block &b, lo
         a.acc_hi[size_t(t) * N + r] = hs;
     };
     const float *row = a.V + size_t(b.field0) * N + r;   // field (i, 0), also where a diagonal block has none
-    float2 v[NP];
+    float2 v[NP], vl[HL ? NP : 1];
 #pragma unroll
-    for (int jp = 0; jp < NP; ++jp)
+    for (int jp = 0; jp < NP; ++jp) {
         v[jp] = make_float2(ld_here(row + 2 * jp * N, 2 * jp < nJ), ld_here(row + (2 * jp + 1) * N, 2 * jp + 1 < nJ));
+        if (HL)
+            vl[jp] = make_float2(ld_here(row + a.lo_off + 2 * jp * N, 2 * jp < nJ),
+                                 ld_here(row + a.lo_off + (2 * jp + 1) * N, 2 * jp + 1 < nJ));
+    }
 #pragma unroll 1
     for (int i = 0; i < nI; ++i) {
         const size_t oi = size_t(b.I0 + i) * N + r;
@@ -1200,26 +1206,31 @@ __device__ __forceinline__ void accum_block(const AccArgs &a, const Block &b, lo
         const bool more = i + 1 < nI;
         // this row's fields have arrived before the next row's are asked for: loads share a few
         // scoreboards, and a value waited for after newer loads on the same one waits for those
-        float2 w[NP];
+        float2 w[NP], wlo[HL ? NP : 1];
 #pragma unroll
         for (int jp = 0; jp < NP; ++jp) {
             asm volatile("" : "+f"(v[jp].x), "+f"(v[jp].y));
             w[jp] = v[jp];
+            if (HL) {
+                asm volatile("" : "+f"(vl[jp].x), "+f"(vl[jp].y));
+                wlo[jp] = vl[jp];
+            }
         }
 #pragma unroll
         for (int jp = 0; jp < NP; ++jp) {   // a diagonal block holds j >= i only, the others count as zero
-            v[jp].x = ld_here(next + 2 * jp * N, more && 2 * jp < nJ && (!kDiag || 2 * jp > i));
-            v[jp].y = ld_here(next + (2 * jp + 1) * N, more && 2 * jp + 1 < nJ && (!kDiag || 2 * jp + 1 > i));
+            const bool ok0 = more && 2 * jp < nJ && (!kDiag || 2 * jp > i);
+            const bool ok1 = more && 2 * jp + 1 < nJ && (!kDiag || 2 * jp + 1 > i);
+            v[jp].x = ld_here(next + 2 * jp * N, ok0);
+            v[jp].y = ld_here(next + (2 * jp + 1) * N, ok1);
+            if (HL) {
+                vl[jp].x = ld_here(next + a.lo_off + 2 * jp * N, ok0);
+                vl[jp].y = ld_here(next + a.lo_off + (2 * jp + 1) * N, ok1);
+            }
         }
 #pragma unroll
         for (int jp = 0; jp < NP; ++jp) {
-            float2 wl = make_float2(0.f, 0.f);
-            const bool ok0 = 2 * jp < nJ, ok1 = 2 * jp + 1 < nJ;
-            if (HL) {
-                wl.x = ok0 && (!kDiag || 2 * jp >= i) ? row[a.lo_off + 2 * jp * N] : 0.f;
-                wl.y = ok1 && (!kDiag || 2 * jp + 1 >= i) ? row[a.lo_off + (2 * jp + 1) * N] : 0.f;
-            }
-            if (!ok0 || (kDiag && 2 * jp + 1 < i)) continue;   // uniform
+            const float2 wl = HL ? wlo[jp] : make_float2(0.f, 0.f);
+            if (2 * jp >= nJ || (kDiag && 2 * jp + 1 < i)) continue;   // uniform
             const float2 nw = __fmul2_rn(w[jp], neg);
             sub_product2<HL>(sj[jp], cj[jp], gi, gi_l, w[jp], nw, wl);
             if (kBoth) {
@@ -1260,7 +1271,7 @@ __device__ __forceinline__ void accum_block(const AccArgs &a, const Block &b, lo
 }
 
 template <bool HL, int NP>
-__global__ void __launch_bounds__(kAccThreads, NP > 4 ? 4 : 6) tc_accum_kernel(const __grid_constant__ AccArgs a)
+__global__ void __launch_bounds__(kAccThreads, NP > 4 ? (HL ? 3 : 4) : (HL ? 5 : 6)) tc_accum_kernel(const __grid_constant__ AccArgs a)
 {
     const Block b = a.blocks[blockIdx.y];
     const long r = long(blockIdx.x) * kAccThreads + threadIdx.x;
