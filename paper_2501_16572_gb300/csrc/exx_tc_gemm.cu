@@ -24,7 +24,7 @@
 // finished chunks.  Cutting inside the GEMM repeated the integer work of every A row for each
 // column tile and left the tensor cores idle meanwhile: both products of ace_apply at
 // n = nphi = 512 on 72 x 72 x 144 points took 65.7 ms, 10.1 ms now (cuts 3.3 ms near the HBM
-// rate, the GEMMs 6.8 ms, of which the tensor pipe's own about 4.7).
+// rate, the GEMMs 6.8 ms, of which the tensor pipe's own 3.7).
 #include "exx_internal.h"
 #include "tc_ptx.cuh"
 
