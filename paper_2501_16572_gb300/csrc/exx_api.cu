@@ -542,6 +542,7 @@ static void tune_set(Plan &P, const TuneVal &v)
     P.t3_znbuf = v.znbuf;
     P.t3_stage = v.stage;
     P.t3_pipe = v.pipe;
+    P.pairs_cap = 0;
     std::fill(P.sched_key, P.sched_key + 4, -1);
     bump_epoch(P);
 }
