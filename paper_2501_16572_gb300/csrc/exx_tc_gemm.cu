@@ -20,11 +20,11 @@
 // Two kernels.  gemm_cut_kernel cuts every operand element once into digit planes in device
 // memory, already in the operand layout of the MMA, and records the row scales;
 // tc_gemm_kernel then only streams 8-byte-per-element blocks of them through shared memory
-// (bulk copies, a producer warp) into the MMAs (one issuing warp) while 8 or 16 warps combine
+// (bulk copies, a producer warp) into the MMAs (one issuing warp) while 8 or 12 warps combine
 // finished chunks.  Cutting inside the GEMM repeated the integer work of every A row for each
 // column tile and left the tensor cores idle meanwhile: both products of ace_apply at
-// n = nphi = 512 on 72 x 72 x 144 points took 65.7 ms, 10.1 ms now (cuts 3.3 ms near the HBM
-// rate, the GEMMs 6.8 ms, of which the tensor pipe's own 3.7).
+// n = nphi = 512 on 72 x 72 x 144 points took 65.7 ms, 9.7 ms now (cuts 3.3 ms near the HBM
+// rate, the GEMMs 6.4 ms, of which the tensor pipe's own 4.2).
 #include "exx_internal.h"
 #include "tc_ptx.cuh"
 
@@ -44,7 +44,7 @@ constexpr int kBlks = 10;            // blocks per exact chunk
 constexpr int kChunk = kBlk * kBlks; // 320: 4 levels x 320 x 3 * 2^14 < 2^24
 constexpr uint64_t kGemmWaitNs = 1000000000ull;
 constexpr uint32_t kSbo = kBlk * 16;           // bytes between 8-row groups of a digit plane
-constexpr int kParts = 4;            // drain warps per 32 TMEM lanes (2 for tiles of up to 32 columns)
+constexpr int kParts = 3;            // drain warps per 32 TMEM lanes (2 for tiles of up to 32 columns)
 constexpr int kNarrow = 32;          // tiles of up to 32 columns: one set of levels, two CTAs per SM
 constexpr int kCutWarps = kBlks;     // gemm_cut_kernel: a warp per k block of a chunk
 
@@ -212,21 +212,23 @@ __device__ __forceinline__ double chunk_value(float h, float l, int ex)
 
 // The CTAs walk the items (split z, row tile, column tile), column tiles fastest so that concurrent
 // CTAs read the same A blocks from L2.  13 digit products per k in 4 MMAs of up to 192 columns
-// (neighbouring B digits feed neighbouring levels): about 284 cycles of the tensor pipe per 16 k of a
+// (neighbouring B digits feed neighbouring levels): 320 cycles of the tensor pipe per 16 k of a
 // 128 x 48 tile, against 22.5 KB of operands.
 //   * SETS = 2 (tiles of 48 columns), one CTA per SM: two sets of level accumulators, so that the
-//     drain warps combine a finished chunk under the next chunk's MMAs.  The combination is
-//     integer work for the most part, about 7 thousand cycles per 128 x 48 chunk where the MMAs
-//     take 5.7 thousand: with one set of 96 columns it was not overlapped, and both products of
-//     ace_apply at n = nphi = 512 on 72 x 72 x 144 points took 15.7 ms, now 10.1.
+//     drain warps combine a finished chunk under the next chunk's MMAs: with one set of 96 columns it
+//     was not overlapped, and both products of ace_apply at n = nphi = 512 on 72 x 72 x 144 points took
+//     15.7 ms, now 9.7.  TMEM loads take about as long for 4 columns as for 8: in groups of 4 the
+//     combination took longer than the MMAs (10.1 ms for that call; 160 columns on 80 x 80 x 60 at
+//     n = 512 3.49 ms, 2.61 in groups of 8 that skip the columns past the last).
 //   * SETS = 1 (tiles of up to 32 columns), two CTAs per SM: bound by the operand blocks' way from L2
 //     and by the chain load - MMA - drain - store of one item.
-// PARTS: drain warps per 32 TMEM lanes (four: 10.1 ms for that call, three 10.2, two 11.1).
+// PARTS: drain warps per 32 TMEM lanes (two cost 160 columns 5% more than three, four nothing less).
 template <int PARTS, int SETS>
 __global__ void __launch_bounds__(128 * PARTS + 64, 3 - SETS) tc_gemm_kernel(const __grid_constant__ GemmArgs a)
 {
     constexpr int kDrainWarps = 4 * PARTS;
-    constexpr int NH = ((SETS == 1 ? kNarrow : kTN) / 4 + PARTS - 1) / PARTS * 4;   // most columns of a drain warp
+    constexpr int GW = 8;                                                       // columns of a group
+    constexpr int NH = ((SETS == 1 ? kNarrow : kTN) / GW + PARTS - 1) / PARTS * GW;   // most columns of a drain warp
     extern __shared__ __align__(1024) uint8_t smem[];
     int *eb = reinterpret_cast<int *>(smem + a.offTab);            // column exponents of a chunk, two sets
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + a.offBar);
@@ -368,11 +370,11 @@ __global__ void __launch_bounds__(128 * PARTS + 64, 3 - SETS) tc_gemm_kernel(con
             }
         }
     } else {
-        // ---- drain warps: TMEM lane `row`, column groups of 4 of this warp's part ----
+        // ---- drain warps: TMEM lane `row`, column groups of this warp's part ----
         const int quarter = warp & 3;
         const int row = quarter * 32 + lane;
         const uint32_t lane_q = uint32_t(quarter * 32) << 16;
-        const int part = (Nt / 4 + PARTS - 1) / PARTS * 4, cbase = (warp >> 2) * part, ncol = min(part, Nt - cbase);
+        const int part = (Nt / GW + PARTS - 1) / PARTS * GW, cbase = (warp >> 2) * part, ncol = min(part, Nt - cbase);
         constexpr int NT = 128 * PARTS;
         int seq = 0;   // chunks drained so far
         bool stop = false;
@@ -406,19 +408,19 @@ __global__ void __launch_bounds__(128 * PARTS + 64, 3 - SETS) tc_gemm_kernel(con
                 tc::tc_fence_after();
                 const uint32_t d0 = tmem + lane_q + uint32_t(set * kLev * Nt);
 #pragma unroll
-                for (int cg = 0; cg < NH / 4; ++cg) {
-                    if (cg * 4 >= ncol || i - lane >= a.m) break;   // uniform
-                    const int cc = cbase + cg * 4;
-                    uint32_t r[kLev][4];
+                for (int cg = 0; cg < NH / GW; ++cg) {
+                    const int cc = cbase + cg * GW;
+                    if (cg * GW >= ncol || j0 + cc >= a.n || i - lane >= a.m) break;   // uniform
+                    uint32_t r[kLev][GW];
 #pragma unroll
-                    for (int l = 0; l < kLev; ++l) tc::tmem_ld4_issue(d0 + uint32_t(l * Nt + cc), r[l]);
+                    for (int l = 0; l < kLev; ++l) tc::tmem_ld8_issue(d0 + uint32_t(l * Nt + cc), r[l]);
                     tc::tmem_wait_ld();
 #pragma unroll
                     for (int l = 0; l < kLev; ++l)
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) tc::order_after_wait(r[l][e]);
+                        for (int e = 0; e < GW; ++e) tc::order_after_wait(r[l][e]);
 #pragma unroll
-                    for (int e = 0; e < 4; e += 2) {
+                    for (int e = 0; e < GW; e += 2) {
                         // levels combined in FP32 down to level 1 (rounding ~2^-32 of level 0's
                         // scale), level 0 added with TwoSum, the pair summed over the chunks in FP64
                         auto lv = [&](int l) { return make_float2(__uint_as_float(r[l][e]), __uint_as_float(r[l][e + 1])); };
@@ -432,8 +434,8 @@ __global__ void __launch_bounds__(128 * PARTS + 64, 3 - SETS) tc_gemm_kernel(con
                         const float2 b0 = __ffma2_rn(l0, m1, h);
                         const float2 lo = __fadd2_rn(__ffma2_rn(__ffma2_rn(b0, m1, h), m1, l0), __ffma2_rn(b0, m1, tl));
                         const int2 ebv = *reinterpret_cast<const int2 *>(ebc + cc + e);
-                        acc[cg * 4 + e] += chunk_value(h.x, lo.x, ea + ebv.x);
-                        acc[cg * 4 + e + 1] += chunk_value(h.y, lo.y, ea + ebv.y);
+                        acc[cg * GW + e] += chunk_value(h.x, lo.x, ea + ebv.x);
+                        acc[cg * GW + e + 1] += chunk_value(h.y, lo.y, ea + ebv.y);
                     }
                 }
                 tc::tc_fence_before();   // TMEM reads before a later chunk's MMAs overwrite them
